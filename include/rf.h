@@ -82,11 +82,13 @@ typedef enum rf_precision {
 } rf_precision;
 
 /* Arithmetic of the closures (Eq. 2-4).  AUTO: FP64 on the RF_PREC_FP64
- * path, double-float on the RF_PREC_MIXED path.  FP64: CUDA's FP64 log and
- * exp.  DOUBLE_FLOAT: pairs of FP32 values (about 48 significant bits: theta*
- * within 1.2e-14 relative, K and C within 2.4e-13), several times faster on
- * GB300, whose FP64 pipe is narrow.  Storage, the chord difference, the
- * operator, the Picard test and the balance are FP64 either way. */
+ * path, double-float on the RF_PREC_MIXED path.  FP64: full FP64 accuracy
+ * (within a few units of the last place), computed in 64-bit fixed point
+ * where the state is in its range (|log2(-alpha h)| < 30, |n log2(-alpha h)|
+ * < 60, n < 16) and in FP64 elsewhere.  DOUBLE_FLOAT: pairs of FP32 values
+ * (about 48 significant bits: theta* within 1.2e-14 relative, K and C within
+ * 2.4e-13).  Storage, the chord difference, the operator, the Picard test and
+ * the balance are FP64 either way. */
 typedef enum rf_closure_arith {
     RF_CLOSURE_AUTO = 0, RF_CLOSURE_FP64 = 1, RF_CLOSURE_DOUBLE_FLOAT = 2
 } rf_closure_arith;

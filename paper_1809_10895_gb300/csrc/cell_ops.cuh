@@ -62,7 +62,8 @@ __device__ __forceinline__ void closure_vg_df(const DevSoil &s, double Ks, doubl
     C = s.cfac * ff_to_d(ff_mul(ys, w));
 }
 
-// The same van Genuchten / Mualem closures (h < 0) in FP64, with the
+// The same van Genuchten / Mualem closures (h < 0) in FP64, for the states
+// outside the fixed-point form's range (fx64.cuh), with the
 // table-driven exp / log of f64m.cuh: with u = -alpha h, L = log u (as a
 // double-double), x = exp(n L), l1 = log1p(x) (double-double):
 //   Se = exp(-m l1), w = 1/(1+x), ys = (x/(1+x))^m = (x/u) Se,
@@ -153,20 +154,13 @@ __device__ __forceinline__ void closure_bc(const DevSoil &s, double Ks, double h
     K = Ks * exp(ls * (2.0 + 3.0 * lam) / lam);
 }
 
-// Closures of one cell at head h: theta*, K, C.  For h >= 0 (tie included)
-// theta* = theta_s + S h, K = Ks, C = S, which makes d(theta*)/dh equal to
-// Eq. 3 on both branches.  fp64 selects FP64 van Genuchten arithmetic
+// Closures of one cell at head h < 0 outside the fixed-point range or of
+// another model or arithmetic.  fp64 selects FP64 van Genuchten arithmetic
 // instead of double-float.  Gardner (Eq. A6, a test model): K = Ks e^(alpha
 // h), theta = theta_r + (theta_s-theta_r) e^(alpha h), in FP64.
-__device__ __forceinline__ void closure(const DevSoil &s, double Ks, double h, const FFTables *__restrict__ tab,
-                                        bool fp64, double &th, double &K, double &C)
+__device__ __forceinline__ void closure_general(const DevSoil &s, double Ks, double h, const FFTables *__restrict__ tab,
+                                                bool fp64, double &th, double &K, double &C)
 {
-    if (h >= 0.0) {
-        th = s.theta_s + s.S * h;
-        K = Ks;
-        C = s.S;
-        return;
-    }
     if (s.model == M_GARDNER) {
         const double dth = s.theta_s - s.theta_r;
         const double e = exp(s.alpha * h);
@@ -181,6 +175,59 @@ __device__ __forceinline__ void closure(const DevSoil &s, double Ks, double h, c
     }
     if (fp64) closure_vg_fp64(s, Ks, h, tab, th, K, C);
     else closure_vg_df(s, Ks, h, tab, th, K, C);
+}
+
+// The same out of line, for the cells that the fixed-point form leaves over.
+struct Closure3 {
+    double th, K, C;
+};
+static __device__ __noinline__ Closure3 closure_rest(const DevSoil *s, double Ks, double h, const FFTables *tab)
+{
+    Closure3 r;
+    closure_general(*s, Ks, h, tab, true, r.th, r.K, r.C);
+    return r;
+}
+
+// Closures of one cell at head h: theta*, K, C.  For h >= 0 (tie included)
+// theta* = theta_s + S h, K = Ks, C = S, which makes d(theta*)/dh equal to
+// Eq. 3 on both branches.  With fp64, van Genuchten cells run in 64-bit fixed
+// point (fx64.cuh; tables fx, global or a shared copy) wherever the state is
+// in its range, and in FP64 elsewhere.
+__device__ __forceinline__ void closure(const DevSoil &s, double Ks, double h, const FFTables *__restrict__ tab,
+                                        const FxTables *__restrict__ fx, bool fp64, double &th, double &K, double &C)
+{
+    const unsigned long long hb = (unsigned long long)__double_as_longlong(h);
+    if (hb <= 0x7ff0000000000000ULL || hb == 0x8000000000000000ULL) {   // h >= 0
+        th = s.theta_s + s.S * h;
+        K = Ks;
+        C = s.S;
+        return;
+    }
+    if (!fp64) {
+        closure_general(s, Ks, h, tab, false, th, K, C);
+        return;
+    }
+    uint64_t se, kr, cr;
+    if (fx_closure_vg(s.fx, hb & 0x7fffffffffffffffULL, fx, se, kr, cr)) {
+        th = fma(s.dth, __longlong_as_double((long long)se), s.theta_r);
+        K = Ks * __longlong_as_double((long long)kr);
+        C = s.cfac * __longlong_as_double((long long)cr);
+        return;
+    }
+    const Closure3 r = closure_rest(&s, Ks, h, tab);
+    th = r.th;
+    K = r.K;
+    C = r.C;
+}
+
+// K at a Dirichlet face's head.  Out of line: the face loops are unrolled and
+// few cells carry such a face.
+static __device__ __noinline__ double closure_face(const DevSoil *s, double Ks, double h, const FFTables *tab,
+                                                   bool fp64)
+{
+    double th, K, C;
+    closure(*s, Ks, h, tab, &tab->fx, fp64, th, K, C);
+    return K;
 }
 
 // Neighbour across face f of cell p = (i,j,k); false when outside the grid.
@@ -292,9 +339,7 @@ __device__ __forceinline__ void assemble_cell(const Grid &g, const DevSoil *__re
             hD = sp.bc_val[f];
         }
         if (type == BC_DIRICHLET) {
-            const DevSoil s = soils[zone[p]];
-            double thD, KD, CD;
-            closure(s, Ks[p], hD, g.tab, g.closure64, thD, KD, CD);
+            const double KD = closure_face(&soils[zone[p]], Ks[p], hD, g.tab, g.closure64);
             const double T = KD * g.wb[f];
             diag += T;
             cb += T;
@@ -340,8 +385,7 @@ __device__ __forceinline__ void boundary_fluxes(const Grid &g, const DevSoil &s,
             hD = sp.bc_val[f];
         }
         if (type == BC_DIRICHLET) {
-            double thD, KD, CD;
-            closure(s, Ksp, hD, g.tab, g.closure64, thD, KD, CD);
+            const double KD = closure_face(&s, Ksp, hD, g.tab, g.closure64);
             const double T = KD * g.wb[f];
             flux = T * hD + gs * KD * g.A[f] - T * xp;
         } else if (type == BC_FLUX) {

@@ -12,14 +12,76 @@
 
 namespace rf {
 
-// Closures of every cell at h; with hprev, also max|h - hprev| and a
-// non-finite flag in v[0], v[1].
+// Largest |h - hprev| of a block's cells and whether one was not finite, as
+// the bits of a non-negative double (order as integers: no FP64 compares).
+struct MaxDh {
+    unsigned long long d;
+    int bad;
+};
+
+// Grid maximum of the blocks' values; true in the last block, whose thread 0
+// then holds the result.
+__device__ __forceinline__ bool grid_max_dh(MaxDh &m, double *partials, unsigned int *ticket)
+{
+    __shared__ unsigned long long sd[RED_THREADS / 32];
+    __shared__ int sb;
+    __shared__ bool am_last;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    auto block = [&]() {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long v = __shfl_xor_sync(0xffffffffu, m.d, o);
+            m.d = v > m.d ? v : m.d;
+        }
+        if (lane == 0) sd[wid] = m.d;
+        m.bad = __syncthreads_or(m.bad);
+        if (threadIdx.x == 0)
+            for (int w = 1; w < RED_THREADS / 32; w++) m.d = sd[w] > m.d ? sd[w] : m.d;
+        __syncthreads();
+    };
+    block();
+    unsigned long long *part = reinterpret_cast<unsigned long long *>(partials);
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = m.d;
+        part[gridDim.x + blockIdx.x] = (unsigned long long)m.bad;
+        __threadfence();
+        am_last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;   // wraps to 0 for the next use
+    }
+    __syncthreads();
+    if (!am_last) return false;
+    __threadfence();
+    m.d = 0;
+    m.bad = 0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += RED_THREADS) {
+        const unsigned long long v = __ldcg(&part[b]);
+        m.d = v > m.d ? v : m.d;
+        m.bad |= __ldcg(&part[gridDim.x + b]) != 0;
+    }
+    block();
+    return true;
+}
+
+// Closures of every cell at h; with hprev, also max|h - hprev| and whether
+// an update was not finite.  In FP64 (table-driven exp and log, 106 FP64
+// instructions a cell) the kernel was bound by the FP64 pipe; in fixed point
+// it is bound by the integer pipes.  512 x 512 x 64 watershed, 12.6 M active
+// cells: 3288 -> 446 us (1.5 TB/s of its 651 MB); 1 M cells: 34 us.  The
+// tables (10 KB) sit in shared memory, where a gather costs its bank
+// conflicts only.
 __device__ __forceinline__ void closure_cells(const Grid &g, const DevSoil *__restrict__ soils,
                                               const uint8_t *__restrict__ zone, const double *__restrict__ Ks,
                                               const uint8_t *__restrict__ flags, const double *__restrict__ h,
                                               const double *__restrict__ hprev, double *__restrict__ theta,
-                                              double *__restrict__ K, double *__restrict__ Can, double (&v)[2])
+                                              double *__restrict__ K, double *__restrict__ Can, MaxDh &m)
 {
+    __shared__ FxTables fx;
+    {
+        const uint64_t *src = reinterpret_cast<const uint64_t *>(&g.tab->fx);
+        uint64_t *dst = reinterpret_cast<uint64_t *>(&fx);
+        for (int i = threadIdx.x; i < (int)(sizeof(FxTables) / 8); i += blockDim.x) dst[i] = src[i];
+    }
+    __syncthreads();
+    m = MaxDh{0, 0};
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < g.N; p += stride) {
         if (!(flags[p] & FLAG_ACTIVE)) {
@@ -30,13 +92,12 @@ __device__ __forceinline__ void closure_cells(const Grid &g, const DevSoil *__re
         }
         const double hp = h[p];
         if (hprev) {
-            const double d = fabs(hp - hprev[p]);
-            if (d <= 1e300) v[0] = fmax(v[0], d);
-            else v[1] = 1.0;           // NaN or inf
+            const unsigned long long d = (unsigned long long)__double_as_longlong(hp - hprev[p]) & 0x7fffffffffffffffULL;
+            if (d <= 0x7e37e43c8800759cULL) m.d = d > m.d ? d : m.d;   // 1e300
+            else m.bad = 1;                                            // NaN or inf
         }
-        const DevSoil s = soils[zone[p]];
         double th, k, c;
-        closure(s, Ks[p], hp, g.tab, g.closure64, th, k, c);
+        closure(soils[zone[p]], Ks[p], hp, g.tab, &fx, g.closure64, th, k, c);
         theta[p] = th;
         K[p] = k;
         Can[p] = c;
@@ -51,12 +112,12 @@ k_closure(Grid g, const DevSoil *__restrict__ soils, const uint8_t *__restrict__
 {
     count_launch(g, KK_CLOSURE);
     count_work(g, KK_CLOSURE);
-    double v[2] = {0.0, 0.0};   // max |h - hprev|, non-finite flag
-    closure_cells(g, soils, zone, Ks, flags, h, hprev, theta, K, Can, v);
+    MaxDh m;
+    closure_cells(g, soils, zone, Ks, flags, h, hprev, theta, K, Can, m);
     if (hprev) {
-        if (grid_reduce<OpMax, 2>(v, partials, ticket) && threadIdx.x == 0) {
-            res->max_dh = v[0];
-            res->nonfinite = v[1] > 0.0;
+        if (grid_max_dh(m, partials, ticket) && threadIdx.x == 0) {
+            res->max_dh = __longlong_as_double((long long)m.d);
+            res->nonfinite = m.bad;
         }
     }
 }
@@ -80,17 +141,18 @@ k_closure_picard(Grid g, const DevSoil *__restrict__ soils, const uint8_t *__res
         return;
     }
     count_work(g, KK_CLOSURE_PICARD);
-    double v[2] = {0.0, 0.0};
-    closure_cells(g, soils, zone, Ks, flags, x, hk, theta, K, Can, v);
-    if (grid_reduce<OpMax, 2>(v, partials, ticket) && threadIdx.x == 0) {
+    MaxDh m;
+    closure_cells(g, soils, zone, Ks, flags, x, hk, theta, K, Can, m);
+    if (grid_max_dh(m, partials, ticket) && threadIdx.x == 0) {
+        const double max_dh = __longlong_as_double((long long)m.d);
         const int it = ++ctl->it;
         if (cg_status->status != CG_OK) {
             ctl->fail = 1;
         } else {
             ctl->cg_total += cg_count->total;
-            ctl->max_dh = v[0];
-            if (v[1] > 0.0) ctl->fail = 1;
-            else if (v[0] <= ctl->tol) {
+            ctl->max_dh = max_dh;
+            if (m.bad) ctl->fail = 1;
+            else if (max_dh <= ctl->tol) {
                 ctl->conv = 1;
                 ctl->mb_pending = 1;
             }
@@ -340,7 +402,7 @@ void launch_state_check_commit(cudaStream_t s, int nblk, const Grid &g, const ui
 // Both precisions' tables: the double-float ones from double arithmetic,
 // the FP64 ones from long double (extended or quadruple precision on the
 // hosts this builds for), each rounded once.
-void make_ff_tables(FFTables *t)
+static void fill_ff_tables(FFTables *t)
 {
     for (int j = 0; j < F64_TAB; j++) {
         const long double e = exp2l((long double)j / (long double)F64_TAB);
@@ -354,6 +416,12 @@ void make_ff_tables(FFTables *t)
         t->lF[j] = make_double2(hi, (double)(lf - (long double)hi));
         t->invF[j] = (double)(1.0L / F);
     }
+    for (int j = 0; j < FX_TAB; j++) {
+        const long double F = 1.0L + (long double)j / (long double)FX_TAB;
+        t->fx.rc[j] = (uint32_t)ceill(2147483648.0L / F);   // rounded up, so that r >= 0
+        t->fx.lg[j] = (uint64_t)rintl(-log2l((long double)t->fx.rc[j] / 2147483648.0L) * 9223372036854775808.0L);
+        t->fx.e2[j] = (uint64_t)rintl(exp2l((long double)j / (long double)FX_TAB) * 9223372036854775808.0L);
+    }
     for (int j = 0; j < 64; j++) {
         const double e = exp2((double)j / 64.0);
         const double c = 1.0 + ((double)j + 0.5) / 64.0;
@@ -363,6 +431,33 @@ void make_ff_tables(FFTables *t)
         t->logc[j] = make_float2(lh, (float)(lc - (double)lh));
         t->invc[j] = make_float2(ih, (float)(ic - (double)ih));
     }
+}
+
+// Constants, computed once per process (quadruple-precision logarithms on a
+// host whose long double is software cost most of a millisecond).
+const FFTables *ff_tables()
+{
+    static FFTables t;
+    static const bool filled = (fill_ff_tables(&t), true);
+    (void)filled;
+    return &t;
+}
+
+FxSoil make_fx_soil(int model, double alpha, double n, double m)
+{
+    FxSoil f{};
+    const long double la = log2l((long double)alpha);
+    // sizes for which every field fits its format; others keep the general closure
+    f.ok = (model == M_VG && n > 1.0 && n < 16.0 && m > 0.0 && la > -20.0L && la < 20.0L) ? 1 : 0;
+    if (!f.ok) return f;
+    f.ne = ilogb(n);
+    f.ea = ilogb(alpha);
+    f.la = (int64_t)rintl(la * 288230376151711744.0L);                          // 2^58
+    f.nm = (uint64_t)ldexpl((long double)n, 63 - f.ne);
+    f.m = (uint64_t)rintl((long double)m * 18446744073709551616.0L);            // 2^64
+    const long double Lm = 60.0L / (long double)n;
+    f.Lmax = (uint64_t)((Lm < 31.5L ? Lm : 31.5L) * 288230376151711744.0L);
+    return f;
 }
 
 void launch_closure(cudaStream_t s, int nblk, const Grid &g, const DevSoil *soils, const uint8_t *zone,

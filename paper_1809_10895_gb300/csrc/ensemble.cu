@@ -688,7 +688,7 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                     else v[1] = 1.0;
                 }
                 double th, k, c;
-                closure(*soil, Ks[p], hp, g.tab, g.closure64, th, k, c);
+                closure(*soil, Ks[p], hp, g.tab, &g.tab->fx, g.closure64, th, k, c);
                 thx[p] = th;
                 Kx[p] = k;
                 Can[p] = c;

@@ -255,8 +255,6 @@ rf_status rf_ens_create(const rf_ens_instance *inst, int n, const rf_solver_para
         return efail(RF_ERR_NOMEM, "rf_ens_create: allocation failed");
     }
 
-    FFTables tab;
-    make_ff_tables(&tab);
     std::vector<uint8_t> flags(N), zone(N, 0);
     std::vector<double> Ks(N);
     e->h0.assign(N, 0.0);
@@ -292,7 +290,8 @@ rf_status rf_ens_create(const rf_ens_instance *inst, int n, const rf_solver_para
         const double m = s.model == RF_VG ? 1.0 - 1.0 / s.n : 0.0;
         const float nh = (float)s.n, mh = (float)m;
         d.soil = DevSoil{s.model, s.theta_r, s.theta_s, s.alpha, s.n, m, s.S, nh, (float)(s.n - (double)nh), mh,
-                         (float)(m - (double)mh), (s.theta_s - s.theta_r) * s.alpha * s.n * m};
+                         (float)(m - (double)mh), (s.theta_s - s.theta_r) * s.alpha * s.n * m,
+                         s.theta_s - s.theta_r, make_fx_soil(s.model, s.alpha, s.n, m)};
         for (int f = 0; f < 6; f++) { d.sp.bc_type[f] = BC_ZERO_FLUX; d.sp.bc_val[f] = 0.0; }
         d.sp.bc_type[F_ZMAX] = a.top_type;
         d.sp.bc_val[F_ZMAX] = a.top_value;
@@ -338,7 +337,7 @@ rf_status rf_ens_create(const rf_ens_instance *inst, int n, const rf_solver_para
     P.outer_max_it = prm.outer_max_it;
     P.zline = prm.precond == RF_PRECOND_ZLINE;
     P.step_budget = 10000000;
-    cudaError_t err = cudaMemcpyAsync(e->tab, &tab, sizeof(FFTables), cudaMemcpyHostToDevice, e->stream);
+    cudaError_t err = cudaMemcpyAsync(e->tab, ff_tables(), sizeof(FFTables), cudaMemcpyHostToDevice, e->stream);
     if (err == cudaSuccess) err = cudaMemcpyAsync(e->B.flags, flags.data(), N, cudaMemcpyHostToDevice, e->stream);
     if (err == cudaSuccess) err = cudaMemcpyAsync(e->B.zone, zone.data(), N, cudaMemcpyHostToDevice, e->stream);
     if (err == cudaSuccess) err = cudaMemcpyAsync(e->B.Ks, Ks.data(), sizeof(double) * N, cudaMemcpyHostToDevice, e->stream);

@@ -1,5 +1,6 @@
-// f64m.cuh -- FP64 exp, log, log1p and expm1 for the closures of the plain
-// FP64 path, by table-driven argument reduction.
+// f64m.cuh -- FP64 exp, log, log1p and expm1, by table-driven argument
+// reduction, for FP64 closures of states outside the range of the
+// fixed-point form (fx64.cuh).
 //
 // Method: P. T. P. Tang, "Table-driven implementation of the exponential
 // function in IEEE floating-point arithmetic", ACM TOMS 15 (1989) 144-157,

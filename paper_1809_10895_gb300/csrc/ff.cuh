@@ -17,13 +17,15 @@
 
 #include <cuda_runtime.h>
 
+#include "fx64.cuh"
+
 namespace rf {
 
 struct ff {
     float hi, lo;
 };
 
-// 64-entry tables, filled on the host (see make_ff_tables).
+// 64-entry tables, filled on the host (see ff_tables).
 // Entries of the FP64 argument-reduction tables (f64m.cuh).
 constexpr int F64_TAB_BITS = 10;
 constexpr int F64_TAB = 1 << F64_TAB_BITS;
@@ -39,6 +41,7 @@ struct FFTables {
     double2 e2[F64_TAB];
     double2 lF[F64_TAB + 1];
     double invF[F64_TAB + 1];
+    FxTables fx;        // fixed-point tables (fx64.cuh)
 };
 
 #ifdef __CUDACC__
@@ -201,6 +204,6 @@ __device__ __forceinline__ ff ff_log(ff a, const FFTables *__restrict__ tab)
 #endif
 
 // Host: fill the tables from double-precision libm values.
-void make_ff_tables(FFTables *t);
+const FFTables *ff_tables();
 
 }  // namespace rf

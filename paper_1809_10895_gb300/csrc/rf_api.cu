@@ -1035,10 +1035,8 @@ rf_status rf_mesh_create(const rf_mesh_desc *mesh, const rf_solver_params *param
     }
     g.ctr = c->ctr;
     g.tab = c->fftab;
-    FFTables tab;
-    make_ff_tables(&tab);
     cudaError_t e = cudaMemcpyAsync(c->flags, c->flags_h.data(), N, cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c->fftab, &tab, sizeof(FFTables), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(c->fftab, ff_tables(), sizeof(FFTables), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ticket, 0, 64 * sizeof(unsigned int), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ctr, 0, 2 * KK_COUNT * sizeof(unsigned long long), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ctl, 0, sizeof(PicardCtl), c->stream);
@@ -1114,7 +1112,8 @@ rf_status rf_soil_set(rf_ctx *c, const rf_soil *zones, int n_zones, const uint8_
         const float nh = (float)s.n, mh = (float)m;
         soils[z] = DevSoil{s.model, s.theta_r, s.theta_s, s.alpha, s.n, m, s.S,
                            nh, (float)(s.n - (double)nh), mh, (float)(m - (double)mh),
-                           (s.theta_s - s.theta_r) * s.alpha * s.n * m};
+                           (s.theta_s - s.theta_r) * s.alpha * s.n * m, s.theta_s - s.theta_r,
+                           make_fx_soil(s.model, s.alpha, s.n, m)};
     }
     const long long N = c->g.N;
     std::vector<uint8_t> zone(N, 0);

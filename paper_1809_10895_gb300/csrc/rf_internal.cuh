@@ -65,6 +65,8 @@ struct DevSoil {
     double theta_r, theta_s, alpha, n, m, S;
     float n_hi, n_lo, m_hi, m_lo;   // n and m as double-float pairs
     double cfac;                    // ((theta_s - theta_r) alpha) n m, the factor of C (Eq. 3)
+    double dth;                     // theta_s - theta_r
+    FxSoil fx;                      // fixed-point copies (van Genuchten)
 };
 
 struct Grid {
@@ -266,6 +268,9 @@ __device__ __forceinline__ void outer_residual_scalars(CgScal *outer, CgScal *in
 
 // Message returned by rf_last_error() on the calling thread.
 void set_last_error(const char *msg);
+
+// Fixed-point copies of a soil's alpha, n and m (closure_assemble.cu).
+FxSoil make_fx_soil(int model, double alpha, double n, double m);
 
 // ---- launch entry points implemented in the .cu files --------------------
 void launch_closure(cudaStream_t s, int nblk, const Grid &g, const DevSoil *soils, const uint8_t *zone,
