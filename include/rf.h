@@ -82,7 +82,7 @@ typedef enum rf_precision {
 } rf_precision;
 
 /* Arithmetic of the closures (Eq. 2-4).  AUTO: FP64 on the RF_PREC_FP64
- * path, double-float on the RF_PREC_MIXED path.  FP64: full FP64 accuracy
+ * and the RF_PREC_MIXED path.  FP64: full FP64 accuracy
  * (within a few units of the last place), computed in 64-bit fixed point
  * where the state is in its range (|log2(-alpha h)| < 30, |n log2(-alpha h)|
  * < 60, n < 16) and in FP64 elsewhere.  DOUBLE_FLOAT: pairs of FP32 values

@@ -279,8 +279,7 @@ rf_status rf_ens_create(const rf_ens_instance *inst, int n, const rf_solver_para
             g.hg[f] = 0.5 * A[f] * g.gf[f];
         }
         // closures in FP64 on the plain path, double-float inside the mixed one (AUTO)
-        g.closure64 = (prm.closure_arith == RF_CLOSURE_FP64 ||
-                       (prm.closure_arith == RF_CLOSURE_AUTO && prm.precision == RF_PREC_FP64)) ? 1 : 0;
+        g.closure64 = prm.closure_arith != RF_CLOSURE_DOUBLE_FLOAT ? 1 : 0;
         for (int ax = 0; ax < 3; ax++) g.w32[ax] = (float)(A[2 * ax] / dd[2 * ax]);
         g.fx = make_fastdiv((unsigned int)a.nx);
         g.fxy = make_fastdiv((unsigned int)g.sxy);

@@ -83,7 +83,7 @@ struct Grid {
     float w32[3];     // A/d per axis, FP32 (mixed-precision operator)
     FastDiv fx, fxy;  // division by nx and by nx*ny
     int cap;          // most blocks a tiled stencil kernel launches (partials hold 8 values per block)
-    int closure64;    // 1: closures in FP64 (CUDA's FP64 log / exp); 0: double-float arithmetic
+    int closure64;    // 1: closures to FP64 accuracy (fixed point, else FP64); 0: double-float arithmetic
     int tilted;       // 1: the elevation gradient has x / y components (gravity on lateral faces)
     int harmonic;     // 1: harmonic interface conductivity; 0: arithmetic mean (linear interpolation)
     int wait_tries;   // polls of a bounded device wait before it gives up (set for tests; 0: default)
