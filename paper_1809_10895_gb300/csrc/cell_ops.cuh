@@ -261,6 +261,34 @@ __device__ __forceinline__ double apply64(const Grid &g, long long p, const doub
     return acc;
 }
 
+// Terms of boundary face f of cell p: diagonal (diag, cb) and right side.
+__device__ __forceinline__ void boundary_face(const Grid &g, const DevSoil *__restrict__ soils,
+                                              const uint8_t *__restrict__ zone, const double *__restrict__ Ks,
+                                              const StepParams &sp, long long p, int f, double hnP, double KP,
+                                              double &diag, double &cb, double &rhs)
+{
+    const double gs = g.gf[f];
+    int type = sp.bc_type[f];
+    double hD = 0.0;
+    if (type == BC_SEEPAGE) {
+        if (hnP >= 0.0) { type = BC_DIRICHLET; hD = 0.0; }
+        else type = BC_ZERO_FLUX;
+    } else if (type == BC_DIRICHLET) {
+        hD = sp.bc_val[f];
+    }
+    if (type == BC_DIRICHLET) {
+        const double KD = closure_face(&soils[zone[p]], Ks[p], hD, g.tab, g.closure64);
+        const double T = KD * g.wb[f];
+        diag += T;
+        cb += T;
+        rhs += T * hD + gs * KD * g.A[f];
+    } else if (type == BC_FLUX) {
+        rhs += sp.bc_val[f] * g.A[f];
+    } else if (type == BC_FREE_DRAINAGE) {
+        rhs += gs * KP * g.A[f];       // unit gradient: gravity outflow K(h^k) A (gs = -1 at a z-up bottom)
+    }
+}
+
 // One cell of the Picard system (Sec. 2.2; see k_assemble):
 //   c = V C^k / dt (chord slope of theta*, or C(h^k) when |h^k - h^n| <= eps),
 //   interior faces T_f = Kbar_f A_f/d_f with Kbar_f = (K_P + K_N)/2 (or the
@@ -328,27 +356,8 @@ __device__ __forceinline__ void assemble_cell(const Grid &g, const DevSoil *__re
                 continue;
             }
         }
-        const double gs = g.gf[f];
         if (!(fl & (1u << f))) continue;    // closed face (lateral face on an inactive cell)
-        int type = sp.bc_type[f];
-        double hD = 0.0;
-        if (type == BC_SEEPAGE) {
-            if (hnP >= 0.0) { type = BC_DIRICHLET; hD = 0.0; }
-            else type = BC_ZERO_FLUX;
-        } else if (type == BC_DIRICHLET) {
-            hD = sp.bc_val[f];
-        }
-        if (type == BC_DIRICHLET) {
-            const double KD = closure_face(&soils[zone[p]], Ks[p], hD, g.tab, g.closure64);
-            const double T = KD * g.wb[f];
-            diag += T;
-            cb += T;
-            rhs += T * hD + gs * KD * g.A[f];
-        } else if (type == BC_FLUX) {
-            rhs += sp.bc_val[f] * g.A[f];
-        } else if (type == BC_FREE_DRAINAGE) {
-            rhs += gs * KP * g.A[f];       // unit gradient: gravity outflow K(h^k) A (gs = -1 at a z-up bottom)
-        }
+        boundary_face(g, soils, zone, Ks, sp, p, f, hnP, KP, diag, cb, rhs);
     }
     out.c = c;
     out.s0 = s0;

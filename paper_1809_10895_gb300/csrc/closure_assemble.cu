@@ -7,8 +7,10 @@
 #include <math.h>
 
 #include "cell_ops.cuh"
+#include "ix64.cuh"
 #include "rf_internal.cuh"
 #include "rf_reduce.cuh"
+#include "tiles.cuh"
 
 namespace rf {
 
@@ -173,6 +175,66 @@ k_closure_picard(Grid g, const DevSoil *__restrict__ soils, const uint8_t *__res
 // interior face), diag(A), 1/diag; FP32 copies of K (NaN on inactive cells,
 // so that max(w (K_P + K_N), 0) closes their faces without a test) and of c
 // plus the Dirichlet diagonal terms for the mixed-precision operator.
+// The Picard attempt is over (skip set): the linear-solve loops that follow
+// are empty.
+template <int MODE>
+__device__ __forceinline__ bool assemble_skipped(const int *skip, const SolveStart &st)
+{
+    if (!(skip && *skip)) return false;
+    if (MODE != ASM_ONLY && blockIdx.x == 0 && threadIdx.x == 0) {
+        st.sc->done = 1;
+        set_cond(st.cond, 0);
+        if (MODE == ASM_MIXED) {
+            st.inner->done = 1;
+            set_cond(st.cond_inner, 0);
+        }
+    }
+    return true;
+}
+
+// Outputs of an inactive cell (hkP: its raw h^k, kept in x).
+template <int MODE>
+__device__ __forceinline__ void assemble_inactive(long long p, double *__restrict__ c_out, double *__restrict__ b,
+                                                  double *__restrict__ Tx, double *__restrict__ Ty,
+                                                  double *__restrict__ Tz, double *__restrict__ diag_out,
+                                                  double *__restrict__ dinv, float *__restrict__ K32,
+                                                  float *__restrict__ cb32, float *__restrict__ dinv32, double hkP,
+                                                  const SolveStart &st)
+{
+    c_out[p] = 0.0; b[p] = 0.0; Tx[p] = 0.0; Ty[p] = 0.0; Tz[p] = 0.0;
+    diag_out[p] = 0.0; dinv[p] = 0.0;
+    K32[p] = __int_as_float(0x7fc00000); cb32[p] = 0.0f; dinv32[p] = 0.0f;   // NaN: fails every K >= 0 test
+    if (MODE != ASM_ONLY) st.x[p] = hkP;
+    if (MODE == ASM_CG64) { st.r[p] = 0.0; st.z[p] = 0.0; }
+    if (MODE == ASM_MIXED) { st.r32[p] = 0.0f; st.z32[p] = 0.0f; st.d32[p] = 0.0f; }
+}
+
+// Start scalars of the linear solve from the reduced norms (v: r.z, r.r, b.b
+// in FP64; a_*: the FP32 seeds').
+template <int MODE>
+__device__ __forceinline__ void assemble_finish(double (&v)[3], float a_rr, float a_bb, float a_rz,
+                                                const SolveStart &st, double *partials, unsigned int *ticket)
+{
+    if (MODE == ASM_CG64) {
+        if (grid_reduce<OpSum, 3>(v, partials, ticket) && threadIdx.x == 0)
+            cg64_start_scalars(st.sc, v, st.tol, st.max_it, st.cond);
+    } else if (MODE == ASM_MIXED) {
+        // the residual is formed in FP64; its norms (a stopping test and CG
+        // seeds) are summed in FP32 within a block, in FP64 across blocks
+        float vf[3] = {a_rr, a_bb, a_rz};
+        double w[3];
+        if (grid_reduce_f32<3>(vf, w, partials, ticket) && threadIdx.x == 0) {
+            const double u[4] = {w[0], w[1], w[0], w[2]};
+            st.sc->iter = 1;
+            st.sc->done = 0;
+            st.sc->status = CG_OK;
+            st.inner->total = 0;
+            outer_residual_scalars(st.sc, st.inner, u, st.tol, st.tol_inner, st.inner_max_it, st.outer_max_it,
+                                   st.cond, st.cond_inner);
+        }
+    }
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(RED_THREADS)
 k_assemble(Grid g, const DevSoil *__restrict__ soils, const uint8_t *__restrict__ zone,
@@ -186,33 +248,17 @@ k_assemble(Grid g, const DevSoil *__restrict__ soils, const uint8_t *__restrict_
            const double *__restrict__ thp)
 {
     count_launch(g, KK_ASSEMBLE);
-    if (skip && *skip) {
-        if (MODE != ASM_ONLY && blockIdx.x == 0 && threadIdx.x == 0) {
-            // the Picard attempt is over: the linear-solve loops that follow are empty
-            st.sc->done = 1;
-            set_cond(st.cond, 0);
-            if (MODE == ASM_MIXED) {
-                st.inner->done = 1;
-                set_cond(st.cond_inner, 0);
-            }
-        }
-        return;
-    }
+    if (assemble_skipped<MODE>(skip, st)) return;
     count_work(g, KK_ASSEMBLE);
     const double eps = spp->eps_chord;
-    const double V_dt = g.V / spp->dt;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    const double V_dt = spp->V_dt;
+    double v[3] = {0.0, 0.0, 0.0};
     float a_rr = 0.0f, a_bb = 0.0f, a_rz = 0.0f;   // mixed start: norms of the FP32 seeds, summed in FP32
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < g.N; p += stride) {
         const uint8_t fl = flags[p];
         if (!(fl & FLAG_ACTIVE)) {
-            c_out[p] = 0.0; b[p] = 0.0; Tx[p] = 0.0; Ty[p] = 0.0; Tz[p] = 0.0;
-            diag_out[p] = 0.0; dinv[p] = 0.0;
-            K32[p] = __int_as_float(0x7fc00000); cb32[p] = 0.0f; dinv32[p] = 0.0f;   // NaN: fails every K >= 0 test
-            if (MODE != ASM_ONLY) st.x[p] = hk[p];
-            if (MODE == ASM_CG64) { st.r[p] = 0.0; st.z[p] = 0.0; }
-            if (MODE == ASM_MIXED) { st.r32[p] = 0.0f; st.z32[p] = 0.0f; st.d32[p] = 0.0f; }
+            assemble_inactive<MODE>(p, c_out, b, Tx, Ty, Tz, diag_out, dinv, K32, cb32, dinv32, hk[p], st);
             continue;
         }
         int i, j, k;
@@ -269,28 +315,245 @@ k_assemble(Grid g, const DevSoil *__restrict__ soils, const uint8_t *__restrict_
             }
         }
     }
-    if (MODE == ASM_CG64) {
-        double w3[3] = {v[0], v[1], v[2]};
-        if (grid_reduce<OpSum, 3>(w3, partials, ticket) && threadIdx.x == 0)
-            cg64_start_scalars(st.sc, w3, st.tol, st.max_it, st.cond);
-    } else if (MODE == ASM_MIXED) {
-        // the residual is formed in FP64; its norms (a stopping test and CG
-        // seeds) are summed in FP32 within a block, in FP64 across blocks
-        float vf[3] = {a_rr, a_bb, a_rz};
-        double w[3];
-        if (grid_reduce_f32<3>(vf, w, partials, ticket) && threadIdx.x == 0) {
-            v[0] = w[0];
-            v[1] = w[1];
-            v[2] = w[0];
-            v[3] = w[2];
-            st.sc->iter = 1;
-            st.sc->done = 0;
-            st.sc->status = CG_OK;
-            st.inner->total = 0;
-            outer_residual_scalars(st.sc, st.inner, v, st.tol, st.tol_inner, st.inner_max_it, st.outer_max_it,
-                                   st.cond, st.cond_inner);
+    assemble_finish<MODE>(v, a_rr, a_bb, a_rz, st, partials, ticket);
+}
+
+// The same assembly for grids that fill the GPU with 32 x 8 column tiles: a
+// block walks its tile's planes upwards, K and h^k of a plane (with a one-cell
+// halo) in shared memory, those of the planes below and above in registers,
+// everything else loaded a plane ahead.  The face coefficients
+// T = (K_P + K_N) hw, their sum and the two reciprocals are positive, so they
+// run in integer arithmetic (ix64.cuh) beside the narrow FP64 pipe, which
+// bounds the kernel; the top face of a plane is the bottom face of the next.
+// FP64 keeps the signed work: about 19 instructions a cell instead of 50.
+// 512 x 512 x 64 watershed (12.6 M active cells): 1105 us with one cell per
+// thread and all of it in FP64, 719 us here; 128 x 128 x 64 box 101 -> 68 us.
+template <int MODE>
+__global__ void __launch_bounds__(RED_THREADS, 2)
+k_assemble_tiled(Grid g, Tiles tw, const DevSoil *__restrict__ soils, const uint8_t *__restrict__ zone,
+                 const double *__restrict__ Ks, const uint8_t *__restrict__ flags,
+                 const StepParams *__restrict__ spp, const double *__restrict__ hk, const double *__restrict__ hn,
+                 const double *__restrict__ thk, const double *__restrict__ thn, const double *__restrict__ K,
+                 const double *__restrict__ Can, double *__restrict__ c_out, double *__restrict__ b,
+                 double *__restrict__ Tx, double *__restrict__ Ty, double *__restrict__ Tz,
+                 double *__restrict__ diag_out, double *__restrict__ dinv, float *__restrict__ K32,
+                 float *__restrict__ cb32, float *__restrict__ dinv32, const int *skip, SolveStart st,
+                 double *partials, unsigned int *ticket, double *__restrict__ s0_out,
+                 const double *__restrict__ thp)
+{
+    count_launch(g, KK_ASSEMBLE);
+    if (assemble_skipped<MODE>(skip, st)) return;
+    count_work(g, KK_ASSEMBLE);
+    __shared__ long long sK[2][TY + 2][TX + 2];
+    __shared__ double sH[2][TY + 2][TX + 2];
+    constexpr long long CLOSED = (long long)0xbff0000000000000ULL;   // K = -1
+    const double eps = spp->eps_chord, V_dt = spp->V_dt;
+    const bool mixed_form = spp->modified || spp->bdf2;
+    const bool Vok = (unsigned)(__double_as_longlong(V_dt) >> 52) - 700u < 650u;   // products stay in the normal range
+    const IxNum hwx = ix_unpack(__double_as_longlong(g.hw[0])), hwy = ix_unpack(__double_as_longlong(g.hw[2]));
+    const IxNum hwz = ix_unpack(__double_as_longlong(g.hw[4])), ixV = ix_unpack(__double_as_longlong(V_dt));
+    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+    int hx = 0, hy = 0;
+    if (threadIdx.x < HALO) halo_cell(threadIdx.x, hx, hy);
+    double v[3] = {0.0, 0.0, 0.0};
+    float a_rr = 0.0f, a_bb = 0.0f, a_rz = 0.0f;   // mixed start: norms of the FP32 seeds, summed in FP32
+    // T of the face between cells with K bits a and b (sign set: closed)
+    auto face = [&](long long a, long long bb, const IxNum &hw, double hwd) -> double {
+        if ((a | bb) < 0) return 0.0;
+        if (!g.harmonic && (unsigned)(a >> 52) - 400u < 1200u && (unsigned)(bb >> 52) - 400u < 1200u)
+            return __longlong_as_double((long long)ix_pack(ix_add_mul(ix_unpack(a), ix_unpack(bb), hw)));
+        const double x = __longlong_as_double(a), y = __longlong_as_double(bb);
+        double s = x + y;
+        if (g.harmonic) s = s > 0.0 ? 4.0 * x * y / s : 0.0;
+        return s * hwd;
+    };
+    struct Pl {
+        double hn, thk, thn, can;
+        uint8_t fl;
+    };
+    for (long long item = blockIdx.x; item < tw.items; item += gridDim.x) {
+        const TileItem it = tile_item(g, tw, item);
+        const int i = it.i0 + tx, j = it.j0 + ty;
+        const bool inside = i < g.nx && j < g.ny;
+        const long long col = i + (long long)g.nx * j;
+        const bool halo = threadIdx.x < HALO && it.i0 + hx >= 0 && it.i0 + hx < g.nx && it.j0 + hy >= 0 &&
+                          it.j0 + hy < g.ny;
+        const long long hcol = (it.i0 + hx) + (long long)g.nx * (it.j0 + hy);
+        auto ldK = [&](int k) -> long long {
+            return inside && k >= 0 && k < g.nz ? __double_as_longlong(K[col + g.sxy * k]) : CLOSED;
+        };
+        auto ldh = [&](int k) -> double { return inside && k >= 0 && k < g.nz ? hk[col + g.sxy * k] : 0.0; };
+        auto load = [&](int k, bool act) {
+            Pl l{0.0, 0.0, 0.0, 0.0, 0};
+            if (act) {
+                const long long p = col + g.sxy * k;
+                l.hn = hn[p];
+                l.thk = thk[p];
+                l.thn = thn[p];
+                l.can = Can[p];
+                l.fl = flags[p];
+            }
+            return l;
+        };
+        long long Kc = ldK(it.k0), Kn = ldK(it.k0 + 1), Kh = CLOSED;
+        double hm = 0.0, hc = ldh(it.k0), hu = ldh(it.k0 + 1), hh = 0.0;
+        if (halo) {
+            Kh = __double_as_longlong(K[hcol + g.sxy * it.k0]);
+            hh = hk[hcol + g.sxy * it.k0];
         }
+        Pl nxt = load(it.k0, Kc >= 0);
+        double Tbot = 0.0;
+        if (it.k0 > 0) {
+            const long long Kb = ldK(it.k0 - 1);
+            Tbot = face(Kb, Kc, hwz, g.hw[4]);
+            hm = Kb >= 0 ? ldh(it.k0 - 1) : 0.0;
+        }
+        for (int k = it.k0; k < it.k1; k++) {
+            const int buf = k & 1;
+            const long long p = col + g.sxy * k;
+            const Pl cur = nxt;
+            sK[buf][ty + 1][tx + 1] = Kc;
+            sH[buf][ty + 1][tx + 1] = Kc >= 0 ? hc : 0.0;    // a closed face's head is multiplied by T = 0
+            if (threadIdx.x < HALO) {
+                sK[buf][hy + 1][hx + 1] = Kh;
+                sH[buf][hy + 1][hx + 1] = Kh >= 0 ? hh : 0.0;
+            }
+            long long K2 = CLOSED;
+            double h2 = 0.0;
+            if (k + 1 < it.k1) {
+                K2 = ldK(k + 2);
+                h2 = ldh(k + 2);
+                nxt = load(k + 1, Kn >= 0);
+                if (halo) {
+                    Kh = __double_as_longlong(K[hcol + g.sxy * (k + 1)]);
+                    hh = hk[hcol + g.sxy * (k + 1)];
+                }
+            }
+            __syncthreads();
+            double Ttop = 0.0;
+            if (Kc >= 0) {
+                const double hkP = hc;
+                double c, s0;
+                if (mixed_form) {
+                    if (spp->bdf2) {
+                        c = V_dt * (spp->a0 * cur.can);
+                        s0 = V_dt * (spp->a0 * cur.can * hkP -
+                                     (spp->a0 * cur.thk - spp->a1 * cur.thn + spp->a2 * thp[p]));
+                    } else {
+                        c = V_dt * cur.can;
+                        s0 = c * hkP - V_dt * (cur.thk - cur.thn);
+                    }
+                } else {
+                    const double dh = hkP - cur.hn;
+                    const long long db = __double_as_longlong(dh) & 0x7fffffffffffffffLL;
+                    if (db > __double_as_longlong(eps)) {
+                        // (theta*^k - theta*^n) (V / dt / |dh|), the factor by integer arithmetic
+                        const double dth = cur.thk - cur.thn;
+                        double f;
+                        if (Vok && (unsigned)(db >> 52) - 700u < 650u) {
+                            const IxNum d = ix_unpack((uint64_t)db);
+                            uint64_t q = fx_mulhi(ix_rcp(d.M), ixV.M);
+                            const int up = (int)(q >> 63);
+                            q = up ? q : q << 1;
+                            f = __longlong_as_double((long long)fx_pack(q, ixV.e - d.e - 1 + up));
+                        } else {
+                            f = V_dt / __longlong_as_double(db);
+                        }
+                        c = __longlong_as_double(__double_as_longlong(dth) ^
+                                                 (__double_as_longlong(dh) & (long long)0x8000000000000000ULL)) * f;
+                    } else {
+                        c = V_dt * cur.can;
+                    }
+                    s0 = c * cur.hn;
+                }
+                const long long kxm = sK[buf][ty + 1][tx], kxp = sK[buf][ty + 1][tx + 2];
+                const long long kym = sK[buf][ty][tx + 1], kyp = sK[buf][ty + 2][tx + 1];
+                const double T0 = face(kxm, Kc, hwx, g.hw[0]), T1 = face(Kc, kxp, hwx, g.hw[0]);
+                const double T2 = face(kym, Kc, hwy, g.hw[2]), T3 = face(Kc, kyp, hwy, g.hw[2]);
+                Ttop = face(Kc, Kn, hwz, g.hw[4]);
+                const double hz = Kn >= 0 ? hu : 0.0;
+                double diag = c + (((T0 + T1) + (T2 + T3)) + (Tbot + Ttop));
+                double rhs = fma(Ttop, g.gd[F_ZMAX], fma(Tbot, g.gd[F_ZMIN], s0));   // explicit gravity
+                if (g.tilted) {
+                    rhs = fma(T0, g.gd[F_XMIN], fma(T1, g.gd[F_XMAX], rhs));
+                    rhs = fma(T2, g.gd[F_YMIN], fma(T3, g.gd[F_YMAX], rhs));
+                }
+                double sT = 0.0;
+                if (MODE != ASM_ONLY) {
+                    sT = T0 * sH[buf][ty + 1][tx];
+                    sT = fma(T1, sH[buf][ty + 1][tx + 2], sT);
+                    sT = fma(T2, sH[buf][ty][tx + 1], sT);
+                    sT = fma(T3, sH[buf][ty + 2][tx + 1], sT);
+                    sT = fma(Tbot, hm, sT);
+                    sT = fma(Ttop, hz, sT);
+                }
+                double cb = c;
+                if (cur.fl & 0x3f) {
+                    const double KP = __longlong_as_double(Kc);
+                    for (int f = 0; f < 6; f++)
+                        if (cur.fl & (1u << f))
+                            boundary_face(g, soils, zone, Ks, *spp, p, f, cur.hn, KP, diag, cb, rhs);
+                }
+                c_out[p] = c;
+                b[p] = rhs;
+                if (s0_out) s0_out[p] = s0;
+                Tx[p] = T1;
+                Ty[p] = T3;
+                Tz[p] = Ttop;
+                const long long gb = __double_as_longlong(diag);
+                double di = 0.0;
+                float di32;
+                if (MODE == ASM_MIXED) {
+                    di32 = __frcp_rn(ix_d2f(diag));
+                } else {
+                    if ((unsigned)(gb >> 52) - 400u < 1200u) {
+                        const IxNum d = ix_unpack((uint64_t)gb);
+                        di = __longlong_as_double((long long)fx_pack(ix_rcp(d.M), -1 - d.e));
+                    } else {
+                        di = 1.0 / diag;
+                    }
+                    dinv[p] = di;
+                    di32 = ix_d2f(di);
+                }
+                diag_out[p] = diag;
+                K32[p] = ix_d2f(__longlong_as_double(Kc));
+                cb32[p] = ix_d2f(cb);
+                dinv32[p] = di32;
+                if (MODE != ASM_ONLY) {
+                    const double rp = rhs - fma(diag, hkP, -sT);     // first residual, x0 = h^k
+                    st.x[p] = hkP;
+                    if (MODE == ASM_CG64) {
+                        const double zp = di * rp;
+                        st.r[p] = rp;
+                        st.z[p] = zp;
+                        v[0] = fma(rp, zp, v[0]);
+                        v[1] = fma(rp, rp, v[1]);
+                        v[2] = fma(rhs, rhs, v[2]);
+                    } else {
+                        const float rf = (float)rp;
+                        const float zf = di32 * rf;
+                        const float bf = (float)rhs;
+                        st.r32[p] = rf;
+                        st.z32[p] = zf;
+                        st.d32[p] = 0.0f;
+                        a_rr = fmaf(rf, rf, a_rr);
+                        a_bb = fmaf(bf, bf, a_bb);
+                        a_rz = fmaf(rf, zf, a_rz);
+                    }
+                }
+            } else if (inside) {
+                assemble_inactive<MODE>(p, c_out, b, Tx, Ty, Tz, diag_out, dinv, K32, cb32, dinv32, hc, st);
+            }
+            Tbot = Ttop;
+            hm = Kc >= 0 ? hc : 0.0;
+            Kc = Kn;
+            Kn = K2;
+            hc = hu;
+            hu = h2;
+        }
+        __syncthreads();
     }
+    assemble_finish<MODE>(v, a_rr, a_bb, a_rz, st, partials, ticket);
 }
 
 // Water balance of the accepted step's last linear system (x = h^{n+1}):
@@ -477,6 +740,16 @@ void launch_closure_picard(cudaStream_t s, int nblk, const Grid &g, const DevSoi
                                                   ctl, cg_status, cg_count, cond);
 }
 
+// Tiles wherever they fill: at least half a tile's row, and enough cells that
+// marching through planes beats one cell per thread (below, every launch is
+// latency and the general kernel's one cell per thread is the shorter chain).
+static bool assemble_tiled(const Grid &g)
+{
+    for (double hw : g.hw)
+        if (!(hw > 1e-90 && hw < 1e90)) return false;     // products of the integer form stay in the normal range
+    return g.nx >= 16 && g.ny >= 4 && g.N >= 32768;
+}
+
 void launch_assemble(cudaStream_t s, int nblk, const Grid &g, const DevSoil *soils, const uint8_t *zone,
                      const double *Ks, const uint8_t *flags, const StepParams *sp, const double *hk,
                      const double *hn, const double *theta_k, const double *theta_n, const double *K,
@@ -487,18 +760,18 @@ void launch_assemble(cudaStream_t s, int nblk, const Grid &g, const DevSoil *soi
 {
     SolveStart st{};
     if (start) st = *start;
-    if (mode == ASM_CG64)
-        k_assemble<ASM_CG64><<<nblk, RED_THREADS, 0, s>>>(g, soils, zone, Ks, flags, sp, hk, hn, theta_k, theta_n, K,
-                                                          Can, c, b, Tx, Ty, Tz, diag, dinv, K32, cb32, dinv32, skip,
-                                                          st, partials, ticket, s0, theta_p);
-    else if (mode == ASM_MIXED)
-        k_assemble<ASM_MIXED><<<nblk, RED_THREADS, 0, s>>>(g, soils, zone, Ks, flags, sp, hk, hn, theta_k, theta_n,
-                                                           K, Can, c, b, Tx, Ty, Tz, diag, dinv, K32, cb32, dinv32,
-                                                           skip, st, partials, ticket, s0, theta_p);
-    else
-        k_assemble<ASM_ONLY><<<nblk, RED_THREADS, 0, s>>>(g, soils, zone, Ks, flags, sp, hk, hn, theta_k, theta_n, K,
-                                                          Can, c, b, Tx, Ty, Tz, diag, dinv, K32, cb32, dinv32, skip,
-                                                          st, partials, ticket, s0, theta_p);
+    if (assemble_tiled(g)) {
+        const Tiles tw = make_tiles(g, nblk);
+        const int nb = tile_blocks(tw, g, nblk);
+        auto *fn = mode == ASM_CG64 ? k_assemble_tiled<ASM_CG64>
+                                    : mode == ASM_MIXED ? k_assemble_tiled<ASM_MIXED> : k_assemble_tiled<ASM_ONLY>;
+        fn<<<nb, RED_THREADS, 0, s>>>(g, tw, soils, zone, Ks, flags, sp, hk, hn, theta_k, theta_n, K, Can, c, b, Tx, Ty,
+                                      Tz, diag, dinv, K32, cb32, dinv32, skip, st, partials, ticket, s0, theta_p);
+        return;
+    }
+    auto *fn = mode == ASM_CG64 ? k_assemble<ASM_CG64> : mode == ASM_MIXED ? k_assemble<ASM_MIXED> : k_assemble<ASM_ONLY>;
+    fn<<<nblk, RED_THREADS, 0, s>>>(g, soils, zone, Ks, flags, sp, hk, hn, theta_k, theta_n, K, Can, c, b, Tx, Ty, Tz,
+                                    diag, dinv, K32, cb32, dinv32, skip, st, partials, ticket, s0, theta_p);
 }
 
 void launch_accept(cudaStream_t s, int nblk, const Grid &g, const double *x_final, double *h,

@@ -1,0 +1,81 @@
+// ix64.cuh -- FP64 operations on positive operands by integer arithmetic.
+//
+// GB300's FP64 pipe issues 2 thread-operations per clock and SM, so an add
+// holds it as long as some thirty integer instructions take.  Sums, scalings
+// and reciprocals of positive numbers need no cancellation handling and are
+// cheap on mantissas and exponents; the assembly runs them beside the FP64
+// pipe instead of on it.  Results are within 0.51 units of the last place.
+// A number is (M, e): M 2^(e - 63) with M's top bit set, or M = 0.
+#pragma once
+
+#include "fx64.cuh"
+
+namespace rf {
+
+struct IxNum {
+    uint64_t M;
+    int e;
+};
+
+// A positive normal double's bits.
+RF_HD IxNum ix_unpack(uint64_t b)
+{
+    return IxNum{(b << 11) | 0x8000000000000000ULL, (int)(b >> 52) - 1023};
+}
+
+// (a + b) c for normalised a, b, c > 0.
+RF_HD IxNum ix_add_mul(IxNum a, IxNum b, IxNum c)
+{
+    const bool sw = a.e < b.e;
+    const int eb = sw ? b.e : a.e;
+    int d = eb - (sw ? a.e : b.e);
+    const uint64_t mb = sw ? b.M : a.M, ms = sw ? a.M : b.M;
+    d = d > 62 ? 62 : d;
+    uint64_t p = fx_mulhi((mb >> 1) + (ms >> (d + 1)), c.M);      // [2^61, 2^64)
+    int e = eb + c.e + 2;
+    if (!(p >> 63)) { p <<= 1; e--; }
+    if (!(p >> 63)) { p <<= 1; e--; }
+    return IxNum{p, e};
+}
+
+RF_HD IxNum ix_add(IxNum a, IxNum b)
+{
+    const bool sw = a.e < b.e;
+    int d = sw ? b.e - a.e : a.e - b.e;
+    const uint64_t mb = sw ? b.M : a.M, ms = sw ? a.M : b.M;
+    d = d > 62 ? 62 : d;
+    uint64_t p = (mb >> 1) + (ms >> (d + 1));                      // [2^62, 2^64)
+    int e = (sw ? b.e : a.e) + 1;
+    if (!(p >> 63)) { p <<= 1; e--; }
+    return IxNum{p, e};
+}
+
+RF_HD uint64_t ix_pack(IxNum a) { return fx_pack(a.M, a.e); }
+
+#ifdef __CUDACC__
+// 1/M for M in [1, 2) (Q63), Q64 in (0.5, 1): the single-precision estimate
+// ri refined by ri (1 + e + e^2), e = 1 - M ri < 2^-21.
+__device__ __forceinline__ uint64_t ix_rcp(uint64_t M)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(0x3f800000u | ((uint32_t)(M >> 40) & 0x7fffffu))));
+    const uint32_t ri = ((__float_as_uint(fminf(r, 0x1.fffffep-1f)) & 0x7fffffu) | 0x800000u) << 8;   // Q32
+    const int64_t e = (int64_t)(0x8000000000000000ULL - fx_mul32(M, ri));                             // Q63
+    const int32_t es = (int32_t)(e >> 11);                                                            // Q52
+    const int64_t s = e + (((int64_t)es * es) >> 41);                                                 // e + e^2
+    const int64_t t = (int64_t)(int32_t)(s >> 32) * ri + (int64_t)(uint32_t)(((uint64_t)(uint32_t)s * ri) >> 32);
+    return ((uint64_t)ri << 32) + (uint64_t)(t << 1);
+}
+
+// The float nearest to a non-negative double (ties to even).
+__device__ __forceinline__ float ix_d2f(double a)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(a);
+    const uint32_t ex = (uint32_t)(b >> 52);
+    if (ex - 897u > 253u) return (float)a;        // zero, subnormal or infinite as a float
+    const uint64_t v = b - (896ULL << 52);
+    return __uint_as_float((uint32_t)((v + 0x0fffffffULL + ((v >> 29) & 1)) >> 29));
+}
+#endif
+
+}  // namespace rf

@@ -24,6 +24,7 @@
 #include "cell_ops.cuh"
 #include "rf_internal.cuh"
 #include "rf_reduce.cuh"
+#include "tiles.cuh"
 #include "tma.cuh"
 
 namespace rf {
@@ -31,98 +32,6 @@ namespace rf {
 #define GRID_STRIDE_LOOP(p)                                                                 \
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < g.N;           \
          p += (long long)gridDim.x * blockDim.x)
-
-// Tiled sweeps for the stencil kernels.  A block owns a TX x TY column tile
-// and a range of z planes and walks up through them: the x/y neighbours of a
-// plane come from shared memory (the plane plus a one-cell halo, double
-// buffered so each plane needs one barrier), the z neighbours from registers
-// (the planes below and above), and the plane above is loaded while the
-// current one is in use.  Blocks loop over (tile, z-range) items; the grid
-// never exceeds the reduction's block count.
-constexpr int TX = 32, TY = RED_THREADS / 32;
-constexpr int HALO = 2 * TY + 2 * TX;   // x- and y-halo cells of a plane (no corners)
-
-struct Tiles {
-    int ntx, nty, zc;       // tiles along x, y; planes per item
-    int tx;                 // tile width in x
-    long long items;
-};
-
-static Tiles make_tiles(const Grid &g, int nblk)
-{
-    if (g.cap > nblk) nblk = g.cap;
-    Tiles t;
-    t.tx = TX;
-    t.ntx = (g.nx + TX - 1) / TX;
-    t.nty = (g.ny + TY - 1) / TY;
-    const long long tiles = (long long)t.ntx * t.nty;
-    // split z so that the items fill the grid in one wave when the tiles alone
-    // do not (every block then walks the same number of planes)
-    const long long want_chunks = nblk / tiles;
-    const int chunks = (int)std::min<long long>(std::max<long long>(want_chunks, 1), g.nz);
-    t.zc = (g.nz + chunks - 1) / chunks;
-    t.items = tiles * ((g.nz + t.zc - 1) / t.zc);
-    return t;
-}
-
-// Tiles with the z split that minimises (waves of `resident` blocks) x
-// (planes per item + the two extra planes an item reads); at most `cap` items
-// per wave are launched.
-static Tiles make_tiles_balanced(const Grid &g, int resident, int tile_x)
-{
-    Tiles t;
-    t.tx = tile_x;
-    t.ntx = (g.nx + tile_x - 1) / tile_x;
-    t.nty = (g.ny + TY - 1) / TY;
-    const long long tiles = (long long)t.ntx * t.nty;
-    long long best = -1;
-    int best_zc = g.nz;
-    for (int ch = 1; ch <= g.nz; ch++) {
-        const int zc = (g.nz + ch - 1) / ch;
-        const long long items = tiles * ((g.nz + zc - 1) / zc);
-        const long long waves = (items + resident - 1) / resident;
-        const long long cost = waves * (zc + 2);
-        if (best < 0 || cost < best) {
-            best = cost;
-            best_zc = zc;
-        }
-    }
-    t.zc = best_zc;
-    t.items = tiles * ((g.nz + t.zc - 1) / t.zc);
-    return t;
-}
-
-static int tile_blocks(const Tiles &t, const Grid &g, int nblk)
-{
-    return (int)std::min<long long>(t.items, g.cap > nblk ? g.cap : nblk);
-}
-
-struct TileItem {
-    int i0, j0, k0, k1;
-};
-
-__device__ __forceinline__ TileItem tile_item(const Grid &g, const Tiles &t, long long item)
-{
-    const long long per_plane = (long long)t.ntx * t.nty;
-    const int chunk = (int)(item / per_plane);
-    const long long r = item - chunk * per_plane;
-    TileItem it;
-    it.j0 = (int)(r / t.ntx) * TY;
-    it.i0 = (int)(r % t.ntx) * t.tx;
-    it.k0 = chunk * t.zc;
-    it.k1 = min(g.nz, it.k0 + t.zc);
-    return it;
-}
-
-// Halo cell h (0 <= h < HALO) of a tile, as offsets (hx, hy) from (i0, j0):
-// -x column, +x column, -y row, +y row.
-__device__ __forceinline__ void halo_cell(int h, int &hx, int &hy)
-{
-    if (h < TY) { hx = -1; hy = h; }
-    else if (h < 2 * TY) { hx = TX; hy = h - TY; }
-    else if (h < 2 * TY + TX) { hx = h - 2 * TY; hy = -1; }
-    else { hx = h - 2 * TY - TX; hy = TY; }
-}
 
 // ---------------------------------------------------------------- FP64 PCG
 __global__ void __launch_bounds__(RED_THREADS)

@@ -189,6 +189,7 @@ void apply_grid_params(Grid &g, const rf_solver_params &p)
     for (int f = 0; f < 6; f++) {
         g.gf[f] = gv[f];
         g.hg[f] = 0.5 * g.A[f] * gv[f];
+        g.gd[f] = gv[f] * (g.A[f] / g.w[f]);
     }
     g.tilted = (p.grav[0] != 0.0 || p.grav[1] != 0.0) ? 1 : 0;
     g.harmonic = p.face_mean == RF_FACE_HARMONIC ? 1 : 0;
@@ -235,6 +236,7 @@ void fill_step_params(rf_ctx *c, double dt)
 {
     StepParams &s = *c->sp_h;
     s.dt = dt;
+    s.V_dt = c->g.V / dt;
     s.t = c->t;
     s.eps_chord = c->prm.eps_chord;
     s.modified = c->prm.picard_form == RF_PICARD_MODIFIED ? 1 : 0;

@@ -80,6 +80,7 @@ struct Grid {
     double hw[6];     // A/(2 d): T_f = (K_P + K_N) hw_f
     double gf[6];     // gravity flux factor of each face, grad(elevation) . n_out: (-gx, gx, -gy, gy, -gz, gz)
     double hg[6];     // gf A / 2: explicit gravity of an interior face is (K_P + K_N) hg_f
+    double gd[6];     // gf d: gravity through an interior face is T_f gd_f
     float w32[3];     // A/d per axis, FP32 (mixed-precision operator)
     FastDiv fx, fxy;  // division by nx and by nx*ny
     int cap;          // most blocks a tiled stencil kernel launches (partials hold 8 values per block)
@@ -95,6 +96,7 @@ struct Grid {
 // be replayed from a CUDA graph.
 struct StepParams {
     double dt, t, eps_chord;
+    double V_dt;    // cell volume / dt
     int bc_type[6];
     double bc_val[6];
     int modified;   // 1: modified Picard (tangent capacity, mixed-form storage); 0: chord capacity
