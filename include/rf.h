@@ -350,7 +350,7 @@ unsigned long long rf_launch_count(rf_ctx *ctx);
  * in order: closure, closure+Picard test, assembly, FP64 CG init, FP64 CG
  * stencil, FP64 CG update, FP64 operator apply, mixed start, FP64 outer
  * residual, FP32 CG stencil, FP32 CG update, correction add, water balance,
- * storage, accept.  Returns the number of values written (<= cap). */
+ * storage, accept, a whole attempt or solve in one launch.  Returns the number of values written (<= cap). */
 int rf_launch_counts(rf_ctx *ctx, unsigned long long *out, int cap);
 
 /* Kernels that rf_profile_kernel can time. */

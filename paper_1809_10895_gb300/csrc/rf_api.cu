@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "dic.cuh"
+#include "grid_red.cuh"
 #include "mg.cuh"
 #include "nn.cuh"
 #include "rf.h"
@@ -77,6 +78,8 @@ struct rf_ctx {
     float *p32[2] = {nullptr, nullptr}, *q32 = nullptr, *d32 = nullptr;
     double *partials = nullptr;
     unsigned int *ticket = nullptr;
+    void *gridred = nullptr;             // barrier and partials of the cooperative kernels
+    int small_blocks[2] = {-1, -1};      // blocks of the small-grid attempt (FP64, mixed; -1: not asked yet)
     CgScal *sc = nullptr, *sc_in = nullptr;
     StepResults *res = nullptr;
     StepParams *sp = nullptr;
@@ -623,8 +626,123 @@ void ws_scalar_features(const rf_ctx *c, const nn::WsScales &sc, double t, doubl
     dt_feat = (float)std::log(dt / sc.t_scale);
 }
 
+// A converged attempt becomes the state: the last iterate and its closures
+// sit in H[f], K[f].
+rf_status accept_iterate(rf_ctx *c, int f)
+{
+    if (c->prm.time_scheme == RF_TIME_BDF2)    // theta*(h^{n-1}) for the next step
+        CUDA_TRY(cudaMemcpyAsync(c->theta_p, c->theta_n, sizeof(double) * c->g.N, cudaMemcpyDeviceToDevice, c->stream));
+    launch_accept(c->stream, c->nblk, c->g, f ? c->x : c->hk, c->h, c->theta_k, c->theta_n, c->K[1], c->K[0], f);
+    return RF_OK;
+}
+
+// The attempt of a small grid: one cooperative launch that starts from h,
+// accepts a converged iterate and reports into pinned host memory.
+rf_status attempt_small(rf_ctx *c, double dt, Attempt &A, bool guess, int blocks)
+{
+    NvtxRange range("rf: Picard attempt");
+    fill_step_params(c, dt);
+    *c->ctl_h = PicardCtl{};
+    if (guess) {
+        float q_feat, dt_feat;
+        ws_scalar_features(c, c->ws_sc, c->t, dt, q_feat, dt_feat);
+        RF_TRY(rf_nn_mesh_guess(c->ws_net, c->stream, c->g, c->flags, c->h, c->Ks, c->ws_sc, q_feat, dt_feat,
+                                c->ws_sc.out_scale * dt, c->hk, c->dev_fault));
+        run_closure(c, c->hk, nullptr, c->theta_k, 0);
+        c->ws_guesses++;
+    }
+    AttemptArgs a{};
+    a.g = c->g;
+    a.sp = *c->sp_h;
+    a.soils = c->soils;
+    a.zone = c->zone;
+    a.flags = c->flags;
+    a.Ks = c->Ks;
+    a.h = c->h;
+    a.H[0] = c->hk;
+    a.H[1] = c->x;
+    a.theta_k = c->theta_k;
+    a.theta_n = c->theta_n;
+    a.theta_p = c->theta_p;
+    a.K[0] = c->K[0];
+    a.K[1] = c->K[1];
+    a.Can = c->Can;
+    a.c = c->c;
+    a.b = c->b;
+    a.s0 = s0_of(c);
+    a.Tx = c->Tx;
+    a.Ty = c->Ty;
+    a.Tz = c->Tz;
+    a.diag = c->diag;
+    a.dinv = c->dinv;
+    a.r = c->r;
+    a.z = c->z;
+    a.q = c->q;
+    a.K32 = c->K32;
+    a.cb32 = c->cb32;
+    a.dinv32 = c->dinv32;
+    a.r32 = c->r32;
+    a.z32 = c->z32;
+    a.q32 = c->q32;
+    a.d32 = c->d32;
+    for (int i = 0; i < 2; i++) {
+        a.p[i] = c->p[i];
+        a.p32[i] = c->p32[i];
+    }
+    a.red = c->gridred;
+    a.fault = c->fault_h;
+    a.ctl = c->ctl_h;
+    a.res = c->res_h;
+    a.tol_picard = c->prm.tol_picard;
+    a.tol_cg = c->prm.tol_cg;
+    a.tol_inner = c->prm.tol_inner;
+    a.n_max = c->prm.n_max;
+    a.cg_max_it = c->prm.cg_max_it;
+    a.inner_max_it = c->prm.inner_max_it;
+    a.outer_max_it = c->prm.outer_max_it;
+    a.copy_h = guess ? 0 : 1;
+    a.do_closure = c->closure_at_h ? 0 : 1;
+    a.keep_theta_p = c->prm.time_scheme == RF_TIME_BDF2 ? 1 : 0;
+    if (guess) RF_TRY(sync(c));     // the network's device waits report through dev_fault
+    *c->fault_h = 0;
+    CUDA_TRY(launch_attempt_small(c->stream, a, c->prm.precision == RF_PREC_MIXED, blocks));
+    c->closure_at_h = false;        // the attempt overwrites K[0] and C; an accepted step sets it again
+    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(cudaStreamSynchronize(c->stream));
+    if (*c->fault_h) {
+        *c->fault_h = 0;
+        CUDA_TRY(cudaMemsetAsync(c->gridred, 0, GR_BYTES, c->stream));   // rounds start afresh
+        CUDA_TRY(cudaStreamSynchronize(c->stream));
+        return fail(RF_ERR_DEVICE_TIMEOUT, "a grid barrier of the small-grid attempt ran out");
+    }
+    const PicardCtl &ctl = *c->ctl_h;
+    A.picard = ctl.it;
+    A.cg = ctl.cg_total;
+    A.max_dh = ctl.max_dh;
+    if (ctl.conv) {
+        A.converged = true;
+        A.mb = *c->res_h;
+        if (blocks > 1) RF_TRY(accept_iterate(c, ctl.it & 1));
+    } else {
+        A.status = ctl.fail ? RF_ERR_CG : RF_ERR_PICARD;
+        if (guess) c->ws_fallbacks++;
+    }
+    return RF_OK;
+}
+
 rf_status attempt(rf_ctx *c, double dt, Attempt &A, bool guess)
 {
+    // Grids on which an attempt is launch latency (measured, one pass of six to
+    // four 60 s steps of the box, graph / one launch): 30 K cells 1585 / 877 us,
+    // 262 K 2150 / 1315, 410 K 2732 / 1766, 786 K 7214 / 5935, 1 M 5665 / 5570;
+    // with hundreds of CG iterations per solve, mixed: 410 K 52.8 / 41.7 ms,
+    // 786 K 55.2 / 63.1.  The other preconditioners run from the graph.
+    constexpr long long SMALL_CELLS = 1 << 19;
+    if (c->prm.precond == RF_PRECOND_JACOBI && c->g.N <= SMALL_CELLS) {
+        int &blocks = c->small_blocks[c->prm.precision == RF_PREC_MIXED ? 1 : 0];
+        if (blocks < 0) blocks = attempt_small_blocks(c->g.N, c->num_sms, c->prm.precision == RF_PREC_MIXED);
+        if (blocks > 0) return attempt_small(c, dt, A, guess, blocks);
+    }
     NvtxRange range("rf: Picard attempt");
     if (!c->picard_exec) RF_TRY(build_picard_graph(c));
     fill_step_params(c, dt);
@@ -661,12 +779,7 @@ rf_status attempt(rf_ctx *c, double dt, Attempt &A, bool guess)
     if (ctl.conv) {
         A.converged = true;
         A.mb = *c->res_h;
-        // the last iterate and its closures: H[it & 1], K[it & 1]
-        const int f = ctl.it & 1;
-        if (c->prm.time_scheme == RF_TIME_BDF2)    // theta*(h^{n-1}) for the next step
-            CUDA_TRY(cudaMemcpyAsync(c->theta_p, c->theta_n, sizeof(double) * c->g.N, cudaMemcpyDeviceToDevice,
-                                     c->stream));
-        launch_accept(c->stream, c->nblk, c->g, f ? c->x : c->hk, c->h, c->theta_k, c->theta_n, c->K[1], c->K[0], f);
+        RF_TRY(accept_iterate(c, ctl.it & 1));
     } else {
         A.status = ctl.fail ? RF_ERR_CG : RF_ERR_PICARD;
         if (guess) c->ws_fallbacks++;
@@ -1018,7 +1131,8 @@ rf_status rf_mesh_create(const rf_mesh_desc *mesh, const rf_solver_params *param
               alloc_n(c, c->sc, 1) && alloc_n(c, c->sc_in, 1) && alloc_n(c, c->res, 1) && alloc_n(c, c->sp, 1) &&
               alloc_n(c, c->ctl, 1) && alloc_n(c, c->ctr, 2 * KK_COUNT) && alloc_n(c, c->fftab, 1) &&
               alloc_n(c, c->dev_fault, 1);
-    if (!ok) {
+    c->gridred = ok ? c->dalloc(GR_BYTES) : nullptr;
+    if (!c->gridred) {
         rf_destroy(c);
         return fail(RF_ERR_NOMEM, "device allocation failed");
     }
@@ -1041,6 +1155,7 @@ rf_status rf_mesh_create(const rf_mesh_desc *mesh, const rf_solver_params *param
     cudaError_t e = cudaMemcpyAsync(c->flags, c->flags_h.data(), N, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->fftab, ff_tables(), sizeof(FFTables), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ticket, 0, 64 * sizeof(unsigned int), c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->gridred, 0, GR_BYTES, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ctr, 0, 2 * KK_COUNT * sizeof(unsigned long long), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ctl, 0, sizeof(PicardCtl), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->dev_fault, 0, sizeof(int), c->stream);

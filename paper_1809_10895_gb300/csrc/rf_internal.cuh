@@ -57,7 +57,7 @@ inline FastDiv make_fastdiv(unsigned int d)
 enum KernelKind {
     KK_CLOSURE = 0, KK_CLOSURE_PICARD, KK_ASSEMBLE, KK_CG64_INIT, KK_CG64_SPMV, KK_CG64_UPDATE, KK_APPLY64,
     KK_MIXED_START, KK_RESID64, KK_CG32_SPMV, KK_CG32_UPDATE, KK_ADD_CORRECTION, KK_MASS_BALANCE, KK_STORAGE,
-    KK_ACCEPT, KK_COUNT
+    KK_ACCEPT, KK_ONE_LAUNCH, KK_COUNT
 };
 
 struct DevSoil {
@@ -273,6 +273,32 @@ void set_last_error(const char *msg);
 
 // Fixed-point copies of a soil's alpha, n and m (closure_assemble.cu).
 FxSoil make_fx_soil(int model, double alpha, double n, double m);
+
+// Everything one Picard attempt of a small grid reads and writes
+// (attempt_small.cu); passed by value.
+struct AttemptArgs {
+    Grid g;
+    StepParams sp;
+    const DevSoil *soils;
+    const uint8_t *zone, *flags;
+    const double *Ks;
+    double *h, *H[2], *theta_k, *theta_n, *theta_p, *K[2], *Can, *c, *b, *s0;
+    double *Tx, *Ty, *Tz, *diag, *dinv, *r, *z, *p[2], *q;
+    float *K32, *cb32, *dinv32, *r32, *z32, *p32[2], *q32, *d32;
+    void *red;                  // grid reductions (grid_red.cuh; zero before the first launch)
+    int *fault;                 // host-visible
+    PicardCtl *ctl;             // host-visible results
+    StepResults *res;
+    double tol_picard, tol_cg, tol_inner;
+    int n_max, cg_max_it, inner_max_it, outer_max_it;
+    int copy_h;                 // start from h (else from H[0], closures done)
+    int do_closure;             // closures at h are not yet in theta_k, K[0], C
+    int keep_theta_p;           // BDF2: theta*(h^{n-1}) kept on acceptance
+    int pad;
+};
+cudaError_t launch_attempt_small(cudaStream_t s, const AttemptArgs &A, int mixed, int blocks);
+// Blocks of that launch (0: cannot run).
+int attempt_small_blocks(long long N, int sms, int mixed);
 
 // ---- launch entry points implemented in the .cu files --------------------
 void launch_closure(cudaStream_t s, int nblk, const Grid &g, const DevSoil *soils, const uint8_t *zone,

@@ -175,7 +175,7 @@ NN_PARAMS = 225793
 NN_LAYERS = 10
 COUNTER_KINDS = ("closure", "closure_picard", "assemble", "cg64_init", "cg64_spmv", "cg64_update", "apply64",
                  "mixed_start", "resid64", "cg32_spmv", "cg32_update", "add_correction", "mass_balance",
-                 "storage", "accept")
+                 "storage", "accept", "one_launch")
 KERNEL_KINDS = {"closure": 0, "assemble": 1, "cg64_spmv": 2, "cg64_update": 3, "resid64": 4, "cg32_spmv": 5,
                 "cg32_update": 6}
 
