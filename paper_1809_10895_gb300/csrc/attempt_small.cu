@@ -210,20 +210,20 @@ k_attempt_small(const __grid_constant__ AttemptArgs A)
             A.Ty[p] = cs.Tup[1];
             A.Tz[p] = cs.Tup[2];
             A.diag[p] = cs.diag;
-            A.K32[p] = (float)cs.KP;
-            A.cb32[p] = (float)cs.cb;
+            A.K32[p] = ix_d2f(cs.KP);
+            A.cb32[p] = ix_d2f(cs.cb);
             const double rp = cs.rhs - (cs.diag * hkP - cs.sT);
             if (PREC == 0) {
-                const double di = rcp64(cs.diag), zp = di * rp;
+                const double di = ix_rcp64(cs.diag), zp = di * rp;
                 A.dinv[p] = di;
-                A.dinv32[p] = (float)di;
+                A.dinv32[p] = ix_d2f(di);
                 rr64[p] = rp;
                 zz64[p] = zp;
                 v[0] = fma(rp, zp, v[0]);
                 v[1] = fma(rp, rp, v[1]);
                 v[2] = fma(cs.rhs, cs.rhs, v[2]);
             } else {
-                const float di = __frcp_rn((float)cs.diag), rf = (float)rp, zf = di * rf, bf = (float)cs.rhs;
+                const float di = __frcp_rn(ix_d2f(cs.diag)), rf = (float)rp, zf = di * rf, bf = (float)cs.rhs;
                 A.dinv32[p] = di;
                 A.r32[p] = rf;
                 A.z32[p] = zf;
@@ -251,12 +251,27 @@ k_attempt_small(const __grid_constant__ AttemptArgs A)
                 const bool first = cg == 0;
                 auto get = [&](long long q) { return first ? zz64[q] : fma(beta, pin[q], zz64[q]); };
                 double w[1] = {0.0};
-                for (int p = p0; p < N; p += stride) {
-                    if (!(A.flags[p] & FLAG_ACTIVE)) continue;
-                    const double pp = get(p), qp = apply64(g, p, A.Tx, A.Ty, A.Tz, A.diag, get);
-                    pout[p] = pp;
-                    A.q[p] = qp;
-                    w[0] = fma(pp, qp, w[0]);
+                if (gridDim.x == 1) {
+                    // one block: p once per cell and a block barrier, instead
+                    // of once per neighbour (a multiply-add each, on a pipe
+                    // that an instruction of seven warps holds 128 cycles)
+                    for (int p = p0; p < N; p += stride)
+                        if (A.flags[p] & FLAG_ACTIVE) pout[p] = get(p);
+                    __syncthreads();
+                    for (int p = p0; p < N; p += stride) {
+                        if (!(A.flags[p] & FLAG_ACTIVE)) continue;
+                        const double qp = apply64(g, p, A.Tx, A.Ty, A.Tz, A.diag, [&](long long q) { return pout[q]; });
+                        A.q[p] = qp;
+                        w[0] = fma(pout[p], qp, w[0]);
+                    }
+                } else {
+                    for (int p = p0; p < N; p += stride) {
+                        if (!(A.flags[p] & FLAG_ACTIVE)) continue;
+                        const double pp = get(p), qp = apply64(g, p, A.Tx, A.Ty, A.Tz, A.diag, get);
+                        pout[p] = pp;
+                        A.q[p] = qp;
+                        w[0] = fma(pp, qp, w[0]);
+                    }
                 }
                 if (!grid_sum<1>(C, w, [&](const double *t) {
                         s.alpha = s.rho * rcp64(t[0]);

@@ -6,6 +6,7 @@
 #include <math.h>
 
 #include "f64m.cuh"
+#include "ix64.cuh"
 #include "rf_internal.cuh"
 
 namespace rf {
@@ -289,12 +290,92 @@ __device__ __forceinline__ void boundary_face(const Grid &g, const DevSoil *__re
     }
 }
 
+// The positive arithmetic of the assembly on the integer pipes (ix64.cuh),
+// with FP64 for operands outside the range in which products of the integer
+// form stay normal numbers.
+constexpr long long K_CLOSED = (long long)0xbff0000000000000ULL;   // bits of K = -1 (inactive, outside)
+
+// T = Kbar A/d of the face between cells with the bits a, b of K (0 when
+// either is closed); hw its A/(2 d), ihw the same unpacked.
+__device__ __forceinline__ double face_coef(const Grid &g, long long a, long long b, double hw, const IxNum &ihw)
+{
+    if ((a | b) < 0) return 0.0;
+    if (g.ix_ok && (unsigned)(a >> 52) - 400u < 1200u && (unsigned)(b >> 52) - 400u < 1200u)
+        return __longlong_as_double((long long)ix_pack(ix_add_mul(ix_unpack(a), ix_unpack(b), ihw)));
+    const double x = __longlong_as_double(a), y = __longlong_as_double(b);
+    double s = x + y;
+    if (g.harmonic) s = s > 0.0 ? 4.0 * x * y / s : 0.0;
+    return s * hw;
+}
+
+// c = V_dt (theta^k - theta^n) / (h^k - h^n), dth and dh the differences.
+__device__ __forceinline__ double chord_c(double dth, double dh, double V_dt)
+{
+    const long long db = __double_as_longlong(dh) & 0x7fffffffffffffffLL, vb = __double_as_longlong(V_dt);
+    double f;
+    if ((unsigned)(vb >> 52) - 700u < 650u && (unsigned)(db >> 52) - 700u < 650u) {
+        const IxNum d = ix_unpack((uint64_t)db), V = ix_unpack((uint64_t)vb);
+        uint64_t q = fx_mulhi(ix_rcp(d.M), V.M);
+        const int up = (int)(q >> 63);
+        q = up ? q : q << 1;
+        f = __longlong_as_double((long long)fx_pack(q, V.e - d.e - 1 + up));
+    } else {
+        f = V_dt / __longlong_as_double(db);
+    }
+    return __longlong_as_double(__double_as_longlong(dth) ^
+                                (__double_as_longlong(dh) & (long long)0x8000000000000000ULL)) * f;
+}
+
+// 1/a for a > 0.
+__device__ __forceinline__ double ix_rcp64(double a)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(a);
+    if ((unsigned)(b >> 52) - 400u < 1200u) {
+        const IxNum d = ix_unpack(b);
+        return __longlong_as_double((long long)fx_pack(ix_rcp(d.M), -1 - d.e));
+    }
+    return 1.0 / a;
+}
+
+// Storage part of a cell: c = V C^k / dt and its share s0 of the right side.
+// form: storage_form(sp), held by the caller.
+enum { STORE_CHORD = 0, STORE_MODIFIED = 1, STORE_BDF2 = 2 };
+__device__ __forceinline__ int storage_form(const StepParams &sp)
+{
+    return sp.bdf2 ? STORE_BDF2 : sp.modified ? STORE_MODIFIED : STORE_CHORD;
+}
+__device__ __forceinline__ void storage_terms(int form, const StepParams &sp, double V_dt, double eps, double hkP,
+                                              double hnP, double thk, double thn, double can,
+                                              const double *__restrict__ thp, long long p, double &c, double &s0)
+{
+    if (form == STORE_BDF2) {
+        // variable-step BDF2 (the multistep alternative Sec. 2.2 names) in the
+        // mixed form V/dt [a0 theta^{n+1} - a1 theta^n + a2 theta^{n-1}],
+        // theta^{n+1} linearised about h^k as in the modified Picard form
+        c = V_dt * (sp.a0 * can);
+        s0 = V_dt * (sp.a0 * can * hkP - (sp.a0 * thk - sp.a1 * thn + sp.a2 * thp[p]));
+    } else if (form == STORE_MODIFIED) {
+        // modified Picard (Sec. 2.2, mass-conservative variant): theta*(h^{k+1})
+        // ~ theta*(h^k) + C(h^k) (h^{k+1} - h^k), so the storage term is
+        // c (h^{k+1} - h^k) + V (theta*(h^k) - theta*(h^n)) / dt
+        c = V_dt * can;
+        s0 = c * hkP - V_dt * (thk - thn);
+    } else {
+        // classical Picard with the chord slope of theta* between h^n and h^k;
+        // |dh| > eps compared on the IEEE bit patterns (both non-negative)
+        const double dh = hkP - hnP;
+        const bool chord = (__double_as_longlong(dh) & 0x7fffffffffffffffLL) > __double_as_longlong(eps);
+        c = chord ? chord_c(thk - thn, dh, V_dt) : V_dt * can;
+        s0 = c * hnP;
+    }
+}
+
 // One cell of the Picard system (Sec. 2.2; see k_assemble):
 //   c = V C^k / dt (chord slope of theta*, or C(h^k) when |h^k - h^n| <= eps),
 //   interior faces T_f = Kbar_f A_f/d_f with Kbar_f = (K_P + K_N)/2 (or the
-//   harmonic mean 2 K_P K_N / (K_P + K_N)) and explicit gravity
-//   gf_f Kbar_f A_f, gf_f the elevation gradient along the face's outward
-//   normal (+1 top, -1 bottom, 0 lateral on a z-up grid),
+//   harmonic mean 2 K_P K_N / (K_P + K_N)) and explicit gravity T_f gd_f,
+//   gd_f the elevation gradient along the face's outward normal times d_f
+//   (+d top, -d bottom, 0 lateral on a z-up grid),
 //   boundary terms of the face classes flagged in fl.
 // With RESID, sT = sum over interior faces of T_f h^k_N (for b - A h^k).
 // thp: theta*(h^{n-1}), read only by the BDF2 storage.
@@ -315,49 +396,31 @@ __device__ __forceinline__ void assemble_cell(const Grid &g, const DevSoil *__re
                                               CellSystem &out)
 {
     const double hkP = hk[p], hnP = hn[p], KP = K[p];
-    double C, s0;
-    if (sp.bdf2) {
-        // variable-step BDF2 (the multistep alternative Sec. 2.2 names) in the
-        // mixed form V/dt [a0 theta^{n+1} - a1 theta^n + a2 theta^{n-1}],
-        // theta^{n+1} linearised about h^k as in the modified Picard form
-        C = sp.a0 * Can[p];
-        s0 = V_dt * (C * hkP - (sp.a0 * thk[p] - sp.a1 * thn[p] + sp.a2 * thp[p]));
-    } else if (sp.modified) {
-        // modified Picard (Sec. 2.2, mass-conservative variant): theta*(h^{k+1})
-        // ~ theta*(h^k) + C(h^k) (h^{k+1} - h^k), so the storage term is
-        // c (h^{k+1} - h^k) + V (theta*(h^k) - theta*(h^n)) / dt
-        C = Can[p];
-        s0 = V_dt * C * hkP - V_dt * (thk[p] - thn[p]);
-    } else {
-        // classical Picard with the chord slope of theta* between h^n and h^k
-        const double dh = hkP - hnP;
-        // |dh| > eps compared on the IEEE bit patterns (both non-negative)
-        const bool chord = (__double_as_longlong(dh) & 0x7fffffffffffffffLL) > __double_as_longlong(eps);
-        C = chord ? (thk[p] - thn[p]) * rcp64(dh) : Can[p];
-        s0 = V_dt * C * hnP;
-    }
-    const double c = V_dt * C;
-    double diag = c, rhs = s0, cb = c;
-    double sT = 0.0;
-    double Tup[3] = {0.0, 0.0, 0.0};
+    const long long kb = __double_as_longlong(KP);
+    double c, s0;
+    storage_terms(storage_form(sp), sp, V_dt, eps, hkP, hnP, thk[p], thn[p], Can[p], thp, p, c, s0);
+    double T[6], sT = 0.0;
 #pragma unroll
     for (int f = 0; f < 6; f++) {
         long long q;
-        if (neighbour(g, p, i, j, k, f, q)) {
-            const double KN = K[q];
-            if (__double_as_longlong(KN) >= 0) {          // active neighbour (K >= 0; inactive K = -1)
-                double Ks2 = KP + KN;                      // 2 Kbar
-                if (g.harmonic) Ks2 = Ks2 > 0.0 ? 4.0 * KP * KN / Ks2 : 0.0;
-                const double T = Ks2 * g.hw[f];            // Kbar A/d
-                diag += T;
-                if (f >= F_ZMIN || g.tilted) rhs = fma(Ks2, g.hg[f], rhs);   // explicit gravity, gf Kbar A
-                if (f & 1) Tup[f >> 1] = T;
-                if (RESID) sT = fma(T, hk[q], sT);
-                continue;
-            }
+        const bool in = neighbour(g, p, i, j, k, f, q);
+        const long long kn = in ? __double_as_longlong(K[q]) : K_CLOSED;
+        T[f] = face_coef(g, kb, kn, g.hw[f], ix_unpack((uint64_t)__double_as_longlong(g.hw[f])));
+        if (RESID) {
+            const double hN = kn >= 0 ? hk[q] : 0.0;
+            sT = f == 0 ? T[f] * hN : fma(T[f], hN, sT);
         }
-        if (!(fl & (1u << f))) continue;    // closed face (lateral face on an inactive cell)
-        boundary_face(g, soils, zone, Ks, sp, p, f, hnP, KP, diag, cb, rhs);
+    }
+    double diag = c + (((T[0] + T[1]) + (T[2] + T[3])) + (T[4] + T[5]));
+    double rhs = fma(T[5], g.gd[F_ZMAX], fma(T[4], g.gd[F_ZMIN], s0));   // explicit gravity
+    if (g.tilted) {
+        rhs = fma(T[0], g.gd[F_XMIN], fma(T[1], g.gd[F_XMAX], rhs));
+        rhs = fma(T[2], g.gd[F_YMIN], fma(T[3], g.gd[F_YMAX], rhs));
+    }
+    double cb = c;
+    if (fl & 0x3f) {
+        for (int f = 0; f < 6; f++)
+            if (fl & (1u << f)) boundary_face(g, soils, zone, Ks, sp, p, f, hnP, KP, diag, cb, rhs);
     }
     out.c = c;
     out.s0 = s0;
@@ -366,9 +429,9 @@ __device__ __forceinline__ void assemble_cell(const Grid &g, const DevSoil *__re
     out.cb = cb;
     out.sT = sT;
     out.KP = KP;
-    out.Tup[0] = Tup[0];
-    out.Tup[1] = Tup[1];
-    out.Tup[2] = Tup[2];
+    out.Tup[0] = T[1];
+    out.Tup[1] = T[3];
+    out.Tup[2] = T[5];
 }
 
 // Boundary inflow (fin >= 0) and outflow (fout >= 0) of one cell's boundary

@@ -26,7 +26,6 @@ struct MaxDh {
 __device__ __forceinline__ bool grid_max_dh(MaxDh &m, double *partials, unsigned int *ticket)
 {
     __shared__ unsigned long long sd[RED_THREADS / 32];
-    __shared__ int sb;
     __shared__ bool am_last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     auto block = [&]() {
@@ -283,7 +282,7 @@ k_assemble(Grid g, const DevSoil *__restrict__ soils, const uint8_t *__restrict_
         if (MODE == ASM_MIXED) {
             di32 = __frcp_rn((float)diag);
         } else {
-            di = rcp64(diag);
+            di = ix_rcp64(diag);
             dinv[p] = di;
             di32 = (float)di;
         }
@@ -346,27 +345,17 @@ k_assemble_tiled(Grid g, Tiles tw, const DevSoil *__restrict__ soils, const uint
     count_work(g, KK_ASSEMBLE);
     __shared__ long long sK[2][TY + 2][TX + 2];
     __shared__ double sH[2][TY + 2][TX + 2];
-    constexpr long long CLOSED = (long long)0xbff0000000000000ULL;   // K = -1
+    constexpr long long CLOSED = K_CLOSED;
     const double eps = spp->eps_chord, V_dt = spp->V_dt;
-    const bool mixed_form = spp->modified || spp->bdf2;
-    const bool Vok = (unsigned)(__double_as_longlong(V_dt) >> 52) - 700u < 650u;   // products stay in the normal range
-    const IxNum hwx = ix_unpack(__double_as_longlong(g.hw[0])), hwy = ix_unpack(__double_as_longlong(g.hw[2]));
-    const IxNum hwz = ix_unpack(__double_as_longlong(g.hw[4])), ixV = ix_unpack(__double_as_longlong(V_dt));
+    const int form = storage_form(*spp);
+    const IxNum hwx = ix_unpack((uint64_t)__double_as_longlong(g.hw[0]));
+    const IxNum hwy = ix_unpack((uint64_t)__double_as_longlong(g.hw[2]));
+    const IxNum hwz = ix_unpack((uint64_t)__double_as_longlong(g.hw[4]));
     const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
     int hx = 0, hy = 0;
     if (threadIdx.x < HALO) halo_cell(threadIdx.x, hx, hy);
     double v[3] = {0.0, 0.0, 0.0};
     float a_rr = 0.0f, a_bb = 0.0f, a_rz = 0.0f;   // mixed start: norms of the FP32 seeds, summed in FP32
-    // T of the face between cells with K bits a and b (sign set: closed)
-    auto face = [&](long long a, long long bb, const IxNum &hw, double hwd) -> double {
-        if ((a | bb) < 0) return 0.0;
-        if (!g.harmonic && (unsigned)(a >> 52) - 400u < 1200u && (unsigned)(bb >> 52) - 400u < 1200u)
-            return __longlong_as_double((long long)ix_pack(ix_add_mul(ix_unpack(a), ix_unpack(bb), hw)));
-        const double x = __longlong_as_double(a), y = __longlong_as_double(bb);
-        double s = x + y;
-        if (g.harmonic) s = s > 0.0 ? 4.0 * x * y / s : 0.0;
-        return s * hwd;
-    };
     struct Pl {
         double hn, thk, thn, can;
         uint8_t fl;
@@ -405,7 +394,7 @@ k_assemble_tiled(Grid g, Tiles tw, const DevSoil *__restrict__ soils, const uint
         double Tbot = 0.0;
         if (it.k0 > 0) {
             const long long Kb = ldK(it.k0 - 1);
-            Tbot = face(Kb, Kc, hwz, g.hw[4]);
+            Tbot = face_coef(g, Kb, Kc, g.hw[4], hwz);
             hm = Kb >= 0 ? ldh(it.k0 - 1) : 0.0;
         }
         for (int k = it.k0; k < it.k1; k++) {
@@ -434,43 +423,12 @@ k_assemble_tiled(Grid g, Tiles tw, const DevSoil *__restrict__ soils, const uint
             if (Kc >= 0) {
                 const double hkP = hc;
                 double c, s0;
-                if (mixed_form) {
-                    if (spp->bdf2) {
-                        c = V_dt * (spp->a0 * cur.can);
-                        s0 = V_dt * (spp->a0 * cur.can * hkP -
-                                     (spp->a0 * cur.thk - spp->a1 * cur.thn + spp->a2 * thp[p]));
-                    } else {
-                        c = V_dt * cur.can;
-                        s0 = c * hkP - V_dt * (cur.thk - cur.thn);
-                    }
-                } else {
-                    const double dh = hkP - cur.hn;
-                    const long long db = __double_as_longlong(dh) & 0x7fffffffffffffffLL;
-                    if (db > __double_as_longlong(eps)) {
-                        // (theta*^k - theta*^n) (V / dt / |dh|), the factor by integer arithmetic
-                        const double dth = cur.thk - cur.thn;
-                        double f;
-                        if (Vok && (unsigned)(db >> 52) - 700u < 650u) {
-                            const IxNum d = ix_unpack((uint64_t)db);
-                            uint64_t q = fx_mulhi(ix_rcp(d.M), ixV.M);
-                            const int up = (int)(q >> 63);
-                            q = up ? q : q << 1;
-                            f = __longlong_as_double((long long)fx_pack(q, ixV.e - d.e - 1 + up));
-                        } else {
-                            f = V_dt / __longlong_as_double(db);
-                        }
-                        c = __longlong_as_double(__double_as_longlong(dth) ^
-                                                 (__double_as_longlong(dh) & (long long)0x8000000000000000ULL)) * f;
-                    } else {
-                        c = V_dt * cur.can;
-                    }
-                    s0 = c * cur.hn;
-                }
+                storage_terms(form, *spp, V_dt, eps, hkP, cur.hn, cur.thk, cur.thn, cur.can, thp, p, c, s0);
                 const long long kxm = sK[buf][ty + 1][tx], kxp = sK[buf][ty + 1][tx + 2];
                 const long long kym = sK[buf][ty][tx + 1], kyp = sK[buf][ty + 2][tx + 1];
-                const double T0 = face(kxm, Kc, hwx, g.hw[0]), T1 = face(Kc, kxp, hwx, g.hw[0]);
-                const double T2 = face(kym, Kc, hwy, g.hw[2]), T3 = face(Kc, kyp, hwy, g.hw[2]);
-                Ttop = face(Kc, Kn, hwz, g.hw[4]);
+                const double T0 = face_coef(g, kxm, Kc, g.hw[0], hwx), T1 = face_coef(g, Kc, kxp, g.hw[0], hwx);
+                const double T2 = face_coef(g, kym, Kc, g.hw[2], hwy), T3 = face_coef(g, Kc, kyp, g.hw[2], hwy);
+                Ttop = face_coef(g, Kc, Kn, g.hw[4], hwz);
                 const double hz = Kn >= 0 ? hu : 0.0;
                 double diag = c + (((T0 + T1) + (T2 + T3)) + (Tbot + Ttop));
                 double rhs = fma(Ttop, g.gd[F_ZMAX], fma(Tbot, g.gd[F_ZMIN], s0));   // explicit gravity
@@ -500,18 +458,12 @@ k_assemble_tiled(Grid g, Tiles tw, const DevSoil *__restrict__ soils, const uint
                 Tx[p] = T1;
                 Ty[p] = T3;
                 Tz[p] = Ttop;
-                const long long gb = __double_as_longlong(diag);
-                double di = 0.0;
                 float di32;
+                double di = 0.0;
                 if (MODE == ASM_MIXED) {
                     di32 = __frcp_rn(ix_d2f(diag));
                 } else {
-                    if ((unsigned)(gb >> 52) - 400u < 1200u) {
-                        const IxNum d = ix_unpack((uint64_t)gb);
-                        di = __longlong_as_double((long long)fx_pack(ix_rcp(d.M), -1 - d.e));
-                    } else {
-                        di = 1.0 / diag;
-                    }
+                    di = ix_rcp64(diag);
                     dinv[p] = di;
                     di32 = ix_d2f(di);
                 }
@@ -530,9 +482,9 @@ k_assemble_tiled(Grid g, Tiles tw, const DevSoil *__restrict__ soils, const uint
                         v[1] = fma(rp, rp, v[1]);
                         v[2] = fma(rhs, rhs, v[2]);
                     } else {
-                        const float rf = (float)rp;
+                        const float rf = ix_d2f(rp);
                         const float zf = di32 * rf;
-                        const float bf = (float)rhs;
+                        const float bf = ix_d2f(rhs);
                         st.r32[p] = rf;
                         st.z32[p] = zf;
                         st.d32[p] = 0.0f;
@@ -745,8 +697,6 @@ void launch_closure_picard(cudaStream_t s, int nblk, const Grid &g, const DevSoi
 // latency and the general kernel's one cell per thread is the shorter chain).
 static bool assemble_tiled(const Grid &g)
 {
-    for (double hw : g.hw)
-        if (!(hw > 1e-90 && hw < 1e90)) return false;     // products of the integer form stay in the normal range
     return g.nx >= 16 && g.ny >= 4 && g.N >= 32768;
 }
 

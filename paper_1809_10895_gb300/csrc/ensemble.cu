@@ -704,10 +704,13 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
             status = ENS_RUNNING;
         }
         bool closure_valid = true;
-        auto sqrt3 = [](const double (&t)[4], double *o) {
-            o[0] = sqrt(t[0]);
-            o[1] = sqrt(t[1]);
-            o[2] = sqrt(t[2]);
+        // of the reduced (r.r, b.b, r.z): whether the residual meets the
+        // tolerance, by squares, and the inner solve's FP32 threshold.  One
+        // thread derives them: an FP64 root is some fifteen dependent
+        // instructions of 64 cycles.
+        auto converged = [&](double rr, double bb, double tol) { return rr <= tol * tol * bb ? 1.0 : 0.0; };
+        auto inner_stop = [&](double rr) {
+            return P.tol_inner * (rr > 1e-30 && rr < 1e30 ? (double)sqrtf((float)rr) : sqrt(rr));
         };
 
         while (status == ENS_RUNNING && t < t_end - t_tol_d(t_end)) {
@@ -736,25 +739,28 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                     const double *hk = H[hkb], *hn = H[hb];
                     double *x = H[xb];
                     // ---- assembly + first residual (Sec. 2.2)
-                    double v[4] = {0.0, 0.0, 0.0, 0.0};
+                    double v[3] = {0.0, 0.0, 0.0};   // r.r, b.b, r.z
                     for (long long p = lo + threadIdx.x; p < hi; p += blockDim.x) {
                         int i, j, k;
                         cell_ijk(g, p, i, j, k);
                         CellSystem cs;
                         assemble_cell<true>(g, soil, zn, Ks, fl[p], sp, p, i, j, k, hk, hn, TH[tn ^ 1], TH[tn],
                                             KB[kin], Can, nullptr, P.eps_chord, V_dt, cs);
-                        const double di = rcp64(cs.diag);
+                        const double di = PREC == 0 ? ix_rcp64(cs.diag) : 0.0;   // the mixed path's scaling is FP32
                         cc[p] = cs.c;
                         bb[p] = cs.rhs;
                         Tx[p] = cs.Tup[0];
                         Ty[p] = cs.Tup[1];
                         Tz[p] = cs.Tup[2];
                         dg[p] = cs.diag;
-                        dinv[p] = di;
-                        K32[p] = (float)cs.KP;
-                        cb32[p] = (float)cs.cb;
-                        const float d32v = (float)di;
-                        di32[p] = d32v;
+                        const float d32v = PREC == 0 ? 0.0f : __frcp_rn(ix_d2f(cs.diag));
+                        if (PREC == 0) {
+                            dinv[p] = di;
+                        } else {
+                            K32[p] = ix_d2f(cs.KP);
+                            cb32[p] = ix_d2f(cs.cb);
+                            di32[p] = d32v;
+                        }
                         const double hkP = hk[p];
                         const double rp = cs.rhs - (cs.diag * hkP - cs.sT);
                         x[p] = hkP;
@@ -762,32 +768,34 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                             const double zp = di * rp;
                             r64[p] = rp;
                             z64[p] = zp;
-                            v[0] += rp * zp;
-                            v[1] += rp * rp;
-                            v[2] += cs.rhs * cs.rhs;
+                            v[0] = fma(rp, rp, v[0]);
+                            v[1] = fma(cs.rhs, cs.rhs, v[1]);
+                            v[2] = fma(rp, zp, v[2]);
                         } else {
                             const float rf = (float)rp;
                             const float zf = d32v * rf;
                             r32[p] = rf;
                             z32[p] = zf;
                             d32[p] = 0.0f;
-                            v[0] += rp * rp;
-                            v[1] += cs.rhs * cs.rhs;
-                            v[2] += (double)(rf * rf);
-                            v[3] += (double)(rf * zf);
+                            v[0] = fma(rp, rp, v[0]);
+                            v[1] = fma(cs.rhs, cs.rhs, v[1]);
+                            if (!P.zline) v[2] += (double)(rf * zf);   // the line solve derives its own
                         }
                     }
-                    double sq[3];   // square roots of the first three sums
-                    cl_reduce<OpSum, 4, 3>(C, v, sq, sqrt3);
+                    double sq[2];   // converged, inner threshold
+                    cl_reduce<OpSum, 3, 2>(C, v, sq, [&](const double (&t)[3], double *o) {
+                        o[0] = converged(t[0], t[1], P.tol_cg);
+                        o[1] = PREC == 0 ? P.tol_cg * P.tol_cg * t[1] : inner_stop(t[0]);
+                    });
                     int cg_it = 0;
                     bool lin_ok = true;
                     if (PREC == 0) {
                         // ---- FP64 Jacobi-PCG
-                        double rho = v[0];
-                        const double stop = P.tol_cg * sq[2];
+                        double rho = v[2];
+                        const double stop2 = sq[1];
                         bool done = !(isfinite(v[0]) && isfinite(v[1]) && isfinite(v[2]));
                         if (done) lin_ok = false;
-                        else done = sq[1] <= stop;
+                        else done = sq[0] != 0.0;
                         double beta = 0.0;
                         int pi = 0;
                         while (!done) {
@@ -818,7 +826,7 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                             }
                             double fb[2];   // stop test passed (1 or 0), beta
                             cl_reduce<OpSum, 2, 2>(C, w2, fb, [&](const double (&t)[2], double *o) {
-                                o[0] = sqrt(t[0]) <= stop ? 1.0 : 0.0;
+                                o[0] = t[0] <= stop2 ? 1.0 : 0.0;
                                 o[1] = t[1] / rho;
                             });
                             cg_it++;
@@ -835,21 +843,21 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                         if (P.zline) zline_factor32(C, geo32(g), K32, cb32, LTi, LTc, LTP, LTQ, LTR);
                         int outer = 1;
                         for (;;) {
-                            const bool finite = isfinite(v[0]) && isfinite(v[1]) && isfinite(v[2]) && isfinite(v[3]);
+                            const bool finite = isfinite(v[0]) && isfinite(v[1]) && isfinite(v[2]);
                             if (!finite) { lin_ok = false; break; }
-                            if (sq[0] <= P.tol_cg * sq[1]) break;
+                            if (sq[0] != 0.0) break;
                             if (outer >= P.outer_max_it) { lin_ok = false; break; }
                             // inner solve A d = r32 from d = 0, FP32 throughout
                             int inner_it = 0;
-                            if (v[2] > 0.0) {
-                                const float stop = (float)(P.tol_inner * sq[2]);
+                            if (v[0] > 0.0) {
+                                const float stop = (float)sq[1];
                                 lin_ok = P.zline
                                              ? inner_pcg32<true>(C, geo32(g), (int)lo, (int)hi, K32, cb32, di32, r32,
                                                                  z32, P32[0], P32[1], q32, d32, LTi, LTc, LTP, LTQ,
                                                                  LTR, 0.0f, stop, P.inner_max_it, inner_it)
                                              : inner_pcg32<false>(C, geo32(g), (int)lo, (int)hi, K32, cb32, di32, r32,
                                                                   z32, P32[0], P32[1], q32, d32, nullptr, nullptr,
-                                                                  nullptr, nullptr, nullptr, (float)v[3], stop,
+                                                                  nullptr, nullptr, nullptr, (float)v[2], stop,
                                                                   P.inner_max_it, inner_it);
                             }
                             cg_it += inner_it;
@@ -857,7 +865,8 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                             for (long long p = lo + threadIdx.x; p < hi; p += blockDim.x) x[p] += (double)d32[p];
                             unit_sync(C);
                             // FP64 outer residual and new inner seeds
-                            v[0] = v[1] = v[2] = v[3] = 0.0;
+                            // (b.b stays in v[1])
+                            double w[2] = {0.0, 0.0};
                             for (long long p = lo + threadIdx.x; p < hi; p += blockDim.x) {
                                 const double bp = bb[p];
                                 const double rp = bp - apply64(g, p, Tx, Ty, Tz, dg, [&](long long qq) { return x[qq]; });
@@ -866,12 +875,16 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                                 r32[p] = rf;
                                 z32[p] = zf;
                                 d32[p] = 0.0f;
-                                v[0] += rp * rp;
-                                v[1] += bp * bp;
-                                v[2] += (double)(rf * rf);
-                                v[3] += (double)(rf * zf);
+                                w[0] = fma(rp, rp, w[0]);
+                                if (!P.zline) w[1] += (double)(rf * zf);
                             }
-                            cl_reduce<OpSum, 4, 3>(C, v, sq, sqrt3);
+                            const double bb = v[1];
+                            cl_reduce<OpSum, 2, 2>(C, w, sq, [&](const double (&t)[2], double *o) {
+                                o[0] = converged(t[0], bb, P.tol_cg);
+                                o[1] = inner_stop(t[0]);
+                            });
+                            v[0] = w[0];
+                            v[2] = w[1];
                             outer++;
                         }
                     }

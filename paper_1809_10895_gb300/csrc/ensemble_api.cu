@@ -275,10 +275,9 @@ rf_status rf_ens_create(const rf_ens_instance *inst, int n, const rf_solver_para
             g.w[f] = A[f] / dd[f];
             g.wb[f] = A[f] / (0.5 * dd[f]);
             g.hw[f] = 0.5 * (A[f] / dd[f]);
-            g.gf[f] = f == F_ZMIN ? -1.0 : (f == F_ZMAX ? 1.0 : 0.0);
-            g.hg[f] = 0.5 * A[f] * g.gf[f];
         }
-        // closures in FP64 on the plain path, double-float inside the mixed one (AUTO)
+        const double up[3] = {0.0, 0.0, 1.0};
+        set_grid_gravity(g, up, false);
         g.closure64 = prm.closure_arith != RF_CLOSURE_DOUBLE_FLOAT ? 1 : 0;
         for (int ax = 0; ax < 3; ax++) g.w32[ax] = (float)(A[2 * ax] / dd[2 * ax]);
         g.fx = make_fastdiv((unsigned int)a.nx);

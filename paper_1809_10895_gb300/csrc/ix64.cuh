@@ -67,14 +67,15 @@ __device__ __forceinline__ uint64_t ix_rcp(uint64_t M)
     return ((uint64_t)ri << 32) + (uint64_t)(t << 1);
 }
 
-// The float nearest to a non-negative double (ties to even).
+// The float nearest to a double (ties to even).
 __device__ __forceinline__ float ix_d2f(double a)
 {
     const uint64_t b = (uint64_t)__double_as_longlong(a);
-    const uint32_t ex = (uint32_t)(b >> 52);
-    if (ex - 897u > 253u) return (float)a;        // zero, subnormal or infinite as a float
-    const uint64_t v = b - (896ULL << 52);
-    return __uint_as_float((uint32_t)((v + 0x0fffffffULL + ((v >> 29) & 1)) >> 29));
+    const uint32_t ex = (uint32_t)(b >> 52) & 0x7ffu;
+    if (ex - 897u > 253u) return (float)a;        // zero, subnormal, infinite or NaN as a float
+    const uint64_t v = (b & 0x7fffffffffffffffULL) - (896ULL << 52);
+    return __uint_as_float((uint32_t)((v + 0x0fffffffULL + ((v >> 29) & 1)) >> 29) |
+                           ((uint32_t)(b >> 32) & 0x80000000u));
 }
 #endif
 

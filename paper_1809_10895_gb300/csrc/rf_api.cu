@@ -188,14 +188,7 @@ rf_status check_params(const rf_solver_params *p)
 // the interface mean and the closure arithmetic.
 void apply_grid_params(Grid &g, const rf_solver_params &p)
 {
-    const double gv[6] = {-p.grav[0], p.grav[0], -p.grav[1], p.grav[1], -p.grav[2], p.grav[2]};
-    for (int f = 0; f < 6; f++) {
-        g.gf[f] = gv[f];
-        g.hg[f] = 0.5 * g.A[f] * gv[f];
-        g.gd[f] = gv[f] * (g.A[f] / g.w[f]);
-    }
-    g.tilted = (p.grav[0] != 0.0 || p.grav[1] != 0.0) ? 1 : 0;
-    g.harmonic = p.face_mean == RF_FACE_HARMONIC ? 1 : 0;
+    set_grid_gravity(g, p.grav, p.face_mean == RF_FACE_HARMONIC);
     // AUTO: the fixed-point form serves both precisions (it is faster than the
     // double-float one as well: 224 against 334 us on 6 M active cells)
     g.closure64 = p.closure_arith != RF_CLOSURE_DOUBLE_FLOAT ? 1 : 0;

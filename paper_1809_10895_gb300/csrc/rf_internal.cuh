@@ -79,13 +79,13 @@ struct Grid {
     double wb[6];     // A/(d/2) for boundary (half-cell) faces
     double hw[6];     // A/(2 d): T_f = (K_P + K_N) hw_f
     double gf[6];     // gravity flux factor of each face, grad(elevation) . n_out: (-gx, gx, -gy, gy, -gz, gz)
-    double hg[6];     // gf A / 2: explicit gravity of an interior face is (K_P + K_N) hg_f
     double gd[6];     // gf d: gravity through an interior face is T_f gd_f
     float w32[3];     // A/d per axis, FP32 (mixed-precision operator)
     FastDiv fx, fxy;  // division by nx and by nx*ny
     int cap;          // most blocks a tiled stencil kernel launches (partials hold 8 values per block)
     int closure64;    // 1: closures to FP64 accuracy (fixed point, else FP64); 0: double-float arithmetic
     int tilted;       // 1: the elevation gradient has x / y components (gravity on lateral faces)
+    int ix_ok;        // 1: arithmetic mean and A/(2 d) within the range of the integer face arithmetic
     int harmonic;     // 1: harmonic interface conductivity; 0: arithmetic mean (linear interpolation)
     int wait_tries;   // polls of a bounded device wait before it gives up (set for tests; 0: default)
     const FFTables *tab;       // double-float exp/log tables (device)
@@ -168,6 +168,20 @@ struct StepResults {
 };
 
 constexpr int RED_THREADS = 256;
+
+// Fields that follow from gravity, the interface mean and the face areas.
+inline void set_grid_gravity(Grid &g, const double grav[3], bool harmonic)
+{
+    const double gv[6] = {-grav[0], grav[0], -grav[1], grav[1], -grav[2], grav[2]};
+    g.ix_ok = harmonic ? 0 : 1;
+    for (int f = 0; f < 6; f++) {
+        g.gf[f] = gv[f];
+        g.gd[f] = gv[f] * (g.A[f] / g.w[f]);
+        if (!(g.hw[f] > 1e-90 && g.hw[f] < 1e90)) g.ix_ok = 0;
+    }
+    g.tilted = (grav[0] != 0.0 || grav[1] != 0.0) ? 1 : 0;
+    g.harmonic = harmonic ? 1 : 0;
+}
 
 #ifdef __CUDACC__
 __device__ __forceinline__ void count_launch(const Grid &g, int kind)
