@@ -373,7 +373,10 @@ k_attempt_small(const __grid_constant__ AttemptArgs A)
                 for (int p = p0; p < N; p += stride) {
                     if (!(A.flags[p] & FLAG_ACTIVE)) continue;
                     const double bp = A.b[p];
-                    const double rp = bp - apply64(g, p, A.Tx, A.Ty, A.Tz, A.diag, [&](long long q) { return x[q]; });
+                    // an inactive neighbour's head may be anything; its face's T = 0 needs a number
+                    const double rp = bp - apply64(g, p, A.Tx, A.Ty, A.Tz, A.diag, [&](long long q) {
+                                          return (A.flags[q] & FLAG_ACTIVE) ? x[q] : 0.0;
+                                      });
                     const float rf = (float)rp, zf = A.dinv32[p] * rf, bf = (float)bp;
                     A.r32[p] = rf;
                     A.z32[p] = zf;

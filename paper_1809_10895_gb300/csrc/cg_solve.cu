@@ -1,0 +1,348 @@
+// cg_solve.cu -- a whole Jacobi-PCG solve in one cooperative launch: FP64, or
+// FP32 inside FP64 defect correction.
+//
+// As two kernels per iteration inside a conditional graph node, an iteration
+// costs 18 us of node latency beside the kernels' own time.  Here the blocks
+// stay resident: stencil products, updates and outer residuals are phases of
+// one loop, each ended by a grid reduction (grid_red.cuh), and every block
+// derives alpha, beta and the stop tests itself.  The sweeps: sweeps.cuh.
+#include <algorithm>
+
+#include "cell_ops.cuh"
+#include "grid_red.cuh"
+#include "rf_internal.cuh"
+#include "sweeps.cuh"
+
+namespace rf {
+
+namespace {
+
+struct CgShared {
+    union {
+        Sweep64Shared w64;
+        Sweep32Shared w32;
+        double part[2][CT];                        // between sweeps
+    };
+    float partf[3][CT / 32];
+    double tot[4];
+    double alpha, beta, rho, stop2;
+    int done, status, iter, abort;
+};
+
+// The block's sum of its threads' values, by one warp per value.
+template <int NV, class Fin>
+__device__ __forceinline__ bool cg_reduce(GridRed &R, CgShared &s, const double (&v)[NV], Fin fin)
+{
+#pragma unroll
+    for (int i = 0; i < NV; i++) s.part[i][threadIdx.x] = v[i];
+    __syncthreads();
+    return grid_red<OpSum, NV>(
+        R, s.tot, &s.abort,
+        [&](int i) {
+            const double *p = &s.part[i][threadIdx.x & 31];
+            return warp_reduce<OpSum>(((p[0] + p[32]) + (p[64] + p[96])) + ((p[128] + p[160]) + (p[192] + p[224])));
+        },
+        fin);
+}
+
+__global__ void __launch_bounds__(CT, SWEEP_OCC)
+k_cg64_solve(Grid g, Tiles tw, const double *__restrict__ Tx, const double *__restrict__ Ty,
+             const double *__restrict__ Tz, const double *__restrict__ diag, const double *__restrict__ dinv,
+             double *x, double *r, double *z, double *p0, double *p1, double *q, void *red, int *fault, CgScal *sc)
+{
+    count_launch(g, KK_ONE_LAUNCH);
+    if (sc->done) return;                          // converged at the start, or the Picard attempt is over
+    count_work(g, KK_ONE_LAUNCH);
+    __shared__ CgShared s;
+    GridRed R = grid_red_begin(red, fault, g.wait_tries);
+    const double stop2 = sc->stop2;
+    const int max_it = sc->max_it;
+    if (threadIdx.x == 0) {
+        s.rho = sc->rho;
+        s.beta = 0.0;
+        s.done = 0;
+        s.status = CG_OK;
+        s.abort = 0;
+    }
+    __syncthreads();
+    const Op64 A{Tx, Ty, Tz, diag};
+    int it = 0;
+    for (;;) {
+        const double beta = s.beta;
+        const bool first = it == 0;
+        const double *pin = (it & 1) ? p1 : p0;
+        double *pout = (it & 1) ? p0 : p1;
+        double acc[1] = {0.0};
+        // ---- p = z + beta p_old, q = A p, p.q
+        struct Raw {
+            double z, o;
+        };
+        sweep64<Raw>(
+            g, tw, A, s.w64, [&](long long c) { return Raw{__ldcs(&z[c]), first ? 0.0 : __ldcs(&pin[c])}; },
+            [&](const Raw &a) { return fma(beta, a.o, a.z); },
+            [&](long long c, double v, double Av, bool) {
+                pout[c] = v;
+                q[c] = Av;
+                acc[0] = fma(v, Av, acc[0]);
+            });
+        if (!cg_reduce<1>(R, s, acc, [&]() {
+                const double pq = s.tot[0];
+                s.alpha = s.rho / pq;
+                if (!(pq > 0.0) || !isfinite(s.alpha)) {
+                    s.status = CG_NONFINITE;
+                    s.done = 1;
+                }
+            }))
+            break;
+        if (s.done) break;
+        // ---- x += alpha p, r -= alpha q, z = D^-1 r, r.r, r.z
+        const double alpha = s.alpha;
+        double v[2] = {0.0, 0.0};
+        cg64_update_cells(g, alpha, dinv, pout, q, x, r, z, v);
+        it++;
+        if (!cg_reduce<2>(R, s, v, [&]() {
+                const double rr = s.tot[0], rz = s.tot[1];
+                if (!isfinite(rr) || !isfinite(rz)) {
+                    s.status = CG_NONFINITE;
+                    s.done = 1;
+                } else if (sqrt(rr) <= stop2) {
+                    s.done = 1;
+                } else if (it >= max_it) {
+                    s.status = CG_MAXIT;
+                    s.done = 1;
+                } else {
+                    s.beta = rz / s.rho;
+                    s.rho = rz;
+                }
+            }))
+            break;
+        if (s.done) break;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        sc->iter = it;
+        sc->total = it;
+        sc->rho = s.rho;
+        sc->rr = s.tot[0];
+        sc->status = s.abort ? CG_NONFINITE : s.status;
+        sc->done = 1;
+    }
+}
+
+// FP32 sums within the block, FP64 across blocks.
+template <int NV, class Fin>
+__device__ __forceinline__ bool cg_reduce_f32(GridRed &R, CgShared &s, float (&v)[NV], Fin fin)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < NV; i++) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+        if (lane == 0) s.partf[i][wid] = v[i];
+    }
+    __syncthreads();
+    return grid_red<OpSum, NV>(
+        R, s.tot, &s.abort,
+        [&](int i) {
+            const float *p = s.partf[i];
+            return (double)(((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7])));
+        },
+        fin);
+}
+
+// Defect correction from the assembly's (or the start kernels') first
+// residual: outer and inner hold its scalars.
+struct MixedArgs {
+    Grid g;
+    Tiles t64, t32;
+    const uint8_t *flags;
+    const double *Tx, *Ty, *Tz, *diag, *b;
+    const float *K32, *cb32, *dinv32;
+    double *x;
+    float *r32, *z32, *d32, *p0, *p1, *q32;
+    void *red;
+    int *fault;
+    CgScal *outer, *inner;
+    double tol, tol_inner;
+    int inner_max_it, outer_max_it;
+};
+
+__global__ void __launch_bounds__(CT, SWEEP_OCC)
+k_mixed_solve(const __grid_constant__ MixedArgs M)
+{
+    const Grid &g = M.g;
+    count_launch(g, KK_ONE_LAUNCH);
+    if (M.outer->done) return;
+    count_work(g, KK_ONE_LAUNCH);
+    __shared__ CgShared s;
+    GridRed R = grid_red_begin(M.red, M.fault, g.wait_tries);
+    if (threadIdx.x == 0) {
+        s.rho = M.inner->rho;
+        s.stop2 = M.inner->stop2;
+        s.beta = 0.0;
+        s.iter = !M.inner->done;                   // an inner solve is due
+        s.done = 0;
+        s.status = CG_OK;
+        s.abort = 0;
+    }
+    __syncthreads();
+    const long long N = g.N, n4 = N / 4, stride = (long long)gridDim.x * CT;
+    const long long t0 = (long long)blockIdx.x * CT + threadIdx.x;
+    int outer = M.outer->iter, total = 0;
+    for (;;) {
+        // ---- inner FP32 PCG, A d = r from d = 0
+        int it = 0;
+        while (s.iter) {
+            const float beta = (float)s.beta;
+            const bool first = it == 0;
+            const float *pin = (it & 1) ? M.p1 : M.p0;
+            float *pout = (it & 1) ? M.p0 : M.p1;
+            float w[1] = {sweep32(g, M.t32, s.w32, M.K32, M.cb32, M.z32, pin, pout, M.q32, beta, first)};
+            if (!cg_reduce_f32<1>(R, s, w, [&]() {
+                    const double pq = s.tot[0];
+                    s.alpha = s.rho / pq;
+                    if (!(pq > 0.0) || !isfinite(s.alpha)) s.status = CG_NONFINITE;
+                }))
+                break;
+            if (s.status != CG_OK) break;
+            const float alpha = (float)s.alpha;
+            float v[2] = {0.0f, 0.0f};
+            cg32_update_cells(g, alpha, first, M.dinv32, pout, M.q32, M.d32, M.r32, M.z32, v);
+            it++;
+            if (!cg_reduce_f32<2>(R, s, v, [&]() {
+                    const double rr = s.tot[0], rz = s.tot[1];
+                    if (!isfinite(rr) || !isfinite(rz)) s.status = CG_NONFINITE;
+                    else if (sqrt(rr) <= s.stop2 || it >= M.inner_max_it) s.iter = 0;   // applied even at the cap
+                    else {
+                        s.beta = rz / s.rho;
+                        s.rho = rz;
+                    }
+                }))
+                break;
+            if (s.status != CG_OK) break;
+        }
+        total += it;
+        if (s.abort || s.status != CG_OK) break;
+        // ---- x += d
+        if (it > 0) {
+            for (long long u = t0; u < n4; u += stride) {
+                const float4 d = reinterpret_cast<const float4 *>(M.d32)[u];
+                double2 a = reinterpret_cast<double2 *>(M.x)[2 * u], c = reinterpret_cast<double2 *>(M.x)[2 * u + 1];
+                a.x += (double)d.x;
+                a.y += (double)d.y;
+                c.x += (double)d.z;
+                c.y += (double)d.w;
+                reinterpret_cast<double2 *>(M.x)[2 * u] = a;
+                reinterpret_cast<double2 *>(M.x)[2 * u + 1] = c;
+            }
+            for (long long c = 4 * n4 + t0; c < N; c += stride) M.x[c] += (double)M.d32[c];
+        }
+        __syncthreads();
+        if (gridDim.x > 1) {
+            if (threadIdx.x == 0 && !grid_red_wait(R)) s.abort = 1;
+            __syncthreads();
+            if (s.abort) break;
+        }
+        // ---- r = b - A x in FP64, seeds of the next inner solve
+        float f[3] = {0.0f, 0.0f, 0.0f};           // r.r, b.b, r.z
+        const Op64 A{M.Tx, M.Ty, M.Tz, M.diag};
+        resid64_sweep(g, M.t64, A, s.w64, M.flags, M.x, M.b, M.dinv32, M.r32, M.z32, nullptr, f);
+        outer++;
+        if (!cg_reduce_f32<3>(R, s, f, [&]() {
+                const double rr = s.tot[0], bb = s.tot[1], rz = s.tot[2];
+                const double rn = sqrt(rr);
+                if (!(isfinite(rr) && isfinite(bb) && isfinite(rz))) {
+                    s.status = CG_NONFINITE;
+                    s.done = 1;
+                } else if (rn <= M.tol * sqrt(bb)) {
+                    s.done = 1;
+                } else if (outer >= M.outer_max_it) {
+                    s.status = CG_MAXIT;
+                    s.done = 1;
+                }
+                s.rho = rz;
+                s.stop2 = M.tol_inner * rn;
+                s.beta = 0.0;
+                s.iter = rr > 0.0;
+            }))
+            break;
+        if (s.done) break;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        M.outer->iter = outer;
+        M.outer->status = s.abort ? CG_NONFINITE : s.status;
+        M.outer->done = 1;
+        M.inner->total += total;
+        M.inner->done = 1;
+    }
+}
+
+}  // namespace
+
+// Blocks of the solve on this grid (0: it cannot run): what fits the GPU at
+// once, but no more than there are tiles and planes to share out.
+int cg64_solve_blocks(const Grid &g, int sms)
+{
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg64_solve, CT, 0) != cudaSuccess || occ < 1) return 0;
+    return std::min(occ * sms, GR_BLOCKS);
+}
+
+cudaError_t launch_cg64_solve(cudaStream_t s, int blocks, const Grid &g, const double *Tx, const double *Ty,
+                              const double *Tz, const double *diag, const double *dinv, double *x, double *r,
+                              double *z, double *p0, double *p1, double *q, void *red, int *fault, CgScal *sc)
+{
+    Grid gg = g;
+    Tiles tw = make_tiles_balanced(g, blocks, CX, CY);
+    blocks = (int)std::min<long long>(blocks, tw.items);
+    void *args[] = {&gg, &tw, &Tx, &Ty, &Tz, &diag, &dinv, &x, &r, &z, &p0, &p1, &q, &red, &fault, &sc};
+    return cudaLaunchCooperativeKernel((void *)k_cg64_solve, dim3((unsigned)blocks), dim3(CT), args, 0, s);
+}
+
+int mixed_solve_blocks(const Grid &g, int sms)
+{
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_mixed_solve, CT, 0) != cudaSuccess || occ < 1) return 0;
+    return std::min(occ * sms, GR_BLOCKS);
+}
+
+cudaError_t launch_mixed_solve(cudaStream_t s, int blocks, const Grid &g, const uint8_t *flags, const double *Tx,
+                               const double *Ty, const double *Tz, const double *diag, const double *b,
+                               const float *K32, const float *cb32, const float *dinv32, double *x, float *r32,
+                               float *z32, float *d32, float *p0, float *p1, float *q32, void *red, int *fault,
+                               CgScal *outer, CgScal *inner, double tol, double tol_inner, int inner_max_it,
+                               int outer_max_it)
+{
+    MixedArgs M{};
+    M.g = g;
+    M.t64 = make_tiles_balanced(g, blocks, CX, CY);
+    M.t32 = make_tiles_balanced(g, blocks, CX, FY);
+    M.flags = flags;
+    M.Tx = Tx;
+    M.Ty = Ty;
+    M.Tz = Tz;
+    M.diag = diag;
+    M.b = b;
+    M.K32 = K32;
+    M.cb32 = cb32;
+    M.dinv32 = dinv32;
+    M.x = x;
+    M.r32 = r32;
+    M.z32 = z32;
+    M.d32 = d32;
+    M.p0 = p0;
+    M.p1 = p1;
+    M.q32 = q32;
+    M.red = red;
+    M.fault = fault;
+    M.outer = outer;
+    M.inner = inner;
+    M.tol = tol;
+    M.tol_inner = tol_inner;
+    M.inner_max_it = inner_max_it;
+    M.outer_max_it = outer_max_it;
+    blocks = (int)std::min<long long>(blocks, std::max(M.t64.items, M.t32.items));
+    void *args[] = {&M};
+    return cudaLaunchCooperativeKernel((void *)k_mixed_solve, dim3((unsigned)blocks), dim3(CT), args, 0, s);
+}
+
+}  // namespace rf

@@ -21,7 +21,9 @@
 #include <mutex>
 
 #include "rf.h"
+#include "cell_ops.cuh"
 #include "rf_internal.cuh"
+#include "rf_reduce.cuh"
 
 using namespace rf;
 
@@ -71,6 +73,79 @@ __global__ void k_noalloc_setup(long long N, const double *__restrict__ diag, do
         dinv[p] = act ? 1.0 / d : 0.0;
         flags[p] = act ? FLAG_ACTIVE : 0;
     }
+}
+
+// The two kernels of an iteration, one cell per thread: the caller's arrays
+// may sit on any 8-byte boundary and may hold anything next to inactive cells,
+// unlike a context's, so the tiled, vectorised forms do not serve them, and at
+// this size (a few MB in L2) they would gain nothing.
+__global__ void __launch_bounds__(RED_THREADS)
+k_noalloc_spmv(Grid g, const uint8_t *__restrict__ flags, const double *__restrict__ z,
+               const double *__restrict__ p_in, double *__restrict__ p_out, double *__restrict__ q,
+               const double *__restrict__ Tx, const double *__restrict__ Ty, const double *__restrict__ Tz,
+               const double *__restrict__ diag, double *partials, unsigned int *ticket, CgScal *sc)
+{
+    if (sc->done) return;
+    const double beta = sc->beta;
+    const bool first = sc->iter == 0;
+    auto val = [&](long long c) { return first ? z[c] : fma(beta, p_in[c], z[c]); };
+    double v[1] = {0.0};
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < g.N; p += stride) {
+        if (!(flags[p] & FLAG_ACTIVE)) {
+            p_out[p] = 0.0;
+            q[p] = 0.0;
+            continue;
+        }
+        int i, j, k;
+        cell_ijk(g, p, i, j, k);
+        const double pp = val(p);
+        double acc = diag[p] * pp;
+        auto face = [&](bool in, long long n, const double *T, long long at) {
+            if (in && (flags[n] & FLAG_ACTIVE)) acc = fma(-T[at], val(n), acc);
+        };
+        face(i > 0, p - 1, Tx, p - 1);
+        face(i < g.nx - 1, p + 1, Tx, p);
+        face(j > 0, p - g.nx, Ty, p - g.nx);
+        face(j < g.ny - 1, p + g.nx, Ty, p);
+        face(k > 0, p - g.sxy, Tz, p - g.sxy);
+        face(k < g.nz - 1, p + g.sxy, Tz, p);
+        p_out[p] = pp;
+        q[p] = acc;
+        v[0] = fma(pp, acc, v[0]);
+    }
+    if (grid_reduce<OpSum, 1>(v, partials, ticket) && threadIdx.x == 0) {
+        sc->pq = v[0];
+        const double a = sc->rho / v[0];
+        if (!(v[0] > 0.0) || !isfinite(a)) {
+            sc->status = CG_NONFINITE;
+            sc->done = 1;
+        }
+        sc->alpha = a;
+    }
+}
+
+__global__ void __launch_bounds__(RED_THREADS)
+k_noalloc_update(Grid g, double *__restrict__ x, double *__restrict__ r, double *__restrict__ z,
+                 const double *__restrict__ pd, const double *__restrict__ q, const double *__restrict__ dinv,
+                 double *partials, unsigned int *ticket, CgScal *sc)
+{
+    if (sc->done) return;
+    const double alpha = sc->alpha;
+    double v[2] = {0.0, 0.0};   // r.r, r.z
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < g.N; p += stride) {
+        const double di = dinv[p];
+        if (di == 0.0) continue;                  // inactive
+        x[p] = fma(alpha, pd[p], x[p]);
+        const double rp = fma(-alpha, q[p], r[p]);
+        const double zp = di * rp;
+        r[p] = rp;
+        z[p] = zp;
+        v[0] = fma(rp, rp, v[0]);
+        v[1] = fma(rp, zp, v[1]);
+    }
+    if (grid_reduce<OpSum, 2>(v, partials, ticket) && threadIdx.x == 0) cg_update_scalars(sc, v);
 }
 
 rf_status noalloc_fail(rf_status s, const char *msg)
@@ -164,8 +239,9 @@ extern "C" rf_status rf_pcg_solve_noalloc(int nx, int ny, int nz, const double *
     for (;;) {
         for (int i = 0; i < chunk; i++, launched++) {
             double *pin = p[launched & 1], *pout = p[(launched + 1) & 1];
-            launch_cg64_spmv(s, nblk, g, flags, z, pin, pout, q, d_Tx, d_Ty, d_Tz, d_diag, partials, ticket, sc);
-            launch_cg64_update(s, nblk, g, d_x, r, z, pout, q, dinv, partials, ticket, sc, none);
+            k_noalloc_spmv<<<nblk, RED_THREADS, 0, s>>>(g, flags, z, pin, pout, q, d_Tx, d_Ty, d_Tz, d_diag, partials,
+                                                        ticket, sc);
+            k_noalloc_update<<<nblk, RED_THREADS, 0, s>>>(g, d_x, r, z, pout, q, dinv, partials, ticket, sc);
         }
         if (cudaGetLastError() != cudaSuccess)
             return noalloc_fail(RF_ERR_CUDA, "rf_pcg_solve_noalloc: kernel launch failed");

@@ -24,6 +24,7 @@
 #include "cell_ops.cuh"
 #include "rf_internal.cuh"
 #include "rf_reduce.cuh"
+#include "sweeps.cuh"
 #include "tiles.cuh"
 #include "tma.cuh"
 
@@ -73,162 +74,31 @@ k_cg64_init(Grid g, const uint8_t *__restrict__ flags, const double *__restrict_
         cg64_start_scalars(sc, v, tol, max_it, cond);
 }
 
-// One plane of the FP64 operator's face coefficients around a tile, staged by
-// the tiled FP64 kernels: Ty of rows j0-1 .. j0+TY-1 and Tx of the -x halo
-// column (the +x / +y / +z coefficients of a cell are its own).
-struct Faces64 {
-    double ty[2][TY + 1][TX];
-    double tx[2][TY];
-};
-
-// Stage the values v (own cell pc, halo via val) and face coefficients of
-// plane k; returns the cell's own coefficients (0 on inactive cells).
-template <class Val>
-__device__ __forceinline__ void stage64(const Grid &g, const TileItem &it, int k, int buf, int tx, int ty, int hx,
-                                        int hy, bool inside, long long c, const uint8_t *__restrict__ flags,
-                                        const double *__restrict__ Tx, const double *__restrict__ Ty,
-                                        const double *__restrict__ Tz, const double *__restrict__ diag, double pc,
-                                        Val val, double (&sP)[2][TY + 2][TX + 2], Faces64 &sF, bool &act,
-                                        double &dg, double &txp, double &typ, double &tzp)
-{
-    sP[buf][ty + 1][tx + 1] = pc;
-    act = inside && (flags[c] & FLAG_ACTIVE);
-    dg = txp = typ = tzp = 0.0;
-    if (act) {
-        dg = diag[c];
-        txp = Tx[c];
-        typ = Ty[c];
-        tzp = Tz[c];
-    }
-    sF.ty[buf][ty + 1][tx] = typ;
-    if (threadIdx.x < HALO) {
-        const int ii = it.i0 + hx, jj = it.j0 + hy;
-        const bool in = ii >= 0 && ii < g.nx && jj >= 0 && jj < g.ny;
-        const long long hc = ii + (long long)g.nx * jj + g.sxy * k;
-        const bool hact = in && (flags[hc] & FLAG_ACTIVE);
-        sP[buf][hy + 1][hx + 1] = hact ? val(hc) : 0.0;
-        if (hx == -1) sF.tx[buf][hy] = hact ? Tx[hc] : 0.0;
-        if (hy == -1) sF.ty[buf][0][hx] = hact ? Ty[hc] : 0.0;
-    }
-}
-
-// (A v)_P = diag_P v_P - sum_f T_f v_N with faces in the order -x +x -y +y -z +z.
-__device__ __forceinline__ double apply64_tile(const Grid &g, int i, int j, int k, int tx, int ty, int buf,
-                                               const double (&sP)[2][TY + 2][TX + 2], const Faces64 &sF,
-                                               double txm_lane, double dg, double txp, double typ, double tzm,
-                                               double tzp, double vm, double vc, double vn)
-{
-    const double txm = tx > 0 ? txm_lane : sF.tx[buf][ty];
-    double acc = dg * vc;
-    if (i > 0) acc -= txm * sP[buf][ty + 1][tx];
-    if (i < g.nx - 1) acc -= txp * sP[buf][ty + 1][tx + 2];
-    if (j > 0) acc -= sF.ty[buf][ty][tx] * sP[buf][ty][tx + 1];
-    if (j < g.ny - 1) acc -= typ * sP[buf][ty + 2][tx + 1];
-    if (k > 0) acc -= tzm * vm;
-    if (k < g.nz - 1) acc -= tzp * vn;
-    return acc;
-}
-
-__global__ void __launch_bounds__(RED_THREADS)
-k_cg64_spmv(Grid g, Tiles tw, const uint8_t *__restrict__ flags, const double *__restrict__ z,
-            const double *__restrict__ p_in, double *__restrict__ p_out, double *__restrict__ q,
-            const double *__restrict__ Tx, const double *__restrict__ Ty, const double *__restrict__ Tz,
-            const double *__restrict__ diag, double *partials, unsigned int *ticket, CgScal *sc)
+__global__ void __launch_bounds__(CT, SWEEP_OCC)
+k_cg64_spmv(Grid g, Tiles tw, const double *__restrict__ z, const double *__restrict__ p_in,
+            double *__restrict__ p_out, double *__restrict__ q, const double *__restrict__ Tx,
+            const double *__restrict__ Ty, const double *__restrict__ Tz, const double *__restrict__ diag,
+            double *partials, unsigned int *ticket, CgScal *sc)
 {
     count_launch(g, KK_CG64_SPMV);
     if (sc->done) return;
     count_work(g, KK_CG64_SPMV);
     const double beta = sc->beta;
     const bool first = sc->iter == 0;
-    auto val = [&](long long c) { return first ? z[c] : fma(beta, p_in[c], z[c]); };
-    // p = z + beta p_old on active cells of the grid, 0 elsewhere
-    auto pval = [&](int i, int j, int k) -> double {
-        if (i >= g.nx || j >= g.ny || k < 0 || k >= g.nz) return 0.0;
-        const long long c = i + (long long)g.nx * j + g.sxy * k;
-        return (flags[c] & FLAG_ACTIVE) ? val(c) : 0.0;
-    };
-    __shared__ double sP[2][TY + 2][TX + 2];
-    __shared__ Faces64 sF;
-    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-    int hx = 0, hy = 0;
-    if (threadIdx.x < HALO) halo_cell(threadIdx.x, hx, hy);
+    __shared__ Sweep64Shared s;
+    const Op64 A{Tx, Ty, Tz, diag};
     double v[1] = {0.0};
-    for (long long item = blockIdx.x; item < tw.items; item += gridDim.x) {
-        const TileItem it = tile_item(g, tw, item);
-        const int i = it.i0 + tx, j = it.j0 + ty;
-        const bool inside = i < g.nx && j < g.ny;
-        double pm = pval(i, j, it.k0 - 1), pc = pval(i, j, it.k0);
-        double tzm = 0.0;
-        if (inside && it.k0 > 0) {
-            const long long cm = i + (long long)g.nx * j + g.sxy * (it.k0 - 1);
-            tzm = (flags[cm] & FLAG_ACTIVE) ? Tz[cm] : 0.0;
-        }
-        // the plane's coefficients and halo, loaded a plane ahead so that
-        // their round trip overlaps the previous plane's work (the kernel is
-        // latency-bound: few FP64 instructions a cell, one barrier a plane)
-        struct Pl {
-            bool act, hact;
-            double dg, txp, typ, tzp, hp, htx, hty;
-        };
-        auto load = [&](int k, long long c) {
-            Pl l;
-            l.act = inside && (flags[c] & FLAG_ACTIVE);
-            l.dg = l.txp = l.typ = l.tzp = 0.0;
-            if (l.act) {
-                l.dg = diag[c];
-                l.txp = Tx[c];
-                l.typ = Ty[c];
-                l.tzp = Tz[c];
-            }
-            l.hact = false;
-            l.hp = l.htx = l.hty = 0.0;
-            if (threadIdx.x < HALO) {
-                const int ii = it.i0 + hx, jj = it.j0 + hy;
-                const bool in = ii >= 0 && ii < g.nx && jj >= 0 && jj < g.ny;
-                const long long hc = ii + (long long)g.nx * jj + g.sxy * k;
-                l.hact = in && (flags[hc] & FLAG_ACTIVE);
-                if (l.hact) {
-                    l.hp = val(hc);
-                    if (hx == -1) l.htx = Tx[hc];
-                    if (hy == -1) l.hty = Ty[hc];
-                }
-            }
-            return l;
-        };
-        Pl nxt = load(it.k0, i + (long long)g.nx * j + g.sxy * it.k0);
-        for (int k = it.k0; k < it.k1; k++) {
-            const int buf = k & 1;
-            const long long c = i + (long long)g.nx * j + g.sxy * k;
-            const Pl cur = nxt;
-            if (k + 1 < it.k1) nxt = load(k + 1, c + g.sxy);
-            sP[buf][ty + 1][tx + 1] = pc;
-            sF.ty[buf][ty + 1][tx] = cur.typ;
-            if (threadIdx.x < HALO) {
-                sP[buf][hy + 1][hx + 1] = cur.hp;
-                if (hx == -1) sF.tx[buf][hy] = cur.htx;
-                if (hy == -1) sF.ty[buf][0][hx] = cur.hty;
-            }
-            const bool act = cur.act;
-            const double dg = cur.dg, txp = cur.txp, typ = cur.typ, tzp = cur.tzp;
-            const double pn = pval(i, j, k + 1);
-            const double txm_lane = __shfl_up_sync(0xffffffffu, txp, 1);
-            __syncthreads();
-            if (act) {
-                const double acc = apply64_tile(g, i, j, k, tx, ty, buf, sP, sF, txm_lane, dg, txp, typ, tzm, tzp,
-                                                pm, pc, pn);
-                p_out[c] = pc;
-                q[c] = acc;
-                v[0] += pc * acc;
-            } else if (inside) {
-                p_out[c] = 0.0;
-                q[c] = 0.0;
-            }
-            tzm = tzp;
-            pm = pc;
-            pc = pn;
-        }
-        __syncthreads();
-    }
+    struct Raw {
+        double z, o;
+    };
+    sweep64<Raw>(
+        g, tw, A, s, [&](long long c) { return Raw{z[c], first ? 0.0 : p_in[c]}; },
+        [&](const Raw &a) { return fma(beta, a.o, a.z); },
+        [&](long long c, double pv, double Ap, bool) {
+            p_out[c] = pv;
+            q[c] = Ap;
+            v[0] = fma(pv, Ap, v[0]);
+        });
     if (grid_reduce<OpSum, 1>(v, partials, ticket) && threadIdx.x == 0) {
         sc->pq = v[0];
         const double a = sc->rho / v[0];
@@ -243,46 +113,14 @@ k_cg64_spmv(Grid g, Tiles tw, const uint8_t *__restrict__ flags, const double *_
 __global__ void __launch_bounds__(RED_THREADS)
 k_cg64_update(Grid g, double *__restrict__ x, double *__restrict__ r, double *__restrict__ z,
               const double *__restrict__ pd, const double *__restrict__ q, const double *__restrict__ dinv,
-              double *partials, unsigned int *ticket, CgScal *sc, CondSet cond)
+              double *partials, unsigned int *ticket, CgScal *sc)
 {
     count_launch(g, KK_CG64_UPDATE);
-    if (sc->done) {             // every launch sets the loop condition
-        if (blockIdx.x == 0 && threadIdx.x == 0) set_cond(cond, 0);
-        return;
-    }
+    if (sc->done) return;
     count_work(g, KK_CG64_UPDATE);
-    const double alpha = sc->alpha;
     double v[2] = {0.0, 0.0};   // r.r, r.z
-    GRID_STRIDE_LOOP(p)
-    {
-        const double di = dinv[p];
-        if (di == 0.0) continue;                  // inactive
-        x[p] = fma(alpha, pd[p], x[p]);
-        const double rp = fma(-alpha, q[p], r[p]);
-        const double zp = di * rp;
-        r[p] = rp;
-        z[p] = zp;
-        v[0] += rp * rp;
-        v[1] += rp * zp;
-    }
-    if (grid_reduce<OpSum, 2>(v, partials, ticket) && threadIdx.x == 0) {
-        sc->iter += 1;
-        sc->total += 1;
-        sc->rr = v[0];
-        if (!isfinite(v[0]) || !isfinite(v[1])) {
-            sc->status = CG_NONFINITE;
-            sc->done = 1;
-        } else if (sqrt(v[0]) <= sc->stop2) {
-            sc->done = 1;
-        } else if (sc->iter >= sc->max_it) {
-            sc->status = CG_MAXIT;
-            sc->done = 1;
-        } else {
-            sc->beta = v[1] / sc->rho;
-            sc->rho = v[1];
-        }
-        set_cond(cond, sc->done ? 0 : 1);
-    }
+    cg64_update_cells(g, sc->alpha, dinv, pd, q, x, r, z, v);
+    if (grid_reduce<OpSum, 2>(v, partials, ticket) && threadIdx.x == 0) cg_update_scalars(sc, v);
 }
 
 __global__ void __launch_bounds__(RED_THREADS)
@@ -325,7 +163,7 @@ k_mixed_start(Grid g, const double *__restrict__ x0, double *__restrict__ x, CgS
 // norms (a stopping test and CG seeds) are summed from the FP32 residual in
 // FP32 within a block, in FP64 across blocks.  Counts outer iterations and
 // fails the solve after outer_max_it residuals without convergence.
-__global__ void __launch_bounds__(RED_THREADS)
+__global__ void __launch_bounds__(CT, SWEEP_OCC)
 k_resid64(Grid g, Tiles tw, const uint8_t *__restrict__ flags, const double *__restrict__ x,
           const double *__restrict__ b, const double *__restrict__ Tx, const double *__restrict__ Ty,
           const double *__restrict__ Tz, const double *__restrict__ diag, const float *__restrict__ dinv32,
@@ -343,64 +181,10 @@ k_resid64(Grid g, Tiles tw, const uint8_t *__restrict__ flags, const double *__r
         return;
     }
     count_work(g, KK_RESID64);
-    auto val = [&](long long c) { return x[c]; };
-    auto xval = [&](int i, int j, int k) -> double {
-        if (i >= g.nx || j >= g.ny || k < 0 || k >= g.nz) return 0.0;
-        const long long c = i + (long long)g.nx * j + g.sxy * k;
-        return (flags[c] & FLAG_ACTIVE) ? x[c] : 0.0;
-    };
-    __shared__ double sP[2][TY + 2][TX + 2];
-    __shared__ Faces64 sF;
-    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-    int hx = 0, hy = 0;
-    if (threadIdx.x < HALO) halo_cell(threadIdx.x, hx, hy);
-    float a_rr = 0.0f, a_bb = 0.0f, a_rz = 0.0f;   // r32.r32, b.b, r32.z32
-    for (long long item = blockIdx.x; item < tw.items; item += gridDim.x) {
-        const TileItem it = tile_item(g, tw, item);
-        const int i = it.i0 + tx, j = it.j0 + ty;
-        const bool inside = i < g.nx && j < g.ny;
-        double xm = xval(i, j, it.k0 - 1), xc = xval(i, j, it.k0);
-        double tzm = 0.0;
-        if (inside && it.k0 > 0) {
-            const long long cm = i + (long long)g.nx * j + g.sxy * (it.k0 - 1);
-            tzm = (flags[cm] & FLAG_ACTIVE) ? Tz[cm] : 0.0;
-        }
-        for (int k = it.k0; k < it.k1; k++) {
-            const int buf = k & 1;
-            const long long c = i + (long long)g.nx * j + g.sxy * k;
-            bool act;
-            double dg, txp, typ, tzp;
-            stage64(g, it, k, buf, tx, ty, hx, hy, inside, c, flags, Tx, Ty, Tz, diag, xc, val, sP, sF, act, dg,
-                    txp, typ, tzp);
-            const double xn = xval(i, j, k + 1);
-            const double bp = act ? b[c] : 0.0;
-            const float di = act ? dinv32[c] : 0.0f;
-            const double txm_lane = __shfl_up_sync(0xffffffffu, txp, 1);
-            __syncthreads();
-            if (act) {
-                const double rp = bp - apply64_tile(g, i, j, k, tx, ty, buf, sP, sF, txm_lane, dg, txp, typ, tzm,
-                                                    tzp, xm, xc, xn);
-                const float rf = (float)rp;
-                const float zf = di * rf;
-                const float bf = (float)bp;
-                r32[c] = rf;
-                z32[c] = zf;
-                d32[c] = 0.0f;
-                a_rr = fmaf(rf, rf, a_rr);
-                a_bb = fmaf(bf, bf, a_bb);
-                a_rz = fmaf(rf, zf, a_rz);
-            } else if (inside) {
-                r32[c] = 0.0f;
-                z32[c] = 0.0f;
-                d32[c] = 0.0f;
-            }
-            tzm = tzp;
-            xm = xc;
-            xc = xn;
-        }
-        __syncthreads();
-    }
-    float vf[3] = {a_rr, a_bb, a_rz};
+    __shared__ Sweep64Shared s;
+    const Op64 A{Tx, Ty, Tz, diag};
+    float vf[3] = {0.0f, 0.0f, 0.0f};   // r32.r32, b.b, r32.z32
+    resid64_sweep(g, tw, A, s, flags, x, b, dinv32, r32, z32, d32, vf);
     double w[3];
     if (grid_reduce_f32<3>(vf, w, partials, ticket) && threadIdx.x == 0) {
         outer->iter += 1;
@@ -409,7 +193,7 @@ k_resid64(Grid g, Tiles tw, const uint8_t *__restrict__ flags, const double *__r
     }
 }
 
-__global__ void __launch_bounds__(RED_THREADS)
+__global__ void __launch_bounds__(CT, SWEEP_OCC)
 k_cg32_spmv(Grid g, Tiles tw, const float *__restrict__ z, const float *__restrict__ p_in, float *__restrict__ p_out,
             float *__restrict__ q, const float *__restrict__ K32, const float *__restrict__ cb32, double *partials,
             unsigned int *ticket, CgScal *sc)
@@ -417,72 +201,8 @@ k_cg32_spmv(Grid g, Tiles tw, const float *__restrict__ z, const float *__restri
     count_launch(g, KK_CG32_SPMV);
     if (sc->done) return;
     count_work(g, KK_CG32_SPMV);
-    const float beta = (float)sc->beta;
-    const bool first = sc->iter == 0;
-    // (p, K) of a cell: p = z + beta p_old, K < 0 marks inactive / outside cells
-    auto load = [&](int i, int j, int k, float &pv, float &kv) {
-        pv = 0.0f;
-        kv = -1.0f;
-        if (i < 0 || i >= g.nx || j < 0 || j >= g.ny || k < 0 || k >= g.nz) return;
-        const long long c = i + (long long)g.nx * j + g.sxy * k;
-        kv = K32[c];
-        if (kv >= 0.0f) pv = first ? z[c] : fmaf(beta, p_in[c], z[c]);
-    };
-    __shared__ float sP[2][TY + 2][TX + 2], sK[2][TY + 2][TX + 2];
-    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-    int hx = 0, hy = 0;
-    if (threadIdx.x < HALO) halo_cell(threadIdx.x, hx, hy);
-    const float wx = g.w32[0] * 0.5f, wy = g.w32[1] * 0.5f, wz = g.w32[2] * 0.5f;
-    float acc = 0.0f;
-    for (long long item = blockIdx.x; item < tw.items; item += gridDim.x) {
-        const TileItem it = tile_item(g, tw, item);
-        const int i = it.i0 + tx, j = it.j0 + ty;
-        const bool inside = i < g.nx && j < g.ny;
-        float pm, km, pc, kc;
-        load(i, j, it.k0 - 1, pm, km);
-        load(i, j, it.k0, pc, kc);
-        for (int k = it.k0; k < it.k1; k++) {
-            const int buf = k & 1;
-            const long long c = i + (long long)g.nx * j + g.sxy * k;
-            sP[buf][ty + 1][tx + 1] = pc;
-            sK[buf][ty + 1][tx + 1] = kc;
-            if (threadIdx.x < HALO) {
-                float hp, hk;
-                load(it.i0 + hx, it.j0 + hy, k, hp, hk);
-                sP[buf][hy + 1][hx + 1] = hp;
-                sK[buf][hy + 1][hx + 1] = hk;
-            }
-            float pn, kn;
-            load(i, j, k + 1, pn, kn);
-            const float cb = (inside && kc >= 0.0f) ? cb32[c] : 0.0f;
-            __syncthreads();
-            if (inside && kc >= 0.0f) {
-                // (A p)_P = cb_P p_P + sum_f w_f (K_P + K_N)/2 (p_P - p_N), faces -x +x -y +y -z +z
-                float qp = cb * pc;
-                auto face = [&](float KN, float vN, float w) {
-                    if (KN >= 0.0f) qp = fmaf(w * (kc + KN), pc - vN, qp);
-                };
-                face(sK[buf][ty + 1][tx], sP[buf][ty + 1][tx], wx);
-                face(sK[buf][ty + 1][tx + 2], sP[buf][ty + 1][tx + 2], wx);
-                face(sK[buf][ty][tx + 1], sP[buf][ty][tx + 1], wy);
-                face(sK[buf][ty + 2][tx + 1], sP[buf][ty + 2][tx + 1], wy);
-                face(km, pm, wz);
-                face(kn, pn, wz);
-                p_out[c] = pc;
-                q[c] = qp;
-                acc = fmaf(pc, qp, acc);
-            } else if (inside) {
-                p_out[c] = 0.0f;
-                q[c] = 0.0f;
-            }
-            pm = pc;
-            km = kc;
-            pc = pn;
-            kc = kn;
-        }
-        __syncthreads();
-    }
-    float vf[1] = {acc};
+    __shared__ Sweep32Shared s;
+    float vf[1] = {sweep32(g, tw, s, K32, cb32, z, p_in, p_out, q, (float)sc->beta, sc->iter == 0)};
     double v[1];
     if (grid_reduce_f32<1>(vf, v, partials, ticket) && threadIdx.x == 0) {
         sc->pq = v[0];
@@ -706,80 +426,15 @@ k_cg32_spmv_tma(Grid g, Tiles tw, const __grid_constant__ TmaMaps32 maps, int pi
 __global__ void __launch_bounds__(RED_THREADS)
 k_cg32_update(Grid g, float *__restrict__ x, float *__restrict__ r, float *__restrict__ z,
               const float *__restrict__ pd, const float *__restrict__ q, const float *__restrict__ dinv,
-              double *partials, unsigned int *ticket, CgScal *sc, CondSet cond)
+              double *partials, unsigned int *ticket, CgScal *sc)
 {
     count_launch(g, KK_CG32_UPDATE);
-    if (sc->done) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) set_cond(cond, 0);
-        return;
-    }
+    if (sc->done) return;
     count_work(g, KK_CG32_UPDATE);
-    const float alpha = (float)sc->alpha;
-    float a0 = 0.0f, a1 = 0.0f;
-    // one cell: inactive cells (dinv 0) keep x and r and hold z = 0 (as set
-    // when the inner solve starts), so z is written without being read
-    auto cell = [&](float di, float pv, float xv, float qv, float rv, float &xo, float &ro, float &zo) {
-        const bool act = di != 0.0f;
-        const float rp = fmaf(-alpha, qv, rv), zp = di * rp;
-        xo = act ? fmaf(alpha, pv, xv) : xv;
-        ro = act ? rp : rv;
-        zo = act ? zp : 0.0f;
-        if (act) {
-            a0 = fmaf(rp, rp, a0);
-            a1 = fmaf(rp, zp, a1);
-        }
-    };
-    const long long N = g.N;
-    const long long stride = (long long)gridDim.x * blockDim.x, t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool vec = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(r) | reinterpret_cast<uintptr_t>(z) |
-                       reinterpret_cast<uintptr_t>(pd) | reinterpret_cast<uintptr_t>(q) |
-                       reinterpret_cast<uintptr_t>(dinv)) & 15u) == 0;
-    long long done = 0;
-    if (vec) {
-        // four cells per thread and pass: 16-byte loads and stores
-        const long long n4 = N / 4;
-        for (long long v = t0; v < n4; v += stride) {
-            const float4 di = reinterpret_cast<const float4 *>(dinv)[v], pv = reinterpret_cast<const float4 *>(pd)[v];
-            const float4 xv = reinterpret_cast<const float4 *>(x)[v], qv = reinterpret_cast<const float4 *>(q)[v];
-            const float4 rv = reinterpret_cast<const float4 *>(r)[v];
-            float4 xo, ro, zo;
-            cell(di.x, pv.x, xv.x, qv.x, rv.x, xo.x, ro.x, zo.x);
-            cell(di.y, pv.y, xv.y, qv.y, rv.y, xo.y, ro.y, zo.y);
-            cell(di.z, pv.z, xv.z, qv.z, rv.z, xo.z, ro.z, zo.z);
-            cell(di.w, pv.w, xv.w, qv.w, rv.w, xo.w, ro.w, zo.w);
-            reinterpret_cast<float4 *>(x)[v] = xo;
-            reinterpret_cast<float4 *>(r)[v] = ro;
-            reinterpret_cast<float4 *>(z)[v] = zo;
-        }
-        done = n4 * 4;
-    }
-    for (long long p = done + t0; p < N; p += stride) {
-        float xo, ro, zo;
-        cell(dinv[p], pd[p], x[p], q[p], r[p], xo, ro, zo);
-        x[p] = xo;
-        r[p] = ro;
-        z[p] = zo;
-    }
-    float vf[2] = {a0, a1};
+    float vf[2] = {0.0f, 0.0f};
+    cg32_update_cells(g, (float)sc->alpha, false, dinv, pd, q, x, r, z, vf);
     double v[2];
-    if (grid_reduce_f32<2>(vf, v, partials, ticket) && threadIdx.x == 0) {
-        sc->iter += 1;
-        sc->total += 1;
-        sc->rr = v[0];
-        if (!isfinite(v[0]) || !isfinite(v[1])) {
-            sc->status = CG_NONFINITE;
-            sc->done = 1;
-        } else if (sqrt(v[0]) <= sc->stop2) {
-            sc->done = 1;
-        } else if (sc->iter >= sc->max_it) {
-            sc->status = CG_MAXIT;
-            sc->done = 1;
-        } else {
-            sc->beta = v[1] / sc->rho;
-            sc->rho = v[1];
-        }
-        set_cond(cond, sc->done ? 0 : 1);
-    }
+    if (grid_reduce_f32<2>(vf, v, partials, ticket) && threadIdx.x == 0) cg_update_scalars(sc, v);
 }
 
 // x += d after an inner solve; a non-finite inner solve fails the outer loop
@@ -812,20 +467,27 @@ void launch_cg64_init(cudaStream_t s, int nblk, const Grid &g, const uint8_t *fl
                                              ticket, sc, skip, cond);
 }
 
-void launch_cg64_spmv(cudaStream_t s, int nblk, const Grid &g, const uint8_t *flags, const double *z,
-                      const double *p_in, double *p_out, double *q, const double *Tx, const double *Ty,
-                      const double *Tz, const double *diag, double *partials, unsigned int *ticket, CgScal *sc)
+// Tiles and blocks of a sweep as a launch of its own: two blocks an SM.
+static int sweep_tiles(const Grid &g, int nblk, int tile_y, Tiles &tw)
 {
-    const Tiles tw = make_tiles(g, nblk);
-    k_cg64_spmv<<<tile_blocks(tw, g, nblk), RED_THREADS, 0, s>>>(g, tw, flags, z, p_in, p_out, q, Tx, Ty, Tz, diag,
-                                                              partials, ticket, sc);
+    const int sms = std::max(1, (g.cap > nblk ? g.cap : nblk) / 8);   // the cap is eight blocks an SM
+    tw = make_tiles_balanced(g, SWEEP_OCC * sms, CX, tile_y);
+    return (int)std::min<long long>(tw.items, SWEEP_OCC * sms);
+}
+
+void launch_cg64_spmv(cudaStream_t s, int nblk, const Grid &g, const double *z, const double *p_in, double *p_out,
+                      double *q, const double *Tx, const double *Ty, const double *Tz, const double *diag,
+                      double *partials, unsigned int *ticket, CgScal *sc)
+{
+    Tiles tw;
+    const int nb = sweep_tiles(g, nblk, CY, tw);
+    k_cg64_spmv<<<nb, CT, 0, s>>>(g, tw, z, p_in, p_out, q, Tx, Ty, Tz, diag, partials, ticket, sc);
 }
 
 void launch_cg64_update(cudaStream_t s, int nblk, const Grid &g, double *x, double *r, double *z, const double *p,
-                        const double *q, const double *dinv, double *partials, unsigned int *ticket, CgScal *sc,
-                        CondSet cond)
+                        const double *q, const double *dinv, double *partials, unsigned int *ticket, CgScal *sc)
 {
-    k_cg64_update<<<nblk, RED_THREADS, 0, s>>>(g, x, r, z, p, q, dinv, partials, ticket, sc, cond);
+    k_cg64_update<<<nblk, RED_THREADS, 0, s>>>(g, x, r, z, p, q, dinv, partials, ticket, sc);
 }
 
 void launch_apply64(cudaStream_t s, int nblk, const Grid &g, const uint8_t *flags, const double *x, double *y,
@@ -846,17 +508,16 @@ void launch_resid64(cudaStream_t s, int nblk, const Grid &g, const uint8_t *flag
                     int outer_max_it, double *partials, unsigned int *ticket, CgScal *outer, CgScal *inner,
                     CondSet cond_outer, CondSet cond_inner)
 {
-    const Tiles tw = make_tiles(g, nblk);
-    k_resid64<<<tile_blocks(tw, g, nblk), RED_THREADS, 0, s>>>(g, tw, flags, x, b, Tx, Ty, Tz, diag, dinv32, r32, z32,
-                                                            d32, tol, tol_inner, inner_max_it, outer_max_it,
-                                                            partials, ticket, outer, inner, cond_outer, cond_inner);
+    Tiles tw;
+    const int nb = sweep_tiles(g, nblk, CY, tw);
+    k_resid64<<<nb, CT, 0, s>>>(g, tw, flags, x, b, Tx, Ty, Tz, diag, dinv32, r32, z32, d32, tol, tol_inner,
+                                inner_max_it, outer_max_it, partials, ticket, outer, inner, cond_outer, cond_inner);
 }
 
 void launch_cg32_spmv(cudaStream_t s, int nblk, const Grid &g, const float *z, const float *p_in, float *p_out,
                       float *q, const float *K32, const float *cb32, double *partials, unsigned int *ticket,
                       CgScal *sc, const TmaMaps32 *tma, int *fault)
 {
-    const Tiles tw = make_tiles(g, nblk);
     if (tma && fault && z == tma->z_ptr && K32 == tma->K_ptr && cb32 == tma->cb_ptr &&
         (p_in == tma->p_ptr[0] || p_in == tma->p_ptr[1]) && TY == 8) {
         // one wave: as many items as blocks resident at this kernel's occupancy
@@ -873,15 +534,15 @@ void launch_cg32_spmv(cudaStream_t s, int nblk, const Grid &g, const float *z, c
             g, tt, *tma, p_in == tma->p_ptr[1] ? 1 : 0, p_out, q, partials, ticket, sc, fault);
         return;
     }
-    k_cg32_spmv<<<tile_blocks(tw, g, nblk), RED_THREADS, 0, s>>>(g, tw, z, p_in, p_out, q, K32, cb32, partials, ticket,
-                                                              sc);
+    Tiles tw;
+    const int nb = sweep_tiles(g, nblk, FY, tw);
+    k_cg32_spmv<<<nb, CT, 0, s>>>(g, tw, z, p_in, p_out, q, K32, cb32, partials, ticket, sc);
 }
 
 void launch_cg32_update(cudaStream_t s, int nblk, const Grid &g, float *x, float *r, float *z, const float *p,
-                        const float *q, const float *dinv, double *partials, unsigned int *ticket, CgScal *sc,
-                        CondSet cond)
+                        const float *q, const float *dinv, double *partials, unsigned int *ticket, CgScal *sc)
 {
-    k_cg32_update<<<nblk, RED_THREADS, 0, s>>>(g, x, r, z, p, q, dinv, partials, ticket, sc, cond);
+    k_cg32_update<<<nblk, RED_THREADS, 0, s>>>(g, x, r, z, p, q, dinv, partials, ticket, sc);
 }
 
 void launch_add_correction(cudaStream_t s, int nblk, const Grid &g, double *x, const float *d, CgScal *outer,

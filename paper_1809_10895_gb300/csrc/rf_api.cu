@@ -79,6 +79,7 @@ struct rf_ctx {
     double *partials = nullptr;
     unsigned int *ticket = nullptr;
     void *gridred = nullptr;             // barrier and partials of the cooperative kernels
+    int cg64_blocks = 0, mixed_blocks = 0;   // of the one-launch solves
     int small_blocks[2] = {-1, -1};      // blocks of the small-grid attempt (FP64, mixed; -1: not asked yet)
     CgScal *sc = nullptr, *sc_in = nullptr;
     StepResults *res = nullptr;
@@ -219,6 +220,7 @@ rf_status sync(rf_ctx *c)
         // reported once: the flag is cleared so that the context stays usable
         *c->fault_h = 0;
         CUDA_TRY(cudaMemsetAsync(c->dev_fault, 0, sizeof(int), c->stream));
+        CUDA_TRY(cudaMemsetAsync(c->gridred, 0, GR_BYTES, c->stream));   // a barrier given up may be left half counted
         CUDA_TRY(cudaStreamSynchronize(c->stream));
         return fail(RF_ERR_DEVICE_TIMEOUT, "a device wait for staged data ran out (the solve was stopped)");
     }
@@ -392,28 +394,33 @@ rf_status capture_solve(rf_ctx *c, cudaGraph_t top, cudaGraph_t parent, std::vec
                              c->prm.tol_cg, c->prm.cg_max_it, c->partials, c->ticket, c->sc, skip, cc);
             RF_TRY(cap_end(c, deps));
         }
-        cudaGraphNode_t wn;
-        cudaGraph_t body;
-        RF_TRY(add_while(parent, deps, cc.h, &wn, &body));
-        RF_TRY(cap_begin(c, body, {}));
-        for (int half = 0; half < 2; half++) {
-            double *pin = c->p[half], *pout = c->p[half ^ 1];
-            launch_cg64_spmv(s, nb, g, c->flags, c->z, pin, pout, c->q, c->Tx, c->Ty, c->Tz, c->diag, c->partials,
-                             c->ticket, c->sc);
-            launch_cg64_update(s, nb, g, x, c->r, c->z, pout, c->q, c->dinv, c->partials, c->ticket, c->sc, cc);
-        }
-        std::vector<cudaGraphNode_t> tmp;
-        RF_TRY(cap_end(c, tmp));
-        out = {wn};
+        RF_TRY(cap_begin(c, parent, deps));
+        CUDA_TRY(launch_cg64_solve(s, c->cg64_blocks, g, c->Tx, c->Ty, c->Tz, c->diag, c->dinv, x, c->r, c->z, c->p[0],
+                                   c->p[1], c->q, c->gridred, c->dev_fault, c->sc));
+        RF_TRY(cap_end(c, out));
         return RF_OK;
     }
     // mixed: WHILE(outer) { WHILE(inner FP32 PCG) ; x += d ; FP64 residual }
     const CondSet co = start->cond, ci = start->cond_inner;
     const bool mg = c->prm.precond == RF_PRECOND_MG, dic = c->prm.precond == RF_PRECOND_DIC;
+    if (!mg && !dic) {
+        RF_TRY(cap_begin(c, parent, deps));
+        if (!fused) {
+            launch_mixed_start(s, nb, g, x0, x, c->sc, c->sc_in, skip, co);
+            launch_resid64(s, nb, g, c->flags, x, c->b, c->Tx, c->Ty, c->Tz, c->diag, c->dinv32, c->r32, c->z32, c->d32,
+                           c->prm.tol_cg, c->prm.tol_inner, c->prm.inner_max_it, c->prm.outer_max_it, c->partials,
+                           c->ticket, c->sc, c->sc_in, co, ci);
+        }
+        CUDA_TRY(launch_mixed_solve(s, c->mixed_blocks, g, c->flags, c->Tx, c->Ty, c->Tz, c->diag, c->b, c->K32, c->cb32,
+                                    c->dinv32, x, c->r32, c->z32, c->d32, c->p32[0], c->p32[1], c->q32, c->gridred,
+                                    c->dev_fault, c->sc, c->sc_in, c->prm.tol_cg, c->prm.tol_inner,
+                                    c->prm.inner_max_it, c->prm.outer_max_it));
+        RF_TRY(cap_end(c, out));
+        return RF_OK;
+    }
     const int *idone = &c->sc_in->done;
     // z = M r for the MG preconditioner
     auto precondition = [&]() { launch_mg_vcycle(s, nb, c->mg, c->K32, c->r32, c->z32, idone); };
-    const CondSet none{0, 0};
     if (!fused) {
         RF_TRY(cap_begin(c, parent, deps));
         launch_mixed_start(s, nb, g, x0, x, c->sc, c->sc_in, skip, co);
@@ -433,15 +440,13 @@ rf_status capture_solve(rf_ctx *c, cudaGraph_t top, cudaGraph_t parent, std::vec
             launch_cg32_rz(s, nb, g, c->r32, c->z32, c->partials, c->ticket, c->sc_in, first, ci);
         }
     };
-    if (mg || dic) {
-        // coarse operators (MG) or pivots (DIC) from this assembly, then
-        // z0 = M r0 and rho = r0.z0
-        RF_TRY(cap_begin(c, parent, deps));
-        if (mg) launch_mg_build(s, nb, c->mg, c->K32, skip);
-        else launch_dic_setup(s, nb, g, c->K32, c->cb32, c->dic_diag, c->dic_rd, skip);
-        precondition_rz(1, false);
-        RF_TRY(cap_end(c, deps));
-    }
+    // coarse operators (MG) or pivots (DIC) from this assembly, then z0 = M r0
+    // and rho = r0.z0
+    RF_TRY(cap_begin(c, parent, deps));
+    if (mg) launch_mg_build(s, nb, c->mg, c->K32, skip);
+    else launch_dic_setup(s, nb, g, c->K32, c->cb32, c->dic_diag, c->dic_rd, skip);
+    precondition_rz(1, false);
+    RF_TRY(cap_end(c, deps));
     cudaGraphNode_t wo, wi;
     cudaGraph_t bo, bi;
     RF_TRY(add_while(parent, deps, co.h, &wo, &bo));
@@ -455,12 +460,9 @@ rf_status capture_solve(rf_ctx *c, cudaGraph_t top, cudaGraph_t parent, std::vec
             launch_cg32_update_dic(s, nb, g, c->d32, c->r32, c->z32, pout, c->q32, c->dinv32, c->dic_rd, c->partials,
                                    c->ticket, c->sc_in);
             precondition_rz(0, true);
-        } else if (mg) {
+        } else {
             launch_cg32_update_mg(s, nb, g, c->d32, c->r32, pout, c->q32, c->dinv32, c->partials, c->ticket, c->sc_in);
             precondition_rz(0, false);
-        } else {
-            launch_cg32_update(s, nb, g, c->d32, c->r32, c->z32, pout, c->q32, c->dinv32, c->partials, c->ticket,
-                               c->sc_in, ci);
         }
     }
     std::vector<cudaGraphNode_t> tmp;
@@ -470,8 +472,7 @@ rf_status capture_solve(rf_ctx *c, cudaGraph_t top, cudaGraph_t parent, std::vec
     launch_resid64(s, nb, g, c->flags, x, c->b, c->Tx, c->Ty, c->Tz, c->diag, c->dinv32, c->r32, c->z32, c->d32,
                    c->prm.tol_cg, c->prm.tol_inner, c->prm.inner_max_it, c->prm.outer_max_it, c->partials, c->ticket,
                    c->sc, c->sc_in, co, ci);
-    if (mg || dic) precondition_rz(1, false);
-    (void)none;
+    precondition_rz(1, false);
     RF_TRY(cap_end(c, tmp));
     out = {wo};
     return RF_OK;
@@ -482,9 +483,9 @@ rf_status make_start(rf_ctx *c, cudaGraph_t G, double *x, SolveStart &st)
 {
     st = SolveStart{};
     cudaGraphConditionalHandle h1, h2;
-    CUDA_TRY(cudaGraphConditionalHandleCreate(&h1, G, 0, 0));
-    st.cond = CondSet{h1, 1};
-    if (c->prm.precision == RF_PREC_MIXED) {
+    if (c->prm.precond != RF_PRECOND_JACOBI) {       // Jacobi solves are one launch, without loop nodes
+        CUDA_TRY(cudaGraphConditionalHandleCreate(&h1, G, 0, 0));
+        st.cond = CondSet{h1, 1};
         CUDA_TRY(cudaGraphConditionalHandleCreate(&h2, G, 0, 0));
         st.cond_inner = CondSet{h2, 1};
     }
@@ -1162,6 +1163,12 @@ rf_status rf_mesh_create(const rf_mesh_desc *mesh, const rf_solver_params *param
         rf_destroy(c);
         return fail(RF_ERR_CUDA, std::string("initialisation: ") + cudaGetErrorString(e));
     }
+    c->cg64_blocks = cg64_solve_blocks(g, c->num_sms);
+    c->mixed_blocks = mixed_solve_blocks(g, c->num_sms);
+    if (c->cg64_blocks < 1 || c->mixed_blocks < 1) {
+        rf_destroy(c);
+        return fail(RF_ERR_CUDA, "cooperative launches are not available on this device");
+    }
     // TMA plane staging for the FP32 stencil (grids with nx a multiple of 4)
     c->tma_ok = make_tma_maps32(g.nx, g.ny, g.nz, c->z32, c->p32[0], c->p32[1], c->K32, c->cb32, &c->tma);
     cudaGetLastError();
@@ -1597,15 +1604,14 @@ rf_status rf_profile_kernel(rf_ctx *c, int kind, int reps, double *avg_ms, doubl
         }
         // one untimed iteration, so the timed ones read the previous direction
         if (kind == RF_K_CG64_SPMV || kind == RF_K_CG64_UPDATE) {
-            launch_cg64_spmv(s, nb, g, c->flags, c->z, c->p[1], c->p[0], c->q, c->Tx, c->Ty, c->Tz, c->diag,
+            launch_cg64_spmv(s, nb, g, c->z, c->p[1], c->p[0], c->q, c->Tx, c->Ty, c->Tz, c->diag,
                              c->partials, c->ticket, c->sc);
-            launch_cg64_update(s, nb, g, c->x, c->r, c->z, c->p[0], c->q, c->dinv, c->partials, c->ticket, c->sc,
-                               none);
+            launch_cg64_update(s, nb, g, c->x, c->r, c->z, c->p[0], c->q, c->dinv, c->partials, c->ticket, c->sc);
         } else if (kind == RF_K_CG32_SPMV || kind == RF_K_CG32_UPDATE) {
             launch_cg32_spmv(s, nb, g, c->z32, c->p32[1], c->p32[0], c->q32, c->K32, c->cb32, c->partials, c->ticket,
                              c->sc_in, c->tma_ok ? &c->tma : nullptr, c->dev_fault);
             launch_cg32_update(s, nb, g, c->d32, c->r32, c->z32, c->p32[0], c->q32, c->dinv32, c->partials,
-                               c->ticket, c->sc_in, none);
+                               c->ticket, c->sc_in);
         }
         return RF_OK;
     };
@@ -1639,17 +1645,16 @@ rf_status rf_profile_kernel(rf_ctx *c, int kind, int reps, double *avg_ms, doubl
         case RF_K_CG64_SPMV:
         case RF_K_CG64_UPDATE:
             if (kind == RF_K_CG64_SPMV)
-                timed([&] { launch_cg64_spmv(s, nb, g, c->flags, c->z, pin, pout, c->q, c->Tx, c->Ty, c->Tz, c->diag,
+                timed([&] { launch_cg64_spmv(s, nb, g, c->z, pin, pout, c->q, c->Tx, c->Ty, c->Tz, c->diag,
                                              c->partials, c->ticket, c->sc); });
             else
-                launch_cg64_spmv(s, nb, g, c->flags, c->z, pin, pout, c->q, c->Tx, c->Ty, c->Tz, c->diag, c->partials,
+                launch_cg64_spmv(s, nb, g, c->z, pin, pout, c->q, c->Tx, c->Ty, c->Tz, c->diag, c->partials,
                                  c->ticket, c->sc);
             if (kind == RF_K_CG64_UPDATE)
                 timed([&] { launch_cg64_update(s, nb, g, c->x, c->r, c->z, pout, c->q, c->dinv, c->partials, c->ticket,
-                                               c->sc, none); });
+                                               c->sc); });
             else
-                launch_cg64_update(s, nb, g, c->x, c->r, c->z, pout, c->q, c->dinv, c->partials, c->ticket, c->sc,
-                                   none);
+                launch_cg64_update(s, nb, g, c->x, c->r, c->z, pout, c->q, c->dinv, c->partials, c->ticket, c->sc);
             break;
         case RF_K_RESID64:
             timed([&] { launch_resid64(s, nb, g, c->flags, c->x, c->b, c->Tx, c->Ty, c->Tz, c->diag, c->dinv32,
@@ -1665,10 +1670,10 @@ rf_status rf_profile_kernel(rf_ctx *c, int kind, int reps, double *avg_ms, doubl
                                  c->sc_in, c->tma_ok ? &c->tma : nullptr, c->dev_fault);
             if (kind == RF_K_CG32_UPDATE)
                 timed([&] { launch_cg32_update(s, nb, g, c->d32, c->r32, c->z32, qout, c->q32, c->dinv32, c->partials,
-                                               c->ticket, c->sc_in, none); });
+                                               c->ticket, c->sc_in); });
             else
                 launch_cg32_update(s, nb, g, c->d32, c->r32, c->z32, qout, c->q32, c->dinv32, c->partials, c->ticket,
-                                   c->sc_in, none);
+                                   c->sc_in);
             break;
         }
     }

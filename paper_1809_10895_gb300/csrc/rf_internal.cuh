@@ -247,6 +247,26 @@ __device__ __forceinline__ void cg64_start_scalars(CgScal *sc, const double (&v)
     set_cond(cond, sc->done ? 0 : 1);
 }
 
+// End of a CG iteration from the reduced (r.r, r.z): stop test or beta.
+__device__ __forceinline__ void cg_update_scalars(CgScal *sc, const double (&v)[2])
+{
+    sc->iter += 1;
+    sc->total += 1;
+    sc->rr = v[0];
+    if (!isfinite(v[0]) || !isfinite(v[1])) {
+        sc->status = CG_NONFINITE;
+        sc->done = 1;
+    } else if (sqrt(v[0]) <= sc->stop2) {
+        sc->done = 1;
+    } else if (sc->iter >= sc->max_it) {
+        sc->status = CG_MAXIT;
+        sc->done = 1;
+    } else {
+        sc->beta = v[1] / sc->rho;
+        sc->rho = v[1];
+    }
+}
+
 // Defect correction: test of an outer FP64 residual (r.r, b.b) and seeds of
 // the inner FP32 solve (r32.r32, r32.z32); outer->iter already counts this
 // residual, and the solve fails after outer_max_it residuals.
@@ -360,12 +380,24 @@ void launch_cg64_init(cudaStream_t s, int nblk, const Grid &g, const uint8_t *fl
                       const double *diag, const double *dinv, double *r, double *z, double tol,
                       int max_it, double *partials, unsigned int *ticket, CgScal *sc, const int *skip,
                       CondSet cond);
-void launch_cg64_spmv(cudaStream_t s, int nblk, const Grid &g, const uint8_t *flags, const double *z,
+void launch_cg64_spmv(cudaStream_t s, int nblk, const Grid &g, const double *z,
                       const double *p_in, double *p_out, double *q, const double *Tx, const double *Ty,
                       const double *Tz, const double *diag, double *partials, unsigned int *ticket, CgScal *sc);
 void launch_cg64_update(cudaStream_t s, int nblk, const Grid &g, double *x, double *r, double *z,
                         const double *p, const double *q, const double *dinv, double *partials,
-                        unsigned int *ticket, CgScal *sc, CondSet cond);
+                        unsigned int *ticket, CgScal *sc);
+// The whole solve in one cooperative launch (cg_solve.cu).
+int cg64_solve_blocks(const Grid &g, int sms);
+cudaError_t launch_cg64_solve(cudaStream_t s, int blocks, const Grid &g, const double *Tx, const double *Ty,
+                              const double *Tz, const double *diag, const double *dinv, double *x, double *r,
+                              double *z, double *p0, double *p1, double *q, void *red, int *fault, CgScal *sc);
+int mixed_solve_blocks(const Grid &g, int sms);
+cudaError_t launch_mixed_solve(cudaStream_t s, int blocks, const Grid &g, const uint8_t *flags, const double *Tx,
+                               const double *Ty, const double *Tz, const double *diag, const double *b,
+                               const float *K32, const float *cb32, const float *dinv32, double *x, float *r32,
+                               float *z32, float *d32, float *p0, float *p1, float *q32, void *red, int *fault,
+                               CgScal *outer, CgScal *inner, double tol, double tol_inner, int inner_max_it,
+                               int outer_max_it);
 void launch_apply64(cudaStream_t s, int nblk, const Grid &g, const uint8_t *flags, const double *x, double *y,
                     const double *Tx, const double *Ty, const double *Tz, const double *diag);
 
@@ -381,8 +413,7 @@ void launch_cg32_spmv(cudaStream_t s, int nblk, const Grid &g, const float *z, c
                       float *q, const float *K32, const float *cb32, double *partials, unsigned int *ticket,
                       CgScal *sc, const TmaMaps32 *tma = nullptr, int *fault = nullptr);
 void launch_cg32_update(cudaStream_t s, int nblk, const Grid &g, float *x, float *r, float *z, const float *p,
-                        const float *q, const float *dinv, double *partials, unsigned int *ticket, CgScal *sc,
-                        CondSet cond);
+                        const float *q, const float *dinv, double *partials, unsigned int *ticket, CgScal *sc);
 void launch_add_correction(cudaStream_t s, int nblk, const Grid &g, double *x, const float *d, CgScal *outer,
                            const CgScal *inner, CondSet cond_outer);
 

@@ -19,7 +19,7 @@ constexpr int HALO = 2 * TY + 2 * TX;   // x- and y-halo cells of a plane (no co
 
 struct Tiles {
     int ntx, nty, zc;       // tiles along x, y; planes per item
-    int tx;                 // tile width in x
+    int tx, ty;             // tile size
     long long items;
 };
 
@@ -28,6 +28,7 @@ inline Tiles make_tiles(const Grid &g, int nblk)
     if (g.cap > nblk) nblk = g.cap;
     Tiles t;
     t.tx = TX;
+    t.ty = TY;
     t.ntx = (g.nx + TX - 1) / TX;
     t.nty = (g.ny + TY - 1) / TY;
     const long long tiles = (long long)t.ntx * t.nty;
@@ -43,12 +44,13 @@ inline Tiles make_tiles(const Grid &g, int nblk)
 // Tiles with the z split that minimises (waves of `resident` blocks) x
 // (planes per item + the two extra planes an item reads); at most `cap` items
 // per wave are launched.
-inline Tiles make_tiles_balanced(const Grid &g, int resident, int tile_x)
+inline Tiles make_tiles_balanced(const Grid &g, int resident, int tile_x, int tile_y = TY)
 {
     Tiles t;
     t.tx = tile_x;
+    t.ty = tile_y;
     t.ntx = (g.nx + tile_x - 1) / tile_x;
-    t.nty = (g.ny + TY - 1) / TY;
+    t.nty = (g.ny + tile_y - 1) / tile_y;
     const long long tiles = (long long)t.ntx * t.nty;
     long long best = -1;
     int best_zc = g.nz;
@@ -83,7 +85,7 @@ __device__ __forceinline__ TileItem tile_item(const Grid &g, const Tiles &t, lon
     const int chunk = (int)(item / per_plane);
     const long long r = item - chunk * per_plane;
     TileItem it;
-    it.j0 = (int)(r / t.ntx) * TY;
+    it.j0 = (int)(r / t.ntx) * t.ty;
     it.i0 = (int)(r % t.ntx) * t.tx;
     it.k0 = chunk * t.zc;
     it.k1 = min(g.nz, it.k0 + t.zc);
