@@ -262,20 +262,24 @@ k_conv3d_tc(TcParams p, const __grid_constant__ CUtensorMap in_map, int cin_mem,
                 tc_fence_after();
                 const uint32_t a_base = smem_addr(sA + s * S::A_BYTES);
                 const uint32_t b_base = smem_addr(sB);
-                for (int rb = 0; rb < TC_RB; rb++) {
-                    const uint32_t d = tmem + (uint32_t)((s * 4 + rb) * NOUT);
-                    const int r0 = TC_ROW0 + 128 * rb;
-                    for (int tap = 0; tap < 27; tap++) {
-                        const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-                        const int off = (dz * TC_HY + dy) * TC_HX + dx;
-                        for (int kc = 0; kc < S::KC; kc++) {
-                            // A: planes 2kc, 2kc+1 (LBO) from row r0 + off; B: k-groups tap CINP/8 + 2kc, + 1
-                            const uint64_t ad =
-                                smem_desc(a_base + (uint32_t)(2 * kc * TC_PLANE_BYTES + (r0 + off) * 16), TC_PLANE_BYTES, 128);
-                            const uint64_t bd = smem_desc(
-                                b_base + (uint32_t)((tap * S::PLANES + 2 * kc) * NOUT * 16), NOUT * 16, 128);
-                            tc_mma(d, ad, bd, S::IDESC, (tap | kc) ? 1u : 0u);
-                        }
+                // row blocks innermost: the four accumulators are independent,
+                // so consecutive MMAs never wait for one another's result
+                // (each accumulator still sums its taps in the same order)
+                const uint32_t d0 = tmem + (uint32_t)(s * 4 * NOUT);
+                for (int tap = 0; tap < 27; tap++) {
+                    const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
+                    const int off = (dz * TC_HY + dy) * TC_HX + dx;
+#pragma unroll
+                    for (int kc = 0; kc < S::KC; kc++) {
+                        // A: planes 2kc, 2kc+1 (LBO) from row r0 + off; B: k-groups tap CINP/8 + 2kc, + 1
+                        const uint64_t ad = smem_desc(
+                            a_base + (uint32_t)(2 * kc * TC_PLANE_BYTES + (TC_ROW0 + off) * 16), TC_PLANE_BYTES, 128);
+                        const uint64_t bd = smem_desc(
+                            b_base + (uint32_t)((tap * S::PLANES + 2 * kc) * NOUT * 16), NOUT * 16, 128);
+#pragma unroll
+                        for (int rb = 0; rb < TC_RB; rb++)   // the next 128 rows: 2048 bytes on, in units of 16
+                            tc_mma(d0 + (uint32_t)(rb * NOUT), ad + (uint64_t)(128 * rb), bd, S::IDESC,
+                                   (tap | kc) ? 1u : 0u);
                     }
                 }
                 tc_commit(&free_bar[s]);
@@ -574,21 +578,23 @@ k_wgrad_tc(const __grid_constant__ CUtensorMap x_map, const __nv_bfloat16 *__res
             if (more) issue_x(tile + gridDim.x);   // lands while the MMAs run
             tc_fence_after();
             const uint32_t tb = smem_addr(sT), gb = smem_addr(sG);
-            for (int c9 = 0; c9 < 9; c9++) {
-                const int dz = c9 / 3 - 1, dxi = c9 % 3;
-                const uint32_t d = tmem + (uint32_t)(c9 * 32);
-                for (int iz = 0; iz < WT_TZ; iz++)
-                    for (int iy = 0; iy < WT_TY; iy++) {
-                        const int m0 = ((iz + 1 + dz) * WT_HY + iy) * 32;   // rows of dy = -1
-                        for (int ks = 0; ks < 2; ks++) {
+            // accumulators innermost, as in the convolution: nine independent
+            // chains, each in the same order as before
+            for (int iz = 0; iz < WT_TZ; iz++)
+                for (int iy = 0; iy < WT_TY; iy++)
+                    for (int ks = 0; ks < 2; ks++) {
+                        const uint64_t bd =
+                            smem_desc(gb + (uint32_t)((iz * WT_TY + iy) * WT_GROW + 2 * ks * 512), 512, 128);
+#pragma unroll
+                        for (int c9 = 0; c9 < 9; c9++) {
+                            const int dz = c9 / 3 - 1, dxi = c9 % 3;
+                            const int m0 = ((iz + 1 + dz) * WT_HY + iy) * 32;   // rows of dy = -1
                             const uint64_t ad =
                                 smem_desc(tb + (uint32_t)(dxi * WT_COPY + 2 * ks * WT_LBO + m0 * 16), WT_LBO, 128);
-                            const uint64_t bd =
-                                smem_desc(gb + (uint32_t)((iz * WT_TY + iy) * WT_GROW + 2 * ks * 512), 512, 128);
-                            tc_mma(d, ad, bd, TcShape<32, 32>::IDESC, (committed | iz | iy | ks) ? 1u : 0u);
+                            tc_mma(tmem + (uint32_t)(c9 * 32), ad, bd, TcShape<32, 32>::IDESC,
+                                   (committed | iz | iy | ks) ? 1u : 0u);
                         }
                     }
-            }
             tc_commit(&mma_bar);
             committed++;
         }
