@@ -17,12 +17,18 @@
 // kernel in the same layout.
 //
 // Warp roles (persistent, one CTA per SM): warp 5 lane 0 issues the tensor
-// copies (two input stages), warp 4 lane 0 the MMAs (two accumulator stages
-// of 4 x 32 TMEM columns), warps 0-3 the epilogue (tcgen05.ld of one TMEM lane
+// copies (two input stages), warp 4 the MMAs (two accumulator stages of
+// 4 x 32 TMEM columns), warps 0-3 the epilogue (tcgen05.ld of one TMEM lane
 // = one voxel's 32 channels per thread; bias, residual, ReLU; BF16 / FP32
 // stores).  Every mbarrier wait is bounded: a wait that runs out raises the
 // CTA's abort flag and the device fault flag, every role leaves its loop,
 // and TMEM is freed before the kernel returns.
+//
+// What bounds it: the MMAs' A reads (4 KB of shared memory for a 128 x 32 x 16
+// product, 32 cycles), once nothing else holds the issue up.  A whole forward
+// pass over 128 x 128 x 32 voxels: 1423 us with each row block's 54 MMAs one
+// after another (each waits for the sum before it), 1073 with the four row
+// blocks innermost, 752 with the loop run by the whole warp (below).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -85,14 +91,18 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
 }
 
 // kind::f16 MMA, M = 128: D FP32, A and B BF16, both K-major (idesc).
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                       uint32_t accum)
+// Run by a whole warp with the same operands on every lane; the lane with
+// `leader` set issues.  Operands that are uniform over the warp stay in
+// uniform registers, which the instruction wants.
+__device__ __forceinline__ void tc_mma_leader(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                              uint32_t accum, uint32_t leader)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum), "r"(leader)
         : "memory");
 }
 
@@ -251,37 +261,46 @@ k_conv3d_tc(TcParams p, const __grid_constant__ CUtensorMap in_map, int cin_mem,
             }
         }
     } else if (warp == 4) {
-        // ---------------- MMA issuer
-        if (lane == 0) {
-            int i = 0;
-            for (long long tile = blockIdx.x; tile < p.tiles; tile += gridDim.x, i++) {
-                const int s = i & 1;
-                if (!wait_or_abort(&full_bar[s], (i >> 1) & 1, abort_flag)) break;
-                s_consumed = i + 1;
-                if (i >= 2 && !wait_or_abort(&tempty_bar[s], ((i >> 1) - 1) & 1, abort_flag)) break;
-                tc_fence_after();
-                const uint32_t a_base = smem_addr(sA + s * S::A_BYTES);
-                const uint32_t b_base = smem_addr(sB);
-                // row blocks innermost: the four accumulators are independent,
-                // so consecutive MMAs never wait for one another's result
-                // (each accumulator still sums its taps in the same order)
-                const uint32_t d0 = tmem + (uint32_t)(s * 4 * NOUT);
-                for (int tap = 0; tap < 27; tap++) {
-                    const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-                    const int off = (dz * TC_HY + dy) * TC_HX + dx;
+        // ---------------- MMA issuer: the whole warp runs the loop, lane 0 issues.
+        // In a branch that only lane 0 takes, the compiler keeps descriptors in
+        // per-lane registers and has to move them to uniform ones for every
+        // MMA: 80 cycles an MMA, issue-bound.  Run by all lanes the operands
+        // are uniform and a descriptor is one uniform add.  Nine taps unrolled
+        // (the offsets fold): a forward pass takes 752 us, against 777 with
+        // three, 862 with one and 916 with all 27 (instruction fetches).
+        const uint32_t leader = lane == 0;
+        const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
+        const uint32_t sa = __shfl_sync(0xffffffffu, smem_addr(sA), 0), sb = __shfl_sync(0xffffffffu, smem_addr(sB), 0);
+        int i = 0;
+        for (long long tile = blockIdx.x; tile < p.tiles; tile += gridDim.x, i++) {
+            const int s = i & 1;
+            if (!__all_sync(0xffffffffu, wait_or_abort(&full_bar[s], (i >> 1) & 1, abort_flag))) break;
+            if (leader) s_consumed = i + 1;
+            if (i >= 2 && !__all_sync(0xffffffffu, wait_or_abort(&tempty_bar[s], ((i >> 1) - 1) & 1, abort_flag))) break;
+            tc_fence_after();
+            // row blocks innermost: the four accumulators are independent,
+            // so consecutive MMAs never wait for one another's result
+            // (each accumulator still sums its taps in the same order)
+            const uint32_t d0 = tmem_u + (uint32_t)(s * 4 * NOUT);
+            // A: planes 2kc, 2kc+1 (LBO) from row r0 + off; B: k-groups tap CINP/8 + 2kc, + 1
+            const uint64_t a0 = smem_desc(sa + (uint32_t)(s * S::A_BYTES + TC_ROW0 * 16), TC_PLANE_BYTES, 128);
+            const uint64_t b0 = smem_desc(sb, NOUT * 16, 128);
+#pragma unroll 9
+            for (int tap = 0; tap < 27; tap++) {
+                const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
+                const int off = (dz * TC_HY + dy) * TC_HX + dx;
 #pragma unroll
-                    for (int kc = 0; kc < S::KC; kc++) {
-                        // A: planes 2kc, 2kc+1 (LBO) from row r0 + off; B: k-groups tap CINP/8 + 2kc, + 1
-                        const uint64_t ad = smem_desc(
-                            a_base + (uint32_t)(2 * kc * TC_PLANE_BYTES + (TC_ROW0 + off) * 16), TC_PLANE_BYTES, 128);
-                        const uint64_t bd = smem_desc(
-                            b_base + (uint32_t)((tap * S::PLANES + 2 * kc) * NOUT * 16), NOUT * 16, 128);
+                for (int kc = 0; kc < S::KC; kc++) {
+                    // descriptor addresses are in units of 16 bytes, one row
+                    const uint64_t ad = a0 + (uint64_t)(int64_t)(2 * kc * (TC_PLANE_BYTES / 16) + off);
+                    const uint64_t bd = b0 + (uint64_t)((tap * S::PLANES + 2 * kc) * NOUT);
 #pragma unroll
-                        for (int rb = 0; rb < TC_RB; rb++)   // the next 128 rows: 2048 bytes on, in units of 16
-                            tc_mma(d0 + (uint32_t)(rb * NOUT), ad + (uint64_t)(128 * rb), bd, S::IDESC,
-                                   (tap | kc) ? 1u : 0u);
-                    }
+                    for (int rb = 0; rb < TC_RB; rb++)
+                        tc_mma_leader(d0 + (uint32_t)(rb * NOUT), ad + (uint64_t)(128 * rb), bd, S::IDESC,
+                                      (tap | kc) ? 1u : 0u, leader);
                 }
+            }
+            if (leader) {
                 tc_commit(&free_bar[s]);
                 tc_commit(&tfull_bar[s]);
                 s_committed = i + 1;
@@ -574,29 +593,37 @@ k_wgrad_tc(const __grid_constant__ CUtensorMap x_map, const __nv_bfloat16 *__res
         fence_proxy_async_smem();   // generic stores, read next by the tensor cores
         __syncthreads();            // operands written, X's stage free
         const bool more = tile + gridDim.x < tiles;
-        if (threadIdx.x == 0) {
-            if (more) issue_x(tile + gridDim.x);   // lands while the MMAs run
+        if (warp == 0) {
+            const uint32_t leader = lane == 0;
+            if (leader && more) issue_x(tile + gridDim.x);   // lands while the MMAs run
+            __syncwarp();
             tc_fence_after();
-            const uint32_t tb = smem_addr(sT), gb = smem_addr(sG);
-            // accumulators innermost, as in the convolution: nine independent
-            // chains, each in the same order as before
-            for (int iz = 0; iz < WT_TZ; iz++)
-                for (int iy = 0; iy < WT_TY; iy++)
-                    for (int ks = 0; ks < 2; ks++) {
-                        const uint64_t bd =
-                            smem_desc(gb + (uint32_t)((iz * WT_TY + iy) * WT_GROW + 2 * ks * 512), 512, 128);
+            // accumulators innermost and the loop run by the whole warp, as in
+            // the convolution: nine independent chains (a gradient over
+            // 128 x 128 x 32 voxels 3980 -> 3455 us, with the convolutions)
+            const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
+            const uint64_t a0 = smem_desc(__shfl_sync(0xffffffffu, smem_addr(sT), 0), WT_LBO, 128);
+            const uint64_t b0 = smem_desc(__shfl_sync(0xffffffffu, smem_addr(sG), 0), 512, 128);
+            const uint32_t fresh = __shfl_sync(0xffffffffu, (uint32_t)committed, 0) == 0;
+#pragma unroll 1
+            for (int row = 0; row < WT_TZ * WT_TY; row++) {
+                const int iz = row / WT_TY, iy = row % WT_TY;
 #pragma unroll
-                        for (int c9 = 0; c9 < 9; c9++) {
-                            const int dz = c9 / 3 - 1, dxi = c9 % 3;
-                            const int m0 = ((iz + 1 + dz) * WT_HY + iy) * 32;   // rows of dy = -1
-                            const uint64_t ad =
-                                smem_desc(tb + (uint32_t)(dxi * WT_COPY + 2 * ks * WT_LBO + m0 * 16), WT_LBO, 128);
-                            tc_mma(tmem + (uint32_t)(c9 * 32), ad, bd, TcShape<32, 32>::IDESC,
-                                   (committed | iz | iy | ks) ? 1u : 0u);
-                        }
+                for (int ks = 0; ks < 2; ks++) {
+                    // descriptor addresses are in units of 16 bytes
+                    const uint64_t bd = b0 + (uint64_t)((row * WT_GROW + 2 * ks * 512) / 16);
+#pragma unroll
+                    for (int c9 = 0; c9 < 9; c9++) {
+                        const int dz = c9 / 3 - 1, dxi = c9 % 3;
+                        const int m0 = ((iz + 1 + dz) * WT_HY + iy) * 32;   // rows of dy = -1
+                        const uint64_t ad = a0 + (uint64_t)((dxi * WT_COPY + 2 * ks * WT_LBO) / 16 + m0);
+                        tc_mma_leader(tmem_u + (uint32_t)(c9 * 32), ad, bd, TcShape<32, 32>::IDESC,
+                                      (fresh && row == 0 && ks == 0) ? 0u : 1u, leader);
                     }
-            tc_commit(&mma_bar);
-            committed++;
+                }
+            }
+            if (leader) tc_commit(&mma_bar);
+            if (leader) committed++;
         }
         if (more) load_g(tile + gridDim.x, gv);   // in flight during the MMAs
         // the operands are rewritten only after the MMAs completed; the
