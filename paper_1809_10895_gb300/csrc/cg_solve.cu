@@ -77,10 +77,11 @@ k_cg64_solve(Grid g, Tiles tw, const double *__restrict__ Tx, const double *__re
         struct Raw {
             double z, o;
         };
-        sweep64<Raw>(
+        sweep64<Raw, NoOwn>(
             g, tw, A, s.w64, [&](long long c) { return Raw{__ldcs(&z[c]), first ? 0.0 : __ldcs(&pin[c])}; },
             [&](const Raw &a) { return fma(beta, a.o, a.z); },
-            [&](long long c, double v, double Av, bool) {
+            [](long long) { return NoOwn{}; },
+            [&](long long c, double v, double Av, bool, NoOwn) {
                 pout[c] = v;
                 q[c] = Av;
                 acc[0] = fma(v, Av, acc[0]);

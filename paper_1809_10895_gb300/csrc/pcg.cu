@@ -91,10 +91,11 @@ k_cg64_spmv(Grid g, Tiles tw, const double *__restrict__ z, const double *__rest
     struct Raw {
         double z, o;
     };
-    sweep64<Raw>(
+    sweep64<Raw, NoOwn>(
         g, tw, A, s, [&](long long c) { return Raw{z[c], first ? 0.0 : p_in[c]}; },
         [&](const Raw &a) { return fma(beta, a.o, a.z); },
-        [&](long long c, double pv, double Ap, bool) {
+        [](long long) { return NoOwn{}; },
+        [&](long long c, double pv, double Ap, bool, NoOwn) {
             p_out[c] = pv;
             q[c] = Ap;
             v[0] = fma(pv, Ap, v[0]);

@@ -55,11 +55,12 @@ struct Op64 {
 };
 
 // Sweep of the FP64 operator over this block's items: value(c) is the vector
-// at cell c as a pair of loads (a, b) combined by mix; out(c, v, Av) takes an
-// in-grid cell's value and product.
-template <class Raw, class Load, class Mix, class Out>
+// at cell c as a pair of loads (a, b) combined by mix; out(c, v, Av, e) takes an
+// in-grid cell's value and product, and what own(c) loaded a plane ahead.
+struct NoOwn {};
+template <class Raw, class Own, class Load, class Mix, class LoadOwn, class Out>
 __device__ __forceinline__ void sweep64(const Grid &g, const Tiles &tw, const Op64 &A, Sweep64Shared &s, Load load,
-                                        Mix mix, Out out)
+                                        Mix mix, LoadOwn own, Out out)
 {
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, h = threadIdx.x;
     int hx, hy;
@@ -81,6 +82,7 @@ __device__ __forceinline__ void sweep64(const Grid &g, const Tiles &tw, const Op
         struct Coef {
             double d0, d1, x0, x1, y0, y1, z0, z1, hT;
             Raw h;
+            Own e0, e1;
         };
         auto coef = [&](int k) {
             Coef a{};
@@ -90,12 +92,14 @@ __device__ __forceinline__ void sweep64(const Grid &g, const Tiles &tw, const Op
                 a.x0 = __ldcs(&A.Tx[c]);
                 a.y0 = __ldcs(&A.Ty[c]);
                 a.z0 = __ldcs(&A.Tz[c]);
+                a.e0 = own(c);
             }
             if (in1) {
                 a.d1 = __ldcs(&A.diag[c + nx]);
                 a.x1 = __ldcs(&A.Tx[c + nx]);
                 a.y1 = __ldcs(&A.Ty[c + nx]);
                 a.z1 = __ldcs(&A.Tz[c + nx]);
+                a.e1 = own(c + nx);
             }
             if (halo) {
                 const long long hc = hcol + sxy * k;
@@ -156,8 +160,8 @@ __device__ __forceinline__ void sweep64(const Grid &g, const Tiles &tw, const Op
                 a0 = fma(-cur.z0, pn0, a0);
                 a1 = fma(-cur.z1, pn1, a1);
             }
-            if (in0) out(c, pc0, a0, act0);
-            if (in1) out(c + nx, pc1, a1, act1);
+            if (in0) out(c, pc0, a0, act0, cur.e0);
+            if (in1) out(c + nx, pc1, a1, act1, cur.e1);
             tzm0 = cur.z0;
             tzm1 = cur.z1;
             pm0 = pc0;
@@ -365,7 +369,11 @@ __device__ __forceinline__ void cg32_update_cells(const Grid &g, float alpha, bo
 }
 
 // FP64 residual r = b - A x over this block's items as FP32 seeds r32 and
-// z32 = D^-1 r32 (d32, when given, becomes 0); v accumulates r.r, b.b and r.z of the seeds in FP32.
+// z32 = D^-1 r32 (d32, when given, becomes 0); v accumulates r.r, b.b and r.z
+// of the seeds in FP32.  b and D^-1 are loaded with the coefficients: loaded
+// where they are used, behind the plane's barrier, they cost a memory latency
+// a plane (384 x 320 x 64 cells, 6.1 M active: 238.6 -> 180.6 us; its 8 FP64
+// instructions a cell alone take 78).
 __device__ __forceinline__ void resid64_sweep(const Grid &g, const Tiles &tw, const Op64 &A, Sweep64Shared &s,
                                               const uint8_t *__restrict__ flags, const double *x,
                                               const double *__restrict__ b, const float *__restrict__ dinv32,
@@ -375,17 +383,22 @@ __device__ __forceinline__ void resid64_sweep(const Grid &g, const Tiles &tw, co
         double x;
         uint8_t fl;
     };
-    sweep64<Raw>(
+    struct Own {
+        double b;
+        float di;
+    };
+    sweep64<Raw, Own>(
         g, tw, A, s, [&](long long c) { return Raw{x[c], flags[c]}; },
         // an inactive cell's head may be anything; its faces' T = 0 needs a number
         [&](const Raw &a) { return (a.fl & FLAG_ACTIVE) ? a.x : 0.0; },
-        [&](long long c, double, double Ax, bool act) {
+        [&](long long c) { return Own{__ldcs(&b[c]), __ldcs(&dinv32[c])}; },
+        [&](long long c, double, double Ax, bool act, const Own &e) {
             float rf = 0.0f, zf = 0.0f;
             if (act) {
-                const double bp = b[c], rp = bp - Ax;
-                const float bf = ix_d2f(bp);
+                const double rp = e.b - Ax;
+                const float bf = ix_d2f(e.b);
                 rf = ix_d2f(rp);
-                zf = dinv32[c] * rf;
+                zf = e.di * rf;
                 v[0] = fmaf(rf, rf, v[0]);
                 v[1] = fmaf(bf, bf, v[1]);
                 v[2] = fmaf(rf, zf, v[2]);
