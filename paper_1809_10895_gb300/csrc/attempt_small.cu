@@ -12,9 +12,11 @@
 // other kernels (cell_ops.cuh).
 //
 // Every reduction is one grid barrier (grid_red.cuh) after which all blocks
-// hold bit-identical scalars and take the same decisions.  FP64 adds are few
-// on purpose (2 thread-operations per clock and SM): threads stage their values
-// in shared memory and warp 0 alone sums them.
+// hold bit-identical scalars and take the same decisions.  Sums run on the
+// integer pipes (ix_sum.cuh) and their scalars without FP64 divisions and
+// compares: of the 7240 cycles of a CG iteration on one block the two sums
+// took 4430, staged in shared memory and added by one warp in FP64 (200 cells,
+// 30 steps: 4.33 -> 3.94 ms; 30 000 cells on 117 blocks, 6 steps: 0.97 -> 0.94).
 //
 // Every loop is bounded as in the graph (max_it, outer_max_it, n_max), and a
 // barrier wait that runs out sets the fault flag and ends the kernel.
@@ -37,7 +39,8 @@ constexpr int AT_NV = 4;
 static_assert(AT_NV <= GR_NV && AT_WARPS == 8, "reduction layout");
 
 struct Shared {
-    double part[AT_NV][AT_THREADS];
+    IxSum part[AT_NV][AT_WARPS];
+    double partm[AT_WARPS];
     double tot[AT_NV];
     float partf[AT_NV][AT_WARPS];
     double alpha, beta, rho, stop2, max_dh;
@@ -67,16 +70,7 @@ template <int NV, class Fin>
 __device__ __forceinline__ bool grid_sum(Ctx &C, double (&v)[NV], Fin fin)
 {
     Shared &s = *C.s;
-#pragma unroll
-    for (int i = 0; i < NV; i++) s.part[i][threadIdx.x] = v[i];
-    __syncthreads();
-    return grid_red<OpSum, NV>(
-        C.R, s.tot, &s.abort,
-        [&](int i) {
-            const double *p = &s.part[i][threadIdx.x & 31];
-            return warp_reduce<OpSum>(((p[0] + p[32]) + (p[64] + p[96])) + ((p[128] + p[160]) + (p[192] + p[224])));
-        },
-        [&]() { fin(s.tot); });
+    return grid_red_sum<NV>(C.R, s.part, s.tot, &s.abort, v, [&]() { fin(s.tot); });
 }
 
 // The same for FP32 thread values: FP32 within a block, FP64 across blocks.
@@ -92,7 +86,7 @@ __device__ __forceinline__ bool grid_sum_f32(Ctx &C, float (&v)[NV], Fin fin)
         if (lane == 0) s.partf[i][wid] = v[i];
     }
     __syncthreads();
-    return grid_red<OpSum, NV>(
+    return grid_red<OpIxSum, NV>(
         C.R, s.tot, &s.abort,
         [&](int i) {
             const float *p = s.partf[i];
@@ -105,14 +99,14 @@ __device__ __forceinline__ bool grid_sum_f32(Ctx &C, float (&v)[NV], Fin fin)
 __device__ __forceinline__ bool grid_max(Ctx &C, unsigned long long m)
 {
     Shared &s = *C.s;
-    const double t = warp_reduce<OpMaxBits>(__longlong_as_double((long long)m));
-    if ((threadIdx.x & 31) == 0) s.part[0][threadIdx.x >> 5] = t;
+    const double t = OpMaxBits::warp(__longlong_as_double((long long)m));
+    if ((threadIdx.x & 31) == 0) s.partm[threadIdx.x >> 5] = t;
     __syncthreads();
     return grid_red<OpMaxBits, 1>(
         C.R, s.tot, &s.abort,
         [&](int) {
             const int lane = threadIdx.x & 31;
-            return warp_reduce<OpMaxBits>(lane < AT_WARPS ? s.part[0][lane] : 0.0);
+            return OpMaxBits::warp(lane < AT_WARPS ? s.partm[lane] : 0.0);
         },
         [&]() { s.max_dh = s.tot[0]; });
 }
@@ -239,8 +233,8 @@ k_attempt_small(const __grid_constant__ AttemptArgs A)
             if (!grid_sum<3>(C, v, [&](const double *t) {
                     s.rho = t[0];
                     s.stop2 = A.tol_cg * A.tol_cg * t[2];
-                    s.ok = isfinite(t[0]) && isfinite(t[1]) && isfinite(t[2]);
-                    s.done = !s.ok || t[1] <= s.stop2;
+                    s.ok = is_finite(t[0]) && is_finite(t[1]) && is_finite(t[2]);
+                    s.done = !s.ok || not_above(t[1], s.stop2);
                     s.beta = 0.0;
                 }))
                 return;
@@ -274,8 +268,8 @@ k_attempt_small(const __grid_constant__ AttemptArgs A)
                     }
                 }
                 if (!grid_sum<1>(C, w, [&](const double *t) {
-                        s.alpha = s.rho * rcp64(t[0]);
-                        if (!(t[0] > 0.0) || !isfinite(s.alpha)) { s.ok = 0; s.done = 1; }
+                        s.alpha = ix_div(s.rho, t[0]);
+                        if (!is_positive(t[0]) || !is_finite(s.alpha)) { s.ok = 0; s.done = 1; }
                     }))
                     return;
                 if (s.done) break;
@@ -293,11 +287,11 @@ k_attempt_small(const __grid_constant__ AttemptArgs A)
                 }
                 cg++;
                 if (!grid_sum<2>(C, w2, [&](const double *t) {
-                        if (!isfinite(t[0]) || !isfinite(t[1])) { s.ok = 0; s.done = 1; }
-                        else if (t[0] <= s.stop2) s.done = 1;
+                        if (!is_finite(t[0]) || !is_finite(t[1])) { s.ok = 0; s.done = 1; }
+                        else if (not_above(t[0], s.stop2)) s.done = 1;
                         else if (cg >= A.cg_max_it) { s.ok = 0; s.done = 1; }
                         else {
-                            s.beta = t[1] * rcp64(s.rho);
+                            s.beta = ix_div(t[1], s.rho);
                             s.rho = t[1];
                         }
                     }))
@@ -307,12 +301,12 @@ k_attempt_small(const __grid_constant__ AttemptArgs A)
         } else {
             // defect correction: outer FP64 residuals, inner FP32 Jacobi-PCG
             auto outer_fin = [&](const double *t) {   // r.r, b.b, r.z of the FP32 seeds
-                s.ok = isfinite(t[0]) && isfinite(t[1]) && isfinite(t[2]);
-                s.done = !s.ok || t[0] <= A.tol_cg * A.tol_cg * t[1];
+                s.ok = is_finite(t[0]) && is_finite(t[1]) && is_finite(t[2]);
+                s.done = !s.ok || not_above(t[0], A.tol_cg * A.tol_cg * t[1]);
                 s.stop2 = A.tol_inner * A.tol_inner * t[0];
                 s.rho = t[2];
                 s.beta = 0.0;
-                s.iter = t[0] > 0.0;
+                s.iter = is_positive(t[0]);
             };
             if (!grid_sum_f32<3>(C, f3, outer_fin)) return;
             int outer = 1;
@@ -335,8 +329,8 @@ k_attempt_small(const __grid_constant__ AttemptArgs A)
                         w[0] = fmaf(pp, qp, w[0]);
                     }
                     if (!grid_sum_f32<1>(C, w, [&](const double *t) {
-                            s.alpha = s.rho * rcp64(t[0]);
-                            if (!(t[0] > 0.0) || !isfinite(s.alpha)) s.ok = 0;
+                            s.alpha = ix_div(s.rho, t[0]);
+                            if (!is_positive(t[0]) || !is_finite(s.alpha)) s.ok = 0;
                         }))
                         return;
                     if (!s.ok) break;
@@ -355,10 +349,10 @@ k_attempt_small(const __grid_constant__ AttemptArgs A)
                     inner++;
                     if (!grid_sum_f32<2>(C, w2, [&](const double *t) {
                             s.iter = 1;
-                            if (!isfinite(t[0]) || !isfinite(t[1])) s.ok = 0;
-                            else if (t[0] <= s.stop2 || inner >= A.inner_max_it) s.iter = 0;
+                            if (!is_finite(t[0]) || !is_finite(t[1])) s.ok = 0;
+                            else if (not_above(t[0], s.stop2) || inner >= A.inner_max_it) s.iter = 0;
                             else {
-                                s.beta = t[1] * rcp64(s.rho);
+                                s.beta = ix_div(t[1], s.rho);
                                 s.rho = t[1];
                             }
                         }))

@@ -326,17 +326,6 @@ __device__ __forceinline__ double chord_c(double dth, double dh, double V_dt)
                                 (__double_as_longlong(dh) & (long long)0x8000000000000000ULL)) * f;
 }
 
-// 1/a for a > 0.
-__device__ __forceinline__ double ix_rcp64(double a)
-{
-    const uint64_t b = (uint64_t)__double_as_longlong(a);
-    if ((unsigned)(b >> 52) - 400u < 1200u) {
-        const IxNum d = ix_unpack(b);
-        return __longlong_as_double((long long)fx_pack(ix_rcp(d.M), -1 - d.e));
-    }
-    return 1.0 / a;
-}
-
 // Storage part of a cell: c = V C^k / dt and its share s0 of the right side.
 // form: storage_form(sp), held by the caller.
 enum { STORE_CHORD = 0, STORE_MODIFIED = 1, STORE_BDF2 = 2 };

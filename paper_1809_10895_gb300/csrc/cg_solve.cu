@@ -21,28 +21,22 @@ struct CgShared {
     union {
         Sweep64Shared w64;
         Sweep32Shared w32;
-        double part[2][CT];                        // between sweeps
     };
+    IxSum part[2][CT / 32];
     float partf[3][CT / 32];
     double tot[4];
     double alpha, beta, rho, stop2;
     int done, status, iter, abort;
 };
 
-// The block's sum of its threads' values, by one warp per value.
+// Sums over the grid's threads.  fin runs on one thread while the rest wait, so
+// it has no FP64 division, root or compare (a microsecond together; an FP32
+// iteration over 256 x 256 x 64 cells took 46.6 us with them and block sums in
+// FP64, 45.7 without).
 template <int NV, class Fin>
 __device__ __forceinline__ bool cg_reduce(GridRed &R, CgShared &s, const double (&v)[NV], Fin fin)
 {
-#pragma unroll
-    for (int i = 0; i < NV; i++) s.part[i][threadIdx.x] = v[i];
-    __syncthreads();
-    return grid_red<OpSum, NV>(
-        R, s.tot, &s.abort,
-        [&](int i) {
-            const double *p = &s.part[i][threadIdx.x & 31];
-            return warp_reduce<OpSum>(((p[0] + p[32]) + (p[64] + p[96])) + ((p[128] + p[160]) + (p[192] + p[224])));
-        },
-        fin);
+    return grid_red_sum<NV>(R, s.part, s.tot, &s.abort, v, fin);
 }
 
 __global__ void __launch_bounds__(CT, SWEEP_OCC)
@@ -55,7 +49,7 @@ k_cg64_solve(Grid g, Tiles tw, const double *__restrict__ Tx, const double *__re
     count_work(g, KK_ONE_LAUNCH);
     __shared__ CgShared s;
     GridRed R = grid_red_begin(red, fault, g.wait_tries);
-    const double stop2 = sc->stop2;
+    const double stop2 = sc->stop2 * sc->stop2;
     const int max_it = sc->max_it;
     if (threadIdx.x == 0) {
         s.rho = sc->rho;
@@ -88,8 +82,8 @@ k_cg64_solve(Grid g, Tiles tw, const double *__restrict__ Tx, const double *__re
             });
         if (!cg_reduce<1>(R, s, acc, [&]() {
                 const double pq = s.tot[0];
-                s.alpha = s.rho / pq;
-                if (!(pq > 0.0) || !isfinite(s.alpha)) {
+                s.alpha = ix_div(s.rho, pq);
+                if (!is_positive(pq) || !is_finite(s.alpha)) {
                     s.status = CG_NONFINITE;
                     s.done = 1;
                 }
@@ -103,16 +97,16 @@ k_cg64_solve(Grid g, Tiles tw, const double *__restrict__ Tx, const double *__re
         it++;
         if (!cg_reduce<2>(R, s, v, [&]() {
                 const double rr = s.tot[0], rz = s.tot[1];
-                if (!isfinite(rr) || !isfinite(rz)) {
+                if (!is_finite(rr) || !is_finite(rz)) {
                     s.status = CG_NONFINITE;
                     s.done = 1;
-                } else if (sqrt(rr) <= stop2) {
+                } else if (not_above(rr, stop2)) {
                     s.done = 1;
                 } else if (it >= max_it) {
                     s.status = CG_MAXIT;
                     s.done = 1;
                 } else {
-                    s.beta = rz / s.rho;
+                    s.beta = ix_div(rz, s.rho);
                     s.rho = rz;
                 }
             }))
@@ -141,7 +135,7 @@ __device__ __forceinline__ bool cg_reduce_f32(GridRed &R, CgShared &s, float (&v
         if (lane == 0) s.partf[i][wid] = v[i];
     }
     __syncthreads();
-    return grid_red<OpSum, NV>(
+    return grid_red<OpIxSum, NV>(
         R, s.tot, &s.abort,
         [&](int i) {
             const float *p = s.partf[i];
@@ -178,7 +172,7 @@ k_mixed_solve(const __grid_constant__ MixedArgs M)
     GridRed R = grid_red_begin(M.red, M.fault, g.wait_tries);
     if (threadIdx.x == 0) {
         s.rho = M.inner->rho;
-        s.stop2 = M.inner->stop2;
+        s.stop2 = M.inner->stop2 * M.inner->stop2;
         s.beta = 0.0;
         s.iter = !M.inner->done;                   // an inner solve is due
         s.done = 0;
@@ -200,8 +194,8 @@ k_mixed_solve(const __grid_constant__ MixedArgs M)
             float w[1] = {sweep32(g, M.t32, s.w32, M.K32, M.cb32, M.z32, pin, pout, M.q32, beta, first)};
             if (!cg_reduce_f32<1>(R, s, w, [&]() {
                     const double pq = s.tot[0];
-                    s.alpha = s.rho / pq;
-                    if (!(pq > 0.0) || !isfinite(s.alpha)) s.status = CG_NONFINITE;
+                    s.alpha = ix_div(s.rho, pq);
+                    if (!is_positive(pq) || !is_finite(s.alpha)) s.status = CG_NONFINITE;
                 }))
                 break;
             if (s.status != CG_OK) break;
@@ -211,10 +205,10 @@ k_mixed_solve(const __grid_constant__ MixedArgs M)
             it++;
             if (!cg_reduce_f32<2>(R, s, v, [&]() {
                     const double rr = s.tot[0], rz = s.tot[1];
-                    if (!isfinite(rr) || !isfinite(rz)) s.status = CG_NONFINITE;
-                    else if (sqrt(rr) <= s.stop2 || it >= M.inner_max_it) s.iter = 0;   // applied even at the cap
+                    if (!is_finite(rr) || !is_finite(rz)) s.status = CG_NONFINITE;
+                    else if (not_above(rr, s.stop2) || it >= M.inner_max_it) s.iter = 0;   // applied even at the cap
                     else {
-                        s.beta = rz / s.rho;
+                        s.beta = ix_div(rz, s.rho);
                         s.rho = rz;
                     }
                 }))
@@ -250,20 +244,19 @@ k_mixed_solve(const __grid_constant__ MixedArgs M)
         outer++;
         if (!cg_reduce_f32<3>(R, s, f, [&]() {
                 const double rr = s.tot[0], bb = s.tot[1], rz = s.tot[2];
-                const double rn = sqrt(rr);
-                if (!(isfinite(rr) && isfinite(bb) && isfinite(rz))) {
+                if (!(is_finite(rr) && is_finite(bb) && is_finite(rz))) {
                     s.status = CG_NONFINITE;
                     s.done = 1;
-                } else if (rn <= M.tol * sqrt(bb)) {
+                } else if (not_above(rr, M.tol * M.tol * bb)) {
                     s.done = 1;
                 } else if (outer >= M.outer_max_it) {
                     s.status = CG_MAXIT;
                     s.done = 1;
                 }
                 s.rho = rz;
-                s.stop2 = M.tol_inner * rn;
+                s.stop2 = M.tol_inner * M.tol_inner * rr;
                 s.beta = 0.0;
-                s.iter = rr > 0.0;
+                s.iter = is_positive(rr);
             }))
             break;
         if (s.done) break;

@@ -9,15 +9,15 @@
 // reduction the blocks publish partials before arriving and each folds all of
 // them, in the same order, after it: results are bit-identical in every block.
 // Partials alternate between two buffers: a block writes one again only two
-// rounds later, when every block has passed the round between.  An FP64
-// instruction occupies a quarter of an SM for 64 cycles, so each value is
-// summed by a warp of its own.  Waits are bounded: one that runs out sets the
-// fault flag and the caller's abort flag.
+// rounds later, when every block has passed the round between.  Each value is
+// summed by a warp of its own, on the integer pipes (ix_sum.cuh).  Waits are
+// bounded: one that runs out sets the fault flag and the caller's abort flag.
 #pragma once
 
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "ix_sum.cuh"
 #include "rf_reduce.cuh"
 
 namespace rf {
@@ -72,6 +72,16 @@ struct OpMaxBits {
     {
         return (unsigned long long)__double_as_longlong(a) > (unsigned long long)__double_as_longlong(b) ? a : b;
     }
+    __device__ static double warp(double v)
+    {
+        return __longlong_as_double((long long)ix_warp_max((uint64_t)__double_as_longlong(v)));
+    }
+};
+
+struct OpIxSum {
+    __device__ static double id() { return 0.0; }
+    __device__ static double op(double a, double b) { return a + b; }
+    __device__ static double warp(double v) { return ix_double(ix_warp_sum(v)); }
 };
 
 // Fold value i of the blocks' partials (whole warp; the total on every lane).
@@ -81,7 +91,7 @@ __device__ __forceinline__ double grid_red_fold(const double *part, int i)
     const double *src = part + i * GR_BLOCKS;
     double t = Op::id();
     for (int b = threadIdx.x & 31; b < (int)gridDim.x; b += 32) t = Op::op(t, __ldcg(src + b));
-    return warp_reduce<Op>(t);
+    return Op::warp(t);
 }
 
 // Block totals (block(i) by warp i < NV, on lane 0 at least) to grid totals in
@@ -114,6 +124,27 @@ __device__ __forceinline__ bool grid_red(GridRed &R, double *tot, int *abort, Bl
     if (threadIdx.x == 0) fin();
     __syncthreads();
     return !*abort;
+}
+
+// Sum NV FP64 thread values of a block of eight warps over the grid; the rest
+// as in grid_red.
+template <int NV, class Fin>
+__device__ __forceinline__ bool grid_red_sum(GridRed &R, IxSum (*part)[8], double *tot, int *abort,
+                                             const double (&v)[NV], Fin fin)
+{
+#pragma unroll
+    for (int i = 0; i < NV; i++) {
+        const IxSum w = ix_warp_sum(v[i]);
+        if ((threadIdx.x & 31) == 0) part[i][threadIdx.x >> 5] = w;
+    }
+    __syncthreads();
+    return grid_red<OpIxSum, NV>(
+        R, tot, abort,
+        [&](int i) {
+            const int lane = threadIdx.x & 31;
+            return ix_fold8(lane < 8 ? part[i][lane] : IxSum{0, {0, 0, 0}});
+        },
+        fin);
 }
 #endif
 

@@ -77,6 +77,37 @@ __device__ __forceinline__ float ix_d2f(double a)
     return __uint_as_float((uint32_t)((v + 0x0fffffffULL + ((v >> 29) & 1)) >> 29) |
                            ((uint32_t)(b >> 32) & 0x80000000u));
 }
+
+// Tests on the bits: a compare of doubles goes to the FP64 pipe.
+__device__ __forceinline__ bool is_finite(double a)
+{
+    return ((uint32_t)__double2hiint(a) & 0x7ff00000u) != 0x7ff00000u;
+}
+__device__ __forceinline__ bool is_positive(double a)            // and no NaN
+{
+    return (unsigned long long)__double_as_longlong(a) - 1ULL < 0x7ff0000000000000ULL;
+}
+__device__ __forceinline__ bool not_above(double a, double b)    // a <= b, both >= 0 and no NaN
+{
+    return __double_as_longlong(a) <= __double_as_longlong(b);
+}
+
+// 1/a.
+__device__ __forceinline__ double ix_rcp64(double a)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(a);
+    if ((unsigned)(b >> 52) - 400u < 1200u) {
+        const IxNum d = ix_unpack(b);
+        return __longlong_as_double((long long)fx_pack(ix_rcp(d.M), -1 - d.e));
+    }
+    return 1.0 / a;
+}
+
+// a/b, to two roundings.
+__device__ __forceinline__ double ix_div(double a, double b)
+{
+    return (unsigned)((uint64_t)__double_as_longlong(b) >> 52) - 400u < 1200u ? a * ix_rcp64(b) : a / b;
+}
 #endif
 
 }  // namespace rf
