@@ -326,6 +326,19 @@ __device__ __forceinline__ double chord_c(double dth, double dh, double V_dt)
                                 (__double_as_longlong(dh) & (long long)0x8000000000000000ULL)) * f;
 }
 
+// Diagonal of a cell: c plus its six face coefficients.  In FP64 the six adds
+// were a quarter of the assembly's instructions on the FP64 pipe.
+__device__ __forceinline__ double diag_sum(double c, const double (&T)[6])
+{
+    const uint64_t b[7] = {(uint64_t)__double_as_longlong(c),    (uint64_t)__double_as_longlong(T[0]),
+                           (uint64_t)__double_as_longlong(T[1]), (uint64_t)__double_as_longlong(T[2]),
+                           (uint64_t)__double_as_longlong(T[3]), (uint64_t)__double_as_longlong(T[4]),
+                           (uint64_t)__double_as_longlong(T[5])};
+    uint64_t s;
+    if (ix_sum7(b, s)) return __longlong_as_double((long long)s);
+    return c + (((T[0] + T[1]) + (T[2] + T[3])) + (T[4] + T[5]));
+}
+
 // Storage part of a cell: c = V C^k / dt and its share s0 of the right side.
 // form: storage_form(sp), held by the caller.
 enum { STORE_CHORD = 0, STORE_MODIFIED = 1, STORE_BDF2 = 2 };
@@ -400,7 +413,7 @@ __device__ __forceinline__ void assemble_cell(const Grid &g, const DevSoil *__re
             sT = f == 0 ? T[f] * hN : fma(T[f], hN, sT);
         }
     }
-    double diag = c + (((T[0] + T[1]) + (T[2] + T[3])) + (T[4] + T[5]));
+    double diag = diag_sum(c, T);
     double rhs = fma(T[5], g.gd[F_ZMAX], fma(T[4], g.gd[F_ZMIN], s0));   // explicit gravity
     if (g.tilted) {
         rhs = fma(T[0], g.gd[F_XMIN], fma(T[1], g.gd[F_XMAX], rhs));

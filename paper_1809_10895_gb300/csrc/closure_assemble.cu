@@ -324,9 +324,10 @@ k_assemble(Grid g, const DevSoil *__restrict__ soils, const uint8_t *__restrict_
 // T = (K_P + K_N) hw, their sum and the two reciprocals are positive, so they
 // run in integer arithmetic (ix64.cuh) beside the narrow FP64 pipe, which
 // bounds the kernel; the top face of a plane is the bottom face of the next.
-// FP64 keeps the signed work: about 19 instructions a cell instead of 50.
-// 512 x 512 x 64 watershed (12.6 M active cells): 1105 us with one cell per
-// thread and all of it in FP64, 719 us here; 128 x 128 x 64 box 101 -> 68 us.
+// FP64 keeps the signed work: 13 instructions a cell instead of 50, 17 with
+// the first residual.  512 x 512 x 64 watershed (12.6 M active cells): 1105 us
+// with one cell per thread and all of it in FP64, 719 us with the diagonal's
+// six adds left in FP64, 652 here; 384 x 320 x 64 mixed 540 -> 381 -> 333 us.
 template <int MODE>
 __global__ void __launch_bounds__(RED_THREADS, 2)
 k_assemble_tiled(Grid g, Tiles tw, const DevSoil *__restrict__ soils, const uint8_t *__restrict__ zone,
@@ -430,7 +431,7 @@ k_assemble_tiled(Grid g, Tiles tw, const DevSoil *__restrict__ soils, const uint
                 const double T2 = face_coef(g, kym, Kc, g.hw[2], hwy), T3 = face_coef(g, Kc, kyp, g.hw[2], hwy);
                 Ttop = face_coef(g, Kc, Kn, g.hw[4], hwz);
                 const double hz = Kn >= 0 ? hu : 0.0;
-                double diag = c + (((T0 + T1) + (T2 + T3)) + (Tbot + Ttop));
+                double diag = diag_sum(c, {T0, T1, T2, T3, Tbot, Ttop});
                 double rhs = fma(Ttop, g.gd[F_ZMAX], fma(Tbot, g.gd[F_ZMIN], s0));   // explicit gravity
                 if (g.tilted) {
                     rhs = fma(T0, g.gd[F_XMIN], fma(T1, g.gd[F_XMAX], rhs));

@@ -52,6 +52,27 @@ RF_HD IxNum ix_add(IxNum a, IxNum b)
 
 RF_HD uint64_t ix_pack(IxNum a) { return fx_pack(a.M, a.e); }
 
+// Sum of seven doubles >= 0 (bits b), zeros among them: significands shifted
+// to the largest exponent with three bits of headroom, one rounding.  False,
+// without a result, when a term is negative or not finite or none exceeds
+// 2^-900.
+RF_HD bool ix_sum7(const uint64_t (&b)[7], uint64_t &sum)
+{
+    uint32_t top = 0;
+    for (int i = 0; i < 7; i++) top = top > (uint32_t)(b[i] >> 32) ? top : (uint32_t)(b[i] >> 32);
+    top >>= 20;
+    if (top - 123u > 1900u) return false;
+    uint64_t s = 0;
+    for (int i = 0; i < 7; i++) {
+        uint32_t d = top + 3 - (uint32_t)(b[i] >> 52);     // zeros and subnormals: more than 63
+        d = d < 63 ? d : 63;
+        s += ((b[i] << 11) | 0x8000000000000000ULL) >> d;
+    }
+    const int z = fx_clz(s);                               // 0 to 3
+    sum = fx_pack(s << z, (int)top - 1020 - z);
+    return true;
+}
+
 #ifdef __CUDACC__
 // 1/M for M in [1, 2) (Q63), Q64 in (0.5, 1): the single-precision estimate
 // ri refined by ri (1 + e + e^2), e = 1 - M ri < 2^-21.

@@ -2,6 +2,7 @@
 // same limbs, warp by warp, with the warp reductions as loops.
 #include <cstring>
 
+#include "ix64.cuh"
 #include "ix_sum.cuh"
 
 using namespace rf;
@@ -36,5 +37,16 @@ extern "C" double ix_sum32(const double *v, int n)
     const uint64_t r = s.e == 0x7ff ? ix_special_bits((uint32_t)s.l[0]) : ix_round(s.e, ix_join(s));
     double d;
     std::memcpy(&d, &r, 8);
+    return d;
+}
+
+// Sum of seven values >= 0; NaN when the integer form refuses them.
+extern "C" double ix_sum_seven(const double *v)
+{
+    uint64_t b[7], s = 0x7ff8000000000000ULL;
+    std::memcpy(b, v, sizeof b);
+    ix_sum7(b, s);
+    double d;
+    std::memcpy(&d, &s, 8);
     return d;
 }

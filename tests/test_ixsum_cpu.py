@@ -24,6 +24,7 @@ def lib(tmp_path_factory):
     L = C.CDLL(so)
     DP = C.POINTER(C.c_double)
     L.ix_sum32.restype, L.ix_sum32.argtypes = C.c_double, [DP, C.c_int]
+    L.ix_sum_seven.restype, L.ix_sum_seven.argtypes = C.c_double, [DP]
     return L, DP
 
 
@@ -57,3 +58,22 @@ def test_edges(sum32):
         assert sum32(np.array(v)) == want, v
     for v in ([np.nan, 1.0], [np.inf, -np.inf], [np.nan, np.inf]):
         assert np.isnan(sum32(np.array(v)))
+
+
+# Seven truncations below 2^-61 of the largest exponent's unit, one rounding.
+@pytest.mark.parametrize("spread", [0, 2, 20, 59, 61, 64, 200, 1100])
+def test_seven_terms(lib, spread):
+    L, DP = lib
+    rng = np.random.default_rng(spread)
+    for k in range(500):
+        v = np.ldexp(rng.uniform(1, 2, 7), rng.integers(-spread // 2, spread // 2 + 1, 7))
+        v[rng.random(7) < 0.3] = 0.0
+        v[k % 7] = max(v[k % 7], 2.0 ** -40)
+        exact = sum(Fraction(float(x)) for x in v)
+        top = Fraction(2) ** int(np.frexp(v.max())[1] - 1)
+        assert abs(Fraction(L.ix_sum_seven(v.ctypes.data_as(DP))) - exact) <= exact / 2 ** 53 + 8 * top / 2 ** 61
+    for bad in (-1.0, np.nan, np.inf, -0.0):
+        v = np.ones(7)
+        v[k % 7] = bad
+        assert np.isnan(L.ix_sum_seven(v.ctypes.data_as(DP)))
+    assert np.isnan(L.ix_sum_seven(np.zeros(7).ctypes.data_as(DP)))
