@@ -217,7 +217,7 @@ k_attempt_small(const __grid_constant__ AttemptArgs A)
                 v[1] = fma(rp, rp, v[1]);
                 v[2] = fma(cs.rhs, cs.rhs, v[2]);
             } else {
-                const float di = __frcp_rn(ix_d2f(cs.diag)), rf = (float)rp, zf = di * rf, bf = (float)cs.rhs;
+                const float di = __frcp_rn(ix_d2f(cs.diag)), rf = ix_d2f(rp), zf = di * rf, bf = ix_d2f(cs.rhs);
                 A.dinv32[p] = di;
                 A.r32[p] = rf;
                 A.z32[p] = zf;
@@ -361,7 +361,7 @@ k_attempt_small(const __grid_constant__ AttemptArgs A)
                 }
                 cg += inner;
                 if (!s.ok) { lin_ok = false; break; }
-                for (int p = p0; p < N; p += stride) x[p] += (double)A.d32[p];
+                for (int p = p0; p < N; p += stride) x[p] += ix_f2d(A.d32[p]);
                 if (!grid_sync(C)) return;
                 float f[3] = {0.0f, 0.0f, 0.0f};
                 for (int p = p0; p < N; p += stride) {
@@ -371,7 +371,7 @@ k_attempt_small(const __grid_constant__ AttemptArgs A)
                     const double rp = bp - apply64(g, p, A.Tx, A.Ty, A.Tz, A.diag, [&](long long q) {
                                           return (A.flags[q] & FLAG_ACTIVE) ? x[q] : 0.0;
                                       });
-                    const float rf = (float)rp, zf = A.dinv32[p] * rf, bf = (float)bp;
+                    const float rf = ix_d2f(rp), zf = A.dinv32[p] * rf, bf = ix_d2f(bp);
                     A.r32[p] = rf;
                     A.z32[p] = zf;
                     A.d32[p] = 0.0f;

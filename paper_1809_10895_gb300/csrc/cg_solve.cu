@@ -222,14 +222,14 @@ k_mixed_solve(const __grid_constant__ MixedArgs M)
             for (long long u = t0; u < n4; u += stride) {
                 const float4 d = reinterpret_cast<const float4 *>(M.d32)[u];
                 double2 a = reinterpret_cast<double2 *>(M.x)[2 * u], c = reinterpret_cast<double2 *>(M.x)[2 * u + 1];
-                a.x += (double)d.x;
-                a.y += (double)d.y;
-                c.x += (double)d.z;
-                c.y += (double)d.w;
+                a.x += ix_f2d(d.x);
+                a.y += ix_f2d(d.y);
+                c.x += ix_f2d(d.z);
+                c.y += ix_f2d(d.w);
                 reinterpret_cast<double2 *>(M.x)[2 * u] = a;
                 reinterpret_cast<double2 *>(M.x)[2 * u + 1] = c;
             }
-            for (long long c = 4 * n4 + t0; c < N; c += stride) M.x[c] += (double)M.d32[c];
+            for (long long c = 4 * n4 + t0; c < N; c += stride) M.x[c] += ix_f2d(M.d32[c]);
         }
         __syncthreads();
         if (gridDim.x > 1) {

@@ -22,6 +22,7 @@
 
 #include "cell_ops.cuh"
 #include "ensemble.cuh"
+#include "ix_sum.cuh"
 #include "rf_reduce.cuh"
 
 namespace cg = cooperative_groups;
@@ -40,11 +41,8 @@ struct ClusterCtx {
     double (*red)[RB_SLOTS][RB_WARPS];     // shared [2][RB_SLOTS][RB_WARPS]: per-warp FP64 partials
     double (*bc)[RB_SLOTS];                // shared [2][RB_SLOTS]: FP64 totals for the whole CTA
     float (*redf)[RB_SLOTS][RB_WARPS];     // shared [2][RB_SLOTS][RB_WARPS]: per-warp FP32 partials
-    double *part;                          // shared [RB_PART][blockDim]: per-thread FP64 partials
     int rb;                                // reduction double-buffer index (same in every CTA)
 };
-
-constexpr int RB_PART = 4;   // FP64 values a single-CTA reduction stages per thread
 
 // Finisher of a reduction that derives nothing.
 struct NoFin {
@@ -74,75 +72,46 @@ __device__ __forceinline__ T warp_allreduce(T x)
     return x;
 }
 
-// Tree reduction to lane 0.
-template <class Op>
-__device__ __forceinline__ double warp_reduce_lane0(double x)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x = Op::op(x, __shfl_down_sync(0xffffffffu, x, o));
-    return x;
-}
-
-// Sum (or max) NV FP64 values over all threads of the instance's CTAs; every
+// Sum NV FP64 values over all threads of the instance's CTAs; every
 // thread gets the totals, bit-identical in every CTA, and the ND scalars
 // fin(totals, d) derives from them (computed once, by one thread, and
 // broadcast: a divide or square root that every thread repeated would cost
-// the narrow FP64 pipe of this GPU hundreds of cycles).  FP64 adds are kept
-// few for the same reason.  On one CTA every thread stages its values in
-// shared memory and warp 0 sums them (nw values a lane, then one tree).  On
-// a cluster each warp reduces its values to lane 0, which publishes them;
-// one cluster barrier; warp 0 of every CTA folds all partials of all CTAs
-// (lane l reads partials l, l+32, ..., remote ones through distributed
-// shared memory, all loads in flight at once), in the same order in every
-// CTA.  A block barrier then hands the results to the other warps.  The
-// double-buffered slots are rewritten two reductions later, after the next
-// barrier, which every reader has passed; the per-thread slots are rewritten
-// only after this reduction's last barrier.
-template <class Op, int NV, int ND = 0, class Fin = NoFin>
-__device__ __forceinline__ void cl_reduce(ClusterCtx &C, double (&v)[NV], double *d = nullptr, Fin fin = Fin{})
+// the narrow FP64 pipe of this GPU hundreds of cycles).  Warps sum on the
+// integer pipes (ix_sum.cuh): an FP64 instruction of every thread holds the
+// pipe for 256 cycles.  Each warp publishes its sums; one barrier; warp 0 of
+// every CTA folds all partials of all CTAs (lane l reads partials l, l+32,
+// ..., remote ones through distributed shared memory, all loads in flight at
+// once), in the same order in every CTA.  A block barrier then hands the
+// results to the other warps.  The double-buffered slots are rewritten two
+// reductions later, after the next barrier, which every reader has passed.
+template <int NV, int ND = 0, class Fin = NoFin>
+__device__ __forceinline__ void cl_sum(ClusterCtx &C, double (&v)[NV], double *d = nullptr, Fin fin = Fin{})
 {
-    static_assert(NV + ND <= RB_SLOTS && NV <= RB_PART, "reduction slots");
+    static_assert(NV + ND <= RB_SLOTS, "reduction slots");
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    double t[NV];
-    if (C.ncta == 1) {
 #pragma unroll
-        for (int i = 0; i < NV; i++) C.part[i * blockDim.x + threadIdx.x] = v[i];
-        __syncthreads();
-        if (wid == 0) {
-#pragma unroll
-            for (int i = 0; i < NV; i++) t[i] = Op::id();
-            for (int w = 0; w < nw; w++) {
-#pragma unroll
-                for (int i = 0; i < NV; i++) t[i] = Op::op(t[i], C.part[i * blockDim.x + 32 * w + lane]);
-            }
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < NV; i++) v[i] = warp_reduce_lane0<Op>(v[i]);
-        if (lane == 0) {
-#pragma unroll
-            for (int i = 0; i < NV; i++) C.red[C.rb][i][wid] = v[i];
-        }
-        unit_sync(C);
-        if (wid == 0) {
-            const int total = C.ncta * nw;   // <= 8 * 16
-#pragma unroll
-            for (int i = 0; i < NV; i++) t[i] = Op::id();
-#pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const int s = lane + 32 * u;
-                if (s < total) {
-                    const int r = s / nw, w = s - r * nw;
-                    const double *src = C.cl.map_shared_rank(&C.red[C.rb][0][w], r);
-#pragma unroll
-                    for (int i = 0; i < NV; i++) t[i] = Op::op(t[i], src[i * RB_WARPS]);
-                }
-            }
-        }
+    for (int i = 0; i < NV; i++) {
+        const double w = ix_double(ix_warp_sum(v[i]));
+        if (lane == 0) C.red[C.rb][i][wid] = w;
     }
+    unit_sync(C);
     if (wid == 0) {
+        const int total = C.ncta * nw;   // <= 8 * 16
+        double t[NV];
 #pragma unroll
-        for (int i = 0; i < NV; i++) t[i] = warp_reduce_lane0<Op>(t[i]);
+        for (int i = 0; i < NV; i++) t[i] = 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int s = lane + 32 * u;
+            if (s < total) {
+                const int r = s / nw, w = s - r * nw;
+                const double *src = C.solo ? &C.red[C.rb][0][w] : C.cl.map_shared_rank(&C.red[C.rb][0][w], r);
+#pragma unroll
+                for (int i = 0; i < NV; i++) t[i] = u == 0 ? src[i * RB_WARPS] : t[i] + src[i * RB_WARPS];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < NV; i++) t[i] = ix_double(ix_warp_sum(t[i]));
         if (lane == 0) {
 #pragma unroll
             for (int i = 0; i < NV; i++) C.bc[C.rb][i] = t[i];
@@ -162,6 +131,29 @@ __device__ __forceinline__ void cl_reduce(ClusterCtx &C, double (&v)[NV], double
         for (int i = 0; i < ND; i++) d[i] = C.bc[C.rb][NV + i];
     }
     C.rb ^= 1;
+}
+
+// Maximum over all threads of the instance's CTAs; every warp folds.
+__device__ __forceinline__ uint64_t cl_max(ClusterCtx &C, uint64_t v)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    v = ix_warp_max(v);
+    if (lane == 0) C.red[C.rb][0][wid] = __longlong_as_double((long long)v);
+    unit_sync(C);
+    const int total = C.ncta * nw;
+    uint64_t m = 0;
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+        const int s = lane + 32 * u;
+        if (s < total) {
+            const int r = s / nw, w = s - r * nw;
+            const double *src = C.solo ? &C.red[C.rb][0][w] : C.cl.map_shared_rank(&C.red[C.rb][0][w], r);
+            const uint64_t o = (uint64_t)__double_as_longlong(*src);
+            m = o > m ? o : m;
+        }
+    }
+    C.rb ^= 1;
+    return ix_warp_max(m);
 }
 
 // FP32 sums for the inner PCG: FP32 adds are cheap, so every warp folds all
@@ -610,8 +602,7 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
     __shared__ double bc[2][RB_SLOTS];
     __shared__ float redf[2][RB_SLOTS][RB_WARPS];
     __shared__ int s_inst;
-    __shared__ double part[RB_PART * THREADS];
-    ClusterCtx C{cg::this_cluster(), 0, 1, false, red, bc, redf, part, 0};
+    ClusterCtx C{cg::this_cluster(), 0, 1, false, red, bc, redf, 0};
     const int cl_rank = (int)C.cl.block_rank(), cl_size = (int)C.cl.num_blocks();
     C.rank = cl_rank;
     C.ncta = cl_size;
@@ -679,13 +670,14 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
         long long budget = P.step_budget;
 
         // closures at the current state h (K, theta*_n, C)
-        auto closure_at = [&](const double *hx, const double *hprev, double *thx, double *Kx, double (&v)[2]) {
+        auto closure_at = [&](const double *hx, const double *hprev, double *thx, double *Kx, uint64_t &mx) {
             for (long long p = lo + threadIdx.x; p < hi; p += blockDim.x) {
                 const double hp = hx[p];
                 if (hprev) {
-                    const double dd = fabs(hp - hprev[p]);
-                    if (dd <= 1e300) v[0] = fmax(v[0], dd);
-                    else v[1] = 1.0;
+                    // |dh| by its bits; all ones above 1e300, infinite or NaN
+                    uint64_t dd = (uint64_t)__double_as_longlong(hp - hprev[p]) & 0x7fffffffffffffffULL;
+                    dd = dd > 0x7e37e43c8800759cULL ? ~0ULL : dd;
+                    mx = dd > mx ? dd : mx;
                 }
                 double th, k, c;
                 closure(*soil, Ks[p], hp, g.tab, &g.tab->fx, g.closure64, th, k, c);
@@ -695,11 +687,11 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
             }
         };
         if (status == ENS_NEW) {
-            double v2[2] = {0.0, 0.0};
-            closure_at(H[hb], nullptr, TH[tn], KB[kb], v2);
+            uint64_t none = 0;
+            closure_at(H[hb], nullptr, TH[tn], KB[kb], none);
             double s1[1] = {0.0};
             for (long long p = lo + threadIdx.x; p < hi; p += blockDim.x) s1[0] += g.V * TH[tn][p];
-            cl_reduce<OpSum, 1>(C, s1);   // also publishes the closures
+            cl_sum<1>(C, s1);   // also publishes the closures
             if (C.rank == 0 && threadIdx.x == 0) d.storage0 = s1[0];
             status = ENS_RUNNING;
         }
@@ -708,9 +700,10 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
         // tolerance, by squares, and the inner solve's FP32 threshold.  One
         // thread derives them: an FP64 root is some fifteen dependent
         // instructions of 64 cycles.
-        auto converged = [&](double rr, double bb, double tol) { return rr <= tol * tol * bb ? 1.0 : 0.0; };
+        auto converged = [&](double rr, double bb, double tol) { return not_above(rr, tol * tol * bb) ? 1.0 : 0.0; };
         auto inner_stop = [&](double rr) {
-            return P.tol_inner * (rr > 1e-30 && rr < 1e30 ? (double)sqrtf((float)rr) : sqrt(rr));
+            const bool f32 = ((uint64_t)__double_as_longlong(rr) >> 52) - 924u < 198u;   // 2^-99 to 2^99
+            return P.tol_inner * (f32 ? ix_f2d(sqrtf(ix_d2f(rr))) : sqrt(rr));
         };
 
         while (status == ENS_RUNNING && t < t_end - t_tol_d(t_end)) {
@@ -728,8 +721,8 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                 int hkb = (hb + 1) % 3, xb = (hb + 2) % 3;
                 for (long long p = lo + threadIdx.x; p < hi; p += blockDim.x) H[hkb][p] = H[hb][p];
                 if (!closure_valid) {
-                    double v2[2] = {0.0, 0.0};
-                    closure_at(H[hkb], nullptr, TH[tn ^ 1], KB[kb], v2);
+                    uint64_t none = 0;
+                    closure_at(H[hkb], nullptr, TH[tn ^ 1], KB[kb], none);
                     closure_valid = true;
                 }
                 unit_sync(C);
@@ -772,18 +765,18 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                             v[1] = fma(cs.rhs, cs.rhs, v[1]);
                             v[2] = fma(rp, zp, v[2]);
                         } else {
-                            const float rf = (float)rp;
+                            const float rf = ix_d2f(rp);
                             const float zf = d32v * rf;
                             r32[p] = rf;
                             z32[p] = zf;
                             d32[p] = 0.0f;
                             v[0] = fma(rp, rp, v[0]);
                             v[1] = fma(cs.rhs, cs.rhs, v[1]);
-                            if (!P.zline) v[2] += (double)(rf * zf);   // the line solve derives its own
+                            if (!P.zline) v[2] += ix_f2d(rf * zf);   // the line solve derives its own
                         }
                     }
                     double sq[2];   // converged, inner threshold
-                    cl_reduce<OpSum, 3, 2>(C, v, sq, [&](const double (&t)[3], double *o) {
+                    cl_sum<3, 2>(C, v, sq, [&](const double (&t)[3], double *o) {
                         o[0] = converged(t[0], t[1], P.tol_cg);
                         o[1] = PREC == 0 ? P.tol_cg * P.tol_cg * t[1] : inner_stop(t[0]);
                     });
@@ -793,7 +786,7 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                         // ---- FP64 Jacobi-PCG
                         double rho = v[2];
                         const double stop2 = sq[1];
-                        bool done = !(isfinite(v[0]) && isfinite(v[1]) && isfinite(v[2]));
+                        bool done = !(is_finite(v[0]) && is_finite(v[1]) && is_finite(v[2]));
                         if (done) lin_ok = false;
                         else done = sq[0] != 0.0;
                         double beta = 0.0;
@@ -811,9 +804,9 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                                 w1[0] += pp * qp;
                             }
                             double alpha;
-                            cl_reduce<OpSum, 1, 1>(C, w1, &alpha,
-                                                   [&](const double (&t)[1], double *o) { o[0] = rho / t[0]; });
-                            if (!(w1[0] > 0.0) || !isfinite(alpha)) { lin_ok = false; break; }
+                            cl_sum<1, 1>(C, w1, &alpha,
+                                                   [&](const double (&t)[1], double *o) { o[0] = ix_div(rho, t[0]); });
+                            if (!is_positive(w1[0]) || !is_finite(alpha)) { lin_ok = false; break; }
                             double w2[2] = {0.0, 0.0};
                             for (long long p = lo + threadIdx.x; p < hi; p += blockDim.x) {
                                 x[p] = fma(alpha, pout[p], x[p]);
@@ -825,14 +818,14 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                                 w2[1] += rp2 * zp2;
                             }
                             double fb[2];   // stop test passed (1 or 0), beta
-                            cl_reduce<OpSum, 2, 2>(C, w2, fb, [&](const double (&t)[2], double *o) {
-                                o[0] = t[0] <= stop2 ? 1.0 : 0.0;
-                                o[1] = t[1] / rho;
+                            cl_sum<2, 2>(C, w2, fb, [&](const double (&t)[2], double *o) {
+                                o[0] = not_above(t[0], stop2) ? 1.0 : 0.0;
+                                o[1] = ix_div(t[1], rho);
                             });
                             cg_it++;
                             pi ^= 1;
-                            if (!isfinite(w2[0]) || !isfinite(w2[1])) { lin_ok = false; break; }
-                            if (fb[0] != 0.0) break;
+                            if (!is_finite(w2[0]) || !is_finite(w2[1])) { lin_ok = false; break; }
+                            if (__double_as_longlong(fb[0]) != 0) break;
                             if (cg_it >= P.cg_max_it) { lin_ok = false; break; }
                             beta = fb[1];
                             rho = w2[1];
@@ -843,26 +836,26 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                         if (P.zline) zline_factor32(C, geo32(g), K32, cb32, LTi, LTc, LTP, LTQ, LTR);
                         int outer = 1;
                         for (;;) {
-                            const bool finite = isfinite(v[0]) && isfinite(v[1]) && isfinite(v[2]);
+                            const bool finite = is_finite(v[0]) && is_finite(v[1]) && is_finite(v[2]);
                             if (!finite) { lin_ok = false; break; }
-                            if (sq[0] != 0.0) break;
+                            if (__double_as_longlong(sq[0]) != 0) break;
                             if (outer >= P.outer_max_it) { lin_ok = false; break; }
                             // inner solve A d = r32 from d = 0, FP32 throughout
                             int inner_it = 0;
-                            if (v[0] > 0.0) {
-                                const float stop = (float)sq[1];
+                            if (is_positive(v[0])) {
+                                const float stop = ix_d2f(sq[1]);
                                 lin_ok = P.zline
                                              ? inner_pcg32<true>(C, geo32(g), (int)lo, (int)hi, K32, cb32, di32, r32,
                                                                  z32, P32[0], P32[1], q32, d32, LTi, LTc, LTP, LTQ,
                                                                  LTR, 0.0f, stop, P.inner_max_it, inner_it)
                                              : inner_pcg32<false>(C, geo32(g), (int)lo, (int)hi, K32, cb32, di32, r32,
                                                                   z32, P32[0], P32[1], q32, d32, nullptr, nullptr,
-                                                                  nullptr, nullptr, nullptr, (float)v[2], stop,
+                                                                  nullptr, nullptr, nullptr, ix_d2f(v[2]), stop,
                                                                   P.inner_max_it, inner_it);
                             }
                             cg_it += inner_it;
                             if (!lin_ok) break;
-                            for (long long p = lo + threadIdx.x; p < hi; p += blockDim.x) x[p] += (double)d32[p];
+                            for (long long p = lo + threadIdx.x; p < hi; p += blockDim.x) x[p] += ix_f2d(d32[p]);
                             unit_sync(C);
                             // FP64 outer residual and new inner seeds
                             // (b.b stays in v[1])
@@ -870,16 +863,16 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                             for (long long p = lo + threadIdx.x; p < hi; p += blockDim.x) {
                                 const double bp = bb[p];
                                 const double rp = bp - apply64(g, p, Tx, Ty, Tz, dg, [&](long long qq) { return x[qq]; });
-                                const float rf = (float)rp;
+                                const float rf = ix_d2f(rp);
                                 const float zf = di32[p] * rf;
                                 r32[p] = rf;
                                 z32[p] = zf;
                                 d32[p] = 0.0f;
                                 w[0] = fma(rp, rp, w[0]);
-                                if (!P.zline) w[1] += (double)(rf * zf);
+                                if (!P.zline) w[1] += ix_f2d(rf * zf);
                             }
                             const double bb = v[1];
-                            cl_reduce<OpSum, 2, 2>(C, w, sq, [&](const double (&t)[2], double *o) {
+                            cl_sum<2, 2>(C, w, sq, [&](const double (&t)[2], double *o) {
                                 o[0] = converged(t[0], bb, P.tol_cg);
                                 o[1] = inner_stop(t[0]);
                             });
@@ -891,14 +884,14 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                     if (!lin_ok) { fail = true; break; }
                     cg_att += cg_it;
                     // ---- closures at the new iterate and the global Picard test (Sec. 2.3)
-                    double w[2] = {0.0, 0.0};
-                    closure_at(x, hk, TH[tn ^ 1], KB[kin ^ 1], w);
-                    cl_reduce<OpMax, 2>(C, w);
+                    uint64_t mx = 0;
+                    closure_at(x, hk, TH[tn ^ 1], KB[kin ^ 1], mx);
+                    mx = cl_max(C, mx);
                     const int kold = kin;
                     kin ^= 1;
                     { const int tmp = hkb; hkb = xb; xb = tmp; }
-                    if (w[1] > 0.0) { fail = true; break; }
-                    if (w[0] <= P.tol_picard) {
+                    if (mx == ~0ULL) { fail = true; break; }
+                    if ((long long)mx <= __double_as_longlong(P.tol_picard)) {
                         conv = true;
                         // water balance of this last linear system (x = H[hkb])
                         double m4[4] = {0.0, 0.0, 0.0, 0.0};
@@ -914,7 +907,7 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                                 m4[3] += dt * fout;
                             }
                         }
-                        cl_reduce<OpSum, 4>(C, m4);
+                        cl_sum<4>(C, m4);
                         const double net = m4[2] - m4[3];
                         in_cum += m4[2];
                         out_cum += m4[3];

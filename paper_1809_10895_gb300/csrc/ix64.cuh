@@ -113,6 +113,15 @@ __device__ __forceinline__ bool not_above(double a, double b)    // a <= b, both
     return __double_as_longlong(a) <= __double_as_longlong(b);
 }
 
+// A float as a double.
+__device__ __forceinline__ double ix_f2d(float a)
+{
+    const uint32_t b = __float_as_uint(a), m = b & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u && m) return (double)a;   // subnormal, infinite or NaN
+    const uint64_t v = m ? ((uint64_t)m << 29) + (896ULL << 52) : 0;
+    return __longlong_as_double((long long)(v | (uint64_t)(b & 0x80000000u) << 32));
+}
+
 // 1/a.
 __device__ __forceinline__ double ix_rcp64(double a)
 {
