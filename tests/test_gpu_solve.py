@@ -54,3 +54,29 @@ def test_masked_cells_may_hold_anything(shape, precision, precond):
         heads.append((s.get_state()[0][act], [(i.picard, i.cg, i.rejected) for i in infos]))
     assert heads[0][1] == heads[1][1]
     assert np.array_equal(heads[0][0], heads[1][0])
+
+
+@pytest.mark.parametrize("shape,precision", [((96, 96, 64), "fp64"), ((96, 96, 64), "mixed"), ((40, 40, 30), "fp64")])
+def test_contexts_step_in_parallel_threads(shape, precision):
+    """Each launch's blocks wait for one another only; two contexts' launches
+    may be on the GPU at once."""
+    import threading
+    case = W.heterogeneous_box(*shape, d=0.25, seed=2, water_table_depth=4.0, rain=2e-6, dt0=30.0)
+
+    def run(out, k):
+        torch.cuda.set_device(0)
+        with torch.cuda.stream(torch.cuda.Stream()):
+            s = rf.Solver.from_case(case, precision=precision)
+            infos = [s.step() for _ in range(4)]
+            out[k] = (s.get_state()[0], [(i.dt, i.picard, i.cg) for i in infos])
+
+    alone, both = {}, {}
+    run(alone, 0)
+    ts = [threading.Thread(target=run, args=(both, k)) for k in range(3)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    for k in range(3):
+        assert both[k][1] == alone[0][1]
+        assert np.array_equal(both[k][0], alone[0][0])
