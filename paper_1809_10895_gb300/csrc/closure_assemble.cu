@@ -66,7 +66,9 @@ __device__ __forceinline__ bool grid_max_dh(MaxDh &m, double *partials, unsigned
 // an update was not finite.  In FP64 (table-driven exp and log, 106 FP64
 // instructions a cell) the kernel was bound by the FP64 pipe; in fixed point
 // it is bound by the integer pipes.  512 x 512 x 64 watershed, 12.6 M active
-// cells: 3288 -> 446 us (1.5 TB/s of its 651 MB); 1 M cells: 34 us.  The
+// cells: 3288 -> 446 us (1.5 TB/s of its 651 MB); 1 M cells: 34 us.  Loading
+// the next cell's inputs ahead takes 80 registers or spills: 5 to 15 % slower;
+// twice the blocks: 2.5 % faster there, 10 % slower on 1 M cells.  The
 // tables (10 KB) sit in shared memory, where a gather costs its bank
 // conflicts only.
 __device__ __forceinline__ void closure_cells(const Grid &g, const DevSoil *__restrict__ soils,
@@ -324,8 +326,8 @@ k_assemble(Grid g, const DevSoil *__restrict__ soils, const uint8_t *__restrict_
 // T = (K_P + K_N) hw, their sum and the two reciprocals are positive, so they
 // run in integer arithmetic (ix64.cuh) beside the narrow FP64 pipe, which
 // bounds the kernel; the top face of a plane is the bottom face of the next.
-// FP64 keeps the signed work: 13 instructions a cell instead of 50, 17 with
-// the first residual.  512 x 512 x 64 watershed (12.6 M active cells): 1105 us
+// FP64 keeps the signed work: 10 instructions a cell (18 with the first residual)
+// instead of 31.  512 x 512 x 64 watershed (12.6 M active cells): 1105 us
 // with one cell per thread and all of it in FP64, 719 us with the diagonal's
 // six adds left in FP64, 652 here; 384 x 320 x 64 mixed 540 -> 381 -> 333 us.
 template <int MODE>
