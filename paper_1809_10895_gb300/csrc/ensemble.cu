@@ -50,10 +50,11 @@ struct NoFin {
     __device__ void operator()(const double (&)[NV], double *) const {}
 };
 
-// Barrier over the threads that share the current instance.
+// Barrier over the threads that share the current instance.  One CTA, also as
+// a cluster of its own, needs no cluster barrier.
 __device__ __forceinline__ void unit_sync(ClusterCtx &C)
 {
-    if (C.solo) __syncthreads();
+    if (C.ncta == 1) __syncthreads();
     else C.cl.sync();
 }
 
@@ -105,7 +106,7 @@ __device__ __forceinline__ void cl_sum(ClusterCtx &C, double (&v)[NV], double *d
             const int s = lane + 32 * u;
             if (s < total) {
                 const int r = s / nw, w = s - r * nw;
-                const double *src = C.solo ? &C.red[C.rb][0][w] : C.cl.map_shared_rank(&C.red[C.rb][0][w], r);
+                const double *src = C.ncta == 1 ? &C.red[C.rb][0][w] : C.cl.map_shared_rank(&C.red[C.rb][0][w], r);
 #pragma unroll
                 for (int i = 0; i < NV; i++) t[i] = u == 0 ? src[i * RB_WARPS] : t[i] + src[i * RB_WARPS];
             }
@@ -147,7 +148,7 @@ __device__ __forceinline__ uint64_t cl_max(ClusterCtx &C, uint64_t v)
         const int s = lane + 32 * u;
         if (s < total) {
             const int r = s / nw, w = s - r * nw;
-            const double *src = C.solo ? &C.red[C.rb][0][w] : C.cl.map_shared_rank(&C.red[C.rb][0][w], r);
+            const double *src = C.ncta == 1 ? &C.red[C.rb][0][w] : C.cl.map_shared_rank(&C.red[C.rb][0][w], r);
             const uint64_t o = (uint64_t)__double_as_longlong(*src);
             m = o > m ? o : m;
         }
@@ -179,7 +180,7 @@ __device__ __forceinline__ void cl_reduce_f32(ClusterCtx &C, float (&v)[NV])
         const int s = lane + 32 * u;
         if (s < total) {
             const int r = s / nw, w = s - r * nw;
-            const float *src = C.solo ? &C.redf[C.rb][0][w] : C.cl.map_shared_rank(&C.redf[C.rb][0][w], r);
+            const float *src = C.ncta == 1 ? &C.redf[C.rb][0][w] : C.cl.map_shared_rank(&C.redf[C.rb][0][w], r);
 #pragma unroll
             for (int i = 0; i < NV; i++) t[i] = FSum::op(t[i], src[i * RB_WARPS]);
         }
