@@ -85,7 +85,7 @@ typedef enum rf_precision {
  * and the RF_PREC_MIXED path.  FP64: full FP64 accuracy
  * (within a few units of the last place), computed in 64-bit fixed point
  * where the state is in its range (|log2(-alpha h)| < 30, |n log2(-alpha h)|
- * < 60, n < 16) and in FP64 elsewhere.  DOUBLE_FLOAT: pairs of FP32 values
+ * < 60, n < 16, 1 - 1/n >= 2^-12) and in FP64 elsewhere.  DOUBLE_FLOAT: pairs of FP32 values
  * (about 48 significant bits: theta* within 1.2e-14 relative, K and C within
  * 2.4e-13).  Storage, the chord difference, the operator, the Picard test and
  * the balance are FP64 either way. */

@@ -661,23 +661,6 @@ const FFTables *ff_tables()
     return &t;
 }
 
-FxSoil make_fx_soil(int model, double alpha, double n, double m)
-{
-    FxSoil f{};
-    const long double la = log2l((long double)alpha);
-    // sizes for which every field fits its format; others keep the general closure
-    f.ok = (model == M_VG && n > 1.0 && n < 16.0 && m > 0.0 && la > -20.0L && la < 20.0L) ? 1 : 0;
-    if (!f.ok) return f;
-    f.ne = ilogb(n);
-    f.ea = ilogb(alpha);
-    f.la = (int64_t)rintl(la * 288230376151711744.0L);                          // 2^58
-    f.nm = (uint64_t)ldexpl((long double)n, 63 - f.ne);
-    f.m = (uint64_t)rintl((long double)m * 18446744073709551616.0L);            // 2^64
-    const long double Lm = 60.0L / (long double)n;
-    f.Lmax = (uint64_t)((Lm < 31.5L ? Lm : 31.5L) * 288230376151711744.0L);
-    return f;
-}
-
 void launch_closure(cudaStream_t s, int nblk, const Grid &g, const DevSoil *soils, const uint8_t *zone,
                     const double *Ks, const uint8_t *flags, const double *h, const double *hprev,
                     double *theta, double *K, double *Can, double *partials, unsigned int *ticket,

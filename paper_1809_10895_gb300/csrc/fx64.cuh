@@ -16,7 +16,10 @@
 // 1 - ys is formed with full relative precision: from the power series of
 // 1 - 2^-q where q = m B < 2^-9 (dry soil), and s likewise from the series of
 // log2(1 + x') where x' = 2^-|y| < 2^-9; both series are the tails of the
-// table-driven functions below, with the table entry 1.
+// table-driven functions below, with the table entry 1.  With a small m, q is
+// small in wet soil too: below FX_M_SMALL it is carried as a significand and
+// an exponent at every head (with q on the grid of 2^-57 K was off by 15 units
+// of the last place at n = 1.01, by 160 at 1.001).
 //
 // Logarithm and power of two: table-driven argument reduction (P. T. P. Tang,
 // ACM TOMS 15 (1989) 144-157 and 16 (1990) 378-400) with 512 entries and the
@@ -26,6 +29,7 @@
 // "Qk" below: an unsigned 64-bit integer v stands for v 2^-k.
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
 
 #ifdef __CUDACC__
@@ -50,12 +54,34 @@ struct FxTables {
 struct FxSoil {
     int64_t la;        // log2(alpha)  Q58
     uint64_t nm;       // n 2^-ne in [1, 2)  Q63
-    uint64_t m;        // m  Q64
+    uint64_t m;        // m  Q64 (exact: m >= 2^-12)
     uint64_t Lmax;     // largest |log2 u| with |y| < 60, Q58
     int ne;            // exponent of n
     int ea;            // floor(log2 alpha)
-    int ok, pad;
+    int ok;
+    int mz;            // leading zeros of m
 };
+
+constexpr int FX_M_SMALL = 4;   // m < 2^-FX_M_SMALL (n < 1.067): q as a significand and an exponent
+
+// Host: the constants of a van Genuchten soil.  Others, and parameters for
+// which a field would not fit its format, get ok = 0.
+inline FxSoil make_fx_soil(bool vg, double alpha, double n, double m)
+{
+    FxSoil f{};
+    const long double la = log2l((long double)alpha);
+    f.ok = (vg && n < 16.0 && m >= 0x1p-12 && la > -20.0L && la < 20.0L) ? 1 : 0;
+    if (!f.ok) return f;
+    f.ne = ilogb(n);
+    f.ea = ilogb(alpha);
+    f.la = (int64_t)rintl(la * 288230376151711744.0L);                          // 2^58
+    f.nm = (uint64_t)ldexpl((long double)n, 63 - f.ne);
+    f.m = (uint64_t)rintl((long double)m * 18446744073709551616.0L);            // 2^64
+    f.mz = -1 - ilogb(m);
+    const long double Lm = 60.0L / (long double)n;
+    f.Lmax = (uint64_t)((Lm < 31.5L ? Lm : 31.5L) * 288230376151711744.0L);
+    return f;
+}
 
 // High 64 bits of a 64 x 64 product, at most 2 units low: the low x low
 // product and one carry are left out (three 32 x 32 multiply-adds).
@@ -151,6 +177,31 @@ RF_HD uint64_t fx_pack(uint64_t M, int e)
     return ((uint64_t)(uint32_t)(e + 1022) << 52) + (M >> 11) + ((M >> 10) & 1);
 }
 
+// 1 - 2^-q = om 2^(eo - 63) for q = m (Bm 2^(eb - 62)), m < 2^-FX_M_SMALL, Bm
+// below 2^63 and the product below 4; mB: q as Q57.
+RF_HD void fx_one_minus_ys_small_m(const FxSoil &s, uint64_t Bm, int eb, uint64_t mB, const FxTables *tab,
+                                   uint64_t &om, int &eo)
+{
+    const int zb = fx_clz(Bm);
+    const uint64_t qm = fx_mulhi(Bm << zb, s.m << s.mz);                            // [2^62, 2^64)
+    const int eq = eb - zb - s.mz;                                                  // q = qm 2^(eq - 62)
+    const uint64_t q63 = eq <= -1 ? qm >> (eq < -64 ? 63 : -1 - eq) : ~0ULL;        // q  Q63 where q < 2
+    if (q63 < 1ULL << 54) {                                                         // q < 2^-9
+        const int sh = eq + 11;
+        const uint64_t gs = sh >= 0 ? qm << sh : qm >> (sh < -63 ? 63 : -sh);       // q 2^73
+        om = fx_mulhi(qm, fx_exp_w<true>(gs));
+        eo = eq + 1;
+        return;
+    }
+    eo = -1;
+    if (q63 >> 63) {                                                                // q >= 1: the bits of Q57 do
+        const int64_t z = -(int64_t)mB;
+        om = 0 - (fx_exp2((uint64_t)z << 7, tab) >> (-(int)(z >> 57) - 1));
+    } else {
+        om = 0 - fx_exp2((0x8000000000000000ULL - q63) << 1, tab);                  // 2^-q = 2^(1 - q) / 2
+    }
+}
+
 // Se, K/Ks and C/cfac (bit patterns of doubles) at |h| = the double with bits
 // hb, h < 0.  Returns false, without results, when the state is outside the
 // range of the fixed-point form (|log2 u| >= 31 or |y| >= 60; zero,
@@ -202,7 +253,9 @@ RF_HD bool fx_closure_vg(const FxSoil &s, uint64_t hb, const FxTables *tab, uint
     const uint64_t q63 = fx_mulhi(s63, s.m);                                        // m s  Q63
     uint64_t om;
     int eo;
-    if (dry && q63 < (1ULL << 54) - 8) {   // margin: fx_mulhi may be 2 units low
+    if (s.mz >= FX_M_SMALL) {
+        fx_one_minus_ys_small_m(s, dry ? sm : B, dry ? es : 5, mB, tab, om, eo);    // B 2^-57 = B 2^(5 - 62)
+    } else if (dry && q63 < (1ULL << 54) - 8) {   // margin: fx_mulhi may be 2 units low
         const int zs = fx_clz(sm);
         const uint64_t qm = fx_mulhi(sm << zs, s.m);                                // q = qm 2^(es - 62) < 2^-9
         es -= zs;

@@ -1231,7 +1231,7 @@ rf_status rf_soil_set(rf_ctx *c, const rf_soil *zones, int n_zones, const uint8_
         soils[z] = DevSoil{s.model, s.theta_r, s.theta_s, s.alpha, s.n, m, s.S,
                            nh, (float)(s.n - (double)nh), mh, (float)(m - (double)mh),
                            (s.theta_s - s.theta_r) * s.alpha * s.n * m, s.theta_s - s.theta_r,
-                           make_fx_soil(s.model, s.alpha, s.n, m)};
+                           make_fx_soil(s.model == RF_VG, s.alpha, s.n, m)};
     }
     const long long N = c->g.N;
     std::vector<uint8_t> zone(N, 0);

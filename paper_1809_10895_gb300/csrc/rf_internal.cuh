@@ -305,9 +305,6 @@ __device__ __forceinline__ void outer_residual_scalars(CgScal *outer, CgScal *in
 // Message returned by rf_last_error() on the calling thread.
 void set_last_error(const char *msg);
 
-// Fixed-point copies of a soil's alpha, n and m (closure_assemble.cu).
-FxSoil make_fx_soil(int model, double alpha, double n, double m);
-
 // Everything one Picard attempt of a small grid reads and writes
 // (attempt_small.cu); passed by value.
 struct AttemptArgs {
