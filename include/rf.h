@@ -331,13 +331,14 @@ rf_status rf_solve(rf_ctx *ctx, double *d_x, int *iters);
 rf_status rf_apply_inner(rf_ctx *ctx, const float *d_z, const float *d_pold, float beta, float *d_p, float *d_q,
                          double *pq);
 
-/* Test hook for the bounded device waits (failure detection): polls that a
- * wait for staged data (the TMA planes of the FP32 stencil) makes before it
- * gives up; polls = 0 restores the default (about a second of suspending
- * polls); polls < 0 makes each such wait a single non-blocking test.  A wait
- * that gives up stops the solve, drains the copies still in flight with the
- * default limit, and the call in progress returns RF_ERR_DEVICE_TIMEOUT with
- * the state unchanged and the context usable. */
+/* Test hook for the context's bounded device waits (failure detection): polls
+ * that a wait makes before it gives up -- for the TMA planes of the FP32
+ * stencil, the grid barriers of the one-launch attempts and solves, and the
+ * staged tiles and MMAs of an attached network's guess.  polls = 0 restores
+ * the default (seconds); polls < 0 makes each such wait a single non-blocking
+ * test.  A wait that gives up ends its kernel, copies still in flight are
+ * drained with the default limit, and the call in progress returns
+ * RF_ERR_DEVICE_TIMEOUT with the state unchanged and the context usable. */
 rf_status rf_set_wait_limit(rf_ctx *ctx, int polls);
 
 /* Number of CUDA kernel launches this context has executed on the device,

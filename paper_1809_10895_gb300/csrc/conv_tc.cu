@@ -80,6 +80,7 @@ struct TcParams {
     int B, D, H, W;
     int ntx, nty, ntz;       // tiles along x, y, z
     long long tiles;
+    int tries;               // of the bounded waits (wait_or_abort)
 };
 
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo)
@@ -164,11 +165,16 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, float (&v)[32])
 }
 
 // Bounded wait that also gives up when another role raised the abort flag.
-__device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, volatile int *abort_flag)
+// tries: polls (a test limit); 0: the default; negative: one non-blocking test.
+__device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, volatile int *abort_flag, int tries = 0)
 {
-    for (int t = 0; t < TC_WAIT_TRIES; t++) {
-        if (mbar_try_wait_sleep(bar, parity, 1000u)) return true;
-        if (*abort_flag) return false;
+    if (tries < 0) {
+        if (mbar_test_wait(bar, parity)) return true;
+    } else {
+        for (int t = 0, n = tries ? tries : TC_WAIT_TRIES; t < n; t++) {
+            if (mbar_try_wait_sleep(bar, parity, 1000u)) return true;
+            if (*abort_flag) return false;
+        }
     }
     *abort_flag = 1;
     return false;
@@ -256,7 +262,7 @@ k_conv3d_tc(TcParams p, const __grid_constant__ CUtensorMap in_map, int cin_mem,
             int i = 0;
             for (long long tile = blockIdx.x; tile < p.tiles; tile += gridDim.x, i++) {
                 const int s = i & 1;
-                if (i >= 2 && !wait_or_abort(&free_bar[s], ((i >> 1) - 1) & 1, abort_flag)) break;
+                if (i >= 2 && !wait_or_abort(&free_bar[s], ((i >> 1) - 1) & 1, abort_flag, p.tries)) break;
                 int b, z0, y0, x0;
                 tile_origin(p, tile, b, z0, y0, x0);
                 mbar_expect_tx(&full_bar[s], loaded * TC_BOX_BYTES);
@@ -286,9 +292,9 @@ k_conv3d_tc(TcParams p, const __grid_constant__ CUtensorMap in_map, int cin_mem,
         int i = 0;
         for (long long tile = blockIdx.x; tile < p.tiles; tile += gridDim.x, i++) {
             const int s = i & 1;
-            if (!__all_sync(0xffffffffu, wait_or_abort(&full_bar[s], (i >> 1) & 1, abort_flag))) break;
+            if (!__all_sync(0xffffffffu, wait_or_abort(&full_bar[s], (i >> 1) & 1, abort_flag, p.tries))) break;
             if (leader) s_consumed = i + 1;
-            if (i >= 2 && !__all_sync(0xffffffffu, wait_or_abort(&tempty_bar[s], ((i >> 1) - 1) & 1, abort_flag))) break;
+            if (i >= 2 && !__all_sync(0xffffffffu, wait_or_abort(&tempty_bar[s], ((i >> 1) - 1) & 1, abort_flag, p.tries))) break;
             tc_fence_after();
             // row blocks innermost: the four accumulators are independent,
             // so consecutive MMAs never wait for one another's result
@@ -324,7 +330,8 @@ k_conv3d_tc(TcParams p, const __grid_constant__ CUtensorMap in_map, int cin_mem,
         const long long HW = (long long)p.H * p.W;
         for (long long tile = blockIdx.x; tile < p.tiles; tile += gridDim.x, i++) {
             const int s = i & 1;
-            if (!wait_or_abort(&tfull_bar[s], (i >> 1) & 1, abort_flag)) break;
+            // a warp gives up as one: the TMEM loads are warp-wide
+            if (!__all_sync(0xffffffffu, wait_or_abort(&tfull_bar[s], (i >> 1) & 1, abort_flag, p.tries))) break;
             if (threadIdx.x == 0) s_drained = i + 1;
             tc_fence_after();
             int b, z0, y0, x0;
@@ -733,7 +740,7 @@ static cudaError_t launch_tc(cudaStream_t s, const CUtensorMap &map, const TcPar
 
 cudaError_t conv3d_tc(cudaStream_t s, int cin_mem, int cinp, int nout, int out_ch, const void *in, const void *Wb,
                       const float *bias, const void *res, void *out_b, float *out_f, int B, int D, int H, int W,
-                      int relu, int *fault, int num_sms)
+                      int relu, int *fault, int num_sms, int tries)
 {
     if (!(cin_mem == 8 || cin_mem == 32) || cin_mem > cinp) return cudaErrorInvalidValue;
     if (out_ch > nout || (nout == 16 && (out_ch != 8 || res || out_b))) return cudaErrorInvalidValue;
@@ -748,6 +755,7 @@ cudaError_t conv3d_tc(cudaStream_t s, int cin_mem, int cinp, int nout, int out_c
     p.nty = (H + TC_TY - 1) / TC_TY;
     p.ntz = (D + TC_TZ - 1) / TC_TZ;
     p.tiles = (long long)p.ntx * p.nty * p.ntz * B;
+    p.tries = tries;
     if (cinp == 32 && nout == 32)
         return launch_tc<32, 32>(s, map, p, cin_mem, out_ch, Wb, bias, res, out_b, out_f, relu, fault, num_sms);
     if (cinp == 16 && nout == 32)

@@ -33,10 +33,11 @@ cudaError_t conv3d(cudaStream_t s, int cin, int cout, const void *in, const void
 // nout x 27 cinp BF16 weights (K = tap cinp + c); nout GEMM columns (16 or
 // 32), of which out_ch are written (the row stride of out_b / out_f; with
 // nout = 16 only out_ch = 8 and FP32 output).  A device wait that runs out
-// sets *fault (and the output is then undefined).
+// (after `tries` polls; 0: the default, negative: one non-blocking test) sets
+// *fault (and the output is then undefined).
 cudaError_t conv3d_tc(cudaStream_t s, int cin_mem, int cinp, int nout, int out_ch, const void *in, const void *Wb,
                       const float *bias, const void *res, void *out_b, float *out_f, int B, int D, int H, int W,
-                      int relu, int *fault, int num_sms);
+                      int relu, int *fault, int num_sms, int tries = 0);
 bool conv3d_tc_available(const void *in, const void *Wb);
 // dst[n][tap cinp + c] = src[n][tap cin + c] (src rows of kp_src), zero for
 // n >= n_src or c >= cin.

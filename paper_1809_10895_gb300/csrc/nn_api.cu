@@ -195,7 +195,7 @@ rf_status ensure_training(rf_nn *n, long long M)
 }
 
 rf_status conv(rf_nn *n, cudaStream_t s, int l, bool transposed, const void *in, const void *res, void *out_b,
-               float *out_f, int B, int D, int H, int W, int relu, int *fault = nullptr)
+               float *out_f, int B, int D, int H, int W, int relu, int *fault = nullptr, int tries = 0)
 {
     const LayerDims &d = n->L[l];
     cudaError_t e;
@@ -205,28 +205,28 @@ rf_status conv(rf_nn *n, cudaStream_t s, int l, bool transposed, const void *in,
     // every layer shape of the network runs on the tcgen05 tensor cores
     if (d.cinp == 32 && d.coutp == 32 && nn::conv3d_tc_available(in, w)) {
         e = nn::conv3d_tc(s, 32, 32, 32, 32, in, w, transposed ? nullptr : n->P + d.b, transposed ? nullptr : res,
-                          out_b, out_f, B, D, H, W, transposed ? 0 : relu, f, n->num_sms);
+                          out_b, out_f, B, D, H, W, transposed ? 0 : relu, f, n->num_sms, tries);
         n->launches++;
         NN_CUDA(e);
         return RF_OK;
     }
     if (l == 0 && !transposed && nn::conv3d_tc_available(in, n->tcw0)) {
         e = nn::conv3d_tc(s, 8, 16, 32, 32, in, n->tcw0, n->P + d.b, res, out_b, out_f, B, D, H, W, relu, f,
-                          n->num_sms);
+                          n->num_sms, tries);
         n->launches++;
         NN_CUDA(e);
         return RF_OK;
     }
     if (last && !transposed && !out_b && !res && nn::conv3d_tc_available(in, n->tcw9)) {
         e = nn::conv3d_tc(s, 32, 32, 16, 8, in, n->tcw9, n->P + d.b, nullptr, nullptr, out_f, B, D, H, W, relu, f,
-                          n->num_sms);
+                          n->num_sms, tries);
         n->launches++;
         NN_CUDA(e);
         return RF_OK;
     }
     if (last && transposed && nn::conv3d_tc_available(in, n->tcw9t)) {
         e = nn::conv3d_tc(s, 8, 16, 32, 32, in, n->tcw9t, nullptr, nullptr, out_b, out_f, B, D, H, W, 0, f,
-                          n->num_sms);
+                          n->num_sms, tries);
         n->launches++;
         NN_CUDA(e);
         return RF_OK;
@@ -244,19 +244,19 @@ rf_status conv(rf_nn *n, cudaStream_t s, int l, bool transposed, const void *in,
 // Inference ping-pongs three M x 32 BF16 buffers; training keeps every
 // activation for the backward pass.
 rf_status forward(rf_nn *n, cudaStream_t s, const void *x, int B, int D, int H, int W, float *y, bool train,
-                  int *fault = nullptr)
+                  int *fault = nullptr, int tries = 0)
 {
     __nv_bfloat16 *A = train ? n->ta[0] : n->iA;
-    NN_TRY(conv(n, s, 0, false, x, nullptr, A, nullptr, B, D, H, W, 1));
+    NN_TRY(conv(n, s, 0, false, x, nullptr, A, nullptr, B, D, H, W, 1, fault, tries));
     for (int blk = 0; blk < 4; blk++) {
         __nv_bfloat16 *U = train ? n->tu[blk] : n->iU;
         __nv_bfloat16 *A2 = train ? n->ta[blk + 1] : n->iA2;
-        NN_TRY(conv(n, s, 1 + 2 * blk, false, A, nullptr, U, nullptr, B, D, H, W, 1, fault));
-        NN_TRY(conv(n, s, 2 + 2 * blk, false, U, A, A2, nullptr, B, D, H, W, 1, fault));
+        NN_TRY(conv(n, s, 1 + 2 * blk, false, A, nullptr, U, nullptr, B, D, H, W, 1, fault, tries));
+        NN_TRY(conv(n, s, 2 + 2 * blk, false, U, A, A2, nullptr, B, D, H, W, 1, fault, tries));
         if (train) A = A2;
         else std::swap(n->iA, n->iA2), A = n->iA;
     }
-    NN_TRY(conv(n, s, 9, false, A, nullptr, nullptr, y, B, D, H, W, 0));
+    NN_TRY(conv(n, s, 9, false, A, nullptr, nullptr, y, B, D, H, W, 0, fault, tries));
     return RF_OK;
 }
 
@@ -368,7 +368,7 @@ rf_status rf_nn_mesh_guess(rf_nn *n, cudaStream_t s, const Grid &g, const uint8_
     NN_TRY(begin(n, s));
     nn::ws_features_bf16(s, g, flags, h, Ks, sc, q_feat, dt_feat, n->ix);
     n->launches++;
-    NN_TRY(forward(n, s, n->ix, 1, g.nz, g.ny, g.nx, n->iy, false, fault));
+    NN_TRY(forward(n, s, n->ix, 1, g.nz, g.ny, g.nx, n->iy, false, fault, g.wait_tries));
     nn::ws_guess(s, g, flags, h, n->iy, scale, hk);
     n->launches++;
     return end(n, s);
