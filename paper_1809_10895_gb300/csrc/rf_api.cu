@@ -643,6 +643,7 @@ rf_status attempt_small(rf_ctx *c, double dt, Attempt &A, bool guess, int blocks
         RF_TRY(rf_nn_mesh_guess(c->ws_net, c->stream, c->g, c->flags, c->h, c->Ks, c->ws_sc, q_feat, dt_feat,
                                 c->ws_sc.out_scale * dt, c->hk, c->dev_fault));
         run_closure(c, c->hk, nullptr, c->theta_k, 0);
+        c->closure_at_h = false;
         c->ws_guesses++;
     }
     AttemptArgs a{};
@@ -699,8 +700,8 @@ rf_status attempt_small(rf_ctx *c, double dt, Attempt &A, bool guess, int blocks
     a.keep_theta_p = c->prm.time_scheme == RF_TIME_BDF2 ? 1 : 0;
     if (guess) RF_TRY(sync(c));     // the network's device waits report through dev_fault
     *c->fault_h = 0;
-    CUDA_TRY(launch_attempt_small(c->stream, a, c->prm.precision == RF_PREC_MIXED, blocks));
     c->closure_at_h = false;        // the attempt overwrites K[0] and C; an accepted step sets it again
+    CUDA_TRY(launch_attempt_small(c->stream, a, c->prm.precision == RF_PREC_MIXED, blocks));
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaStreamSynchronize(c->stream));
     if (*c->fault_h) {

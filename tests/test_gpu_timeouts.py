@@ -57,3 +57,18 @@ def test_network_guess():
         c.step()
     _times_out(s)
     _same_steps(s, ref, 3)
+
+
+def test_plain_step_after_a_guess_that_timed_out():
+    """The closures of the guess (here metres off, left in the network's
+    output by the step before) do not pass for the state's."""
+    case, net = _box(), _network()
+    sc = warmstart.scales_for(case, out_scale=5.0 / 60.0)
+    s, ref = rf.Solver.from_case(case), rf.Solver.from_case(case)
+    for c in (s, ref):
+        c.ws_attach(net, sc)
+        c.step()
+    _times_out(s)
+    for c in (s, ref):
+        c.ws_attach(None)
+    _same_steps(s, ref, 3)
