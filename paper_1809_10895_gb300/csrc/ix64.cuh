@@ -8,6 +8,9 @@
 // A number is (M, e): M 2^(e - 63) with M's top bit set, or M = 0.
 #pragma once
 
+#include <math.h>
+#include <string.h>
+
 #include "fx64.cuh"
 
 namespace rf {
@@ -73,14 +76,24 @@ RF_HD bool ix_sum7(const uint64_t (&b)[7], uint64_t &sum)
     return true;
 }
 
-#ifdef __CUDACC__
-// 1/M for M in [1, 2) (Q63), Q64 in (0.5, 1): the single-precision estimate
-// ri refined by ri (1 + e + e^2), e = 1 - M ri < 2^-21.
-__device__ __forceinline__ uint64_t ix_rcp(uint64_t M)
+// The 24-bit estimate r of 1/M as Q32 in [1/2, 1): rcp.approx, off by up to
+// 2^-23, may return 1 next to M = 1 and less than 1/2 next to M = 2.
+RF_HD uint32_t ix_rcp_seed(float r)
 {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(0x3f800000u | ((uint32_t)(M >> 40) & 0x7fffffu))));
-    const uint32_t ri = ((__float_as_uint(fminf(r, 0x1.fffffep-1f)) & 0x7fffffu) | 0x800000u) << 8;   // Q32
+    r = fminf(fmaxf(r, 0.5f), 0x1.fffffep-1f);
+    uint32_t b;
+#ifdef __CUDA_ARCH__
+    b = __float_as_uint(r);
+#else
+    memcpy(&b, &r, 4);
+#endif
+    return ((b & 0x7fffffu) | 0x800000u) << 8;
+}
+
+// 1/M for M in [1, 2) (Q63), Q64 in (0.5, 1): the seed ri refined by
+// ri (1 + e + e^2), |e| = |1 - M ri| < 2^-21.
+RF_HD uint64_t ix_rcp_refine(uint64_t M, uint32_t ri)
+{
     const int64_t e = (int64_t)(0x8000000000000000ULL - fx_mul32(M, ri));                             // Q63
     const int32_t es = (int32_t)(e >> 11);                                                            // Q52
     const int64_t s = e + (((int64_t)es * es) >> 41);                                                 // e + e^2
@@ -88,15 +101,39 @@ __device__ __forceinline__ uint64_t ix_rcp(uint64_t M)
     return ((uint64_t)ri << 32) + (uint64_t)(t << 1);
 }
 
+// The float nearest to the double with bits b (ties to even); false where it
+// is zero, subnormal, infinite or NaN as a float.
+RF_HD bool ix_d2f_bits(uint64_t b, uint32_t &f)
+{
+    if (((uint32_t)(b >> 52) & 0x7ffu) - 897u > 253u) return false;
+    const uint64_t v = (b & 0x7fffffffffffffffULL) - (896ULL << 52);
+    f = (uint32_t)((v + 0x0fffffffULL + ((v >> 29) & 1)) >> 29) | ((uint32_t)(b >> 32) & 0x80000000u);
+    return true;
+}
+
+// The float with bits b as a double; false for subnormal, infinite or NaN.
+RF_HD bool ix_f2d_bits(uint32_t b, uint64_t &d)
+{
+    const uint32_t m = b & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u && m) return false;
+    d = (m ? ((uint64_t)m << 29) + (896ULL << 52) : 0) | (uint64_t)(b & 0x80000000u) << 32;
+    return true;
+}
+
+#ifdef __CUDACC__
+// 1/M for M in [1, 2) (Q63), Q64 in (0.5, 1).
+__device__ __forceinline__ uint64_t ix_rcp(uint64_t M)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(0x3f800000u | ((uint32_t)(M >> 40) & 0x7fffffu))));
+    return ix_rcp_refine(M, ix_rcp_seed(r));
+}
+
 // The float nearest to a double (ties to even).
 __device__ __forceinline__ float ix_d2f(double a)
 {
-    const uint64_t b = (uint64_t)__double_as_longlong(a);
-    const uint32_t ex = (uint32_t)(b >> 52) & 0x7ffu;
-    if (ex - 897u > 253u) return (float)a;        // zero, subnormal, infinite or NaN as a float
-    const uint64_t v = (b & 0x7fffffffffffffffULL) - (896ULL << 52);
-    return __uint_as_float((uint32_t)((v + 0x0fffffffULL + ((v >> 29) & 1)) >> 29) |
-                           ((uint32_t)(b >> 32) & 0x80000000u));
+    uint32_t f;
+    return ix_d2f_bits((uint64_t)__double_as_longlong(a), f) ? __uint_as_float(f) : (float)a;
 }
 
 // Tests on the bits: a compare of doubles goes to the FP64 pipe.
@@ -116,10 +153,8 @@ __device__ __forceinline__ bool not_above(double a, double b)    // a <= b, both
 // A float as a double.
 __device__ __forceinline__ double ix_f2d(float a)
 {
-    const uint32_t b = __float_as_uint(a), m = b & 0x7fffffffu;
-    if (m - 0x00800000u >= 0x7f000000u && m) return (double)a;   // subnormal, infinite or NaN
-    const uint64_t v = m ? ((uint64_t)m << 29) + (896ULL << 52) : 0;
-    return __longlong_as_double((long long)(v | (uint64_t)(b & 0x80000000u) << 32));
+    uint64_t d;
+    return ix_f2d_bits(__float_as_uint(a), d) ? __longlong_as_double((long long)d) : (double)a;
 }
 
 // 1/a.

@@ -1,0 +1,61 @@
+// Host build of the integer forms of FP64 arithmetic (csrc/ix64.cuh) for the
+// CPU test: the same source that the kernels include; the estimate of a
+// reciprocal, an instruction there, is a rounded quotient `ulps` units off.
+#include <cmath>
+#include <cstring>
+
+#include "ix64.cuh"
+
+using namespace rf;
+
+static uint64_t bits(double a)
+{
+    uint64_t b;
+    std::memcpy(&b, &a, 8);
+    return b;
+}
+static double value(uint64_t b)
+{
+    double a;
+    std::memcpy(&a, &b, 8);
+    return a;
+}
+
+static uint64_t rcp(uint64_t M, int ulps)
+{
+    const uint32_t xb = 0x3f800000u | ((uint32_t)(M >> 40) & 0x7fffffu);
+    float x;
+    std::memcpy(&x, &xb, 4);
+    const float r = 1.0f / x, unit = 0x1p-24f;      // of a result in [1/2, 1)
+    return ix_rcp_refine(M, ix_rcp_seed(r + (float)ulps * unit));
+}
+
+extern "C" double ix_h_rcp(double a, int ulps)
+{
+    const IxNum d = ix_unpack(bits(a));
+    return value(fx_pack(rcp(d.M, ulps), -1 - d.e));
+}
+
+extern "C" double ix_h_add_mul(double a, double b, double c)
+{
+    return value(ix_pack(ix_add_mul(ix_unpack(bits(a)), ix_unpack(bits(b)), ix_unpack(bits(c)))));
+}
+
+extern "C" double ix_h_add(double a, double b) { return value(ix_pack(ix_add(ix_unpack(bits(a)), ix_unpack(bits(b))))); }
+
+// NaN where the integer form leaves the conversion to the instruction.
+extern "C" float ix_h_d2f(double a)
+{
+    uint32_t f;
+    float v = NAN;
+    if (ix_d2f_bits(bits(a), f)) std::memcpy(&v, &f, 4);
+    return v;
+}
+
+extern "C" double ix_h_f2d(float a)
+{
+    uint32_t b;
+    uint64_t d;
+    std::memcpy(&b, &a, 4);
+    return ix_f2d_bits(b, d) ? value(d) : NAN;
+}
