@@ -311,17 +311,7 @@ __device__ __forceinline__ double face_coef(const Grid &g, long long a, long lon
 // c = V_dt (theta^k - theta^n) / (h^k - h^n), dth and dh the differences.
 __device__ __forceinline__ double chord_c(double dth, double dh, double V_dt)
 {
-    const long long db = __double_as_longlong(dh) & 0x7fffffffffffffffLL, vb = __double_as_longlong(V_dt);
-    double f;
-    if ((unsigned)(vb >> 52) - 700u < 650u && (unsigned)(db >> 52) - 700u < 650u) {
-        const IxNum d = ix_unpack((uint64_t)db), V = ix_unpack((uint64_t)vb);
-        uint64_t q = fx_mulhi(ix_rcp(d.M), V.M);
-        const int up = (int)(q >> 63);
-        q = up ? q : q << 1;
-        f = __longlong_as_double((long long)fx_pack(q, V.e - d.e - 1 + up));
-    } else {
-        f = V_dt / __longlong_as_double(db);
-    }
+    const double f = ix_div(V_dt, __longlong_as_double(__double_as_longlong(dh) & 0x7fffffffffffffffLL));
     return __longlong_as_double(__double_as_longlong(dth) ^
                                 (__double_as_longlong(dh) & (long long)0x8000000000000000ULL)) * f;
 }

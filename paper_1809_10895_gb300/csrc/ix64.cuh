@@ -101,6 +101,22 @@ RF_HD uint64_t ix_rcp_refine(uint64_t M, uint32_t ri)
     return ((uint64_t)ri << 32) + (uint64_t)(t << 1);
 }
 
+// a r 2^(-eb), r = 1/M of a number M 2^eb (ix_rcp).
+RF_HD uint64_t ix_quot(IxNum a, uint64_t r, int eb)
+{
+    uint64_t q = fx_mulhi(a.M, r);                                 // [2^62, 2^64)
+    const int up = (int)(q >> 63);
+    q = up ? q : q << 1;
+    return fx_pack(q, a.e - eb - 1 + up);
+}
+
+// Exponents for which quotients stay normal (a negative number's sign bit
+// fails the test).
+RF_HD bool ix_quot_ok(uint64_t a, uint64_t b)
+{
+    return (uint32_t)(a >> 52) - 700u < 650u && (uint32_t)(b >> 52) - 700u < 650u;
+}
+
 // The float nearest to the double with bits b (ties to even); false where it
 // is zero, subnormal, infinite or NaN as a float.
 RF_HD bool ix_d2f_bits(uint64_t b, uint32_t &f)
@@ -168,10 +184,13 @@ __device__ __forceinline__ double ix_rcp64(double a)
     return 1.0 / a;
 }
 
-// a/b, to two roundings.
+// a/b.
 __device__ __forceinline__ double ix_div(double a, double b)
 {
-    return (unsigned)((uint64_t)__double_as_longlong(b) >> 52) - 400u < 1200u ? a * ix_rcp64(b) : a / b;
+    const uint64_t ab = (uint64_t)__double_as_longlong(a), bb = (uint64_t)__double_as_longlong(b);
+    if (!ix_quot_ok(ab, bb)) return a / b;
+    const IxNum d = ix_unpack(bb);
+    return __longlong_as_double((long long)ix_quot(ix_unpack(ab), ix_rcp(d.M), d.e));
 }
 #endif
 

@@ -36,6 +36,14 @@ extern "C" double ix_h_rcp(double a, int ulps)
     return value(fx_pack(rcp(d.M, ulps), -1 - d.e));
 }
 
+// NaN where the integer form leaves the division to the instruction.
+extern "C" double ix_h_div(double a, double b, int ulps)
+{
+    if (!ix_quot_ok(bits(a), bits(b))) return NAN;
+    const IxNum d = ix_unpack(bits(b));
+    return value(ix_quot(ix_unpack(bits(a)), rcp(d.M, ulps), d.e));
+}
+
 extern "C" double ix_h_add_mul(double a, double b, double c)
 {
     return value(ix_pack(ix_add_mul(ix_unpack(bits(a)), ix_unpack(bits(b)), ix_unpack(bits(c)))));

@@ -24,7 +24,8 @@ def lib(tmp_path_factory):
     subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I", CSRC,
                     os.path.join(HERE, "c", "ix64_host.cpp"), "-o", so], check=True)
     L = C.CDLL(so)
-    for name, res, args in (("rcp", D, [D, C.c_int]), ("add_mul", D, [D, D, D]), ("add", D, [D, D]), ("d2f", F, [D]),
+    for name, res, args in (("rcp", D, [D, C.c_int]), ("div", D, [D, D, C.c_int]),
+                            ("add_mul", D, [D, D, D]), ("add", D, [D, D]), ("d2f", F, [D]),
                             ("f2d", D, [F])):
         f = getattr(L, "ix_h_" + name)
         f.restype, f.argtypes = res, args
@@ -59,6 +60,18 @@ def test_reciprocal(lib, ulps):
     for m in significands(rng, 3000):
         a = float(np.ldexp(m, int(rng.integers(-600, 600))))
         assert ulps_off(lib.ix_h_rcp(a, ulps), 1 / Fraction(a)) <= TOL, (m, ulps)
+
+
+@pytest.mark.parametrize("ulps", [-2, 0, 2])
+def test_quotient(lib, ulps):
+    rng = np.random.default_rng(4)
+    sig = significands(rng, 3000)
+    for m in sig:
+        a = float(np.ldexp(m, int(rng.integers(-320, 320))))
+        b = float(np.ldexp(rng.choice(sig), int(rng.integers(-320, 320))))
+        assert ulps_off(lib.ix_h_div(a, b, ulps), Fraction(a) / Fraction(b)) <= TOL, (a, b)
+    for a, b in ((-1.0, 1.0), (1.0, -1.0), (0.0, 1.0), (1.0, 0.0), (np.inf, 1.0), (1.0, np.nan), (2.0 ** -400, 1.0)):
+        assert np.isnan(lib.ix_h_div(a, b, ulps))
 
 
 @pytest.mark.parametrize("spread", [0, 1, 3, 52, 61, 62, 63, 64, 200])
