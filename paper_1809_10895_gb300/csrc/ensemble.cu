@@ -702,14 +702,10 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
         }
         bool closure_valid = true;
         // of the reduced (r.r, b.b, r.z): whether the residual meets the
-        // tolerance, by squares, and the inner solve's FP32 threshold.  One
-        // thread derives them: an FP64 root is some fifteen dependent
-        // instructions of 64 cycles.
+        // tolerance, by squares, and the inner solve's threshold.  One thread
+        // derives them.
         auto converged = [&](double rr, double bb, double tol) { return not_above(rr, tol * tol * bb) ? 1.0 : 0.0; };
-        auto inner_stop = [&](double rr) {
-            const bool f32 = ((uint64_t)__double_as_longlong(rr) >> 52) - 924u < 198u;   // 2^-99 to 2^99
-            return P.tol_inner * (f32 ? ix_f2d(sqrtf(ix_d2f(rr))) : sqrt(rr));
-        };
+        auto inner_stop = [&](double rr) { return P.tol_inner * ix_sqrt(rr); };
 
         while (status == ENS_RUNNING && t < t_end - t_tol_d(t_end)) {
             if (--budget < 0) { status = ENS_BUDGET; break; }
@@ -744,14 +740,14 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                         CellSystem cs;
                         assemble_cell<true>(g, soil, zn, Ks, fl[p], sp, p, i, j, k, hk, hn, TH[tn ^ 1], TH[tn],
                                             KB[kin], Can, nullptr, P.eps_chord, V_dt, cs);
-                        const double di = PREC == 0 ? ix_rcp64(cs.diag) : 0.0;   // the mixed path's scaling is FP32
+                        const double di = ix_rcp64(cs.diag);
                         cc[p] = cs.c;
                         bb[p] = cs.rhs;
                         Tx[p] = cs.Tup[0];
                         Ty[p] = cs.Tup[1];
                         Tz[p] = cs.Tup[2];
                         dg[p] = cs.diag;
-                        const float d32v = PREC == 0 ? 0.0f : __frcp_rn(ix_d2f(cs.diag));
+                        const float d32v = PREC == 0 ? 0.0f : ix_d2f(di);
                         if (PREC == 0) {
                             dinv[p] = di;
                         } else {

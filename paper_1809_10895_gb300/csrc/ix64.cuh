@@ -136,6 +136,14 @@ RF_HD bool ix_f2d_bits(uint32_t b, uint64_t &d)
     return true;
 }
 
+// Square root of a in [2^-99, 2^99], relative error below 2^-44: the float
+// root s plus (a - s^2) / (2 s), of which only the difference and the sum need
+// FP64 (an FP64 root is some fifteen dependent instructions of 64 cycles).
+RF_HD double ix_root_step(double a, double s, float sf)
+{
+    return s + (double)((float)fma(-s, s, a) * (0.5f / sf));
+}
+
 #ifdef __CUDACC__
 // 1/M for M in [1, 2) (Q63), Q64 in (0.5, 1).
 __device__ __forceinline__ uint64_t ix_rcp(uint64_t M)
@@ -182,6 +190,14 @@ __device__ __forceinline__ double ix_rcp64(double a)
         return __longlong_as_double((long long)fx_pack(ix_rcp(d.M), -1 - d.e));
     }
     return 1.0 / a;
+}
+
+// Square root, relative error below 2^-44.
+__device__ __forceinline__ double ix_sqrt(double a)
+{
+    if ((uint32_t)((uint64_t)__double_as_longlong(a) >> 52) - 924u >= 198u) return sqrt(a);
+    const float sf = sqrtf(ix_d2f(a));
+    return ix_root_step(a, ix_f2d(sf), sf);
 }
 
 // a/b.

@@ -51,6 +51,22 @@ extern "C" double ix_h_add_mul(double a, double b, double c)
 
 extern "C" double ix_h_add(double a, double b) { return value(ix_pack(ix_add(ix_unpack(bits(a)), ix_unpack(bits(b))))); }
 
+extern "C" double ix_h_sqrt(double a)
+{
+    const float s = sqrtf((float)a);
+    return ix_root_step(a, (double)s, s);
+}
+
+// The FP32 reciprocal as the ensemble's Jacobi scaling forms it.
+extern "C" float ix_h_rcp32(double a, int ulps)
+{
+    const double r = ix_h_rcp(a, ulps);
+    uint32_t f;
+    float v = NAN;
+    if (ix_d2f_bits(bits(r), f)) std::memcpy(&v, &f, 4);
+    return v;
+}
+
 // NaN where the integer form leaves the conversion to the instruction.
 extern "C" float ix_h_d2f(double a)
 {

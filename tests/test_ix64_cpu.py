@@ -25,7 +25,7 @@ def lib(tmp_path_factory):
                     os.path.join(HERE, "c", "ix64_host.cpp"), "-o", so], check=True)
     L = C.CDLL(so)
     for name, res, args in (("rcp", D, [D, C.c_int]), ("div", D, [D, D, C.c_int]),
-                            ("add_mul", D, [D, D, D]), ("add", D, [D, D]), ("d2f", F, [D]),
+                            ("sqrt", D, [D]), ("rcp32", F, [D, C.c_int]), ("add_mul", D, [D, D, D]), ("add", D, [D, D]), ("d2f", F, [D]),
                             ("f2d", D, [F])):
         f = getattr(L, "ix_h_" + name)
         f.restype, f.argtypes = res, args
@@ -72,6 +72,24 @@ def test_quotient(lib, ulps):
         assert ulps_off(lib.ix_h_div(a, b, ulps), Fraction(a) / Fraction(b)) <= TOL, (a, b)
     for a, b in ((-1.0, 1.0), (1.0, -1.0), (0.0, 1.0), (1.0, 0.0), (np.inf, 1.0), (1.0, np.nan), (2.0 ** -400, 1.0)):
         assert np.isnan(lib.ix_h_div(a, b, ulps))
+
+
+# s is within 2^-24 of the root, so the step leaves 2^-48 / 2, the float
+# arithmetic of the correction 2^-24 (2^-24 + 2^-23): below 2^-45 together.
+def test_square_root(lib):
+    rng = np.random.default_rng(8)
+    for m in significands(rng, 3000):
+        a = float(np.ldexp(m, int(rng.integers(-99, 99))))
+        assert abs(Fraction(lib.ix_h_sqrt(a)) ** 2 / Fraction(a) - 1) <= 2 * Fraction(1, 2 ** 44), a
+
+
+# An FP64 reciprocal (0.51 units of its last place) rounded once to FP32.
+@pytest.mark.parametrize("ulps", [-2, 0, 2])
+def test_fp32_reciprocal(lib, ulps):
+    rng = np.random.default_rng(9)
+    for m in significands(rng, 3000):
+        a = float(np.ldexp(m, int(rng.integers(-100, 100))))
+        assert ulps_off(lib.ix_h_rcp32(a, ulps), 1 / Fraction(a)) <= Fraction(2 ** 29) * (Fraction(1, 2) + Fraction(1, 2 ** 20)), a
 
 
 @pytest.mark.parametrize("spread", [0, 1, 3, 52, 61, 62, 63, 64, 200])
