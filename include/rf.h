@@ -341,6 +341,13 @@ rf_status rf_apply_inner(rf_ctx *ctx, const float *d_z, const float *d_pold, flo
  * RF_ERR_DEVICE_TIMEOUT with the state unchanged and the context usable. */
 rf_status rf_set_wait_limit(rf_ctx *ctx, int polls);
 
+/* Test and diagnostic hook: whether Jacobi contexts run small grids' Picard
+ * attempts (attempts != 0) and linear solves (solves != 0) as one cooperative
+ * launch, the default.  With 0 they run as the launches of a CUDA graph, which
+ * is also what a context falls back to where the stream's SMs cannot hold a
+ * cooperative launch's blocks at once.  Results agree to rounding. */
+rf_status rf_set_one_launch(rf_ctx *ctx, int attempts, int solves);
+
 /* Number of CUDA kernel launches this context has executed on the device,
  * counted by the kernels themselves (loop bodies replayed from CUDA graphs
  * included).  Synchronises the context's stream. */

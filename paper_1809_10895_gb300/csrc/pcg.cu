@@ -114,14 +114,20 @@ k_cg64_spmv(Grid g, Tiles tw, const double *__restrict__ z, const double *__rest
 __global__ void __launch_bounds__(RED_THREADS)
 k_cg64_update(Grid g, double *__restrict__ x, double *__restrict__ r, double *__restrict__ z,
               const double *__restrict__ pd, const double *__restrict__ q, const double *__restrict__ dinv,
-              double *partials, unsigned int *ticket, CgScal *sc)
+              double *partials, unsigned int *ticket, CgScal *sc, CondSet cond)
 {
     count_launch(g, KK_CG64_UPDATE);
-    if (sc->done) return;
+    if (sc->done) {             // every launch sets the loop condition
+        if (blockIdx.x == 0 && threadIdx.x == 0) set_cond(cond, 0);
+        return;
+    }
     count_work(g, KK_CG64_UPDATE);
     double v[2] = {0.0, 0.0};   // r.r, r.z
     cg64_update_cells(g, sc->alpha, dinv, pd, q, x, r, z, v);
-    if (grid_reduce<OpSum, 2>(v, partials, ticket) && threadIdx.x == 0) cg_update_scalars(sc, v);
+    if (grid_reduce<OpSum, 2>(v, partials, ticket) && threadIdx.x == 0) {
+        cg_update_scalars(sc, v);
+        set_cond(cond, sc->done ? 0 : 1);
+    }
 }
 
 __global__ void __launch_bounds__(RED_THREADS)
@@ -427,15 +433,21 @@ k_cg32_spmv_tma(Grid g, Tiles tw, const __grid_constant__ TmaMaps32 maps, int pi
 __global__ void __launch_bounds__(RED_THREADS)
 k_cg32_update(Grid g, float *__restrict__ x, float *__restrict__ r, float *__restrict__ z,
               const float *__restrict__ pd, const float *__restrict__ q, const float *__restrict__ dinv,
-              double *partials, unsigned int *ticket, CgScal *sc)
+              double *partials, unsigned int *ticket, CgScal *sc, CondSet cond)
 {
     count_launch(g, KK_CG32_UPDATE);
-    if (sc->done) return;
+    if (sc->done) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) set_cond(cond, 0);
+        return;
+    }
     count_work(g, KK_CG32_UPDATE);
     float vf[2] = {0.0f, 0.0f};
     cg32_update_cells(g, (float)sc->alpha, false, dinv, pd, q, x, r, z, vf);
     double v[2];
-    if (grid_reduce_f32<2>(vf, v, partials, ticket) && threadIdx.x == 0) cg_update_scalars(sc, v);
+    if (grid_reduce_f32<2>(vf, v, partials, ticket) && threadIdx.x == 0) {
+        cg_update_scalars(sc, v);
+        set_cond(cond, sc->done ? 0 : 1);
+    }
 }
 
 // x += d after an inner solve; a non-finite inner solve fails the outer loop
@@ -486,9 +498,10 @@ void launch_cg64_spmv(cudaStream_t s, int nblk, const Grid &g, const double *z, 
 }
 
 void launch_cg64_update(cudaStream_t s, int nblk, const Grid &g, double *x, double *r, double *z, const double *p,
-                        const double *q, const double *dinv, double *partials, unsigned int *ticket, CgScal *sc)
+                        const double *q, const double *dinv, double *partials, unsigned int *ticket, CgScal *sc,
+                        CondSet cond)
 {
-    k_cg64_update<<<nblk, RED_THREADS, 0, s>>>(g, x, r, z, p, q, dinv, partials, ticket, sc);
+    k_cg64_update<<<nblk, RED_THREADS, 0, s>>>(g, x, r, z, p, q, dinv, partials, ticket, sc, cond);
 }
 
 void launch_apply64(cudaStream_t s, int nblk, const Grid &g, const uint8_t *flags, const double *x, double *y,
@@ -541,9 +554,10 @@ void launch_cg32_spmv(cudaStream_t s, int nblk, const Grid &g, const float *z, c
 }
 
 void launch_cg32_update(cudaStream_t s, int nblk, const Grid &g, float *x, float *r, float *z, const float *p,
-                        const float *q, const float *dinv, double *partials, unsigned int *ticket, CgScal *sc)
+                        const float *q, const float *dinv, double *partials, unsigned int *ticket, CgScal *sc,
+                        CondSet cond)
 {
-    k_cg32_update<<<nblk, RED_THREADS, 0, s>>>(g, x, r, z, p, q, dinv, partials, ticket, sc);
+    k_cg32_update<<<nblk, RED_THREADS, 0, s>>>(g, x, r, z, p, q, dinv, partials, ticket, sc, cond);
 }
 
 void launch_add_correction(cudaStream_t s, int nblk, const Grid &g, double *x, const float *d, CgScal *outer,

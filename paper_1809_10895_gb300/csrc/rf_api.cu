@@ -79,8 +79,9 @@ struct rf_ctx {
     double *partials = nullptr;
     unsigned int *ticket = nullptr;
     void *gridred = nullptr;             // barrier and partials of the cooperative kernels
-    int cg64_blocks = 0, mixed_blocks = 0;   // of the one-launch solves
-    int small_blocks[2] = {-1, -1};      // blocks of the small-grid attempt (FP64, mixed; -1: not asked yet)
+    int cg64_blocks = 0, mixed_blocks = 0;   // of the one-launch solves (0: cooperative launches not possible)
+    int small_blocks[2] = {-1, -1};      // blocks of the small-grid attempt (FP64, mixed; -1: not asked yet; 0: not possible)
+    bool small_on = true, solve_on = true;   // small-grid attempts and one-launch solves wanted (rf_set_one_launch)
     CgScal *sc = nullptr, *sc_in = nullptr;
     StepResults *res = nullptr;
     StepParams *sp = nullptr;
@@ -225,6 +226,14 @@ rf_status sync(rf_ctx *c)
         return fail(RF_ERR_DEVICE_TIMEOUT, "a device wait for staged data ran out (the solve was stopped)");
     }
     return RF_OK;
+}
+
+// Jacobi solves run as one cooperative launch, unless the device or the stream
+// cannot hold its blocks at once: then as loops of a graph.
+bool one_launch_solve(const rf_ctx *c)
+{
+    return c->prm.precond == RF_PRECOND_JACOBI && c->solve_on &&
+           (c->prm.precision == RF_PREC_FP64 ? c->cg64_blocks : c->mixed_blocks) > 0;
 }
 
 // storage part of b, written and read only with modified Picard
@@ -394,30 +403,33 @@ rf_status capture_solve(rf_ctx *c, cudaGraph_t top, cudaGraph_t parent, std::vec
                              c->prm.tol_cg, c->prm.cg_max_it, c->partials, c->ticket, c->sc, skip, cc);
             RF_TRY(cap_end(c, deps));
         }
-        RF_TRY(cap_begin(c, parent, deps));
-        CUDA_TRY(launch_cg64_solve(s, c->cg64_blocks, g, c->Tx, c->Ty, c->Tz, c->diag, c->dinv, x, c->r, c->z, c->p[0],
-                                   c->p[1], c->q, c->gridred, c->dev_fault, c->sc));
-        RF_TRY(cap_end(c, out));
+        if (one_launch_solve(c)) {
+            RF_TRY(cap_begin(c, parent, deps));
+            const cudaError_t e =
+                launch_cg64_solve(s, c->cg64_blocks, g, c->Tx, c->Ty, c->Tz, c->diag, c->dinv, x, c->r, c->z, c->p[0],
+                                  c->p[1], c->q, c->gridred, c->dev_fault, c->sc);
+            RF_TRY(cap_end(c, out));
+            CUDA_TRY(e);
+            return RF_OK;
+        }
+        cudaGraphNode_t wn;
+        cudaGraph_t body;
+        RF_TRY(add_while(parent, deps, cc.h, &wn, &body));
+        RF_TRY(cap_begin(c, body, {}));
+        for (int half = 0; half < 2; half++) {
+            double *pin = c->p[half], *pout = c->p[half ^ 1];
+            launch_cg64_spmv(s, nb, g, c->z, pin, pout, c->q, c->Tx, c->Ty, c->Tz, c->diag, c->partials, c->ticket,
+                             c->sc);
+            launch_cg64_update(s, nb, g, x, c->r, c->z, pout, c->q, c->dinv, c->partials, c->ticket, c->sc, cc);
+        }
+        std::vector<cudaGraphNode_t> tmp;
+        RF_TRY(cap_end(c, tmp));
+        out = {wn};
         return RF_OK;
     }
     // mixed: WHILE(outer) { WHILE(inner FP32 PCG) ; x += d ; FP64 residual }
     const CondSet co = start->cond, ci = start->cond_inner;
     const bool mg = c->prm.precond == RF_PRECOND_MG, dic = c->prm.precond == RF_PRECOND_DIC;
-    if (!mg && !dic) {
-        RF_TRY(cap_begin(c, parent, deps));
-        if (!fused) {
-            launch_mixed_start(s, nb, g, x0, x, c->sc, c->sc_in, skip, co);
-            launch_resid64(s, nb, g, c->flags, x, c->b, c->Tx, c->Ty, c->Tz, c->diag, c->dinv32, c->r32, c->z32, c->d32,
-                           c->prm.tol_cg, c->prm.tol_inner, c->prm.inner_max_it, c->prm.outer_max_it, c->partials,
-                           c->ticket, c->sc, c->sc_in, co, ci);
-        }
-        CUDA_TRY(launch_mixed_solve(s, c->mixed_blocks, g, c->flags, c->Tx, c->Ty, c->Tz, c->diag, c->b, c->K32, c->cb32,
-                                    c->dinv32, x, c->r32, c->z32, c->d32, c->p32[0], c->p32[1], c->q32, c->gridred,
-                                    c->dev_fault, c->sc, c->sc_in, c->prm.tol_cg, c->prm.tol_inner,
-                                    c->prm.inner_max_it, c->prm.outer_max_it));
-        RF_TRY(cap_end(c, out));
-        return RF_OK;
-    }
     const int *idone = &c->sc_in->done;
     // z = M r for the MG preconditioner
     auto precondition = [&]() { launch_mg_vcycle(s, nb, c->mg, c->K32, c->r32, c->z32, idone); };
@@ -428,6 +440,17 @@ rf_status capture_solve(rf_ctx *c, cudaGraph_t top, cudaGraph_t parent, std::vec
                        c->prm.tol_cg, c->prm.tol_inner, c->prm.inner_max_it, c->prm.outer_max_it, c->partials,
                        c->ticket, c->sc, c->sc_in, co, ci);
         RF_TRY(cap_end(c, deps));
+    }
+    if (one_launch_solve(c)) {
+        RF_TRY(cap_begin(c, parent, deps));
+        const cudaError_t e =
+            launch_mixed_solve(s, c->mixed_blocks, g, c->flags, c->Tx, c->Ty, c->Tz, c->diag, c->b, c->K32, c->cb32,
+                               c->dinv32, x, c->r32, c->z32, c->d32, c->p32[0], c->p32[1], c->q32, c->gridred,
+                               c->dev_fault, c->sc, c->sc_in, c->prm.tol_cg, c->prm.tol_inner, c->prm.inner_max_it,
+                               c->prm.outer_max_it);
+        RF_TRY(cap_end(c, out));
+        CUDA_TRY(e);
+        return RF_OK;
     }
     // z = M r and rho = r.z (start) or beta (inner iterations); DIC folds
     // r.z into its two sweeps, and within the loop its red pass into the update
@@ -441,12 +464,14 @@ rf_status capture_solve(rf_ctx *c, cudaGraph_t top, cudaGraph_t parent, std::vec
         }
     };
     // coarse operators (MG) or pivots (DIC) from this assembly, then z0 = M r0
-    // and rho = r0.z0
-    RF_TRY(cap_begin(c, parent, deps));
-    if (mg) launch_mg_build(s, nb, c->mg, c->K32, skip);
-    else launch_dic_setup(s, nb, g, c->K32, c->cb32, c->dic_diag, c->dic_rd, skip);
-    precondition_rz(1, false);
-    RF_TRY(cap_end(c, deps));
+    // and rho = r0.z0 (Jacobi: z and rho come with the residual)
+    if (mg || dic) {
+        RF_TRY(cap_begin(c, parent, deps));
+        if (mg) launch_mg_build(s, nb, c->mg, c->K32, skip);
+        else launch_dic_setup(s, nb, g, c->K32, c->cb32, c->dic_diag, c->dic_rd, skip);
+        precondition_rz(1, false);
+        RF_TRY(cap_end(c, deps));
+    }
     cudaGraphNode_t wo, wi;
     cudaGraph_t bo, bi;
     RF_TRY(add_while(parent, deps, co.h, &wo, &bo));
@@ -460,9 +485,12 @@ rf_status capture_solve(rf_ctx *c, cudaGraph_t top, cudaGraph_t parent, std::vec
             launch_cg32_update_dic(s, nb, g, c->d32, c->r32, c->z32, pout, c->q32, c->dinv32, c->dic_rd, c->partials,
                                    c->ticket, c->sc_in);
             precondition_rz(0, true);
-        } else {
+        } else if (mg) {
             launch_cg32_update_mg(s, nb, g, c->d32, c->r32, pout, c->q32, c->dinv32, c->partials, c->ticket, c->sc_in);
             precondition_rz(0, false);
+        } else {
+            launch_cg32_update(s, nb, g, c->d32, c->r32, c->z32, pout, c->q32, c->dinv32, c->partials, c->ticket,
+                               c->sc_in, ci);
         }
     }
     std::vector<cudaGraphNode_t> tmp;
@@ -472,7 +500,7 @@ rf_status capture_solve(rf_ctx *c, cudaGraph_t top, cudaGraph_t parent, std::vec
     launch_resid64(s, nb, g, c->flags, x, c->b, c->Tx, c->Ty, c->Tz, c->diag, c->dinv32, c->r32, c->z32, c->d32,
                    c->prm.tol_cg, c->prm.tol_inner, c->prm.inner_max_it, c->prm.outer_max_it, c->partials, c->ticket,
                    c->sc, c->sc_in, co, ci);
-    precondition_rz(1, false);
+    if (mg || dic) precondition_rz(1, false);
     RF_TRY(cap_end(c, tmp));
     out = {wo};
     return RF_OK;
@@ -483,11 +511,13 @@ rf_status make_start(rf_ctx *c, cudaGraph_t G, double *x, SolveStart &st)
 {
     st = SolveStart{};
     cudaGraphConditionalHandle h1, h2;
-    if (c->prm.precond != RF_PRECOND_JACOBI) {       // Jacobi solves are one launch, without loop nodes
+    if (!one_launch_solve(c)) {                      // a one-launch solve has no loop nodes
         CUDA_TRY(cudaGraphConditionalHandleCreate(&h1, G, 0, 0));
         st.cond = CondSet{h1, 1};
-        CUDA_TRY(cudaGraphConditionalHandleCreate(&h2, G, 0, 0));
-        st.cond_inner = CondSet{h2, 1};
+        if (c->prm.precision == RF_PREC_MIXED) {
+            CUDA_TRY(cudaGraphConditionalHandleCreate(&h2, G, 0, 0));
+            st.cond_inner = CondSet{h2, 1};
+        }
     }
     st.x = x;
     st.r = c->r;
@@ -587,11 +617,28 @@ rf_status build_solve_graph(rf_ctx *c)
     return RF_OK;
 }
 
+// Build a graph unless it is there, and launch it.  Where that fails with
+// one-launch solves in it (more blocks than the SMs of the stream hold at once:
+// a stream or a process limited to some of them), the solves become loops.
+rf_status launch_graph(rf_ctx *c, cudaGraphExec_t rf_ctx::*exec, rf_status (*build)(rf_ctx *))
+{
+    auto run = [&]() -> rf_status {
+        if (!(c->*exec)) RF_TRY(build(c));
+        CUDA_TRY(cudaGraphLaunch(c->*exec, c->stream));
+        return RF_OK;
+    };
+    const rf_status st = run();
+    if (st != RF_ERR_CUDA || !one_launch_solve(c)) return st;
+    cudaGetLastError();
+    destroy_graphs(c);
+    c->cg64_blocks = c->mixed_blocks = 0;
+    return run();
+}
+
 // Solve the assembled system from hk into x (kernel-level entry point).
 rf_status solve_system(rf_ctx *c, int *iters)
 {
-    if (!c->solve_exec) RF_TRY(build_solve_graph(c));
-    CUDA_TRY(cudaGraphLaunch(c->solve_exec, c->stream));
+    RF_TRY(launch_graph(c, &rf_ctx::solve_exec, build_solve_graph));
     CUDA_TRY(cudaMemcpyAsync(c->sc_h, c->sc, sizeof(CgScal), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(cudaMemcpyAsync(c->sc_in_h, c->sc_in, sizeof(CgScal), cudaMemcpyDeviceToHost, c->stream));
     RF_TRY(sync(c));
@@ -632,7 +679,9 @@ rf_status accept_iterate(rf_ctx *c, int f)
 
 // The attempt of a small grid: one cooperative launch that starts from h,
 // accepts a converged iterate and reports into pinned host memory.
-rf_status attempt_small(rf_ctx *c, double dt, Attempt &A, bool guess, int blocks)
+// refused: the stream's SMs do not hold the launch's blocks at once, and
+// nothing has run.
+rf_status attempt_small(rf_ctx *c, double dt, Attempt &A, bool guess, int blocks, bool &refused)
 {
     NvtxRange range("rf: Picard attempt");
     fill_step_params(c, dt);
@@ -701,7 +750,14 @@ rf_status attempt_small(rf_ctx *c, double dt, Attempt &A, bool guess, int blocks
     if (guess) RF_TRY(sync(c));     // the network's device waits report through dev_fault
     *c->fault_h = 0;
     c->closure_at_h = false;        // the attempt overwrites K[0] and C; an accepted step sets it again
-    CUDA_TRY(launch_attempt_small(c->stream, a, c->prm.precision == RF_PREC_MIXED, blocks));
+    const cudaError_t e = launch_attempt_small(c->stream, a, c->prm.precision == RF_PREC_MIXED, blocks);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        refused = true;
+        if (guess) c->ws_guesses--;
+        return RF_OK;
+    }
+    CUDA_TRY(e);
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaStreamSynchronize(c->stream));
     if (*c->fault_h) {
@@ -733,13 +789,17 @@ rf_status attempt(rf_ctx *c, double dt, Attempt &A, bool guess)
     // with hundreds of CG iterations per solve, mixed: 410 K 52.8 / 41.7 ms,
     // 786 K 55.2 / 63.1.  The other preconditioners run from the graph.
     constexpr long long SMALL_CELLS = 1 << 19;
-    if (c->prm.precond == RF_PRECOND_JACOBI && c->g.N <= SMALL_CELLS) {
+    if (c->prm.precond == RF_PRECOND_JACOBI && c->small_on && c->g.N <= SMALL_CELLS) {
         int &blocks = c->small_blocks[c->prm.precision == RF_PREC_MIXED ? 1 : 0];
         if (blocks < 0) blocks = attempt_small_blocks(c->g.N, c->num_sms, c->prm.precision == RF_PREC_MIXED);
-        if (blocks > 0) return attempt_small(c, dt, A, guess, blocks);
+        bool refused = false;
+        if (blocks > 0) {
+            const rf_status st = attempt_small(c, dt, A, guess, blocks, refused);
+            if (!refused) return st;
+            blocks = 0;
+        }
     }
     NvtxRange range("rf: Picard attempt");
-    if (!c->picard_exec) RF_TRY(build_picard_graph(c));
     fill_step_params(c, dt);
     PicardCtl &ctl = *c->ctl_h;
     ctl = PicardCtl{};
@@ -763,7 +823,7 @@ rf_status attempt(rf_ctx *c, double dt, Attempt &A, bool guess)
             c->closure_at_h = true;
         }
     }
-    CUDA_TRY(cudaGraphLaunch(c->picard_exec, c->stream));
+    RF_TRY(launch_graph(c, &rf_ctx::picard_exec, build_picard_graph));
     c->closure_at_h = false;     // the attempt overwrites K[0] and C; an accepted step sets it again
     CUDA_TRY(cudaMemcpyAsync(c->ctl_h, c->ctl, sizeof(PicardCtl), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(cudaMemcpyAsync(c->res_h, c->res, sizeof(StepResults), cudaMemcpyDeviceToHost, c->stream));
@@ -1166,10 +1226,6 @@ rf_status rf_mesh_create(const rf_mesh_desc *mesh, const rf_solver_params *param
     }
     c->cg64_blocks = cg64_solve_blocks(g, c->num_sms);
     c->mixed_blocks = mixed_solve_blocks(g, c->num_sms);
-    if (c->cg64_blocks < 1 || c->mixed_blocks < 1) {
-        rf_destroy(c);
-        return fail(RF_ERR_CUDA, "cooperative launches are not available on this device");
-    }
     // TMA plane staging for the FP32 stencil (grids with nx a multiple of 4)
     c->tma_ok = make_tma_maps32(g.nx, g.ny, g.nz, c->z32, c->p32[0], c->p32[1], c->K32, c->cb32, &c->tma);
     cudaGetLastError();
@@ -1547,6 +1603,16 @@ rf_status rf_set_wait_limit(rf_ctx *c, int polls)
     return RF_OK;
 }
 
+rf_status rf_set_one_launch(rf_ctx *c, int attempts, int solves)
+{
+    if (!c) return fail(RF_ERR_ARG, "null context");
+    CUDA_TRY(cudaStreamSynchronize(c->stream));
+    c->small_on = attempts != 0;
+    c->solve_on = solves != 0;
+    destroy_graphs(c);
+    return RF_OK;
+}
+
 unsigned long long rf_launch_count(rf_ctx *c)
 {
     if (!c) return 0ULL;
@@ -1607,12 +1673,13 @@ rf_status rf_profile_kernel(rf_ctx *c, int kind, int reps, double *avg_ms, doubl
         if (kind == RF_K_CG64_SPMV || kind == RF_K_CG64_UPDATE) {
             launch_cg64_spmv(s, nb, g, c->z, c->p[1], c->p[0], c->q, c->Tx, c->Ty, c->Tz, c->diag,
                              c->partials, c->ticket, c->sc);
-            launch_cg64_update(s, nb, g, c->x, c->r, c->z, c->p[0], c->q, c->dinv, c->partials, c->ticket, c->sc);
+            launch_cg64_update(s, nb, g, c->x, c->r, c->z, c->p[0], c->q, c->dinv, c->partials, c->ticket, c->sc,
+                               none);
         } else if (kind == RF_K_CG32_SPMV || kind == RF_K_CG32_UPDATE) {
             launch_cg32_spmv(s, nb, g, c->z32, c->p32[1], c->p32[0], c->q32, c->K32, c->cb32, c->partials, c->ticket,
                              c->sc_in, c->tma_ok ? &c->tma : nullptr, c->dev_fault);
             launch_cg32_update(s, nb, g, c->d32, c->r32, c->z32, c->p32[0], c->q32, c->dinv32, c->partials,
-                               c->ticket, c->sc_in);
+                               c->ticket, c->sc_in, none);
         }
         return RF_OK;
     };
@@ -1653,9 +1720,10 @@ rf_status rf_profile_kernel(rf_ctx *c, int kind, int reps, double *avg_ms, doubl
                                  c->ticket, c->sc);
             if (kind == RF_K_CG64_UPDATE)
                 timed([&] { launch_cg64_update(s, nb, g, c->x, c->r, c->z, pout, c->q, c->dinv, c->partials, c->ticket,
-                                               c->sc); });
+                                               c->sc, none); });
             else
-                launch_cg64_update(s, nb, g, c->x, c->r, c->z, pout, c->q, c->dinv, c->partials, c->ticket, c->sc);
+                launch_cg64_update(s, nb, g, c->x, c->r, c->z, pout, c->q, c->dinv, c->partials, c->ticket, c->sc,
+                                   none);
             break;
         case RF_K_RESID64:
             timed([&] { launch_resid64(s, nb, g, c->flags, c->x, c->b, c->Tx, c->Ty, c->Tz, c->diag, c->dinv32,
@@ -1671,10 +1739,10 @@ rf_status rf_profile_kernel(rf_ctx *c, int kind, int reps, double *avg_ms, doubl
                                  c->sc_in, c->tma_ok ? &c->tma : nullptr, c->dev_fault);
             if (kind == RF_K_CG32_UPDATE)
                 timed([&] { launch_cg32_update(s, nb, g, c->d32, c->r32, c->z32, qout, c->q32, c->dinv32, c->partials,
-                                               c->ticket, c->sc_in); });
+                                               c->ticket, c->sc_in, none); });
             else
                 launch_cg32_update(s, nb, g, c->d32, c->r32, c->z32, qout, c->q32, c->dinv32, c->partials, c->ticket,
-                                   c->sc_in);
+                                   c->sc_in, none);
             break;
         }
     }

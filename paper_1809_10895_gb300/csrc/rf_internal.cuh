@@ -382,7 +382,7 @@ void launch_cg64_spmv(cudaStream_t s, int nblk, const Grid &g, const double *z,
                       const double *Tz, const double *diag, double *partials, unsigned int *ticket, CgScal *sc);
 void launch_cg64_update(cudaStream_t s, int nblk, const Grid &g, double *x, double *r, double *z,
                         const double *p, const double *q, const double *dinv, double *partials,
-                        unsigned int *ticket, CgScal *sc);
+                        unsigned int *ticket, CgScal *sc, CondSet cond);
 // The whole solve in one cooperative launch (cg_solve.cu).
 int cg64_solve_blocks(const Grid &g, int sms);
 cudaError_t launch_cg64_solve(cudaStream_t s, int blocks, const Grid &g, const double *Tx, const double *Ty,
@@ -410,7 +410,8 @@ void launch_cg32_spmv(cudaStream_t s, int nblk, const Grid &g, const float *z, c
                       float *q, const float *K32, const float *cb32, double *partials, unsigned int *ticket,
                       CgScal *sc, const TmaMaps32 *tma = nullptr, int *fault = nullptr);
 void launch_cg32_update(cudaStream_t s, int nblk, const Grid &g, float *x, float *r, float *z, const float *p,
-                        const float *q, const float *dinv, double *partials, unsigned int *ticket, CgScal *sc);
+                        const float *q, const float *dinv, double *partials, unsigned int *ticket, CgScal *sc,
+                        CondSet cond);
 void launch_add_correction(cudaStream_t s, int nblk, const Grid &g, double *x, const float *d, CgScal *outer,
                            const CgScal *inner, CondSet cond_outer);
 

@@ -138,6 +138,7 @@ SIGNATURES = {
     "rf_solve": (C.c_int, [_VP, _VP, C.POINTER(C.c_int)]),
     "rf_apply_inner": (C.c_int, [_VP, _VP, _VP, C.c_float, _VP, _VP, _DP]),
     "rf_set_wait_limit": (C.c_int, [_VP, C.c_int]),
+    "rf_set_one_launch": (C.c_int, [_VP, C.c_int, C.c_int]),
     "rf_launch_count": (C.c_ulonglong, [_VP]),
     "rf_profile_kernel": (C.c_int, [_VP, C.c_int, C.c_int, _DP, _DP]),
     "rf_launch_counts": (C.c_int, [_VP, C.POINTER(C.c_ulonglong), C.c_int]),
@@ -449,6 +450,11 @@ class Solver:
     def set_wait_limit(self, polls: int):
         """Test hook of the bounded device waits (0: default; < 0: one non-blocking test)."""
         _check(load().rf_set_wait_limit(self.ctx, int(polls)), "rf_set_wait_limit")
+
+    def set_one_launch(self, attempts: bool = True, solves: bool = True):
+        """Whether small grids' Picard attempts and Jacobi solves run as one cooperative launch (the
+        default) or as a graph's launches."""
+        _check(load().rf_set_one_launch(self.ctx, int(attempts), int(solves)), "rf_set_one_launch")
 
     # -- learned warm start
     def ws_features(self, scales: "rf_ws_scales", t: float, dt: float, out, h=None):
