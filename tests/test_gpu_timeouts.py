@@ -40,6 +40,42 @@ def _times_out(s):
     assert np.array_equal(h0, h1) and m0 == m1
 
 
+# Each kind of bounded wait in a step: the small-grid attempt's barrier, the
+# one-launch solves' in the Picard graph, the TMA planes of the FP32 stencil
+# (DIC and multigrid, and Jacobi's loops; nx a multiple of 4).
+@pytest.mark.parametrize("precision,precond,route", [
+    ("fp64", "jacobi", (True, True)), ("mixed", "jacobi", (True, True)), ("fp64", "jacobi", (False, True)),
+    ("mixed", "jacobi", (False, True)), ("mixed", "jacobi", (False, False)), ("mixed", "dic", (True, True)),
+    ("mixed", "mg", (True, True))])
+def test_step(precision, precond, route):
+    case = W.heterogeneous_box(136, 20, 12, d=0.25, seed=21, water_table_depth=2.0, rain=4e-6, dt0=60.0)
+    s, ref = (rf.Solver.from_case(case, precision=precision, precond=precond) for _ in range(2))
+    for c in (s, ref):
+        c.set_one_launch(*route)
+        c.step()
+    _times_out(s)
+    _times_out(s)
+    _same_steps(s, ref, 3)
+
+
+def test_solve():
+    """The stored system's solve, and the next one."""
+    case = W.heterogeneous_box(136, 20, 12, d=0.25, seed=21, water_table_depth=2.0, rain=4e-6)
+    h = torch.as_tensor(case.h0, dtype=torch.float64, device="cuda")
+    for precision in ("fp64", "mixed"):
+        s = rf.Solver.from_case(case, precision=precision)
+        s.assemble(h, h, 60.0, 0.0)
+        x, y = h.clone(), h.clone()
+        it = s.solve(x)
+        s.set_wait_limit(-1)
+        with pytest.raises(rf.RFError) as e:
+            s.solve(y)
+        assert e.value.status == rf.RF_ERR_DEVICE_TIMEOUT
+        s.set_wait_limit(0)
+        y = h.clone()
+        assert s.solve(y) == it and torch.equal(x, y)
+
+
 def _same_steps(a, b, n):
     for _ in range(n):
         i, j = a.step(), b.step()
