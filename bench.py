@@ -434,11 +434,38 @@ def native(args):
         return out
 
     names = {"closure": "k_closure_picard", "assemble": "k_assemble_tiled", "cg64_spmv": "k_cg64_spmv",
-             "cg64_update": "k_cg64_update", "resid64": "k_resid64", "cg32_spmv": "k_cg32_spmv_tma",
+             "cg64_update": "k_cg64_update", "resid64": "k_resid64", "cg32_spmv": "k_cg32_spmv",
              "cg32_update": "k_cg32_update"}
+
+    def one_launch(s, kernel):
+        """The one-launch solve of the system at the window's end state, from x0 = 0 (start kernels and
+        copies included), timed by events around rf_solve."""
+        h = torch.empty(case.N, dtype=torch.float64, device="cuda")
+        s.get_state_device(h)
+        s.assemble(h, h, 60.0, meta0["t"])
+        x = torch.empty_like(h)
+        best = None
+        for _ in range(4):
+            x.zero_()
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record(s.stream)
+            it = s.solve(x)
+            b.record(s.stream)
+            b.synchronize()
+            ms = a.elapsed_time(b)
+            best = ms if best is None else min(best, ms)
+        return {"kernel": kernel, "ms": best, "iterations": it, "ms_per_iteration": best / max(it, 1)}
+
+    # phases of the one-launch solves: timed here as launches of their own; they
+    # run once an iteration inside the solve, without a launch
+    phase_of = {"cg64_spmv": "k_cg64_solve", "cg64_update": "k_cg64_solve", "resid64": "k_mixed_solve",
+                "cg32_spmv": "k_mixed_solve", "cg32_update": "k_mixed_solve"}
+
+    def count(kind, n):
+        return {"phase_of": phase_of[kind], "iterations": n} if kind in phase_of else {"launches_worked": n}
+
     kern64 = kernel_table(s64, ("closure", "assemble", "cg64_spmv", "cg64_update"))
     work64 = {"closure": counts64["closure_picard"][1] + counts64["closure"][1],
-              # the CG phases run inside the one-launch solves, once an iteration
               "assemble": counts64["assemble"][1], "cg64_spmv": st64["cg"], "cg64_update": st64["cg"]}
     est = {k: work64[k] * kern64[k]["avg_ms"] for k in work64}
     dom = max(est, key=lambda k: est[k])
@@ -466,8 +493,9 @@ def native(args):
                 "traffic": tr, "algorithmic_bytes_per_launch": kd["bytes"], "avg_launch_ms": kd["avg_ms"]}
 
     roof = roof_of(dom, kern64[dom])
-    kernels64 = {names[k]: dict(roof_of(k, v), launches_worked=work64[k], est_ms=est[k],
-                                share_of_window=est[k] / ms64) for k, v in kern64.items()}
+    kernels64 = {names[k]: dict(roof_of(k, v), est_ms=est[k], share_of_window=est[k] / ms64, **count(k, work64[k]))
+                 for k, v in kern64.items()}
+    kernels64["one_launch_solve"] = one_launch(s64, "k_cg64_solve")
     kernels_mix = None
     if s_mix is not None:
         km = kernel_table(s_mix, ("closure", "assemble", "resid64", "cg32_spmv", "cg32_update"))
@@ -476,8 +504,9 @@ def native(args):
               # Picard iteration, one stencil and one update an inner iteration
               "assemble": counts_mix["assemble"][1], "resid64": counts_mix["assemble"][1],
               "cg32_spmv": leg_mix["cg_iters"], "cg32_update": leg_mix["cg_iters"]}
-        kernels_mix = {names[k]: dict(roof_of(k, v), launches_worked=wm[k], est_ms=wm[k] * v["avg_ms"])
+        kernels_mix = {names[k]: dict(roof_of(k, v), est_ms=wm[k] * v["avg_ms"], **count(k, wm[k]))
                        for k, v in km.items()}
+        kernels_mix["one_launch_solve"] = one_launch(s_mix, "k_mixed_solve")
         s_mix.close()
 
     # ---- end to end through the C ABI with host buffers: every step uploads

@@ -318,8 +318,10 @@ rf_status rf_apply(rf_ctx *ctx, const double *d_x, double *d_y);
 rf_status rf_solve(rf_ctx *ctx, double *d_x, int *iters);
 
 /* The stencil step of the FP32 inner PCG of the mixed path (Sec. 2.2's PCG
- * run in FP32, the kernel its iterations launch: TMA-staged planes when nx
- * is a multiple of 4, plain tiles otherwise) on the last assembled system.
+ * run in FP32) on the last assembled system, as its iterations run it: the
+ * tiled sweep of the one-launch solve, or, where the solve is a graph's loops
+ * (the other preconditioners, rf_set_one_launch), the kernel they launch, which
+ * stages its planes by TMA when nx is a multiple of 4.
  * With p = d_z + beta d_pold on active cells (beta == 0: p = d_z, d_pold
  * unread), it writes d_p = p and d_q = A32 p, where
  *     (A32 v)_P = cb_P v_P + sum_f w_f (K_P + K_N)/2 (v_P - v_N)
@@ -358,10 +360,13 @@ unsigned long long rf_launch_count(rf_ctx *ctx);
  * in order: closure, closure+Picard test, assembly, FP64 CG init, FP64 CG
  * stencil, FP64 CG update, FP64 operator apply, mixed start, FP64 outer
  * residual, FP32 CG stencil, FP32 CG update, correction add, water balance,
- * storage, accept, a whole attempt or solve in one launch.  Returns the number of values written (<= cap). */
+ * storage, accept, a whole attempt or solve in one launch.  Returns the
+ * number of values written (<= cap). */
 int rf_launch_counts(rf_ctx *ctx, unsigned long long *out, int cap);
 
-/* Kernels that rf_profile_kernel can time. */
+/* Kernels that rf_profile_kernel can time.  The phases of a CG iteration and
+ * the outer residual are timed as launches of their own; a one-launch solve
+ * runs the same sweeps without the launches between them. */
 typedef enum rf_kernel_kind {
     RF_K_CLOSURE = 0,      /* closures at h with max|h - h_prev|            */
     RF_K_ASSEMBLE = 1,     /* Picard-system assembly                        */

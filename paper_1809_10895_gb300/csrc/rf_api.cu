@@ -236,6 +236,10 @@ bool one_launch_solve(const rf_ctx *c)
            (c->prm.precision == RF_PREC_FP64 ? c->cg64_blocks : c->mixed_blocks) > 0;
 }
 
+// The FP32 stencil as launches of its own stages its planes by TMA (nx a
+// multiple of 4); inside the one-launch solve it is the plain sweep.
+const TmaMaps32 *inner_tma(const rf_ctx *c) { return c->tma_ok && !one_launch_solve(c) ? &c->tma : nullptr; }
+
 // storage part of b, written and read only with modified Picard
 double *s0_of(rf_ctx *c) { return c->prm.picard_form == RF_PICARD_MODIFIED ? c->s0 : nullptr; }
 
@@ -480,7 +484,7 @@ rf_status capture_solve(rf_ctx *c, cudaGraph_t top, cudaGraph_t parent, std::vec
     for (int half = 0; half < 2; half++) {
         float *pin = c->p32[half], *pout = c->p32[half ^ 1];
         launch_cg32_spmv(s, nb, g, c->z32, pin, pout, c->q32, c->K32, c->cb32, c->partials, c->ticket, c->sc_in,
-                         c->tma_ok ? &c->tma : nullptr, c->dev_fault);
+                         inner_tma(c), c->dev_fault);
         if (dic) {
             launch_cg32_update_dic(s, nb, g, c->d32, c->r32, c->z32, pout, c->q32, c->dinv32, c->dic_rd, c->partials,
                                    c->ticket, c->sc_in);
@@ -1584,7 +1588,7 @@ rf_status rf_apply_inner(rf_ctx *c, const float *d_z, const float *d_pold, float
     h.max_it = 1;
     CUDA_TRY(cudaMemcpyAsync(c->sc_in, c->sc_in_h, sizeof(CgScal), cudaMemcpyHostToDevice, s));
     launch_cg32_spmv(s, c->nblk, g, c->z32, c->p32[1], c->p32[0], c->q32, c->K32, c->cb32, c->partials, c->ticket,
-                     c->sc_in, c->tma_ok ? &c->tma : nullptr, c->dev_fault);
+                     c->sc_in, inner_tma(c), c->dev_fault);
     CUDA_TRY(cudaMemcpyAsync(d_p, c->p32[0], nb, cudaMemcpyDeviceToDevice, s));
     CUDA_TRY(cudaMemcpyAsync(d_q, c->q32, nb, cudaMemcpyDeviceToDevice, s));
     CUDA_TRY(cudaMemcpyAsync(c->sc_in_h, c->sc_in, sizeof(CgScal), cudaMemcpyDeviceToHost, s));
@@ -1677,7 +1681,7 @@ rf_status rf_profile_kernel(rf_ctx *c, int kind, int reps, double *avg_ms, doubl
                                none);
         } else if (kind == RF_K_CG32_SPMV || kind == RF_K_CG32_UPDATE) {
             launch_cg32_spmv(s, nb, g, c->z32, c->p32[1], c->p32[0], c->q32, c->K32, c->cb32, c->partials, c->ticket,
-                             c->sc_in, c->tma_ok ? &c->tma : nullptr, c->dev_fault);
+                             c->sc_in, inner_tma(c), c->dev_fault);
             launch_cg32_update(s, nb, g, c->d32, c->r32, c->z32, c->p32[0], c->q32, c->dinv32, c->partials,
                                c->ticket, c->sc_in, none);
         }
@@ -1733,10 +1737,10 @@ rf_status rf_profile_kernel(rf_ctx *c, int kind, int reps, double *avg_ms, doubl
         default:
             if (kind == RF_K_CG32_SPMV)
                 timed([&] { launch_cg32_spmv(s, nb, g, c->z32, qin, qout, c->q32, c->K32, c->cb32, c->partials,
-                                             c->ticket, c->sc_in, c->tma_ok ? &c->tma : nullptr, c->dev_fault); });
+                                             c->ticket, c->sc_in, inner_tma(c), c->dev_fault); });
             else
                 launch_cg32_spmv(s, nb, g, c->z32, qin, qout, c->q32, c->K32, c->cb32, c->partials, c->ticket,
-                                 c->sc_in, c->tma_ok ? &c->tma : nullptr, c->dev_fault);
+                                 c->sc_in, inner_tma(c), c->dev_fault);
             if (kind == RF_K_CG32_UPDATE)
                 timed([&] { launch_cg32_update(s, nb, g, c->d32, c->r32, c->z32, qout, c->q32, c->dinv32, c->partials,
                                                c->ticket, c->sc_in, none); });
