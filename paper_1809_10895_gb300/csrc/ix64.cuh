@@ -9,7 +9,6 @@
 #pragma once
 
 #include <math.h>
-#include <string.h>
 
 #include "fx64.cuh"
 
@@ -76,27 +75,20 @@ RF_HD bool ix_sum7(const uint64_t (&b)[7], uint64_t &sum)
     return true;
 }
 
-// The 24-bit estimate r of 1/M as Q32 in [1/2, 1): rcp.approx, off by up to
-// 2^-23, may return 1 next to M = 1 and less than 1/2 next to M = 2.
-RF_HD uint32_t ix_rcp_seed(float r)
-{
-    r = fminf(fmaxf(r, 0.5f), 0x1.fffffep-1f);
-    uint32_t b;
-#ifdef __CUDA_ARCH__
-    b = __float_as_uint(r);
-#else
-    memcpy(&b, &r, 4);
-#endif
-    return ((b & 0x7fffffu) | 0x800000u) << 8;
-}
+// The float (bits) whose reciprocal is estimated for M in [1, 2) (Q63): M's
+// leading bits with the last three set to 2, so that an estimate off by up to
+// 2^-23 lies in [1/2, 1) however close M is to 1 or 2.
+RF_HD uint32_t ix_rcp_arg(uint64_t M) { return ((uint32_t)(M >> 40) & 0x7ffff8u) | 0x3f800002u; }
 
-// 1/M for M in [1, 2) (Q63), Q64 in (0.5, 1): the seed ri refined by
-// ri (1 + e + e^2), |e| = |1 - M ri| < 2^-21.
-RF_HD uint64_t ix_rcp_refine(uint64_t M, uint32_t ri)
+// 1/M, Q64 in (0.5, 1), from the estimate (bits rb): ri (1 + e + e^2) with ri
+// the estimate (Q32) and |e| = |1 - M ri| <= 2^-20 (6 + 2 units of 2^-23); e^3
+// is below 0.008 units of a double's last place.
+RF_HD uint64_t ix_rcp_refine(uint64_t M, uint32_t rb)
 {
+    const uint32_t ri = (rb << 8) | 0x80000000u;
     const int64_t e = (int64_t)(0x8000000000000000ULL - fx_mul32(M, ri));                             // Q63
-    const int32_t es = (int32_t)(e >> 11);                                                            // Q52
-    const int64_t s = e + (((int64_t)es * es) >> 41);                                                 // e + e^2
+    const int32_t es = (int32_t)(e >> 13);                                                            // Q50
+    const int64_t s = e + (((int64_t)es * es) >> 37);                                                 // e + e^2
     const int64_t t = (int64_t)(int32_t)(s >> 32) * ri + (int64_t)(uint32_t)(((uint64_t)(uint32_t)s * ri) >> 32);
     return ((uint64_t)ri << 32) + (uint64_t)(t << 1);
 }
@@ -117,23 +109,26 @@ RF_HD bool ix_quot_ok(uint64_t a, uint64_t b)
     return (uint32_t)(a >> 52) - 700u < 650u && (uint32_t)(b >> 52) - 700u < 650u;
 }
 
-// The float nearest to the double with bits b (ties to even); false where it
-// is zero, subnormal, infinite or NaN as a float.
-RF_HD bool ix_d2f_bits(uint64_t b, uint32_t &f)
+// The bits of the float nearest to the double with bits b (ties to even);
+// not where it is zero, subnormal, infinite or NaN as a float.
+RF_HD bool ix_d2f_ok(uint64_t b) { return ((uint32_t)(b >> 52) & 0x7ffu) - 897u <= 253u; }
+RF_HD uint32_t ix_d2f_bits(uint64_t b)
 {
-    if (((uint32_t)(b >> 52) & 0x7ffu) - 897u > 253u) return false;
     const uint64_t v = (b & 0x7fffffffffffffffULL) - (896ULL << 52);
-    f = (uint32_t)((v + 0x0fffffffULL + ((v >> 29) & 1)) >> 29) | ((uint32_t)(b >> 32) & 0x80000000u);
-    return true;
+    return (uint32_t)((v + 0x0fffffffULL + ((v >> 29) & 1)) >> 29) | ((uint32_t)(b >> 32) & 0x80000000u);
 }
 
-// The float with bits b as a double; false for subnormal, infinite or NaN.
-RF_HD bool ix_f2d_bits(uint32_t b, uint64_t &d)
+// The bits of the float with bits b as a double; not where it is subnormal,
+// infinite or NaN.
+RF_HD bool ix_f2d_ok(uint32_t b)
 {
     const uint32_t m = b & 0x7fffffffu;
-    if (m - 0x00800000u >= 0x7f000000u && m) return false;
-    d = (m ? ((uint64_t)m << 29) + (896ULL << 52) : 0) | (uint64_t)(b & 0x80000000u) << 32;
-    return true;
+    return m - 0x00800000u < 0x7f000000u || !m;
+}
+RF_HD uint64_t ix_f2d_bits(uint32_t b)
+{
+    const uint32_t m = b & 0x7fffffffu;
+    return (m ? ((uint64_t)m << 29) + (896ULL << 52) : 0) | (uint64_t)(b & 0x80000000u) << 32;
 }
 
 // Square root of a in [2^-99, 2^99], relative error below 2^-44: the float
@@ -149,15 +144,16 @@ RF_HD double ix_root_step(double a, double s, float sf)
 __device__ __forceinline__ uint64_t ix_rcp(uint64_t M)
 {
     float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(0x3f800000u | ((uint32_t)(M >> 40) & 0x7fffffu))));
-    return ix_rcp_refine(M, ix_rcp_seed(r));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(ix_rcp_arg(M))));
+    return ix_rcp_refine(M, __float_as_uint(r));
 }
 
 // The float nearest to a double (ties to even).
 __device__ __forceinline__ float ix_d2f(double a)
 {
-    uint32_t f;
-    return ix_d2f_bits((uint64_t)__double_as_longlong(a), f) ? __uint_as_float(f) : (float)a;
+    const uint64_t b = (uint64_t)__double_as_longlong(a);
+    if (!ix_d2f_ok(b)) return (float)a;
+    return __uint_as_float(ix_d2f_bits(b));
 }
 
 // Tests on the bits: a compare of doubles goes to the FP64 pipe.
@@ -177,8 +173,9 @@ __device__ __forceinline__ bool not_above(double a, double b)    // a <= b, both
 // A float as a double.
 __device__ __forceinline__ double ix_f2d(float a)
 {
-    uint64_t d;
-    return ix_f2d_bits(__float_as_uint(a), d) ? __longlong_as_double((long long)d) : (double)a;
+    const uint32_t b = __float_as_uint(a);
+    if (!ix_f2d_ok(b)) return (double)a;
+    return __longlong_as_double((long long)ix_f2d_bits(b));
 }
 
 // 1/a.

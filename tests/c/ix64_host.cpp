@@ -23,11 +23,13 @@ static double value(uint64_t b)
 
 static uint64_t rcp(uint64_t M, int ulps)
 {
-    const uint32_t xb = 0x3f800000u | ((uint32_t)(M >> 40) & 0x7fffffu);
+    const uint32_t xb = ix_rcp_arg(M);
+    uint32_t rb;
     float x;
     std::memcpy(&x, &xb, 4);
-    const float r = 1.0f / x, unit = 0x1p-24f;      // of a result in [1/2, 1)
-    return ix_rcp_refine(M, ix_rcp_seed(r + (float)ulps * unit));
+    const float r = 1.0f / x + (float)ulps * 0x1p-24f;      // units of a result in [1/2, 1)
+    std::memcpy(&rb, &r, 4);
+    return ix_rcp_refine(M, rb);
 }
 
 extern "C" double ix_h_rcp(double a, int ulps)
@@ -61,25 +63,24 @@ extern "C" double ix_h_sqrt(double a)
 extern "C" float ix_h_rcp32(double a, int ulps)
 {
     const double r = ix_h_rcp(a, ulps);
-    uint32_t f;
+    const uint32_t f = ix_d2f_bits(bits(r));
     float v = NAN;
-    if (ix_d2f_bits(bits(r), f)) std::memcpy(&v, &f, 4);
+    if (ix_d2f_ok(bits(r))) std::memcpy(&v, &f, 4);
     return v;
 }
 
 // NaN where the integer form leaves the conversion to the instruction.
 extern "C" float ix_h_d2f(double a)
 {
-    uint32_t f;
+    const uint32_t f = ix_d2f_bits(bits(a));
     float v = NAN;
-    if (ix_d2f_bits(bits(a), f)) std::memcpy(&v, &f, 4);
+    if (ix_d2f_ok(bits(a))) std::memcpy(&v, &f, 4);
     return v;
 }
 
 extern "C" double ix_h_f2d(float a)
 {
     uint32_t b;
-    uint64_t d;
     std::memcpy(&b, &a, 4);
-    return ix_f2d_bits(b, d) ? value(d) : NAN;
+    return ix_f2d_ok(b) ? value(ix_f2d_bits(b)) : NAN;
 }

@@ -49,7 +49,7 @@ def ulps_off(got, exact):
 
 
 # One rounding plus what the 64-bit significand loses: a few units of 2^-63,
-# below a hundredth of a unit of the last place.
+# and of a reciprocal e^3 <= 2^-60: below a hundredth of a unit of the last place.
 TOL = Fraction(51, 100)
 
 
