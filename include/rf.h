@@ -81,14 +81,15 @@ typedef enum rf_precision {
     RF_PREC_MIXED = 1
 } rf_precision;
 
-/* Arithmetic of the closures (Eq. 2-4).  AUTO: FP64 on the RF_PREC_FP64
- * and the RF_PREC_MIXED path.  FP64: full FP64 accuracy
- * (within a few units of the last place), computed in 64-bit fixed point
- * where the state is in its range (|log2(-alpha h)| < 30, |n log2(-alpha h)|
- * < 60, n < 16, 1 - 1/n >= 2^-12) and in FP64 elsewhere.  DOUBLE_FLOAT: pairs of FP32 values
+/* Arithmetic of the closures (Eq. 2-4).  FP64: full FP64 accuracy (within a
+ * few units of the last place), computed in 64-bit fixed point where the state
+ * is in its range (|log2(-alpha h)| < 30, |n log2(-alpha h)| < 60, n < 16,
+ * 1 - 1/n >= 2^-12) and in FP64 elsewhere.  DOUBLE_FLOAT: pairs of FP32 values
  * (about 48 significant bits: theta* within 1.2e-14 relative, K and C within
- * 2.4e-13).  Storage, the chord difference, the operator, the Picard test and
- * the balance are FP64 either way. */
+ * 2.4e-13).  AUTO: FP64 on the RF_PREC_FP64 path; on the RF_PREC_MIXED path
+ * fixed point in its range and DOUBLE_FLOAT elsewhere, which takes a quarter of
+ * FP64's time.  Storage, the chord difference, the operator, the Picard test
+ * and the balance are FP64 either way. */
 typedef enum rf_closure_arith {
     RF_CLOSURE_AUTO = 0, RF_CLOSURE_FP64 = 1, RF_CLOSURE_DOUBLE_FLOAT = 2
 } rf_closure_arith;

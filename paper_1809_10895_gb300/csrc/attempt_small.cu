@@ -153,7 +153,7 @@ k_attempt_small(const __grid_constant__ AttemptArgs A)
     __syncthreads();
     auto cell_closure = [&](int p, double hp, double *K) {
         double th, k, c;
-        closure(A.soils[A.zone[p]], A.Ks[p], hp, g.tab, &s.fx, g.closure64, th, k, c);
+        closure(A.soils[A.zone[p]], A.Ks[p], hp, g.tab, &s.fx, g.arith, th, k, c);
         A.theta_k[p] = th;
         K[p] = k;
         A.Can[p] = c;

@@ -178,7 +178,8 @@ __device__ __forceinline__ void closure_general(const DevSoil &s, double Ks, dou
     else closure_vg_df(s, Ks, h, tab, th, K, C);
 }
 
-// The same out of line, for the cells that the fixed-point form leaves over.
+// The same out of line, for the cells that the fixed-point form leaves over:
+// two functions (4.2 M cells in range: 145 us; 154 with one and a switch).
 struct Closure3 {
     double th, K, C;
 };
@@ -188,14 +189,21 @@ static __device__ __noinline__ Closure3 closure_rest(const DevSoil *s, double Ks
     closure_general(*s, Ks, h, tab, true, r.th, r.K, r.C);
     return r;
 }
+static __device__ __noinline__ Closure3 closure_rest_df(const DevSoil *s, double Ks, double h, const FFTables *tab)
+{
+    Closure3 r;
+    closure_general(*s, Ks, h, tab, false, r.th, r.K, r.C);
+    return r;
+}
 
 // Closures of one cell at head h: theta*, K, C.  For h >= 0 (tie included)
 // theta* = theta_s + S h, K = Ks, C = S, which makes d(theta*)/dh equal to
-// Eq. 3 on both branches.  With fp64, van Genuchten cells run in 64-bit fixed
-// point (fx64.cuh; tables fx, global or a shared copy) wherever the state is
-// in its range, and in FP64 elsewhere.
+// Eq. 3 on both branches.  Unless arith is ARITH_DF, van Genuchten cells run in
+// 64-bit fixed point (fx64.cuh; tables fx, global or a shared copy) wherever
+// the state is in its range; the others in FP64, or with ARITH_FX_DF in
+// double-float arithmetic (4.2 M cells all out of range: 975 and 213 us).
 __device__ __forceinline__ void closure(const DevSoil &s, double Ks, double h, const FFTables *__restrict__ tab,
-                                        const FxTables *__restrict__ fx, bool fp64, double &th, double &K, double &C)
+                                        const FxTables *__restrict__ fx, int arith, double &th, double &K, double &C)
 {
     const unsigned long long hb = (unsigned long long)__double_as_longlong(h);
     if (hb <= 0x7ff0000000000000ULL || hb == 0x8000000000000000ULL) {   // h >= 0
@@ -204,30 +212,40 @@ __device__ __forceinline__ void closure(const DevSoil &s, double Ks, double h, c
         C = s.S;
         return;
     }
-    if (!fp64) {
-        closure_general(s, Ks, h, tab, false, th, K, C);
-        return;
-    }
     uint64_t se, kr, cr;
-    if (fx_closure_vg(s.fx, hb & 0x7fffffffffffffffULL, fx, se, kr, cr)) {
+    if (arith != ARITH_DF && fx_closure_vg(s.fx, hb & 0x7fffffffffffffffULL, fx, se, kr, cr)) {
         th = fma(s.dth, __longlong_as_double((long long)se), s.theta_r);
         K = Ks * __longlong_as_double((long long)kr);
         C = s.cfac * __longlong_as_double((long long)cr);
         return;
     }
-    const Closure3 r = closure_rest(&s, Ks, h, tab);
+    const Closure3 r = arith == ARITH_FP64 ? closure_rest(&s, Ks, h, tab) : closure_rest_df(&s, Ks, h, tab);
     th = r.th;
     K = r.K;
     C = r.C;
 }
 
+// The same in double-float arithmetic throughout, inline: for the closure
+// kernels' instance of that choice (4.2 M cells: 233 us, out of line 246).
+__device__ __forceinline__ void closure_df(const DevSoil &s, double Ks, double h, const FFTables *__restrict__ tab,
+                                           double &th, double &K, double &C)
+{
+    if (h >= 0.0) {
+        th = s.theta_s + s.S * h;
+        K = Ks;
+        C = s.S;
+        return;
+    }
+    closure_general(s, Ks, h, tab, false, th, K, C);
+}
+
 // K at a Dirichlet face's head.  Out of line: the face loops are unrolled and
 // few cells carry such a face.
 static __device__ __noinline__ double closure_face(const DevSoil *s, double Ks, double h, const FFTables *tab,
-                                                   bool fp64)
+                                                   int arith)
 {
     double th, K, C;
-    closure(*s, Ks, h, tab, &tab->fx, fp64, th, K, C);
+    closure(*s, Ks, h, tab, &tab->fx, arith, th, K, C);
     return K;
 }
 
@@ -278,7 +296,7 @@ __device__ __forceinline__ void boundary_face(const Grid &g, const DevSoil *__re
         hD = sp.bc_val[f];
     }
     if (type == BC_DIRICHLET) {
-        const double KD = closure_face(&soils[zone[p]], Ks[p], hD, g.tab, g.closure64);
+        const double KD = closure_face(&soils[zone[p]], Ks[p], hD, g.tab, g.arith);
         const double T = KD * g.wb[f];
         diag += T;
         cb += T;
@@ -449,7 +467,7 @@ __device__ __forceinline__ void boundary_fluxes(const Grid &g, const DevSoil &s,
             hD = sp.bc_val[f];
         }
         if (type == BC_DIRICHLET) {
-            const double KD = closure_face(&s, Ksp, hD, g.tab, g.closure64);
+            const double KD = closure_face(&s, Ksp, hD, g.tab, g.arith);
             const double T = KD * g.wb[f];
             flux = T * hD + gs * KD * g.A[f] - T * xp;
         } else if (type == BC_FLUX) {

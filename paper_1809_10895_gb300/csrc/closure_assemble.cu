@@ -71,6 +71,7 @@ __device__ __forceinline__ bool grid_max_dh(MaxDh &m, double *partials, unsigned
 // twice the blocks: 2.5 % faster there, 10 % slower on 1 M cells.  The
 // tables (10 KB) sit in shared memory, where a gather costs its bank
 // conflicts only.
+template <bool DF>
 __device__ __forceinline__ void closure_cells(const Grid &g, const DevSoil *__restrict__ soils,
                                               const uint8_t *__restrict__ zone, const double *__restrict__ Ks,
                                               const uint8_t *__restrict__ flags, const double *__restrict__ h,
@@ -78,7 +79,7 @@ __device__ __forceinline__ void closure_cells(const Grid &g, const DevSoil *__re
                                               double *__restrict__ K, double *__restrict__ Can, MaxDh &m)
 {
     __shared__ FxTables fx;
-    {
+    if (!DF) {
         const uint64_t *src = reinterpret_cast<const uint64_t *>(&g.tab->fx);
         uint64_t *dst = reinterpret_cast<uint64_t *>(&fx);
         for (int i = threadIdx.x; i < (int)(sizeof(FxTables) / 8); i += blockDim.x) dst[i] = src[i];
@@ -100,13 +101,15 @@ __device__ __forceinline__ void closure_cells(const Grid &g, const DevSoil *__re
             else m.bad = 1;                                            // NaN or inf
         }
         double th, k, c;
-        closure(soils[zone[p]], Ks[p], hp, g.tab, &fx, g.closure64, th, k, c);
+        if (DF) closure_df(soils[zone[p]], Ks[p], hp, g.tab, th, k, c);
+        else closure(soils[zone[p]], Ks[p], hp, g.tab, &fx, g.arith, th, k, c);
         theta[p] = th;
         K[p] = k;
         Can[p] = c;
     }
 }
 
+template <bool DF>
 __global__ void __launch_bounds__(RED_THREADS)
 k_closure(Grid g, const DevSoil *__restrict__ soils, const uint8_t *__restrict__ zone,
           const double *__restrict__ Ks, const uint8_t *__restrict__ flags, const double *__restrict__ h,
@@ -116,7 +119,7 @@ k_closure(Grid g, const DevSoil *__restrict__ soils, const uint8_t *__restrict__
     count_launch(g, KK_CLOSURE);
     count_work(g, KK_CLOSURE);
     MaxDh m;
-    closure_cells(g, soils, zone, Ks, flags, h, hprev, theta, K, Can, m);
+    closure_cells<DF>(g, soils, zone, Ks, flags, h, hprev, theta, K, Can, m);
     if (hprev) {
         if (grid_max_dh(m, partials, ticket) && threadIdx.x == 0) {
             res->max_dh = __longlong_as_double((long long)m.d);
@@ -131,6 +134,7 @@ k_closure(Grid g, const DevSoil *__restrict__ soils, const uint8_t *__restrict__
 // and the loop control.  A failed linear solve or a non-finite update fails
 // the attempt.  The last block sets the Picard loop condition; every launch
 // sets it, so the loop always terminates (at the latest after n_max).
+template <bool DF>
 __global__ void __launch_bounds__(RED_THREADS)
 k_closure_picard(Grid g, const DevSoil *__restrict__ soils, const uint8_t *__restrict__ zone,
                  const double *__restrict__ Ks, const uint8_t *__restrict__ flags, const double *__restrict__ x,
@@ -145,7 +149,7 @@ k_closure_picard(Grid g, const DevSoil *__restrict__ soils, const uint8_t *__res
     }
     count_work(g, KK_CLOSURE_PICARD);
     MaxDh m;
-    closure_cells(g, soils, zone, Ks, flags, x, hk, theta, K, Can, m);
+    closure_cells<DF>(g, soils, zone, Ks, flags, x, hk, theta, K, Can, m);
     if (grid_max_dh(m, partials, ticket) && threadIdx.x == 0) {
         const double max_dh = __longlong_as_double((long long)m.d);
         const int it = ++ctl->it;
@@ -666,7 +670,8 @@ void launch_closure(cudaStream_t s, int nblk, const Grid &g, const DevSoil *soil
                     double *theta, double *K, double *Can, double *partials, unsigned int *ticket,
                     StepResults *res)
 {
-    k_closure<<<nblk, RED_THREADS, 0, s>>>(g, soils, zone, Ks, flags, h, hprev, theta, K, Can, partials, ticket, res);
+    auto *fn = g.arith == ARITH_DF ? k_closure<true> : k_closure<false>;
+    fn<<<nblk, RED_THREADS, 0, s>>>(g, soils, zone, Ks, flags, h, hprev, theta, K, Can, partials, ticket, res);
 }
 
 void launch_closure_picard(cudaStream_t s, int nblk, const Grid &g, const DevSoil *soils, const uint8_t *zone,
@@ -674,8 +679,9 @@ void launch_closure_picard(cudaStream_t s, int nblk, const Grid &g, const DevSoi
                            double *theta, double *K, double *Can, double *partials, unsigned int *ticket,
                            PicardCtl *ctl, const CgScal *cg_status, const CgScal *cg_count, CondSet cond)
 {
-    k_closure_picard<<<nblk, RED_THREADS, 0, s>>>(g, soils, zone, Ks, flags, x, hk, theta, K, Can, partials, ticket,
-                                                  ctl, cg_status, cg_count, cond);
+    auto *fn = g.arith == ARITH_DF ? k_closure_picard<true> : k_closure_picard<false>;
+    fn<<<nblk, RED_THREADS, 0, s>>>(g, soils, zone, Ks, flags, x, hk, theta, K, Can, partials, ticket, ctl, cg_status,
+                                    cg_count, cond);
 }
 
 // Tiles wherever they fill: at least half a tile's row, and enough cells that

@@ -685,7 +685,7 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                     mx = dd > mx ? dd : mx;
                 }
                 double th, k, c;
-                closure(*soil, Ks[p], hp, g.tab, &g.tab->fx, g.closure64, th, k, c);
+                closure(*soil, Ks[p], hp, g.tab, &g.tab->fx, g.arith, th, k, c);
                 thx[p] = th;
                 Kx[p] = k;
                 Can[p] = c;

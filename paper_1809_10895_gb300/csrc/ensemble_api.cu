@@ -278,7 +278,8 @@ rf_status rf_ens_create(const rf_ens_instance *inst, int n, const rf_solver_para
         }
         const double up[3] = {0.0, 0.0, 1.0};
         set_grid_gravity(g, up, false);
-        g.closure64 = prm.closure_arith != RF_CLOSURE_DOUBLE_FLOAT ? 1 : 0;
+        g.arith = closure_arith_of(prm.closure_arith == RF_CLOSURE_DOUBLE_FLOAT, prm.closure_arith == RF_CLOSURE_AUTO,
+                                   prm.precision == RF_PREC_MIXED);
         for (int ax = 0; ax < 3; ax++) g.w32[ax] = (float)(A[2 * ax] / dd[2 * ax]);
         g.fx = make_fastdiv((unsigned int)a.nx);
         g.fxy = make_fastdiv((unsigned int)g.sxy);

@@ -193,7 +193,8 @@ void apply_grid_params(Grid &g, const rf_solver_params &p)
     set_grid_gravity(g, p.grav, p.face_mean == RF_FACE_HARMONIC);
     // AUTO: the fixed-point form serves both precisions (it is faster than the
     // double-float one as well: 224 against 334 us on 6 M active cells)
-    g.closure64 = p.closure_arith != RF_CLOSURE_DOUBLE_FLOAT ? 1 : 0;
+    g.arith = closure_arith_of(p.closure_arith == RF_CLOSURE_DOUBLE_FLOAT, p.closure_arith == RF_CLOSURE_AUTO,
+                               p.precision == RF_PREC_MIXED);
 }
 
 double series_at(const BcSeries &b, double t)

@@ -83,7 +83,7 @@ struct Grid {
     float w32[3];     // A/d per axis, FP32 (mixed-precision operator)
     FastDiv fx, fxy;  // division by nx and by nx*ny
     int cap;          // most blocks a tiled stencil kernel launches (partials hold 8 values per block)
-    int closure64;    // 1: closures to FP64 accuracy (fixed point, else FP64); 0: double-float arithmetic
+    int arith;        // closure arithmetic, ARITH_*
     int tilted;       // 1: the elevation gradient has x / y components (gravity on lateral faces)
     int ix_ok;        // 1: arithmetic mean and A/(2 d) within the range of the integer face arithmetic
     int harmonic;     // 1: harmonic interface conductivity; 0: arithmetic mean (linear interpolation)
@@ -168,6 +168,14 @@ struct StepResults {
 };
 
 constexpr int RED_THREADS = 256;
+
+// Closure arithmetic: double-float; fixed point, else FP64; fixed point, else
+// double-float.  AUTO keeps to FP64 accuracy on the FP64 path only.
+enum { ARITH_DF = 0, ARITH_FP64 = 1, ARITH_FX_DF = 2 };
+inline int closure_arith_of(bool df, bool automatic, bool mixed)
+{
+    return df ? ARITH_DF : automatic && mixed ? ARITH_FX_DF : ARITH_FP64;
+}
 
 // Fields that follow from gravity, the interface mean and the face areas.
 inline void set_grid_gravity(Grid &g, const double grav[3], bool harmonic)
