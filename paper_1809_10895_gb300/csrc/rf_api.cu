@@ -133,8 +133,16 @@ struct rf_ctx {
         void *ptr = nullptr;
         if (has_alloc) ptr = alloc.alloc(bytes, alloc.user);
         else if (cudaMalloc(&ptr, bytes) != cudaSuccess) ptr = nullptr;
+        // the kernels load 16 bytes at a time: a caller's pointer off the
+        // 256-byte boundary that rf_allocator asks for is moved up to one
+        uintptr_t at = reinterpret_cast<uintptr_t>(ptr);
+        if (at & 255) {
+            alloc.free(ptr, alloc.user);
+            ptr = alloc.alloc(bytes + 255, alloc.user);
+            at = (reinterpret_cast<uintptr_t>(ptr) + 255) & ~uintptr_t(255);
+        }
         if (ptr) allocations.push_back(ptr);
-        return ptr;
+        return ptr ? reinterpret_cast<void *>(at) : nullptr;
     }
 };
 
