@@ -1,9 +1,11 @@
 // grid_red.cuh -- barriers and reductions over the blocks of a running
 // cooperative kernel.
 //
-// The barrier is one counter: a block arrives with an acquire-release atomic
-// and polls until the top bit flips, which the last arrival causes, so nothing
-// is reset between launches (1.2 us over 152 blocks; adding __threadfence() on
+// The barrier is one counter, as in CUDA's cooperative-groups grid barrier: block
+// 0 adds 2^31 - (blocks - 1) and the others 1, so that the last arrival flips
+// the top bit, and nothing is reset between launches.  Here a block arrives with
+// an acquire-release atomic and polls with acquire loads, a bounded number of
+// times (1.2 us over 152 blocks; adding __threadfence() on
 // both sides costs 0.1 us, an all-gather in which every block polls every
 // block's slot costs 2-3 us more, and clusters in front of it 0.4 us).  For a
 // reduction the blocks publish partials before arriving and each folds all of

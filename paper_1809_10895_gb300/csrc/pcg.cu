@@ -10,7 +10,9 @@
 //   (A v)_P = cb_P v_P + sum_f w_f (K_P + K_N)/2 (v_P - v_N)
 // where cb = c + Dirichlet half-cell terms; inactive neighbours carry K < 0.
 //
-// One PCG iteration is two kernels:
+// Jacobi solves run in one launch (cg_solve.cu).  As launches of their own, for
+// the loops of the other preconditioners and of streams that cannot hold a
+// cooperative launch, and for the profiler, an iteration is two kernels:
 //   spmv   : p = z + beta p_old (recomputed for the stencil neighbours, so p
 //            ping-pongs between two buffers), q = A p, partial p.q;
 //   update : x += alpha p, r -= alpha q, z = D^-1 r, partial r.r and r.z.

@@ -796,11 +796,14 @@ rf_status attempt_small(rf_ctx *c, double dt, Attempt &A, bool guess, int blocks
 
 rf_status attempt(rf_ctx *c, double dt, Attempt &A, bool guess)
 {
-    // Grids on which an attempt is launch latency (measured, one pass of six to
-    // four 60 s steps of the box, graph / one launch): 30 K cells 1585 / 877 us,
-    // 262 K 2150 / 1315, 410 K 2732 / 1766, 786 K 7214 / 5935, 1 M 5665 / 5570;
-    // with hundreds of CG iterations per solve, mixed: 410 K 52.8 / 41.7 ms,
-    // 786 K 55.2 / 63.1.  The other preconditioners run from the graph.
+    // Grids on which an attempt is launch latency.  Four steps of the box, some
+    // seven CG iterations a step, graph / one launch in ms: FP64 30 K cells 0.76 /
+    // 0.51, 99 K 1.00 / 0.71, 262 K 1.49 / 1.01, 524 K 2.16 / 1.65; mixed 0.89 / 0.64,
+    // 1.15 / 0.91, 1.46 / 1.21, 2.04 / 1.86.  The line is drawn for such steps.  Saturated
+    // blocks whose solves take 100 to 400 iterations prefer the graph's tiled
+    // sweeps earlier: FP64 30 K 7.2 / 6.4, 99 K 13.9 / 15.0, 262 K 26.0 / 31.7, 524 K
+    // 55.1 / 61.2; mixed 8.6 / 9.1, 15.6 / 18.0, 24.4 / 37.3, 39.6 / 69.2 (columns never:
+    // 2000 cells 147 / 65, 196 / 91).  The other preconditioners run from the graph.
     constexpr long long SMALL_CELLS = 1 << 19;
     if (c->prm.precond == RF_PRECOND_JACOBI && c->small_on && c->g.N <= SMALL_CELLS) {
         int &blocks = c->small_blocks[c->prm.precision == RF_PREC_MIXED ? 1 : 0];
