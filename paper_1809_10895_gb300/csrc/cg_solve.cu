@@ -39,6 +39,7 @@ __device__ __forceinline__ bool cg_reduce(GridRed &R, CgShared &s, const double 
     return grid_red_sum<NV>(R, s.part, s.tot, &s.abort, v, fin);
 }
 
+template <bool NARROW>
 __global__ void __launch_bounds__(CT, SWEEP_OCC)
 k_cg64_solve(Grid g, Tiles tw, const double *__restrict__ Tx, const double *__restrict__ Ty,
              const double *__restrict__ Tz, const double *__restrict__ diag, const double *__restrict__ dinv,
@@ -71,15 +72,18 @@ k_cg64_solve(Grid g, Tiles tw, const double *__restrict__ Tx, const double *__re
         struct Raw {
             double z, o;
         };
-        sweep64<Raw, NoOwn>(
-            g, tw, A, s.w64, [&](long long c) { return Raw{__ldcs(&z[c]), first ? 0.0 : __ldcs(&pin[c])}; },
-            [&](const Raw &a) { return fma(beta, a.o, a.z); },
-            [](long long) { return NoOwn{}; },
-            [&](long long c, double v, double Av, bool, NoOwn) {
-                pout[c] = v;
-                q[c] = Av;
-                acc[0] = fma(v, Av, acc[0]);
-            });
+        auto none = [](long long) { return NoOwn{}; };
+        auto out = [&](long long c, double v, double Av, bool, NoOwn) {
+            pout[c] = v;
+            q[c] = Av;
+            acc[0] = fma(v, Av, acc[0]);
+        };
+        if (NARROW)
+            cells64<NoOwn>(g, A, [&](long long c) { return first ? z[c] : fma(beta, pin[c], z[c]); }, none, out);
+        else
+            sweep64<Raw, NoOwn>(
+                g, tw, A, s.w64, [&](long long c) { return Raw{__ldcs(&z[c]), first ? 0.0 : __ldcs(&pin[c])}; },
+                [&](const Raw &a) { return fma(beta, a.o, a.z); }, none, out);
         if (!cg_reduce<1>(R, s, acc, [&]() {
                 const double pq = s.tot[0];
                 s.alpha = ix_div(s.rho, pq);
@@ -161,6 +165,7 @@ struct MixedArgs {
     int inner_max_it, outer_max_it;
 };
 
+template <bool NARROW>
 __global__ void __launch_bounds__(CT, SWEEP_OCC)
 k_mixed_solve(const __grid_constant__ MixedArgs M)
 {
@@ -191,7 +196,8 @@ k_mixed_solve(const __grid_constant__ MixedArgs M)
             const bool first = it == 0;
             const float *pin = (it & 1) ? M.p1 : M.p0;
             float *pout = (it & 1) ? M.p0 : M.p1;
-            float w[1] = {sweep32(g, M.t32, s.w32, M.K32, M.cb32, M.z32, pin, pout, M.q32, beta, first)};
+            float w[1] = {NARROW ? cells32(g, M.K32, M.cb32, M.z32, pin, pout, M.q32, beta, first)
+                                 : sweep32(g, M.t32, s.w32, M.K32, M.cb32, M.z32, pin, pout, M.q32, beta, first)};
             if (!cg_reduce_f32<1>(R, s, w, [&]() {
                     const double pq = s.tot[0];
                     s.alpha = ix_div(s.rho, pq);
@@ -240,7 +246,7 @@ k_mixed_solve(const __grid_constant__ MixedArgs M)
         // ---- r = b - A x in FP64, seeds of the next inner solve
         float f[3] = {0.0f, 0.0f, 0.0f};           // r.r, b.b, r.z
         const Op64 A{M.Tx, M.Ty, M.Tz, M.diag};
-        resid64_sweep(g, M.t64, A, s.w64, M.flags, M.x, M.b, M.dinv32, M.r32, M.z32, nullptr, f);
+        resid64_sweep<NARROW>(g, M.t64, A, s.w64, M.flags, M.x, M.b, M.dinv32, M.r32, M.z32, nullptr, f);
         outer++;
         if (!cg_reduce_f32<3>(R, s, f, [&]() {
                 const double rr = s.tot[0], bb = s.tot[1], rz = s.tot[2];
@@ -272,14 +278,26 @@ k_mixed_solve(const __grid_constant__ MixedArgs M)
 
 }  // namespace
 
-// Blocks of the solve on this grid (0: it cannot run): what fits the GPU at
-// once, but no more than there are tiles and planes to share out.
-int cg64_solve_blocks(const Grid &g, int sms)
+// Instances, and their blocks on this grid (0: it cannot run): what fits the
+// GPU at once, but no more than there are tiles and planes, or cells, to share out.
+static auto *cg64_fn(const Grid &g) { return narrow_grid(g, CX, CY) ? k_cg64_solve<true> : k_cg64_solve<false>; }
+static auto *mixed_fn(const Grid &g) { return narrow_grid(g, CX, CY) ? k_mixed_solve<true> : k_mixed_solve<false>; }
+
+static int solve_blocks(const void *fn, int sms)
 {
     int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg64_solve, CT, 0) != cudaSuccess || occ < 1) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, CT, 0) != cudaSuccess || occ < 1) return 0;
     return std::min(occ * sms, GR_BLOCKS);
 }
+
+static int blocks_for(const Grid &g, int blocks, long long items)
+{
+    const long long shares = narrow_grid(g, CX, CY) ? (g.N + CT - 1) / CT : items;
+    return (int)std::min<long long>(blocks, shares);
+}
+
+int cg64_solve_blocks(const Grid &g, int sms) { return solve_blocks((const void *)cg64_fn(g), sms); }
+int mixed_solve_blocks(const Grid &g, int sms) { return solve_blocks((const void *)mixed_fn(g), sms); }
 
 cudaError_t launch_cg64_solve(cudaStream_t s, int blocks, const Grid &g, const double *Tx, const double *Ty,
                               const double *Tz, const double *diag, const double *dinv, double *x, double *r,
@@ -287,16 +305,9 @@ cudaError_t launch_cg64_solve(cudaStream_t s, int blocks, const Grid &g, const d
 {
     Grid gg = g;
     Tiles tw = make_tiles_balanced(g, blocks, CX, CY);
-    blocks = (int)std::min<long long>(blocks, tw.items);
+    blocks = blocks_for(g, blocks, tw.items);
     void *args[] = {&gg, &tw, &Tx, &Ty, &Tz, &diag, &dinv, &x, &r, &z, &p0, &p1, &q, &red, &fault, &sc};
-    return cudaLaunchCooperativeKernel((void *)k_cg64_solve, dim3((unsigned)blocks), dim3(CT), args, 0, s);
-}
-
-int mixed_solve_blocks(const Grid &g, int sms)
-{
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_mixed_solve, CT, 0) != cudaSuccess || occ < 1) return 0;
-    return std::min(occ * sms, GR_BLOCKS);
+    return cudaLaunchCooperativeKernel((void *)cg64_fn(g), dim3((unsigned)blocks), dim3(CT), args, 0, s);
 }
 
 cudaError_t launch_mixed_solve(cudaStream_t s, int blocks, const Grid &g, const uint8_t *flags, const double *Tx,
@@ -334,9 +345,9 @@ cudaError_t launch_mixed_solve(cudaStream_t s, int blocks, const Grid &g, const 
     M.tol_inner = tol_inner;
     M.inner_max_it = inner_max_it;
     M.outer_max_it = outer_max_it;
-    blocks = (int)std::min<long long>(blocks, std::max(M.t64.items, M.t32.items));
+    blocks = blocks_for(g, blocks, std::max(M.t64.items, M.t32.items));
     void *args[] = {&M};
-    return cudaLaunchCooperativeKernel((void *)k_mixed_solve, dim3((unsigned)blocks), dim3(CT), args, 0, s);
+    return cudaLaunchCooperativeKernel((void *)mixed_fn(g), dim3((unsigned)blocks), dim3(CT), args, 0, s);
 }
 
 }  // namespace rf

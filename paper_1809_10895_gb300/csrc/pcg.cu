@@ -76,6 +76,7 @@ k_cg64_init(Grid g, const uint8_t *__restrict__ flags, const double *__restrict_
         cg64_start_scalars(sc, v, tol, max_it, cond);
 }
 
+template <bool NARROW>
 __global__ void __launch_bounds__(CT, SWEEP_OCC)
 k_cg64_spmv(Grid g, Tiles tw, const double *__restrict__ z, const double *__restrict__ p_in,
             double *__restrict__ p_out, double *__restrict__ q, const double *__restrict__ Tx,
@@ -93,15 +94,16 @@ k_cg64_spmv(Grid g, Tiles tw, const double *__restrict__ z, const double *__rest
     struct Raw {
         double z, o;
     };
-    sweep64<Raw, NoOwn>(
-        g, tw, A, s, [&](long long c) { return Raw{z[c], first ? 0.0 : p_in[c]}; },
-        [&](const Raw &a) { return fma(beta, a.o, a.z); },
-        [](long long) { return NoOwn{}; },
-        [&](long long c, double pv, double Ap, bool, NoOwn) {
-            p_out[c] = pv;
-            q[c] = Ap;
-            v[0] = fma(pv, Ap, v[0]);
-        });
+    auto load = [&](long long c) { return Raw{z[c], first ? 0.0 : p_in[c]}; };
+    auto mix = [&](const Raw &a) { return fma(beta, a.o, a.z); };
+    auto none = [](long long) { return NoOwn{}; };
+    auto out = [&](long long c, double pv, double Ap, bool, NoOwn) {
+        p_out[c] = pv;
+        q[c] = Ap;
+        v[0] = fma(pv, Ap, v[0]);
+    };
+    if (NARROW) cells64<NoOwn>(g, A, [&](long long c) { return mix(load(c)); }, none, out);
+    else sweep64<Raw, NoOwn>(g, tw, A, s, load, mix, none, out);
     if (grid_reduce<OpSum, 1>(v, partials, ticket) && threadIdx.x == 0) {
         sc->pq = v[0];
         const double a = sc->rho / v[0];
@@ -172,6 +174,7 @@ k_mixed_start(Grid g, const double *__restrict__ x0, double *__restrict__ x, CgS
 // norms (a stopping test and CG seeds) are summed from the FP32 residual in
 // FP32 within a block, in FP64 across blocks.  Counts outer iterations and
 // fails the solve after outer_max_it residuals without convergence.
+template <bool NARROW>
 __global__ void __launch_bounds__(CT, SWEEP_OCC)
 k_resid64(Grid g, Tiles tw, const uint8_t *__restrict__ flags, const double *__restrict__ x,
           const double *__restrict__ b, const double *__restrict__ Tx, const double *__restrict__ Ty,
@@ -193,7 +196,7 @@ k_resid64(Grid g, Tiles tw, const uint8_t *__restrict__ flags, const double *__r
     __shared__ Sweep64Shared s;
     const Op64 A{Tx, Ty, Tz, diag};
     float vf[3] = {0.0f, 0.0f, 0.0f};   // r32.r32, b.b, r32.z32
-    resid64_sweep(g, tw, A, s, flags, x, b, dinv32, r32, z32, d32, vf);
+    resid64_sweep<NARROW>(g, tw, A, s, flags, x, b, dinv32, r32, z32, d32, vf);
     double w[3];
     if (grid_reduce_f32<3>(vf, w, partials, ticket) && threadIdx.x == 0) {
         outer->iter += 1;
@@ -202,6 +205,7 @@ k_resid64(Grid g, Tiles tw, const uint8_t *__restrict__ flags, const double *__r
     }
 }
 
+template <bool NARROW>
 __global__ void __launch_bounds__(CT, SWEEP_OCC)
 k_cg32_spmv(Grid g, Tiles tw, const float *__restrict__ z, const float *__restrict__ p_in, float *__restrict__ p_out,
             float *__restrict__ q, const float *__restrict__ K32, const float *__restrict__ cb32, double *partials,
@@ -211,7 +215,10 @@ k_cg32_spmv(Grid g, Tiles tw, const float *__restrict__ z, const float *__restri
     if (sc->done) return;
     count_work(g, KK_CG32_SPMV);
     __shared__ Sweep32Shared s;
-    float vf[1] = {sweep32(g, tw, s, K32, cb32, z, p_in, p_out, q, (float)sc->beta, sc->iter == 0)};
+    const float beta = (float)sc->beta;
+    const bool first = sc->iter == 0;
+    float vf[1] = {NARROW ? cells32(g, K32, cb32, z, p_in, p_out, q, beta, first)
+                          : sweep32(g, tw, s, K32, cb32, z, p_in, p_out, q, beta, first)};
     double v[1];
     if (grid_reduce_f32<1>(vf, v, partials, ticket) && threadIdx.x == 0) {
         sc->pq = v[0];
@@ -482,9 +489,12 @@ void launch_cg64_init(cudaStream_t s, int nblk, const Grid &g, const uint8_t *fl
                                              ticket, sc, skip, cond);
 }
 
-// Tiles and blocks of a sweep as a launch of its own: two blocks an SM.
+// Tiles and blocks of a sweep as a launch of its own: two blocks an SM (cell by
+// cell: all that the reductions hold).
 static int sweep_tiles(const Grid &g, int nblk, int tile_y, Tiles &tw)
 {
+    tw = Tiles{};
+    if (narrow_grid(g, CX, CY)) return nblk;
     const int sms = std::max(1, (g.cap > nblk ? g.cap : nblk) / 8);   // the cap is eight blocks an SM
     tw = make_tiles_balanced(g, SWEEP_OCC * sms, CX, tile_y);
     return (int)std::min<long long>(tw.items, SWEEP_OCC * sms);
@@ -496,7 +506,8 @@ void launch_cg64_spmv(cudaStream_t s, int nblk, const Grid &g, const double *z, 
 {
     Tiles tw;
     const int nb = sweep_tiles(g, nblk, CY, tw);
-    k_cg64_spmv<<<nb, CT, 0, s>>>(g, tw, z, p_in, p_out, q, Tx, Ty, Tz, diag, partials, ticket, sc);
+    auto *fn = narrow_grid(g, CX, CY) ? k_cg64_spmv<true> : k_cg64_spmv<false>;
+    fn<<<nb, CT, 0, s>>>(g, tw, z, p_in, p_out, q, Tx, Ty, Tz, diag, partials, ticket, sc);
 }
 
 void launch_cg64_update(cudaStream_t s, int nblk, const Grid &g, double *x, double *r, double *z, const double *p,
@@ -526,8 +537,9 @@ void launch_resid64(cudaStream_t s, int nblk, const Grid &g, const uint8_t *flag
 {
     Tiles tw;
     const int nb = sweep_tiles(g, nblk, CY, tw);
-    k_resid64<<<nb, CT, 0, s>>>(g, tw, flags, x, b, Tx, Ty, Tz, diag, dinv32, r32, z32, d32, tol, tol_inner,
-                                inner_max_it, outer_max_it, partials, ticket, outer, inner, cond_outer, cond_inner);
+    auto *fn = narrow_grid(g, CX, CY) ? k_resid64<true> : k_resid64<false>;
+    fn<<<nb, CT, 0, s>>>(g, tw, flags, x, b, Tx, Ty, Tz, diag, dinv32, r32, z32, d32, tol, tol_inner, inner_max_it,
+                         outer_max_it, partials, ticket, outer, inner, cond_outer, cond_inner);
 }
 
 void launch_cg32_spmv(cudaStream_t s, int nblk, const Grid &g, const float *z, const float *p_in, float *p_out,
@@ -552,7 +564,8 @@ void launch_cg32_spmv(cudaStream_t s, int nblk, const Grid &g, const float *z, c
     }
     Tiles tw;
     const int nb = sweep_tiles(g, nblk, FY, tw);
-    k_cg32_spmv<<<nb, CT, 0, s>>>(g, tw, z, p_in, p_out, q, K32, cb32, partials, ticket, sc);
+    auto *fn = narrow_grid(g, CX, CY) ? k_cg32_spmv<true> : k_cg32_spmv<false>;
+    fn<<<nb, CT, 0, s>>>(g, tw, z, p_in, p_out, q, K32, cb32, partials, ticket, sc);
 }
 
 void launch_cg32_update(cudaStream_t s, int nblk, const Grid &g, float *x, float *r, float *z, const float *p,

@@ -173,6 +173,66 @@ __device__ __forceinline__ void sweep64(const Grid &g, const Tiles &tw, const Op
     }
 }
 
+// The same cell by cell, for grids that do not fill a tile (narrow_grid): values
+// of the neighbours are formed again, terms added in the same order.
+template <class Own, class Value, class LoadOwn, class Out>
+__device__ __forceinline__ void cells64(const Grid &g, const Op64 &A, Value value, LoadOwn own, Out out)
+{
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < g.N; c += stride) {
+        int i, j, k;
+        cell_ijk(g, c, i, j, k);
+        const Own e = own(c);
+        const double d = A.diag[c], v = value(c);
+        const bool act = __double_as_longlong(d) != 0;
+        double a = 0.0;
+        if (act) {
+            a = d * v;
+            if (i > 0) a = fma(-A.Tx[c - 1], value(c - 1), a);
+            if (i < g.nx - 1) a = fma(-A.Tx[c], value(c + 1), a);
+            if (j > 0) a = fma(-A.Ty[c - g.nx], value(c - g.nx), a);
+            if (j < g.ny - 1) a = fma(-A.Ty[c], value(c + g.nx), a);
+            if (k > 0) a = fma(-A.Tz[c - g.sxy], value(c - g.sxy), a);
+            if (k < g.nz - 1) a = fma(-A.Tz[c], value(c + g.sxy), a);
+        }
+        out(c, v, a, act, e);
+    }
+}
+
+// FP32 stencil product cell by cell (as sweep32).
+__device__ __forceinline__ float cells32(const Grid &g, const float *__restrict__ K32, const float *__restrict__ cb32,
+                                         const float *z, const float *pin, float *pout, float *q, float beta,
+                                         bool first)
+{
+    const float wx = g.w32[0] * 0.5f, wy = g.w32[1] * 0.5f, wz = g.w32[2] * 0.5f;
+    float acc = 0.0f;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < g.N; c += stride) {
+        int i, j, k;
+        cell_ijk(g, c, i, j, k);
+        const float K = K32[c];
+        auto value = [&](long long n) { return first ? z[n] : fmaf(beta, pin[n], z[n]); };
+        float v = 0.0f, a = 0.0f;
+        if (K >= 0.0f) {
+            v = value(c);
+            a = cb32[c] * v;
+            auto face = [&](bool in, long long n, float w) {
+                if (in) a = fmaf(fmaxf(w * (K + K32[n]), 0.0f), v - value(n), a);
+            };
+            face(i > 0, c - 1, wx);
+            face(i < g.nx - 1, c + 1, wx);
+            face(j > 0, c - g.nx, wy);
+            face(j < g.ny - 1, c + g.nx, wy);
+            face(k > 0, c - g.sxy, wz);
+            face(k < g.nz - 1, c + g.sxy, wz);
+        }
+        pout[c] = v;
+        q[c] = a;
+        acc = fmaf(v, a, acc);
+    }
+    return acc;
+}
+
 // FP32 stencil product over this block's items: p = z + beta p_old, q = A p;
 // returns this thread's p.q.
 __device__ __forceinline__ float sweep32(const Grid &g, const Tiles &tw, Sweep32Shared &s, const float *__restrict__ K32,
@@ -374,6 +434,7 @@ __device__ __forceinline__ void cg32_update_cells(const Grid &g, float alpha, bo
 // where they are used, behind the plane's barrier, they cost a memory latency
 // a plane (384 x 320 x 64 cells, 6.1 M active: 238.6 -> 180.6 us; its 8 FP64
 // instructions a cell alone take 78).
+template <bool NARROW>
 __device__ __forceinline__ void resid64_sweep(const Grid &g, const Tiles &tw, const Op64 &A, Sweep64Shared &s,
                                               const uint8_t *__restrict__ flags, const double *x,
                                               const double *__restrict__ b, const float *__restrict__ dinv32,
@@ -387,26 +448,27 @@ __device__ __forceinline__ void resid64_sweep(const Grid &g, const Tiles &tw, co
         double b;
         float di;
     };
-    sweep64<Raw, Own>(
-        g, tw, A, s, [&](long long c) { return Raw{x[c], flags[c]}; },
-        // an inactive cell's head may be anything; its faces' T = 0 needs a number
-        [&](const Raw &a) { return (a.fl & FLAG_ACTIVE) ? a.x : 0.0; },
-        [&](long long c) { return Own{__ldcs(&b[c]), __ldcs(&dinv32[c])}; },
-        [&](long long c, double, double Ax, bool act, const Own &e) {
-            float rf = 0.0f, zf = 0.0f;
-            if (act) {
-                const double rp = e.b - Ax;
-                const float bf = ix_d2f(e.b);
-                rf = ix_d2f(rp);
-                zf = e.di * rf;
-                v[0] = fmaf(rf, rf, v[0]);
-                v[1] = fmaf(bf, bf, v[1]);
-                v[2] = fmaf(rf, zf, v[2]);
-            }
-            r32[c] = rf;
-            z32[c] = zf;
-            if (d32) d32[c] = 0.0f;
-        });
+    auto own = [&](long long c) { return Own{__ldcs(&b[c]), __ldcs(&dinv32[c])}; };
+    // an inactive cell's head may be anything; its faces' T = 0 needs a number
+    auto mix = [&](const Raw &a) { return (a.fl & FLAG_ACTIVE) ? a.x : 0.0; };
+    auto load = [&](long long c) { return Raw{x[c], flags[c]}; };
+    auto out = [&](long long c, double, double Ax, bool act, const Own &e) {
+        float rf = 0.0f, zf = 0.0f;
+        if (act) {
+            const double rp = e.b - Ax;
+            const float bf = ix_d2f(e.b);
+            rf = ix_d2f(rp);
+            zf = e.di * rf;
+            v[0] = fmaf(rf, rf, v[0]);
+            v[1] = fmaf(bf, bf, v[1]);
+            v[2] = fmaf(rf, zf, v[2]);
+        }
+        r32[c] = rf;
+        z32[c] = zf;
+        if (d32) d32[c] = 0.0f;
+    };
+    if (NARROW) cells64<Own>(g, A, [&](long long c) { return mix(load(c)); }, own, out);
+    else sweep64<Raw, Own>(g, tw, A, s, load, mix, own, out);
 }
 
 #endif

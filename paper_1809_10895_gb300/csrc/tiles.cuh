@@ -69,6 +69,18 @@ inline Tiles make_tiles_balanced(const Grid &g, int resident, int tile_x, int ti
     return t;
 }
 
+// Whether a plane of the grid leaves more than three quarters of its tiles
+// empty: columns and vertical sections, which a walk plane by plane serves with
+// a few threads; they run cell by cell.  us a CG iteration, 600 000 cells, tiled /
+// cell by cell: FP64 1 x 1 x 600000 2009 / 23, 600 x 1 x 1000 107 / 26, 600 x 4 x 250
+// 42 / 30, 16 x 16 x 2500 39 / 32, 64 x 64 x 150 28 / 30; mixed 1515 / 16, 60 / 18,
+// 26 / 21, 19 / 19, 13 / 20.
+inline bool narrow_grid(const Grid &g, int tile_x, int tile_y)
+{
+    const long long tiles = (long long)((g.nx + tile_x - 1) / tile_x) * ((g.ny + tile_y - 1) / tile_y);
+    return 4 * g.sxy < tiles * tile_x * tile_y;
+}
+
 inline int tile_blocks(const Tiles &t, const Grid &g, int nblk)
 {
     return (int)std::min<long long>(t.items, g.cap > nblk ? g.cap : nblk);
