@@ -684,12 +684,20 @@ void launch_closure_picard(cudaStream_t s, int nblk, const Grid &g, const DevSoi
                                     cg_count, cond);
 }
 
-// Tiles wherever they fill: at least half a tile's row, and enough cells that
-// marching through planes beats one cell per thread (below, every launch is
-// latency and the general kernel's one cell per thread is the shorter chain).
+// Tiles where the planes fill them and there are enough cells that marching
+// through planes beats one cell per thread (below, every launch is latency and
+// the general kernel's one cell per thread is the shorter chain).  us, tiled / one
+// cell per thread, alone (fused with the first residual the tiled form gains
+// some 30 us more on 600 000 cells): 256 x 256 x 64 199 / 267, 128 x 128 x 64 61 /
+// 72, 45 x 45 x 60 (0.66 of the tiles filled) 19 / 16, 33 x 33 x 500 (0.43) 66 / 39,
+// 16 x 4 x 10000 (0.25) 95 / 44; steps of 600 000 cells: 0.75 filled 23.2 / 23.4 ms,
+// 0.62 30.7 / 30.8, 0.5 equal, 0.43 25.6 / 25.5.  The harmonic mean divides in FP64
+// for every face, each twice in a tile's walk but for the vertical ones: 0.75
+// filled 152 / 120, 0.94 185 / 170, full 107 / 113 (642 000 cells).
 static bool assemble_tiled(const Grid &g)
 {
-    return g.nx >= 16 && g.ny >= 4 && g.N >= 32768;
+    const long long area = (long long)((g.nx + TX - 1) / TX) * TX * ((g.ny + TY - 1) / TY) * TY;
+    return g.N >= 32768 && (g.harmonic ? 16 * g.sxy > 15 * area : 8 * g.sxy >= 5 * area);
 }
 
 void launch_assemble(cudaStream_t s, int nblk, const Grid &g, const DevSoil *soils, const uint8_t *zone,
