@@ -740,7 +740,7 @@ k_ensemble(EnsDesc *__restrict__ D, int n_inst, EnsBuffers B, EnsParams P, const
                         CellSystem cs;
                         assemble_cell<true>(g, soil, zn, Ks, fl[p], sp, p, i, j, k, hk, hn, TH[tn ^ 1], TH[tn],
                                             KB[kin], Can, nullptr, P.eps_chord, V_dt, cs);
-                        const double di = ix_rcp64(cs.diag);
+                        const double di = PREC == 0 || !P.zline ? ix_rcp64(cs.diag) : 0.0;   // unread with the line solve
                         cc[p] = cs.c;
                         bb[p] = cs.rhs;
                         Tx[p] = cs.Tup[0];
