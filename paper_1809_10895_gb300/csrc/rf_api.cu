@@ -311,10 +311,12 @@ rf_status cap_end(rf_ctx *c, std::vector<cudaGraphNode_t> &leaves)
     cudaStreamCaptureStatus st;
     const cudaGraphNode_t *d = nullptr;
     size_t n = 0;
-    CUDA_TRY(cudaStreamGetCaptureInfo(c->cap, &st, nullptr, nullptr, &d, nullptr, &n));
-    leaves.assign(d, d + n);
+    const cudaError_t e = cudaStreamGetCaptureInfo(c->cap, &st, nullptr, nullptr, &d, nullptr, &n);
+    if (e == cudaSuccess) leaves.assign(d, d + n);
     cudaGraph_t out;
-    CUDA_TRY(cudaStreamEndCapture(c->cap, &out));
+    const cudaError_t e_end = cudaStreamEndCapture(c->cap, &out);   // also of a capture that a launch invalidated
+    CUDA_TRY(e);
+    CUDA_TRY(e_end);
     CUDA_TRY(cudaGetLastError());
     return RF_OK;
 }
